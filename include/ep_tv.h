@@ -321,11 +321,11 @@ ep_tv_status ep_tv_trace_read(ep_tv_ctx* ctx, int32_t kernel, double* ms, int64_
    not allocate after start-up, or runs inside an allocator or host runtime that
    owns the device memory and only hands out the buffers it was asked for.  The
    caller passes every input and output; the scratch the pass needs (one FP64
-   partial sum of E|u| per work unit of 16 row pairs of a 60-column strip, a
+   partial sum of E|u| per work unit of up to 16 row pairs of a 60-column strip, a
    status word, counters) lives in a file-scope device array of 65536 + 8 doubles
    (512 KB) that every GPU loading the library holds until the process exits.
-     height, width  image size; its ceil(width / 60) * ceil(((height + 1) / 2 + 1) / 16)
-                    work units (about 126 M pixels at most) must not exceed 65536, and
+     height, width  image size; ceil(width / 60) * ceil(((height + 1) / 2 + 1) / 16)
+                    (about 126 M pixels at most) must not exceed 65536, and
                     height * width must not exceed 2^31, else EP_TV_ERR_ARG.
      p              uses damping, var_cap, periodic, precision (0 or 1), the prior and
                     its omega, s1_sq, s2_sq, and xi when y is given.

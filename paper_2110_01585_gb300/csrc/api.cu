@@ -862,7 +862,7 @@ struct ep_tv_batch {
   BatchItem* h_items[2] = {nullptr, nullptr};
   cudaEvent_t items_ev[2] = {nullptr, nullptr};
   int slot = 0;
-  long long total_units = 0;             // prior-sweep work units of all images
+  long long total_steps = 0;             // prior-sweep row-pair steps of all images
   std::vector<int> lik;                 // contexts with a likelihood state
   std::vector<cudaStream_t> wstream;    // one worker stream per such context
   std::vector<cudaEvent_t> wdone;
@@ -886,7 +886,7 @@ namespace {
 
 // Image table of a sweep with every context's prior buffers at parity cur ^ flip.
 void fill_items(ep_tv_batch* b, BatchItem* h, int flip) {
-  long long unit = 0;
+  long long step = 0;
   for (size_t i = 0; i < b->ctx.size(); ++i) {
     ep_tv_ctx* c = b->ctx[i];
     h[i].a = sweep_args(c, 0x4321);
@@ -899,9 +899,10 @@ void fill_items(ep_tv_batch* b, BatchItem* h, int flip) {
     prior_sweep_prepare(h[i].a);
     h[i].site0_from_y = site0_from_y(c);
     h[i].units = prior_sweep_blocks(c->height, c->width);
-    h[i].unit_begin = unit;
-    unit += h[i].units;
+    h[i].step_begin = step;
+    step += h[i].units << h[i].a.unit_shift;
   }
+  b->total_steps = step;
 }
 
 // Graph of `period` batch sweeps from the contexts' current parities (captured on
@@ -937,7 +938,7 @@ cudaGraphExec_t batch_graph(ep_tv_batch* b, int period, int em_every) {
     return nullptr;
   }
   for (int t = 0; t < period; ++t) {
-    launch_prior_sweep_batch(b->g_items[t & 1], (int)n, b->total_units, b->stream);
+    launch_prior_sweep_batch(b->g_items[t & 1], (int)n, b->total_steps, b->stream);
     if (em_every > 0 && (t + 1) % em_every == 0)
       for (ep_tv_ctx* c : b->ctx) {
         const int cur = c->cur ^ ((t + 1) & 1);  // the contexts' parity after sweep t
@@ -1023,7 +1024,6 @@ ep_tv_status ep_tv_batch_create(int32_t n, ep_tv_ctx* const* ctxs, ep_tv_batch**
   b->stream = ctxs[0]->stream;
   b->device = ctxs[0]->device;
   for (int i = 0; i < n; ++i) {
-    b->total_units += prior_sweep_blocks(ctxs[i]->height, ctxs[i]->width);
     if (ctxs[i]->lik) b->lik.push_back(i);
   }
   bool ok = true;
@@ -1089,7 +1089,7 @@ ep_tv_status ep_tv_batch_sweep(ep_tv_batch* b, int32_t n_sweeps, int32_t em_ever
     CK(cudaMemcpyAsync(b->d_items[b->slot], h, sizeof(BatchItem) * n, cudaMemcpyHostToDevice,
                        b->stream));
     CK(cudaEventRecord(b->items_ev[b->slot], b->stream));
-    launch_prior_sweep_batch(b->d_items[b->slot], n, b->total_units, b->stream);
+    launch_prior_sweep_batch(b->d_items[b->slot], n, b->total_steps, b->stream);
     b->slot ^= 1;
     for (ep_tv_ctx* c : b->ctx) {
       c->cur ^= 1;

@@ -115,6 +115,7 @@ struct SweepArgs {
   float mix_v1, mix_v2;       // MoG2 / BG: component variances (BG: v2 = 0, the point mass)
   double* abar_partial;       // one FP64 partial sum of E|u| per work unit
   int vec2;                   // set by prior_sweep_prepare: float2 loads and stores allowed
+  int unit_shift;             // set by prior_sweep_prepare: log2 of the row-pair steps per unit
   unsigned* status;
   unsigned long long* counters;
 };
@@ -124,7 +125,7 @@ struct BatchItem {
   SweepArgs a;
   int site0_from_y;
   long long units;        // work units of this image
-  long long unit_begin;   // first unit of this image in the launch
+  long long step_begin;   // first step of this image in the launch (units << unit_shift each)
 };
 
 // Whether the prior fields of p are valid, and their copy into the sweep arguments.
@@ -138,11 +139,11 @@ double prior_sweep_bytes_per_pixel(bool site0_from_y);
 // Runs the per-device set-up of the prior-pass launchers (occupancy queries and
 // attributes) so that a later launch inside a stream capture makes no such calls.
 void prior_sweep_prewarm();
-// Fills the fields of `a` that the launch derives (vector access).
+// Fills the fields of `a` that the launch derives (vector access, unit length).
 void prior_sweep_prepare(SweepArgs& a);
 // Work units (and E|u| partial sums) of one image's prior-site pass.
 int prior_sweep_blocks(int height, int width);
-void launch_prior_sweep_batch(const BatchItem* items, int n_items, long long total_units,
+void launch_prior_sweep_batch(const BatchItem* items, int n_items, long long total_steps,
                               cudaStream_t s);
 
 // abar = sum(partials) in a fixed order; if do_em, beta = n / abar.

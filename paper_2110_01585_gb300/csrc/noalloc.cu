@@ -25,8 +25,9 @@
 namespace eptv {
 namespace {
 
-// One work unit is 16 row pairs of a 60-column strip, so 65536 units hold images
-// of up to about 65536 * 32 * 60 = 126 M pixels.
+// Large images are cut into units of 16 row pairs of a 60-column strip, so 65536 units
+// hold images of up to about 65536 * 32 * 60 = 126 M pixels.  Shorter units are taken
+// only by images of fewer than 7296 of those, which have fewer than 2 * 7296 units.
 constexpr int kNoAllocMaxBlocks = 65536;
 constexpr int kNoAllocDoubles = kNoAllocMaxBlocks + 8;
 constexpr int kMaxDevices = 64;
@@ -82,12 +83,12 @@ extern "C" ep_tv_status ep_tv_prior_sweep_noalloc(int32_t height, int32_t width,
   if (!(p->damping > 0.0 && p->damping <= 1.0) || !(p->var_cap > 0.0)) return EP_TV_ERR_ARG;
   if (y && !(p->xi > 0.0)) return EP_TV_ERR_ARG;
   if (tau_in == tau_out || nu_in == nu_out) return EP_TV_ERR_ARG;
-  // Work units in 64-bit: ceil(width / 60) * ceil(((height + 1) / 2 + 1) / 16), the
-  // count prior_sweep_blocks returns, without its int overflow for huge sizes.
+  // Units of 16 row pairs in 64-bit: ceil(width / 60) * ceil(((height + 1) / 2 + 1) / 16),
+  // without the int overflow of prior_sweep_blocks for huge sizes.
   const long long units = ((long long)width + 59) / 60 * ((((long long)height + 1) / 2 + 1 + 15) / 16);
   if (units > kNoAllocMaxBlocks) return EP_TV_ERR_ARG;  // image larger than the fixed scratch
   const int nblk = prior_sweep_blocks(height, width);
-  if (nblk != units) return EP_TV_ERR_ARG;
+  if (nblk > kNoAllocMaxBlocks) return EP_TV_ERR_ARG;
   int order = 0x4321;
   if (k_order) {
     int seen = 0;

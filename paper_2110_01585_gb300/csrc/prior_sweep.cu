@@ -25,11 +25,11 @@
 // staging slots for the next row pair, the parked carried row and a copy of the
 // loop's arguments: 12.9 KB per warp); there is no block barrier.
 //
-// Work units are 16 row pairs of one strip.  A persistent grid of warps takes
-// contiguous ranges of units (images of a batch laid end to end), so one launch
-// serves any number of images.  The E|u| sum of each unit is reduced in FP64 in
-// a fixed order and stored in its own slot, which makes the result independent
-// of how units are spread over warps.
+// Work units are 1, 2, 4, 8 or 16 row pairs of one strip, by the size of the image
+// (unit_shift).  A persistent grid of warps takes contiguous ranges of units
+// (images of a batch laid end to end), so one launch serves any number of images.
+// The E|u| sum of each unit is reduced in FP64 in a fixed order and stored in its
+// own slot, which makes the result independent of how units are spread over warps.
 //
 // Arithmetic: FP32 with the cancellation-free forms below; the new precision
 // uses tau_i = rho / (c_j + q c_i), which equals 1/Var_i - 1/c_i of Eq. update_qk_x
@@ -47,7 +47,8 @@ namespace eptv {
 namespace {
 
 constexpr int kStripCols = 60;     // owned columns per warp (lanes 1..30, two each)
-constexpr int kStepsPerUnit = 16;  // row-pair steps per work unit
+constexpr int kMaxUnitShift = 4;   // at most 16 row-pair steps per work unit
+constexpr long long kWantUnits = 4 * 1824;  // units a whole image is cut into, if it has them
 constexpr int kWarpsPerBlock = 4;
 constexpr int kThreads = 32 * kWarpsPerBlock;
 constexpr int kMinBlocks = 3;      // blocks per SM the register budget is sized for
@@ -465,6 +466,7 @@ struct __align__(16) Io {
   int height, width;
   bool periodic, vec2;  // periodic: the rows wrap (columns: SweepArgs::periodic)
   float inv_xi;
+  int unit_shift;
 };
 
 static_assert(sizeof(Io) <= kIoBytes, "argument copy exceeds its shared-memory slot");
@@ -483,6 +485,7 @@ __device__ __forceinline__ Io make_io(const SweepArgs& a, bool site0_from_y) {
   io.periodic = a.periodic_rows != 0;
   io.vec2 = a.vec2 != 0;
   io.inv_xi = a.inv_xi;
+  io.unit_shift = a.unit_shift;
   return io;
 }
 
@@ -688,8 +691,8 @@ __device__ __forceinline__ void load_saved_row(const float2* src, bool ok, Row& 
 // the later vertical update of the order, 1 when V3 is); one spare step covers
 // both offsets and odd heights.
 __host__ __device__ __forceinline__ int steps_of(int height) { return (height + 1) / 2 + 1; }
-__host__ __device__ __forceinline__ int units_per_strip(int height) {
-  return (steps_of(height) + kStepsPerUnit - 1) / kStepsPerUnit;
+__host__ __device__ __forceinline__ int units_per_strip(int height, int shift) {
+  return (steps_of(height) + (1 << shift) - 1) >> shift;
 }
 __host__ __device__ __forceinline__ int strips_of(int width) {
   return (width + kStripCols - 1) / kStripCols;
@@ -713,7 +716,7 @@ __device__ __noinline__ void run_strip(const SweepArgs& a, int strip, int b_lo, 
                                        long long unit_base, float2* stage) {
   constexpr int kI = 7 - kX;
   constexpr int kOff = kX == 4 ? 0 : 1;
-  const int W = a.width, H = a.height;
+  const int W = a.width;
   Lane L;
   L.lane = threadIdx.x & 31;
   const int gc0 = strip * kStripCols - 2 + 2 * L.lane;  // unwrapped column of the left pixel
@@ -832,8 +835,9 @@ __device__ __noinline__ void run_strip(const SweepArgs& a, int strip, int b_lo, 
     if (!warm) {
       store_row(io, c, L, gcol, row0 - 1, carry);
       store_row(io, c, L, gcol, row0, r0);
-      if ((b + 1) % kStepsPerUnit == 0 || b + 1 == b_hi) {
-        flush_unit(abar_partial, c.eab, unit_base + b / kStepsPerUnit);
+      const int shift = io.unit_shift, next = b + 1;
+      if ((next >> shift) << shift == next || next == b_hi) {
+        flush_unit(abar_partial, c.eab, unit_base + (b >> shift));
         c.eab = 0.0f;
       }
     }
@@ -856,7 +860,8 @@ __host__ __device__ __forceinline__ int later_vertical(int order) {
 // Units [u_lo, u_hi) of one image (strip-major: unit = strip * units_per_strip + block).
 template <bool kSite0FromY, int kX, int kEdge>
 __device__ void run_units(const SweepArgs& a, long long u_lo, long long u_hi, float2* stage) {
-  const int ups = units_per_strip(a.height);
+  const int shift = a.unit_shift;
+  const int ups = units_per_strip(a.height, shift);
   const int nsteps = steps_of(a.height);
   long long u = u_lo;
   while (u < u_hi) {
@@ -864,7 +869,7 @@ __device__ void run_units(const SweepArgs& a, long long u_lo, long long u_hi, fl
     const long long strip_end = (long long)(strip + 1) * ups;
     const long long e = u_hi < strip_end ? u_hi : strip_end;
     const int k_lo = (int)(u - (long long)strip * ups), k_hi = (int)(e - (long long)strip * ups);
-    run_strip<kSite0FromY, kX, kEdge>(a, strip, k_lo * kStepsPerUnit, min(k_hi * kStepsPerUnit, nsteps),
+    run_strip<kSite0FromY, kX, kEdge>(a, strip, k_lo << shift, min(k_hi << shift, nsteps),
                                (long long)strip * ups, stage);
     u = e;
   }
@@ -901,13 +906,15 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) prior_sweep_kernel(Sweep
   const int w = global_warp();
   if (w >= S * n_seg) return;
   const int strip = w % S, seg = w / S;
-  const long long ups = units_per_strip(a.height);
+  const long long ups = units_per_strip(a.height, a.unit_shift);
   const long long lo = ups * seg / n_seg, hi = ups * (seg + 1) / n_seg;
   if (lo < hi) run_units<kSite0FromY, kX, kEdge>(a, strip * ups + lo, strip * ups + hi, warp_stage());
 }
 
-// Many images in one launch; units of image i start at items[i].unit_begin and
-// warp w of n_warps takes units [U w / n_warps, U (w + 1) / n_warps).
+// Many images in one launch.  Images are laid end to end in units of one row-pair
+// step (a unit of image i counts 1 << unit_shift of them, so that images cut into
+// longer units weigh more); warp w of n_warps takes the units whose first step is in
+// [T w / n_warps, T (w + 1) / n_warps), T the total.
 __global__ void __launch_bounds__(kThreads, kMinBlocks) prior_sweep_batch_kernel(const BatchItem* items,
                                                                      int n_items, long long total,
                                                                      int n_warps) {
@@ -918,17 +925,20 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) prior_sweep_batch_kernel
   int it = 0, top = n_items - 1;
   while (it < top) {  // last image whose first unit is <= lo
     const int mid = (it + top + 1) >> 1;
-    if (items[mid].unit_begin <= lo) it = mid; else top = mid - 1;
+    if (items[mid].step_begin <= lo) it = mid; else top = mid - 1;
   }
   long long u = lo;
   while (u < hi && it < n_items) {
     const BatchItem& b = items[it];
-    const long long end = b.unit_begin + b.units;
+    const int shift = b.a.unit_shift;
+    const long long up = (1ll << shift) - 1;  // a unit belongs to the range of its first step
+    const long long end = b.step_begin + (b.units << shift);
     const long long e = hi < end ? hi : end;
     if (e > u) {
       const int kind = edge_kind(b.a);
-      const long long ulo = u - b.unit_begin, uhi = e - b.unit_begin;
-      if (b.site0_from_y) {
+      const long long ulo = (u - b.step_begin + up) >> shift, uhi = (e - b.step_begin + up) >> shift;
+      if (ulo >= uhi) {
+      } else if (b.site0_from_y) {
         if (kind == kEdgeMix) run_units_any<true, kEdgeMix>(b.a, ulo, uhi, warp_stage());
         else if (kind == kEdgeL1Q) run_units_any<true, kEdgeL1Q>(b.a, ulo, uhi, warp_stage());
         else run_units_any<true, kEdgeL1>(b.a, ulo, uhi, warp_stage());
@@ -947,7 +957,17 @@ __global__ void abar_reduce_kernel(const double* partial, int n, double* dscal, 
                                    int do_em) {
   __shared__ double buf[1024];
   double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s += partial[i];
+  // one block: the latency of its loads is the whole time, so eight are in flight
+  for (int i0 = threadIdx.x; i0 < n; i0 += 8 * blockDim.x) {
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int i = i0 + k * blockDim.x;
+      v[k] = i < n ? partial[i] : 0.0;
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s += v[k];
+  }
   buf[threadIdx.x] = s;
   __syncthreads();
   for (int w = blockDim.x / 2; w > 0; w >>= 1) {
@@ -996,11 +1016,15 @@ void launch_single(const SweepArgs& a, cudaStream_t s) {
   // occupancy cache slot of this instantiation: 0..3 and 5..12 (4 is the batch kernel's)
   const int slot = kEdge * 4 + (kSite0FromY ? 0 : 2) + (kX == 4 ? 0 : 1) + (kEdge ? 1 : 0);
   const int S = strips_of(a.width);
-  const int ups = units_per_strip(a.height);
+  const int ups = units_per_strip(a.height, a.unit_shift);
   const int resident = resident_warps(prior_sweep_kernel<kSite0FromY, kX, kEdge>, slot);
   int n_seg = resident / S;
   if (n_seg < 1) n_seg = 1;
   if (n_seg > ups) n_seg = ups;
+  // the longest range is ceil(ups / n_seg) units: no more ranges than that length needs
+  // (each costs a warm-up step and a warp's share of its SM)
+  const int per_seg = (ups + n_seg - 1) / n_seg;
+  n_seg = (ups + per_seg - 1) / per_seg;
   const int blocks = (S * n_seg + kWarpsPerBlock - 1) / kWarpsPerBlock;
   prior_sweep_kernel<kSite0FromY, kX, kEdge><<<blocks, kThreads, kSmemBytes, s>>>(a, n_seg);
 }
@@ -1021,14 +1045,31 @@ double prior_sweep_bytes_per_pixel(bool site0_from_y) {
   return site0_from_y ? (9 + 8) * 4.0 : (10 + 8) * 4.0;
 }
 
+// Row-pair steps per work unit, as a power of two: the longest unit (16 steps at most)
+// that still cuts the image into kWantUnits units, four per warp the GPU holds
+// (152 SMs x 12 warps), so that the warps' ranges differ by a quarter at most; small
+// images come down to units of one step.  A warp runs its steps one after another
+// (about 2.4 us each while few warps are resident, 3.7 us with twelve per SM), and a range
+// of any length starts with one warm-up step.  By size only, so that an image's E|u|
+// sums do not depend on the device or on the batch it is in.  With units of 16 steps
+// always, a 64^2 to 1024^2 sweep took 41-42 us, one warp's 17 steps; now 8.3 us at 64^2
+// and 15 us at 512^2.  Eight units per warp made 4096^2 1.3% slower (units of 8 steps,
+// whose FP64 sums cost more than the finer ranges gave).
+static int unit_shift(int height, int width) {
+  int shift = kMaxUnitShift;
+  while (shift > 0 && (long long)strips_of(width) * units_per_strip(height, shift) < kWantUnits) --shift;
+  return shift;
+}
+
 void prior_sweep_prepare(SweepArgs& a) {
+  a.unit_shift = unit_shift(a.height, a.width);
   auto al = [](const void* p) { return ((uintptr_t)p & 7) == 0; };
   a.vec2 = (a.width % 2 == 0) && al(a.tau0) && al(a.nu0) && al(a.tin) && al(a.nin) && al(a.tout) &&
            al(a.nout) && al(a.y);
 }
 
 int prior_sweep_blocks(int height, int width) {
-  return strips_of(width) * units_per_strip(height);
+  return strips_of(width) * units_per_strip(height, unit_shift(height, width));
 }
 
 void prior_sweep_prewarm() {
@@ -1047,11 +1088,11 @@ void prior_sweep_prewarm() {
   resident_warps(prior_sweep_kernel<false, 3, kEdgeMix>, 12);
 }
 
-void launch_prior_sweep_batch(const BatchItem* items, int n_items, long long total_units,
+void launch_prior_sweep_batch(const BatchItem* items, int n_items, long long total_steps,
                               cudaStream_t s) {
   int n_warps, blocks;
-  launch_units(total_units, resident_warps(prior_sweep_batch_kernel, 4), n_warps, blocks);
-  prior_sweep_batch_kernel<<<blocks, kThreads, kSmemBytes, s>>>(items, n_items, total_units, n_warps);
+  launch_units(total_steps, resident_warps(prior_sweep_batch_kernel, 4), n_warps, blocks);
+  prior_sweep_batch_kernel<<<blocks, kThreads, kSmemBytes, s>>>(items, n_items, total_steps, n_warps);
 }
 
 void launch_prior_sweep(const SweepArgs& args, bool site0_from_y, cudaStream_t s) {

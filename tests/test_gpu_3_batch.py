@@ -73,3 +73,33 @@ def test_batch_denoise_matches_oracle():
         mu, var = (t.cpu().numpy() for t in e.posterior())
         assert_parity(mu, var, *o.posterior(), p.y)
         e.close()
+
+
+@pytest.mark.parametrize("h,w", [(2, 2), (3, 61), (66, 120), (30000, 62)])
+def test_unit_lengths_batch_and_statistic(h, w):
+    """Work units of one row-pair step (the small sizes) and of four (30000 x 62): an
+    image swept in a batch with one of another unit length gives the bits of the image
+    alone, and a_u, whose partial sums are one per unit, is the oracle's (FP32 terms of
+    relative error below 1e-6 summed in FP32 per lane and unit, then in FP64)."""
+    torch = cuda()
+    stream = torch.cuda.Stream()
+    periodic = int(h % 2 == 0 and w % 2 == 0)
+    p = syn.denoise_problem(h, w, sigma=0.1, beta=4.0, seed=h + w)
+    q = syn.denoise_problem(96, 64, sigma=0.1, beta=4.0, seed=8)
+    kw = {"periodic": periodic}
+    single = [_make(torch, "denoise", p, kw, stream), _make(torch, "denoise", q, {}, stream)]
+    batched = [_make(torch, "denoise", p, kw, stream), _make(torch, "denoise", q, {}, stream)]
+    for e in single:
+        e.sweep(1)
+    with Batch(batched[::-1]) as b:
+        b.sweep(1)
+    for e1, e2 in zip(single, batched):
+        assert e1.em_beta() == e2.em_beta()
+        for a1, a2 in zip(e1.sites(), e2.sites()):
+            torch.cuda.synchronize()
+            assert torch.equal(a1, a2)
+    o = EPOracle("denoise", p.y.astype(np.float32), p.xi, p.beta, h, w, periodic=bool(periodic))
+    o.run(1)
+    assert abs(single[0].em_beta()[1] / o.abar - 1.0) < 2e-6
+    for e in single + batched:
+        e.close()

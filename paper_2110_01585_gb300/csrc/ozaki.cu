@@ -6,7 +6,7 @@
 // Splitting (Ozaki's error-free splitting of a product into exact slice
 // products).  Every operand row r is scaled by 2^-e_r, e_r the binary exponent
 // of its largest entry, so that every scaled entry x lies in (-1, 1).  x is then
-// written as eight 7-bit digits by round-to-nearest,
+// written as eight 7-bit digits by rounding to the nearest multiple of 2^-56,
 //   x = sum_{s=1..8} d_s 2^{-7 s} + rho,   |d_1| <= 128, |d_s| <= 64 (s > 1), |rho| <= 2^-57,
 // each step exact in FP64.  The slice d_s 2^{-7 s} has at most 8 significant bits, so
 // it is exact in BF16, and the product of two slices is exact in FP32.  For a
@@ -30,8 +30,8 @@
 // Kernel: one CTA per 128 x 64 output tile; K in stages of 16 (one MMA K step),
 // four shared-memory stages filled by bulk asynchronous copies (cp.async.bulk,
 // the TMA engine) from operands packed in the tensor core's shared-memory
-// core-matrix order, so that a stage is two contiguous copies (A: 128 rows, B:
-// 64 rows, 8 slices each).  Warp-specialised: one thread issues the copies and
+// core-matrix order, so that a stage is three contiguous copies of 64 rows (two for
+// A, one for B, 8 slices each).  Warp-specialised: one thread issues the copies and
 // waits only for stages to free up, one thread issues the 36 MMAs of a stage
 // (M = 128, N = 64, K = 16, BF16 inputs, FP32 accumulators in tensor memory) and
 // waits only for stages to land, and sixteen warps read the accumulators back
@@ -59,8 +59,7 @@ constexpr int kTM = 128;             // output tile rows; packing row tile
 constexpr int kTN = 64;              // output tile columns
 constexpr int kKS = 16;              // K per stage (one MMA K step)
 constexpr int kCore = 128;           // one core matrix: 8 rows x 16 bytes
-constexpr int kSliceKc = kTM / 8 * kCore;               // 16 row groups: 2048 bytes
-constexpr int kSliceKcB = kTN / 8 * kCore;              // 8 row groups: 1024 bytes
+constexpr int kSliceStep = 2 * kCore;  // from one slice of an 8-row group to the next
 constexpr int kTmemCols = 512;  // the accumulators (at most 7 of 64 columns), rounded up
 
 // Shapes that depend on the number of digit slices S (8 for the operator
@@ -78,8 +77,9 @@ struct Split {
   static constexpr int kExact = S <= 8 ? 5 : 7;
   static constexpr int kChunkStages = S <= 8 ? 16 : 8;
   static_assert(kTN * (kExact + 1) <= kTmemCols, "tensor memory");
-  static constexpr int kAStage = S * 2 * kSliceKc;
-  static constexpr int kBStage = S * 2 * kSliceKcB;
+  static constexpr int kGroup = S * kSliceStep;         // 8 rows, all slices
+  static constexpr int kAStage = kTM / 8 * kGroup;
+  static constexpr int kBStage = kTN / 8 * kGroup;
   static constexpr int kStageBytes = kAStage + kBStage;
   static constexpr int kStages = S <= 8 ? 4 : 3;
   // the stages, 8 KB of slack past the last stage (so that every descriptor
@@ -195,104 +195,207 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
 }
 
 // ---- packing
+//
+// GB300 retires about two FP64 operations per clock and SM, so the splitting is done
+// on the bit fields of the operands with integer instructions.  With the digits formed
+// by FP64 multiplies and rounding (about 40 FP64 operations per entry, a pass for the
+// exponents and another packing for the other side of a symmetric product), packing took
+// as long as the tensor-core work of all but the largest products; now a pack takes 6 us
+// on average over the factorisation of 1228 rows.
 
-// Operand entry X(r, k) = X[r * ld + k] (X[k * ld + r] when trans), times ks[k]
-// when a k scale is given.
-template <typename T>
-__device__ __forceinline__ double entry(const T* X, long long ld, int trans, const double* ks, int r, int k) {
-  const double x = (double)(trans ? X[(long long)k * ld + r] : X[(long long)r * ld + k]);
-  return ks ? x * ks[k] : x;
+// Bits of the FP64 value of an FP32 number.
+__device__ __forceinline__ unsigned long long f64_bits(float x) {
+  const unsigned u = __float_as_uint(x), e = (u >> 23) & 0xFFu;
+  if (e - 1u >= 254u) return (unsigned long long)__double_as_longlong((double)x);  // zero, subnormal, Inf, NaN
+  return ((unsigned long long)(u & 0x80000000u) << 32) | ((unsigned long long)(e + 896u) << 52) |
+         ((unsigned long long)(u & 0x7FFFFFu) << 29);
+}
+__device__ __forceinline__ unsigned long long f64_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x);
 }
 
-// e[r] = binary exponent of max_k |X(r, k)| (0 for a zero row): |X(r, k)| 2^-e[r] < 1.
+// Bits of entry X[at] times ks[k] when a k scale is given.
 template <typename T>
-__global__ void row_exponent_kernel(const T* X, long long ld, int trans, const double* ks, int R, int K,
-                                    int* e) {
-  if (!trans) {
-    const int r = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (r >= R) return;
-    double m = 0.0;
-    for (int k = lane; k < K; k += 32) m = fmax(m, fabs(entry(X, ld, 0, ks, r, k)));
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if (lane == 0) {
-      int ex = 0;
-      if (m > 0.0) frexp(m, &ex);
-      e[r] = ex;
-    }
+__device__ __forceinline__ unsigned long long entry_bits(T x, const double* ks, int k) {
+  return ks ? f64_bits(__longlong_as_double((long long)f64_bits(x)) * ks[k]) : f64_bits(x);
+}
+
+// The exponent e of the smallest power of two above every entry of a row, from the
+// largest |bits| (the order of the bits of non-negative FP64 numbers is theirs); 0 for
+// a row of zeros and for one with an Inf or NaN.
+__device__ __forceinline__ int row_exponent(unsigned long long mx) {
+  const int ef = (int)(mx >> 52);
+  return mx == 0ull || ef == 0x7FF ? 0 : max(ef, 1) - 1022;
+}
+
+// Digits of |x| 2^-ex < 1 to base 128, d[0] the leading one, by rounding to a multiple of
+// 2^-7S and then from the last digit up: d = ((q + 64) mod 128) - 64, carry into the
+// next.  |d[0]| <= 128, |d[s]| <= 64.
+template <int S>
+__device__ __forceinline__ void slice_digits(unsigned long long u, int ex, int (&d)[S]) {
+  constexpr int H = S / 2, kLow = kDigitBits * H;  // the lower H digits, then the upper ones
+  constexpr unsigned long long kMask = (1ull << kLow) - 1;
+  const int ef = (int)((u >> 52) & 0x7FFull);
+  unsigned long long m = u & 0xFFFFFFFFFFFFFull;
+  if (ef) m |= 1ull << 52;
+  // |x| 2^(7S - ex) = m 2^sh; |x| < 2^ex bounds sh by 7 S - 53
+  const int sh = max(ef, 1) - 1075 + kDigitBits * S - ex;
+  unsigned long long lo, hi;
+  if (sh >= 0) {
+    lo = (m << sh) & kMask;
+    hi = m >> (kLow - sh);
   } else {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R) return;
-    double m = 0.0;
-    for (int k = 0; k < K; ++k) m = fmax(m, fabs(entry(X, ld, 1, ks, r, k)));
-    int ex = 0;
-    if (m > 0.0) frexp(m, &ex);
-    e[r] = ex;
+    const int r = -sh;
+    const unsigned long long q = r > 53 ? 0ull : (m + (1ull << (r - 1))) >> r;
+    lo = q & kMask;
+    hi = q >> kLow;
   }
+  const bool neg = (long long)u < 0;
+#pragma unroll
+  for (int s = S - 1; s >= H; --s) {
+    const int t = (int)(lo & 127u);
+    lo = (lo + 64u) >> 7;
+    d[s] = t >= 64 ? t - 128 : t;
+  }
+  hi += lo;
+#pragma unroll
+  for (int s = H - 1; s >= 1; --s) {
+    const int t = (int)(hi & 127u);
+    hi = (hi + 64u) >> 7;
+    d[s] = t >= 64 ? t - 128 : t;
+  }
+  d[0] = (int)hi;
+#pragma unroll
+  for (int s = 0; s < S; ++s) d[s] = neg ? -d[s] : d[s];
 }
 
-// Digits of 8 consecutive k of one row, written as 8 slices of 16 bytes into the
-// packed layout: blocks of (tile rows TR) x (one K stage of 16) holding, for slice s
-// and K half kc (8 values of k), TR / 8 core matrices of 8 rows x 16 bytes:
-// byte ((s * 2 + kc) * TR / 8 + g) * 128 + w * 16 of the block for row 8 g + w.
-// Every block is one contiguous bulk copy.  Rows >= R and k >= K (the padding)
-// are written as zeros.
+// Packs one octet (8 values of k of one row): slice s to base + s * kSliceStep.  An Inf or
+// NaN becomes NaN in every slice, which the FP32 tail accumulator carries to the output.
+template <int S>
+__device__ __forceinline__ void store_octet(const unsigned long long (&v)[8], int ex, uint8_t* base) {
+  uint32_t out[S][4];
+#pragma unroll
+  for (int i = 0; i < 8; i += 2) {
+    int d0[S], d1[S];
+    slice_digits<S>(v[i], ex, d0);
+    slice_digits<S>(v[i + 1], ex, d1);
+    const bool bad0 = ((v[i] >> 52) & 0x7FFull) == 0x7FFull, bad1 = ((v[i + 1] >> 52) & 0x7FFull) == 0x7FFull;
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      // integer to float by the bits of 1.5 2^23 + d (exact), scaled to d 2^-7(s+1);
+      // at most 8 significant bits, so the upper half of the word is the BF16 value
+      const float w_s = exp2f(-(float)(kDigitBits * (s + 1)));
+      float f0 = (__int_as_float(0x4B400000 + d0[s]) - 12582912.0f) * w_s;
+      float f1 = (__int_as_float(0x4B400000 + d1[s]) - 12582912.0f) * w_s;
+      if (bad0) f0 = __int_as_float(0x7FFFFFFF);
+      if (bad1) f1 = __int_as_float(0x7FFFFFFF);
+      out[s][i / 2] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+    }
+  }
+#pragma unroll
+  for (int s = 0; s < S; ++s)
+    *reinterpret_cast<uint4*>(base + s * kSliceStep) = make_uint4(out[s][0], out[s][1], out[s][2], out[s][3]);
+}
+
+// Address of octet o of row r in the packed form: blocks of (64 rows) x (one K stage of
+// 16), row tile outermost, each holding 8 groups of 8 rows; a group holds, for slice s
+// and K half kc (8 values of k), one core matrix of 8 rows x 16 bytes at
+// s * kSliceStep + kc * kCore.  A 64-row block is one contiguous bulk copy and a left
+// operand's 128 rows are two that lie one after the other in shared memory, with the
+// same distance between 8-row groups, so one packing serves both sides of a product.
+template <int S>
+__device__ __forceinline__ uint8_t* octet_addr(uint8_t* out, int r, int o, int nkt) {
+  const long long blk = (long long)(r >> 6) * nkt + (o >> 1);
+  return out + (blk * 8 + ((r & 63) >> 3)) * (S * kSliceStep) + (o & 1) * kCore + (r & 7) * 16;
+}
+
+constexpr int kPackThreads = 256;
+
+// Rows r0 .. r0 + 7 of X(r, k) = X[r * ld + k] (times ks[k]): the rows' exponents, then
+// their digits.  Thread t takes row t & 7 and octets t >> 3, + 32, ...: a warp reads 256
+// contiguous bytes of each of 8 rows and writes whole core matrices.  vec: two values per
+// load (16-byte aligned rows of FP64).  Rows >= R and k >= K are written as zeros.
 template <typename T, int S>
-__global__ void pack_kernel(const T* X, long long ld, int trans, const double* ks, int R, int K, const int* e,
-                            uint8_t* out, int tile_rows, int r_pad, int n_oct) {
-  const long long total = (long long)r_pad * n_oct;
-  const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= total) return;
-  int r, o;
-  if (trans) {  // consecutive threads: consecutive rows (columns of X) -> coalesced reads
-    r = (int)(idx % r_pad);
-    o = (int)(idx / r_pad);
-  } else {
-    o = (int)(idx % n_oct);
-    r = (int)(idx / n_oct);
-  }
-  const int k0 = o * 8;
-  double v[8];
-  const bool row_ok = r < R;
-  const int ex = row_ok ? e[r] : 0;
+__global__ void __launch_bounds__(kPackThreads) pack_rows_kernel(const T* X, long long ld, const double* ks, int R,
+                                                                 int K, int* e, uint8_t* out, int n_oct, int vec) {
+  __shared__ unsigned long long red[8][8];
+  const int w = threadIdx.x & 7, r = blockIdx.x * 8 + w, o0 = threadIdx.x >> 3;
+  const T* row = X + (long long)r * ld;
+  auto load = [&](int o, unsigned long long (&v)[8]) {
+    const int k0 = 8 * o;
+    if (r < R && k0 + 8 <= K && vec && sizeof(T) == 8) {
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int k = k0 + i;
-    double x = 0.0;
-    if (row_ok && k < K) x = entry(X, ld, trans, ks, r, k);
-    v[i] = ldexp(x, -ex);
-  }
-  const int nkt = n_oct / 2;
-  const int groups = tile_rows / 8;
-  const int rt = r / tile_rows, rr = r % tile_rows, g = rr / 8, w = rr % 8;
-  const int kt = o / 2, kc = o % 2;
-  const long long block_bytes = (long long)S * 2 * groups * kCore;
-  uint8_t* base = out + ((long long)rt * nkt + kt) * block_bytes + ((long long)kc * groups + g) * kCore + w * 16;
+      for (int i = 0; i < 8; i += 2) {
+        const double2 x = *reinterpret_cast<const double2*>(reinterpret_cast<const double*>(row) + k0 + i);
+        v[i] = entry_bits(x.x, ks, k0 + i);
+        v[i + 1] = entry_bits(x.y, ks, k0 + i + 1);
+      }
+    } else {
 #pragma unroll
-  for (int s = 0; s < S; ++s) {
-    const float w_s = exp2f(-(float)(kDigitBits * (s + 1)));
-    uint32_t packed[4];
-#pragma unroll
-    for (int i = 0; i < 8; i += 2) {
-      const double x0 = v[i] * 128.0, x1 = v[i + 1] * 128.0;
-      const double d0 = rint(x0), d1 = rint(x1);
-      v[i] = x0 - d0;
-      v[i + 1] = x1 - d1;
-      const unsigned short b0 = __bfloat16_as_ushort(__float2bfloat16_rn((float)d0 * w_s));
-      const unsigned short b1 = __bfloat16_as_ushort(__float2bfloat16_rn((float)d1 * w_s));
-      packed[i / 2] = (uint32_t)b0 | ((uint32_t)b1 << 16);
+      for (int i = 0; i < 8; ++i) v[i] = r < R && k0 + i < K ? entry_bits(row[k0 + i], ks, k0 + i) : 0ull;
     }
-    *reinterpret_cast<uint4*>(base + (long long)s * 2 * groups * kCore) =
-        make_uint4(packed[0], packed[1], packed[2], packed[3]);
+  };
+  unsigned long long mx = 0;
+  for (int o = o0; o < n_oct; o += kPackThreads / 8) {
+    unsigned long long v[8];
+    load(o, v);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) mx = max(mx, v[i] & 0x7FFFFFFFFFFFFFFFull);
+  }
+#pragma unroll
+  for (int off = 8; off <= 16; off <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+  if ((threadIdx.x & 31) < 8) red[threadIdx.x >> 5][w] = mx;
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < 8; ++u) mx = max(mx, red[u][w]);
+  const int ex = row_exponent(mx);
+  if (threadIdx.x < 8 && r < R) e[r] = ex;
+  for (int o = o0; o < n_oct; o += kPackThreads / 8) {
+    unsigned long long v[8];
+    load(o, v);
+    store_octet<S>(v, ex, octet_addr<S>(out, r, o, n_oct >> 1));
+  }
+}
+
+// The same for X(r, k) = X[k * ld + r]: rows r0 .. r0 + 31, one per lane (coalesced over r);
+// warp w takes octets w, w + 8, ...
+template <typename T, int S>
+__global__ void __launch_bounds__(kPackThreads) pack_cols_kernel(const T* X, long long ld, const double* ks, int R,
+                                                                 int K, int* e, uint8_t* out, int n_oct) {
+  __shared__ unsigned long long red[kPackThreads / 32][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, r = blockIdx.x * 32 + lane;
+  auto load = [&](int o, unsigned long long (&v)[8]) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = 8 * o + i;
+      v[i] = r < R && k < K ? entry_bits(X[(long long)k * ld + r], ks, k) : 0ull;
+    }
+  };
+  unsigned long long mx = 0;
+  for (int o = w; o < n_oct; o += kPackThreads / 32) {
+    unsigned long long v[8];
+    load(o, v);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) mx = max(mx, v[i] & 0x7FFFFFFFFFFFFFFFull);
+  }
+  red[w][lane] = mx;
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < kPackThreads / 32; ++u) mx = max(mx, red[u][lane]);
+  const int ex = row_exponent(mx);
+  if (w == 0 && r < R) e[r] = ex;
+  for (int o = w; o < n_oct; o += kPackThreads / 32) {
+    unsigned long long v[8];
+    load(o, v);
+    store_octet<S>(v, ex, octet_addr<S>(out, r, o, n_oct >> 1));
   }
 }
 
 // ---- the product
 
 struct GemmArgs {
-  const uint8_t* pa;   // packed A (rows of the output), 128-row tiles
-  const uint8_t* pb;   // packed B (columns of the output), 64-row tiles
+  const uint8_t* pa;   // packed A (rows of the output)
+  const uint8_t* pb;   // packed B (columns of the output)
   const int* ea;
   const int* eb;
   int nkt;             // K stages of both packings
@@ -302,6 +405,7 @@ struct GemmArgs {
   double alpha, beta;
   int lower_only;      // write only col <= row; skip tiles above the diagonal
   int a_lower;         // A lower triangular: row tile i reads k < 128 (i + 1)
+  int vec;             // C's rows are 16-byte aligned: two columns per access
   unsigned* status;
 };
 
@@ -314,6 +418,25 @@ struct GemmArgs {
 constexpr int kEpiWarps = 16;
 constexpr int kEpiCols = kTN / 4;  // output columns per reading warp
 constexpr int kThreads = (kEpiWarps + 2) * 32;
+
+// beta 2^ex (hi 2^-28 + lo 2^-7(kExact+1) + tail) in six FP64 operations: the integers
+// (|.| < 2^51) become doubles by the bits of 1.5 2^52 + i, the scales by their exponent
+// fields.  Exponents outside +-800 take ldexp.
+template <int kExact>
+__device__ __noinline__ double out_value_far(double dh, double dl, double dt, int ex, double beta) {
+  return beta * (ldexp(dh, ex - kDigitBits * 4) + (ldexp(dl, ex - kDigitBits * (kExact + 1)) + ldexp(dt, ex)));
+}
+
+template <int kExact>
+__device__ __forceinline__ double out_value(long long hi, long long lo, uint32_t tail, int ex, double beta) {
+  const double dh = __longlong_as_double(0x4338000000000000ll + hi) - 6755399441055744.0;
+  const double dl = __longlong_as_double(0x4338000000000000ll + lo) - 6755399441055744.0;
+  const double dt = __longlong_as_double((long long)f64_bits(__uint_as_float(tail)));
+  if (ex > 800 || ex < -800) return out_value_far<kExact>(dh, dl, dt, ex, beta);
+  auto pow2 = [](int e) { return __longlong_as_double((long long)(1023 + e) << 52); };
+  const double v = fma(dh, pow2(-kDigitBits * 4), fma(dl, pow2(-kDigitBits * (kExact + 1)), dt));
+  return v * (beta * pow2(ex));
+}
 
 template <int S>
 __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(GemmArgs a) {
@@ -364,9 +487,9 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(GemmArgs a) {
   const uint32_t sbase = smem_u32(smem);
 
   if (warp == kEpiWarps + 1) {
-    // producer: one A block (128 x 16, 32 KB) and one B block (64 x 16, 16 KB) per stage
+    // producer: two blocks of 64 x 16 for A and one for B per stage
     if (lane == 0) {
-      const uint8_t* pa = a.pa + (long long)blockIdx.y * a.nkt * kAStage;
+      const uint8_t* pa = a.pa + (long long)(2 * blockIdx.y) * a.nkt * kBStage;
       const uint8_t* pb = a.pb + (long long)blockIdx.x * a.nkt * kBStage;
       int st = 0;
       for (; st < nst && !*abort_flag; ++st) {
@@ -377,7 +500,8 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(GemmArgs a) {
         }
         const uint32_t bar = full0 + 8 * b, dst = sbase + b * kStageBytes;
         expect_tx(bar, kStageBytes);
-        bulk_load(dst, pa + (long long)st * kAStage, kAStage, bar);
+        bulk_load(dst, pa + (long long)st * kBStage, kBStage, bar);
+        bulk_load(dst + kBStage, pa + (long long)(a.nkt + st) * kBStage, kBStage, bar);
         bulk_load(dst + kAStage, pb + (long long)st * kBStage, kBStage, bar);
       }
       *produced_out = st;
@@ -407,11 +531,11 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(GemmArgs a) {
           // index is a compile-time constant and the flags stay in registers
 #pragma unroll
           for (int s = 0; s < S; ++s) {
-            const uint64_t ad = smem_desc(ab + s * 2 * kSliceKc, kSliceKc, kCore);
+            const uint64_t ad = smem_desc(ab + s * kSliceStep, kCore, Sh::kGroup);
 #pragma unroll
             for (int t = 0; t < S - s; ++t) {
               const int q = s + t < kExact ? s + t : kExact;
-              const uint64_t bd = smem_desc(bb + t * 2 * kSliceKcB, kSliceKcB, kCore);
+              const uint64_t bd = smem_desc(bb + t * kSliceStep, kCore, Sh::kGroup);
               uint32_t accumulate;
               if (q < kExact) {
                 accumulate = (started >> q) & 1u;
@@ -475,15 +599,27 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(GemmArgs a) {
           tmem_ld16(lane_addr + kExact * kTN + cb * 16, r);
           if (row < a.m) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
+            for (int i = 0; i < 16; i += 2) {
               const int col = col0 + c_part * kEpiCols + cb * 16 + i;
-              if (col >= a.n || (a.lower_only && col > row)) continue;
-              const int ex = ei + a.eb[col];
-              const double v = ldexp((double)acc_hi[cb * 16 + i], ex - kDigitBits * 4) +
-                               ldexp((double)acc_lo[cb * 16 + i], ex - kDigitBits * (kExact + 1)) +
-                               ldexp((double)__uint_as_float(r[i]), ex);
+              const int n_ok = a.lower_only ? min(a.n, row + 1) : a.n;  // columns written: [0, n_ok)
+              if (col >= n_ok) continue;
+              const int j = cb * 16 + i;
               double* cp = a.C + (long long)row * a.ldc + col;
-              *cp = a.alpha == 0.0 ? a.beta * v : a.alpha * *cp + a.beta * v;
+              const bool two = col + 1 < n_ok;
+              const double v0 = out_value<kExact>(acc_hi[j], acc_lo[j], r[i], ei + a.eb[col], a.beta);
+              const double v1 =
+                  two ? out_value<kExact>(acc_hi[j + 1], acc_lo[j + 1], r[i + 1], ei + a.eb[col + 1], a.beta) : 0.0;
+              if (two && a.vec) {
+                double2 c = make_double2(v0, v1);
+                if (a.alpha != 0.0) {
+                  const double2 old = *reinterpret_cast<const double2*>(cp);
+                  c = make_double2(fma(a.alpha, old.x, v0), fma(a.alpha, old.y, v1));
+                }
+                *reinterpret_cast<double2*>(cp) = c;
+              } else {
+                cp[0] = a.alpha == 0.0 ? v0 : fma(a.alpha, cp[0], v0);
+                if (two) cp[1] = a.alpha == 0.0 ? v1 : fma(a.alpha, cp[1], v1);
+              }
             }
           }
         }
@@ -511,14 +647,10 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(GemmArgs a) {
   }
 }
 
-inline unsigned blocks_for(long long n, int threads) {
-  return (unsigned)std::max<long long>(1, (n + threads - 1) / threads);
-}
-
 }  // namespace
 
 size_t ozaki_pack_bytes(int rows, int k, int slices) {
-  const long long r_pad = (long long)(rows + kTM - 1) / kTM * kTM;  // covers both tile heights
+  const long long r_pad = (long long)(rows + kTM - 1) / kTM * kTM;
   const long long k_pad = (long long)(k + kKS - 1) / kKS * kKS;
   return (size_t)(r_pad * k_pad * slices * 2);
 }
@@ -533,36 +665,36 @@ ep_tv_status ozaki_init() {
 
 namespace {
 
-template <typename T>
+template <typename T, int S>
 void pack_any(const T* X, long long ld, bool trans, int rows, int k, const double* kscale, int* e, uint8_t* out,
-              OzakiSide side, bool exponents, int slices, cudaStream_t s) {
+              cudaStream_t s) {
   if (rows <= 0 || k <= 0) return;
-  if (exponents) {
-    if (trans)
-      row_exponent_kernel<T><<<blocks_for(rows, 256), 256, 0, s>>>(X, ld, 1, kscale, rows, k, e);
-    else
-      row_exponent_kernel<T><<<blocks_for(rows, 8), 256, 0, s>>>(X, ld, 0, kscale, rows, k, e);
-  }
-  const int tile_rows = side == OzakiSide::kLeft ? kTM : kTN;
-  const int r_pad = (rows + tile_rows - 1) / tile_rows * tile_rows;
+  const int r_pad = (rows + kTM - 1) / kTM * kTM;
   const int n_oct = (k + kKS - 1) / kKS * 2;
-  const unsigned nb = blocks_for((long long)r_pad * n_oct, 256);
-  if (slices == 10)
-    pack_kernel<T, 10><<<nb, 256, 0, s>>>(X, ld, trans ? 1 : 0, kscale, rows, k, e, out, tile_rows, r_pad, n_oct);
-  else
-    pack_kernel<T, 8><<<nb, 256, 0, s>>>(X, ld, trans ? 1 : 0, kscale, rows, k, e, out, tile_rows, r_pad, n_oct);
+  if (trans) {
+    pack_cols_kernel<T, S><<<r_pad / 32, kPackThreads, 0, s>>>(X, ld, kscale, rows, k, e, out, n_oct);
+  } else {
+    const int vec = ((uintptr_t)X & 15) == 0 && (ld & 1) == 0;
+    pack_rows_kernel<T, S><<<r_pad / 8, kPackThreads, 0, s>>>(X, ld, kscale, rows, k, e, out, n_oct, vec);
+  }
 }
 
 }  // namespace
 
 void ozaki_pack(const double* X, long long ld, bool trans, int rows, int k, const double* kscale, int* e,
-                uint8_t* out, OzakiSide side, bool exponents, cudaStream_t s, int slices) {
-  pack_any(X, ld, trans, rows, k, kscale, e, out, side, exponents, slices, s);
+                uint8_t* out, cudaStream_t s, int slices) {
+  if (slices == 10)
+    pack_any<double, 10>(X, ld, trans, rows, k, kscale, e, out, s);
+  else
+    pack_any<double, 8>(X, ld, trans, rows, k, kscale, e, out, s);
 }
 
 void ozaki_pack(const float* X, long long ld, bool trans, int rows, int k, const double* kscale, int* e,
-                uint8_t* out, OzakiSide side, bool exponents, cudaStream_t s, int slices) {
-  pack_any(X, ld, trans, rows, k, kscale, e, out, side, exponents, slices, s);
+                uint8_t* out, cudaStream_t s, int slices) {
+  if (slices == 10)
+    pack_any<float, 10>(X, ld, trans, rows, k, kscale, e, out, s);
+  else
+    pack_any<float, 8>(X, ld, trans, rows, k, kscale, e, out, s);
 }
 
 void ozaki_gemm(const OzakiOperand& A, const OzakiOperand& B, int k, double* C, long long ldc, int m, int n,
@@ -582,6 +714,7 @@ void ozaki_gemm(const OzakiOperand& A, const OzakiOperand& B, int k, double* C, 
   g.beta = beta;
   g.lower_only = lower_only ? 1 : 0;
   g.a_lower = a_lower ? 1 : 0;
+  g.vec = ((uintptr_t)C & 15) == 0 && (ldc & 1) == 0;
   g.status = status;
   dim3 grid((n + kTN - 1) / kTN, (m + kTM - 1) / kTM);
   if (A.slices == 10)
@@ -606,8 +739,8 @@ ep_tv_status ozaki_gemm_standalone(const double* A, const double* B, double* C, 
   unsigned h_status = 0;
   if (st == EP_TV_OK) {
     cudaMemsetAsync(status, 0, sizeof(unsigned), s);
-    ozaki_pack(A, k, false, m, k, nullptr, ea, pa, OzakiSide::kLeft, true, s, slices);
-    ozaki_pack(B, k, false, n, k, nullptr, eb, pb, OzakiSide::kRight, true, s, slices);
+    ozaki_pack(A, k, false, m, k, nullptr, ea, pa, s, slices);
+    ozaki_pack(B, k, false, n, k, nullptr, eb, pb, s, slices);
     ozaki_gemm(OzakiOperand{pa, ea, slices}, OzakiOperand{pb, eb, slices}, k, C, n, m, n, 0.0, 1.0, false, false,
                status, s);
     if (cudaMemcpyAsync(&h_status, status, sizeof(unsigned), cudaMemcpyDeviceToHost, s) != cudaSuccess ||

@@ -16,25 +16,19 @@ struct OzakiOperand {
   int slices = 8;  // digit slices per entry: 8 or 10 (both operands of a product alike)
 };
 
-// Which operand a packing is for: left (rows of the output, 128-row tiles) or
-// right (columns of the output, 64-row tiles).
-enum class OzakiSide { kLeft, kRight };
-
-// Bytes of the packed form of a rows x k operand (either side).
+// Bytes of the packed form of a rows x k operand (the same for either side of a product).
 size_t ozaki_pack_bytes(int rows, int k, int slices = 8);
 // Raises the kernel's dynamic shared-memory limit (once per process and device).
 ep_tv_status ozaki_init();
 // Packs rows x k operand X(r, k) = X[r * ld + k] (trans: X[k * ld + r]), times
-// kscale[k] when kscale is not NULL, into out (ozaki_pack_bytes(rows, k) bytes);
-// with exponents, first writes its row exponents into e (rows ints), else
-// uses those in e (packing one matrix for both sides).
+// kscale[k] when kscale is not NULL, into out (ozaki_pack_bytes(rows, k) bytes), and
+// writes its row exponents into e (rows ints).
 // slices: 8 (error about 2^-56 of the rows' largest entries) or 10 (2^-70).
 void ozaki_pack(const double* X, long long ld, bool trans, int rows, int k, const double* kscale, int* e,
-                uint8_t* out, OzakiSide side, bool exponents, cudaStream_t s, int slices = 8);
+                uint8_t* out, cudaStream_t s, int slices = 8);
 void ozaki_pack(const float* X, long long ld, bool trans, int rows, int k, const double* kscale, int* e,
-                uint8_t* out, OzakiSide side, bool exponents, cudaStream_t s, int slices = 8);
-// C = alpha C + beta A B^T for packed A (m x k, left side) and B (n x k, right
-// side); C row-major, ldc.
+                uint8_t* out, cudaStream_t s, int slices = 8);
+// C = alpha C + beta A B^T for packed A (m x k) and B (n x k; may be A); C row-major, ldc.
 // With 10 slices k must be at most 8192.
 // lower_only: only entries with col <= row are written.  a_lower: A is lower
 // triangular (row i has no entries beyond k = i), so row tiles stop early.

@@ -155,3 +155,36 @@ def test_slice_count_is_checked():
     assert lib.ep_tv_tc_gemm_f64(ctypes.c_void_p(8), ctypes.c_void_p(8), ctypes.c_void_p(8), 1, 1, 8193, 10,
                                  None) == 1
 
+
+
+@pytest.mark.parametrize("m,n,k,slices", [(129, 65, 17, 8), (127, 63, 15, 10), (8, 200, 129, 10), (65, 129, 258, 8)])
+def test_packing_edges(m, n, k, slices):
+    """Sizes one off the packing's tiles (8-row groups, 64- and 128-row blocks, octets of
+    k; odd k leaves rows unaligned for paired loads), zeros, the smallest normal
+    numbers, entries a rounding below a power of two, and row scales at both ends of
+    the range, within the bound of the split form."""
+    rng = np.random.default_rng(m + k)
+    A, B = rng.standard_normal((m, k)), rng.standard_normal((n, k))
+    A[0] = np.nextafter(2.0, 0.0)
+    A[1, ::2] = 0.0
+    B[0] = -np.nextafter(0.5, 0.0)
+    _check(A, B, _tc_product(A, B, slices), n_samples=10, slices=slices)
+    # power-of-two scalings move the result exactly, also past the fast exponent range
+    C = _tc_product(A, B, slices)
+    for ea, eb in ((-900, 20), (880, 30), (-990, 900)):
+        D = _tc_product(np.ldexp(A, ea), np.ldexp(B, eb), slices)
+        np.testing.assert_array_equal(D, np.ldexp(C, ea + eb))
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("slices", [8, 10])
+def test_non_finite_entries_reach_their_rows(value, slices):
+    """A NaN or an infinity in a row of A makes that row of the product NaN and leaves the
+    others alone."""
+    rng = np.random.default_rng(3)
+    A, B = rng.standard_normal((70, 40)), rng.standard_normal((66, 40))
+    C = _tc_product(A, B, slices)
+    A[13, 21] = value
+    D = _tc_product(A, B, slices)
+    assert np.all(np.isnan(D[13]))
+    np.testing.assert_array_equal(np.delete(D, 13, 0), np.delete(C, 13, 0))

@@ -147,17 +147,44 @@ __global__ void f32_to_f64_kernel(const float* in, double* out, int n) {
   if (i < n) out[i] = (double)in[i];
 }
 
-// w[i] = sum_m W[m, i]^2 (column sums, FP64)
-__global__ void colsq_kernel(const double* W, int M, int N, double* w) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// Column sums of W (M x N) over the rows of chunk blockIdx.y: pw[chunk][i] = sum W[m, i]^2 and
+// pg[chunk][i] = sum W[m, i] v[m], one thread per column; cs_site0_kernel adds the chunks.
+// One pass over W, which is its cost (W is 644 MB at M = 4915, N = 16384; as two kernels with
+// one thread per column over all rows the sums took 1.70 ms there; 0.31 ms here).
+constexpr int kSumThreads = 128;
+__global__ void __launch_bounds__(kSumThreads) col_sums_kernel(const double* W, const double* v, int M, int N,
+                                                               int rows_per, double* pw, double* pg) {
+  const int i = blockIdx.x * kSumThreads + threadIdx.x;
   if (i >= N) return;
-  double s = 0.0;
-  for (int m = 0; m < M; ++m) {
-    const double v = W[(long long)m * N + i];
-    s = fma(v, v, s);
+  const int m0 = blockIdx.y * rows_per, m1 = min(M, m0 + rows_per);
+  double w = 0.0, g = 0.0;
+  int m = m0;
+  for (; m + 4 <= m1; m += 4) {
+    double x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = W[(long long)(m + u) * N + i];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      w = fma(x[u], x[u], w);
+      g = fma(x[u], v[m + u], g);
+    }
   }
-  w[i] = s;
+  for (; m < m1; ++m) {
+    const double x = W[(long long)m * N + i];
+    w = fma(x, x, w);
+    g = fma(x, v[m], g);
+  }
+  pw[(long long)blockIdx.y * N + i] = w;
+  pg[(long long)blockIdx.y * N + i] = g;
 }
+
+// Rows per chunk: at least 16, and chunks enough for about eight blocks per SM.
+int sum_rows(int M, int N) {
+  const int cols = (N + kSumThreads - 1) / kSumThreads;
+  const int want = std::max(1, 8 * 152 / cols);
+  return std::max(16, (M + want - 1) / want);
+}
+int sum_chunks(int M, int N) { return (M + sum_rows(M, N) - 1) / sum_rows(M, N); }
 
 // t = y - A m  (one warp per row)
 __global__ void resid_vec_kernel(const float* A, const float* y, const double* m, int M, int N,
@@ -170,15 +197,6 @@ __global__ void resid_vec_kernel(const float* A, const float* y, const double* m
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
   if (lane == 0) t[row] = (double)y[row] - s;
-}
-
-// g = W^T v  (one thread per column)
-__global__ void wtv_kernel(const double* W, const double* v, int M, int N, double* g) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  double s = 0.0;
-  for (int m = 0; m < M; ++m) s = fma(W[(long long)m * N + i], v[m], s);
-  g[i] = s;
 }
 
 // Cavity of site 0 from the prior sites: d = sum tau_k, n = sum nu_k; c = 1/d, m = n/d.
@@ -195,16 +213,31 @@ __global__ void cs_cavity_kernel(const float* tp, const float* np, long long N, 
 }
 
 // Eq. update_q0_x: tau = w / (1 - c w) (= 1/Var - 1/c), cap, nu = tau E + (E - m)/c, damp.
-__global__ void cs_site0_kernel(const double* w, const double* g, const double* c, const double* m,
+// w and g: the chunks of col_sums_kernel, added in order.
+__global__ void cs_site0_kernel(const double* pw, const double* pg, int chunks, const double* c, const double* m,
                                 long long N, float* tau0, float* nu0, float min_tau, float damping,
                                 unsigned* status, unsigned long long* counters) {
   unsigned capped = 0;
   bool bad = false;
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N;
        p += (long long)gridDim.x * blockDim.x) {
+    double w = 0.0, g = 0.0;
+    for (int u0 = 0; u0 < chunks; u0 += 8) {
+      double a[8], b[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        a[u] = u0 + u < chunks ? pw[(u0 + u) * N + p] : 0.0;
+        b[u] = u0 + u < chunks ? pg[(u0 + u) * N + p] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        w += a[u];
+        g += b[u];
+      }
+    }
     const double ci = c[p];
-    const double E = m[p] + ci * g[p];
-    double tn = w[p] / (1.0 - ci * w[p]);
+    const double E = m[p] + ci * g;
+    double tn = w / (1.0 - ci * w);
     if (!(tn >= (double)min_tau)) {
       tn = min_tau;
       ++capped;
@@ -223,26 +256,64 @@ __global__ void cs_site0_kernel(const double* w, const double* g, const double* 
 // ---- Hadamard operator
 //
 // Fast Walsh-Hadamard transform (Sylvester order, unnormalised) of rows of n
-// doubles, n a power of two: one row per block in shared memory (n <= 16384), the
-// butterflies (a, b) -> (a + b, a - b) at strides 1, 2, 4, ...
+// doubles, n a power of two: one row per block in shared memory (n <= 16384).  The
+// butterflies (a, b) -> (a + b, a - b) of the different strides commute: two strides of 32
+// and more at a time pass through shared memory (neighbouring lanes on neighbouring
+// words), those below 32 run between the lanes of a warp.  Bound by FP64 additions,
+// n log2 n of them at two per clock and SM (60 us for n = 16384).
+// With Z the row is not read: it is L^{-1} S / sqrt(M) of the Hadamard operator, row
+// blockIdx.x of the lower-triangular Z (M x M) scattered to the columns sel.
 constexpr int kFwhtThreads = 1024;
 constexpr int kFwhtMaxSmem = 16384;
 
-__global__ void __launch_bounds__(kFwhtThreads) fwht_rows_smem_kernel(double* rows, int n) {
+__global__ void __launch_bounds__(kFwhtThreads) fwht_rows_smem_kernel(double* rows, int n, const double* Z, int M,
+                                                                      const int* sel) {
   extern __shared__ double v[];
   double* row = rows + (long long)blockIdx.x * n;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) v[i] = row[i];
+  if (Z) {
+    const double scale = 1.0 / sqrt((double)M);
+    const double* z = Z + (long long)blockIdx.x * M;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) v[i] = 0.0;
+    __syncthreads();
+    for (int j = threadIdx.x; j <= blockIdx.x; j += blockDim.x) v[sel[j]] = z[j] * scale;
+  } else {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) v[i] = row[i];
+  }
   __syncthreads();
-  for (int h = 1; h < n; h <<= 1) {
-    for (int t = threadIdx.x; t < n / 2; t += blockDim.x) {
-      const int i = (t / h) * 2 * h + (t % h), j = i + h;
-      const double a = v[i], b = v[j];
-      v[i] = a + b;
-      v[j] = a - b;
+  int h = n;  // strides h and more are done
+  for (; h >= 128; h >>= 2) {
+    const int q = h >> 2;  // strides h / 2 and h / 4
+    for (int t = threadIdx.x; t < n / 4; t += blockDim.x) {
+      const int i = (t / q) * h + (t & (q - 1));
+      const double a = v[i], b = v[i + q], c = v[i + 2 * q], d = v[i + 3 * q];
+      const double ac = a + c, bd = b + d, a_c = a - c, b_d = b - d;
+      v[i] = ac + bd;
+      v[i + q] = ac - bd;
+      v[i + 2 * q] = a_c + b_d;
+      v[i + 3 * q] = a_c - b_d;
     }
     __syncthreads();
   }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) row[i] = v[i];
+  if (h == 64) {
+    for (int t = threadIdx.x; t < n / 2; t += blockDim.x) {
+      const int i = (t >> 5) * 64 + (t & 31);
+      const double a = v[i], b = v[i + 32];
+      v[i] = a + b;
+      v[i + 32] = a - b;
+    }
+    __syncthreads();
+    h = 32;
+  }
+  // strides below 32 (the block is a multiple of a warp, so whole warps take part)
+  for (int i0 = 0; i0 < n; i0 += blockDim.x) {
+    const int i = i0 + threadIdx.x;
+    double x = i < n ? v[i] : 0.0;
+    for (int s = h >> 1; s >= 1; s >>= 1) {
+      const double o = __shfl_xor_sync(0xffffffffu, x, s);
+      x = threadIdx.x & s ? o - x : x + o;
+    }
+    if (i < n) row[i] = x;
+  }
 }
 
 // One butterfly stage (stride h) over rows rows of n doubles in global memory.
@@ -259,21 +330,19 @@ __global__ void fwht_stage_kernel(double* rows, int n, int h, long long pairs) {
   }
 }
 
-// K = diag(xi) + (W c)[s_m ^ s_m'] / M, from wc = W c.
+// K = diag(xi) + (W c)[s_m ^ s_m'] / M, from wc = W c: the lower triangle, which is all
+// the factorisation reads; row blockIdx.x, 256 columns per block.
 __global__ void hadamard_k_kernel(double* K, int M, const int* sel, const double* wc, double xi,
                                   const double* xi_v) {
-  const long long total = (long long)M * M;
-  const double inv_m = 1.0 / (double)M;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(e / M), j = (int)(e - (long long)i * M);
-    double v = wc[sel[i] ^ sel[j]] * inv_m;
-    if (i == j) v += xi_v ? xi_v[i] : xi;
-    K[e] = v;
-  }
+  const int i = blockIdx.x, j = blockIdx.y * blockDim.x + threadIdx.x;
+  if (j > i) return;
+  double v = wc[sel[i] ^ sel[j]] * (1.0 / (double)M);
+  if (i == j) v += xi_v ? xi_v[i] : xi;
+  K[(long long)i * M + j] = v;
 }
 
-// G = 0, then G[m, s_j] = Z[m, j] / sqrt(M) for the lower triangle of Z (L^{-1} is lower).
+// G = 0, then G[m, s_j] = Z[m, j] / sqrt(M) for the lower triangle of Z (L^{-1} is lower):
+// rows longer than fwht_rows_smem_kernel holds.
 __global__ void hadamard_scatter_kernel(const double* Z, int M, const int* sel, double* G, int N) {
   const long long total = (long long)M * M;
   const double scale = 1.0 / sqrt((double)M);
@@ -328,14 +397,16 @@ __device__ __forceinline__ double recip_f64(double d) {
 // rows are factored in four panels of 16 whose bulk work is spread over the cluster's SMs
 // (CTA c owns the rows, and then the columns of Z, that are c modulo the cluster's size),
 // each CTA keeping the block in its own shared memory:
-//   - the 16 x 16 diagonal block by Gaussian elimination on [S | I] in place, in the
-//     registers of one warp, in every CTA alike: S = L1 D L1^T, L_pp^{-1} = D^{-1/2} L1^{-1},
-//     one reciprocal per pivot (the square roots are taken once, at the end);
+//   - the 16 x 16 diagonal block by Gaussian elimination on [S | I] in place, two entries
+//     per thread (a warp's FP64 instruction holds its quarter of the SM for 64 clocks), in
+//     every CTA alike: S = L1 D L1^T, L_pp^{-1} = D^{-1/2} L1^{-1}, one reciprocal per pivot
+//     (the square roots are taken once, at the end);
 //   - the owned rows of the panel, L21 = S21 L_pp^{-T}, written to every CTA;
 //   - the owned rows of the trailing update; the next diagonal block's written to every CTA;
 //   - at the end the owned columns of Z by block forward substitution.
 // Measured for 64 rows: 287 us as a one-block Cholesky with square root and division
-// per pivot and a one-thread-per-column inverse, 72 us in this form.
+// per pivot and a one-thread-per-column inverse, 72 us with a diagonal block held by one
+// warp, 49 us in this form.
 constexpr int kBlkCtas = 8;
 constexpr int kBlkThreads = 128;
 constexpr int kPan = 16;
@@ -349,6 +420,7 @@ __global__ void __cluster_dims__(kBlkCtas, 1, 1) __launch_bounds__(kBlkThreads)
   __shared__ double S[kNb * kPitch];
   __shared__ double Zd[kNb / kPan][kPan][kPan + 1];
   __shared__ double Y[kNb][kNb / kBlkCtas + 1];
+  __shared__ double prow[2][kPan];
   const int tid = threadIdx.x, lane = tid & 31;
   for (int e = tid; e < kNb * kNb; e += kBlkThreads) {
     const int i = e / kNb, j = e % kNb;  // rows beyond n: the unit matrix
@@ -357,42 +429,40 @@ __global__ void __cluster_dims__(kBlkCtas, 1, 1) __launch_bounds__(kBlkThreads)
   cl.sync();  // every CTA's copy is loaded before another writes into it
   for (int p = 0; p < kNb / kPan; ++p) {
     const int o = kPan * p;
-    if (tid < 32) {
-      // lane: row i, columns 8 h .. 8 h + 7
-      const int i = lane >> 1, h = lane & 1;
-      double a[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int k = 8 * h + u;
-        a[u] = S[(o + max(i, k)) * kPitch + o + min(i, k)];
-      }
+    {
+      // row i = tid / 8, columns k0 and k0 + 1; a warp holds four whole rows
+      const int i = tid >> 3, k0 = 2 * (tid & 7);
+      auto sym = [&](int k) { return S[(o + max(i, k)) * kPitch + o + min(i, k)]; };
+      double a0 = sym(k0), a1 = sym(k0 + 1), piv = 1.0;
       bool bad = false;
-      double piv = 1.0;  // the row's pivot
 #pragma unroll
       for (int j = 0; j < kPan; ++j) {
-        double d = __shfl_sync(0xffffffffu, a[j & 7], 2 * j + (j >> 3));
+        double* row = prow[j & 1];  // row j, published by its owners after step j - 1
+        if (i == j) {
+          row[k0] = a0;
+          row[k0 + 1] = a1;
+        }
+        const double cij = __shfl_sync(0xffffffffu, j & 1 ? a1 : a0, (lane & ~7) | (j >> 1));
+        __syncthreads();
+        double d = row[j];
         if (!(d > 0.0)) {
           bad = true;
           d = 1e-300;
         }
         if (i == j) piv = d;
-        const double cij = __shfl_sync(0xffffffffu, a[j & 7], (lane & ~1) | (j >> 3));
-        double t[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) t[u] = cij * __shfl_sync(0xffffffffu, a[u], 2 * j + h);
-        const double r = recip_f64(d);
-        if (i > j) {
-#pragma unroll
-          for (int u = 0; u < 8; ++u) a[u] = 8 * h + u == j ? -cij * r : fma(-t[u], r, a[u]);
+        if ((tid >> 5) * 4 + 3 > j) {  // warps whose rows are all done have nothing to update
+          const double t0 = cij * row[k0], t1 = cij * row[k0 + 1];
+          const double r = recip_f64(d);
+          if (i > j) {
+            a0 = k0 == j ? -cij * r : fma(-t0, r, a0);
+            a1 = k0 + 1 == j ? -cij * r : fma(-t1, r, a1);
+          }
         }
       }
-      if (bad && rank == 0 && lane == 0) atomicOr(status, ST_NONFINITE);
+      if (bad && rank == 0 && tid == 0) atomicOr(status, ST_NONFINITE);
       const double y = rsqrt(piv);
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int k = 8 * h + u;
-        Zd[p][i][k] = k < i ? a[u] * y : (k == i ? y : 0.0);
-      }
+      Zd[p][i][k0] = k0 < i ? a0 * y : (k0 == i ? y : 0.0);
+      Zd[p][i][k0 + 1] = k0 + 1 < i ? a1 * y : (k0 + 1 == i ? y : 0.0);
     }
     __syncthreads();
     if (o + kPan >= kNb) break;
@@ -479,9 +549,9 @@ inline int g1d(long long n) {
 void fwht_rows(double* rows, long long nrows, int n, cudaStream_t s) {
   if (n < 2 || nrows < 1) return;
   const int chunk = std::min(n, kFwhtMaxSmem);
-  const int threads = std::min(kFwhtThreads, std::max(32, chunk / 2));
+  const int threads = std::min(kFwhtThreads, std::max(32, chunk / 4));
   fwht_rows_smem_kernel<<<(unsigned)(nrows * (n / chunk)), threads, sizeof(double) * chunk, s>>>(
-      rows, chunk);
+      rows, chunk, nullptr, 0, nullptr);
   const long long pairs = nrows * (n / 2);
   for (int h = chunk; h < n; h <<= 1) fwht_stage_kernel<<<g1d(pairs), 256, 0, s>>>(rows, n, h, pairs);
 }
@@ -515,8 +585,8 @@ struct CsState {
   double* c = nullptr;
   double* sqc = nullptr;
   double* m = nullptr;
-  double* w = nullptr;
-  double* g = nullptr;
+  double* sums = nullptr;     // 2 x chunks x N: column sums of W^2 and W v (col_sums_kernel)
+  double* g = nullptr;        // N, Hadamard: input and output of the transforms
   double* t = nullptr;        // M
   double* v = nullptr;        // M
   double* xi_v = nullptr;     // M noise variances (diagonal noise covariance), or NULL
@@ -544,7 +614,7 @@ void cs_free(CsState* S) {
   cudaFree(S->c);
   cudaFree(S->sqc);
   cudaFree(S->m);
-  cudaFree(S->w);
+  cudaFree(S->sums);
   cudaFree(S->g);
   cudaFree(S->t);
   cudaFree(S->v);
@@ -589,22 +659,21 @@ constexpr int kMmaMin = 64;
 constexpr int kFactorSlices = 10;
 constexpr int kFactorMaxK = 8192;  // the 10-slice product's integer accumulators hold k <= 8192
 
-// C = alpha C + beta X Y^T, X (m x k) row-major at ldx, Y(j, kk) = Y[j * ldy + kk]
+// C = (add ? C : 0) +- X Y^T (- when negate), X (m x k) row-major at ldx, Y(j, kk) = Y[j * ldy + kk]
 // or, when y_trans, Y[kk * ldy + j]; x_lower / y_lower: the stored X / Y is lower
-// triangular (the SIMT GEMM skips the zero products; the split product stops a
-// row tile of a triangular X at its diagonal).  same: Y is X.
+// triangular (both products skip the ranges of k that are zero).  same: Y is X.
 void product(CsState* S, const double* X, long long ldx, bool x_lower, const double* Y, long long ldy,
-             bool y_trans, bool y_lower, bool same, int m, int n, int k, double* C, long long ldc, double alpha,
-             double beta, bool lower_only, cudaStream_t s) {
+             bool y_trans, bool y_lower, bool same, int m, int n, int k, double* C, long long ldc, bool add,
+             bool negate, bool lower_only, cudaStream_t s) {
   if (m <= 0 || n <= 0 || k <= 0) return;
   if (std::min(m, n) < kMmaMin || k < kMmaMin || k > kFactorMaxK) {
-    gemm(!y_trans, m, n, k, X, (int)ldx, Y, (int)ldy, C, (int)ldc, alpha, beta, lower_only, s, x_lower,
-         y_lower);
+    gemm(!y_trans, m, n, k, X, (int)ldx, Y, (int)ldy, C, (int)ldc, add ? 1.0 : 0.0, negate ? -1.0 : 1.0, lower_only, s,
+         x_lower, y_lower);
     S->simt_flops += (x_lower || y_lower ? 1.0 : 2.0) * m * n * k;  // a triangle halves the products
     return;
   }
   const int sl = kFactorSlices;
-  const double f = ozaki_tensor_flops(m, n, k, sl) * (x_lower || lower_only ? 0.5 : 1.0);
+  const double f = ozaki_tensor_flops(m, n, k, sl) * (x_lower || y_lower || lower_only ? 0.5 : 1.0);
   S->mma_flops += f;
   Segment seg(S, s, f);
   ozaki_pack(X, ldx, false, m, k, nullptr, S->exp_a, S->pack_a, s, sl);
@@ -614,7 +683,8 @@ void product(CsState* S, const double* X, long long ldx, bool x_lower, const dou
     ozaki_pack(Y, ldy, y_trans, n, k, nullptr, S->exp_b, S->pack_b, s, sl);
     b = OzakiOperand{S->pack_b, S->exp_b, sl};
   }
-  ozaki_gemm(a, b, k, C, ldc, m, n, alpha, beta, lower_only, x_lower, S->status, s);
+  const OzakiTri tri = !y_lower ? OzakiTri::kNone : y_trans ? OzakiTri::kUpper : OzakiTri::kLower;
+  ozaki_gemm(a, b, k, C, ldc, m, n, add, negate, lower_only, x_lower, tri, S->status, s);
 }
 
 int split_point(int n) {
@@ -647,11 +717,11 @@ void chol_inv(CsState* S, double* K, long long ld, double* Z, long long ldz, int
   double* L21 = pool;                       // n2 x n1
   double* T = pool + (long long)n2 * n1;    // n2 x n1
   double* rest = T + (long long)n2 * n1;
-  product(S, K21, ld, false, Z, ldz, false, true, false, n2, n1, n1, L21, n1, 0.0, 1.0, false, s);
-  product(S, L21, n1, false, L21, n1, false, false, true, n2, n2, n1, K22, ld, 1.0, -1.0, true, s);
+  product(S, K21, ld, false, Z, ldz, false, true, false, n2, n1, n1, L21, n1, false, false, false, s);
+  product(S, L21, n1, false, L21, n1, false, false, true, n2, n2, n1, K22, ld, true, true, true, s);
   chol_inv(S, K22, ld, Z22, ldz, n2, rest, s);
-  product(S, L21, n1, false, Z, ldz, true, true, false, n2, n1, n1, T, n1, 0.0, 1.0, false, s);
-  product(S, Z22, ldz, true, T, n1, true, false, false, n2, n1, n2, Z21, ldz, 0.0, -1.0, false, s);
+  product(S, L21, n1, false, Z, ldz, true, true, false, n2, n1, n1, T, n1, false, false, false, s);
+  product(S, Z22, ldz, true, T, n1, true, false, false, n2, n1, n2, Z21, ldz, false, true, false, s);
 }
 
 unsigned bit_reverse(unsigned k, int bits) {
@@ -682,7 +752,7 @@ bool alloc_common(CsState* S) {
          cudaMalloc(&S->c, sizeof(double) * N) == cudaSuccess &&
          cudaMalloc(&S->sqc, sizeof(double) * N) == cudaSuccess &&
          cudaMalloc(&S->m, sizeof(double) * N) == cudaSuccess &&
-         cudaMalloc(&S->w, sizeof(double) * N) == cudaSuccess &&
+         cudaMalloc(&S->sums, sizeof(double) * 2 * sum_chunks(M, N) * N) == cudaSuccess &&
          cudaMalloc(&S->g, sizeof(double) * N) == cudaSuccess &&
          cudaMalloc(&S->t, sizeof(double) * M) == cudaSuccess &&
          cudaMalloc(&S->v, sizeof(double) * M) == cudaSuccess &&
@@ -791,7 +861,7 @@ ep_tv_status cs_update(CsState* S, float* tau0, float* nu0, const float* tp, con
     if (cudaMemcpyAsync(S->g, S->c, sizeof(double) * N, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
       return EP_TV_ERR_CUDA;
     fwht_rows(S->g, 1, N, s);
-    hadamard_k_kernel<<<g1d(MM), 256, 0, s>>>(S->K, M, S->sel, S->g, S->xi, S->xi_v);
+    hadamard_k_kernel<<<dim3(M, (M + 255) / 256), 256, 0, s>>>(S->K, M, S->sel, S->g, S->xi, S->xi_v);
   } else {
     // K = diag(xi) + (A C^{1/2})(A C^{1/2})^T, lower triangle, on the tensor cores
     init_k_kernel<<<g1d(MM), 256, 0, s>>>(S->K, M, S->xi, S->xi_v);
@@ -800,7 +870,7 @@ ep_tv_status cs_update(CsState* S, float* tau0, float* nu0, const float* tp, con
     Segment seg(S, s, f);
     ozaki_pack(S->A, N, false, M, N, S->sqc, S->exp_a, S->pack_a, s);
     const OzakiOperand g{S->pack_a, S->exp_a};
-    ozaki_gemm(g, g, N, S->K, M, M, M, 1.0, 1.0, true, false, status, s);
+    ozaki_gemm(g, g, N, S->K, M, M, M, true, false, true, false, OzakiTri::kNone, status, s);
   }
   // K = L L^T and Z = L^{-1}
   if (cudaMemsetAsync(S->Z, 0, sizeof(double) * MM, s) != cudaSuccess) return EP_TV_ERR_CUDA;
@@ -808,19 +878,23 @@ ep_tv_status cs_update(CsState* S, float* tau0, float* nu0, const float* tp, con
   if (S->hadamard) {
     // W = (L^{-1} S) W_N / sqrt(M): the lower inverse scattered to the selected
     // columns, then a fast transform of every row
-    if (cudaMemsetAsync(S->G, 0, sizeof(double) * MN, s) != cudaSuccess) return EP_TV_ERR_CUDA;
-    hadamard_scatter_kernel<<<g1d(MM), 256, 0, s>>>(S->Z, M, S->sel, S->G, N);
-    fwht_rows(S->G, M, N, s);
+    if (N <= kFwhtMaxSmem) {
+      fwht_rows_smem_kernel<<<M, std::min(kFwhtThreads, std::max(32, N / 4)), sizeof(double) * N, s>>>(S->G, N, S->Z,
+                                                                                                    M, S->sel);
+    } else {
+      if (cudaMemsetAsync(S->G, 0, sizeof(double) * MN, s) != cudaSuccess) return EP_TV_ERR_CUDA;
+      hadamard_scatter_kernel<<<g1d(MM), 256, 0, s>>>(S->Z, M, S->sel, S->G, N);
+      fwht_rows(S->G, M, N, s);
+    }
   } else {
     // W = Z A on the tensor cores (Z lower triangular)
     const double f = ozaki_tensor_flops(M, N, M) / 2.0;
     S->mma_flops += f;
     Segment seg(S, s, f);
     ozaki_pack(S->Z, M, false, M, M, nullptr, S->exp_a, S->pack_a, s);
-    ozaki_gemm(OzakiOperand{S->pack_a, S->exp_a}, OzakiOperand{S->pack_at, S->exp_at}, M, S->G, N, M, N, 0.0,
-               1.0, false, true, status, s);
+    ozaki_gemm(OzakiOperand{S->pack_a, S->exp_a}, OzakiOperand{S->pack_at, S->exp_at}, M, S->G, N, M, N, false,
+               false, false, true, OzakiTri::kNone, status, s);
   }
-  colsq_kernel<<<(N + 255) / 256, 256, 0, s>>>(S->G, M, N, S->w);
   // mean: t = y - A m, v = L^{-1} t, g = W^T v, E = m + c g
   if (S->hadamard) {
     if (cudaMemcpyAsync(S->g, S->m, sizeof(double) * N, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
@@ -831,8 +905,11 @@ ep_tv_status cs_update(CsState* S, float* tau0, float* nu0, const float* tp, con
     resid_vec_kernel<<<(M + 7) / 8, 256, 0, s>>>(S->A, S->y, S->m, M, N, S->t);
   }
   trmv_lower_kernel<<<(M + 7) / 8, 256, 0, s>>>(S->Z, M, S->t, S->v);
-  wtv_kernel<<<(N + 255) / 256, 256, 0, s>>>(S->G, S->v, M, N, S->g);
-  cs_site0_kernel<<<g1d(N), 256, 0, s>>>(S->w, S->g, S->c, S->m, N, tau0, nu0, S->min_tau, S->damping,
+  const int chunks = sum_chunks(M, N);
+  double* const pg = S->sums + (long long)chunks * N;
+  col_sums_kernel<<<dim3((N + kSumThreads - 1) / kSumThreads, chunks), kSumThreads, 0, s>>>(
+      S->G, S->v, M, N, sum_rows(M, N), S->sums, pg);
+  cs_site0_kernel<<<g1d(N), 256, 0, s>>>(S->sums, pg, chunks, S->c, S->m, N, tau0, nu0, S->min_tau, S->damping,
                                          status, counters);
   tr->end(s, (double)N);
   return cudaGetLastError() == cudaSuccess ? EP_TV_OK : EP_TV_ERR_CUDA;

@@ -402,9 +402,10 @@ struct GemmArgs {
   double* C;
   long long ldc;
   int m, n;
-  double alpha, beta;
+  int add, negate;     // C = (add ? C : 0) +- A B^T
   int lower_only;      // write only col <= row; skip tiles above the diagonal
   int a_lower;         // A lower triangular: row tile i reads k < 128 (i + 1)
+  int b_tri;           // OzakiTri of B: a column tile reads k < 64 (j + 1), or k >= 64 j
   int vec;             // C's rows are 16-byte aligned: two columns per access
   unsigned* status;
 };
@@ -419,23 +420,30 @@ constexpr int kEpiWarps = 16;
 constexpr int kEpiCols = kTN / 4;  // output columns per reading warp
 constexpr int kThreads = (kEpiWarps + 2) * 32;
 
-// beta 2^ex (hi 2^-28 + lo 2^-7(kExact+1) + tail) in six FP64 operations: the integers
-// (|.| < 2^51) become doubles by the bits of 1.5 2^52 + i, the scales by their exponent
-// fields.  Exponents outside +-800 take ldexp.
-template <int kExact>
-__device__ __noinline__ double out_value_far(double dh, double dl, double dt, int ex, double beta) {
-  return beta * (ldexp(dh, ex - kDigitBits * 4) + (ldexp(dl, ex - kDigitBits * (kExact + 1)) + ldexp(dt, ex)));
-}
+__device__ __noinline__ double scale_far(double v, int ex) { return ldexp(v, ex); }
 
+// +-2^ex (hi 2^-28 + lo 2^-7(kExact+1) + tail), rounded once, without FP64 arithmetic (an
+// output tile has 8192 of these; with ldexp and FP64 sums they took longer than a short
+// product's MMAs): the sum in 128-bit fixed point of unit 2^-64 (|hi|, |lo| < 2^51,
+// |tail| < 2^-17), its leading 64 bits rounded to 53, and the exponent field.
 template <int kExact>
-__device__ __forceinline__ double out_value(long long hi, long long lo, uint32_t tail, int ex, double beta) {
-  const double dh = __longlong_as_double(0x4338000000000000ll + hi) - 6755399441055744.0;
-  const double dl = __longlong_as_double(0x4338000000000000ll + lo) - 6755399441055744.0;
-  const double dt = __longlong_as_double((long long)f64_bits(__uint_as_float(tail)));
-  if (ex > 800 || ex < -800) return out_value_far<kExact>(dh, dl, dt, ex, beta);
-  auto pow2 = [](int e) { return __longlong_as_double((long long)(1023 + e) << 52); };
-  const double v = fma(dh, pow2(-kDigitBits * 4), fma(dl, pow2(-kDigitBits * (kExact + 1)), dt));
-  return v * (beta * pow2(ex));
+__device__ __forceinline__ double out_value(long long hi, long long lo, uint32_t tail, int ex, bool negate) {
+  if ((tail & 0x7F800000u) == 0x7F800000u) return __longlong_as_double(0x7FF8000000000000ll);  // an Inf or NaN in
+  const long long tl = __float2ll_rn(__uint_as_float(tail) * 18446744073709551616.0f);
+  const __int128 t = ((__int128)hi << (64 - kDigitBits * 4)) + ((__int128)lo << (64 - kDigitBits * (kExact + 1))) + tl;
+  const unsigned __int128 u = (unsigned __int128)(t < 0 ? -t : t);
+  const unsigned long long up = (unsigned long long)(u >> 64), low = (unsigned long long)u;
+  if ((up | low) == 0ull) return 0.0;
+  const int lz = up ? __clzll((long long)up) : __clzll((long long)low);
+  // the leading 64 bits and their weight: the top one is 2^msb units
+  const unsigned long long m = up ? (lz ? (up << lz) | (low >> (64 - lz)) : up) : low << lz;
+  const int msb = (up ? 127 : 63) - lz;
+  const unsigned long long r = (m >> 11) + ((m >> 10) & 1ull);  // 53 bits, or 2^53
+  const unsigned long long sign = (t < 0) != negate ? 1ull << 63 : 0ull;
+  const int e = msb - 64 + ex;
+  if (e < -1020 || e > 1020)
+    return scale_far(__longlong_as_double((long long)((((unsigned long long)(1022 + msb - 64)) << 52) + r | sign)), ex);
+  return __longlong_as_double((long long)((((unsigned long long)(1022 + e)) << 52) + r | sign));
 }
 
 template <int S>
@@ -453,10 +461,16 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(GemmArgs a) {
   int* committed_out = reinterpret_cast<int*>(tmem_slot + 3);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int row0 = blockIdx.y * kTM, col0 = blockIdx.x * kTN;
+  // tiles with the longest range of k first, so that the last wave is of short ones
+  const int by = a.a_lower ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
+  const int bx = a.b_tri == (int)OzakiTri::kLower ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+  const int row0 = by * kTM, col0 = bx * kTN;
   if (a.lower_only && col0 > row0 + kTM - 1) return;
   int nst = a.nkt;
   if (a.a_lower) nst = min(nst, (row0 + kTM + kKS - 1) / kKS);
+  if (a.b_tri == (int)OzakiTri::kLower) nst = min(nst, (col0 + kTN + kKS - 1) / kKS);
+  const int st0 = a.b_tri == (int)OzakiTri::kUpper ? min(col0 / kKS, nst - 1) : 0;  // first stage
+  nst -= st0;
   const int n_chunks = (nst + kChunkStages - 1) / kChunkStages;
 
   const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kStages);
@@ -489,8 +503,8 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(GemmArgs a) {
   if (warp == kEpiWarps + 1) {
     // producer: two blocks of 64 x 16 for A and one for B per stage
     if (lane == 0) {
-      const uint8_t* pa = a.pa + (long long)(2 * blockIdx.y) * a.nkt * kBStage;
-      const uint8_t* pb = a.pb + (long long)blockIdx.x * a.nkt * kBStage;
+      const uint8_t* pa = a.pa + ((long long)(2 * by) * a.nkt + st0) * kBStage;
+      const uint8_t* pb = a.pb + ((long long)bx * a.nkt + st0) * kBStage;
       int st = 0;
       for (; st < nst && !*abort_flag; ++st) {
         const int b = st % kStages;
@@ -590,7 +604,7 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(GemmArgs a) {
       }
       if (c == n_chunks - 1) {
         // the tail accumulator, then
-        // C = alpha C + beta 2^{e_i + f_j} (acc_hi 2^-28 + acc_lo 2^-7 (kExact + 1) + tail)
+        // C = C or 0, +- 2^{e_i + f_j} (acc_hi 2^-28 + acc_lo 2^-7 (kExact + 1) + tail)
         const int row = row0 + quarter * 32 + lane;
         const int ei = row < a.m ? a.ea[row] : 0;
 #pragma unroll
@@ -606,19 +620,19 @@ __global__ void __launch_bounds__(kThreads, 1) ozaki_gemm_kernel(GemmArgs a) {
               const int j = cb * 16 + i;
               double* cp = a.C + (long long)row * a.ldc + col;
               const bool two = col + 1 < n_ok;
-              const double v0 = out_value<kExact>(acc_hi[j], acc_lo[j], r[i], ei + a.eb[col], a.beta);
+              const double v0 = out_value<kExact>(acc_hi[j], acc_lo[j], r[i], ei + a.eb[col], a.negate);
               const double v1 =
-                  two ? out_value<kExact>(acc_hi[j + 1], acc_lo[j + 1], r[i + 1], ei + a.eb[col + 1], a.beta) : 0.0;
+                  two ? out_value<kExact>(acc_hi[j + 1], acc_lo[j + 1], r[i + 1], ei + a.eb[col + 1], a.negate) : 0.0;
               if (two && a.vec) {
                 double2 c = make_double2(v0, v1);
-                if (a.alpha != 0.0) {
+                if (a.add) {
                   const double2 old = *reinterpret_cast<const double2*>(cp);
-                  c = make_double2(fma(a.alpha, old.x, v0), fma(a.alpha, old.y, v1));
+                  c = make_double2(old.x + v0, old.y + v1);
                 }
                 *reinterpret_cast<double2*>(cp) = c;
               } else {
-                cp[0] = a.alpha == 0.0 ? v0 : fma(a.alpha, cp[0], v0);
-                if (two) cp[1] = a.alpha == 0.0 ? v1 : fma(a.alpha, cp[1], v1);
+                cp[0] = a.add ? cp[0] + v0 : v0;
+                if (two) cp[1] = a.add ? cp[1] + v1 : v1;
               }
             }
           }
@@ -698,7 +712,8 @@ void ozaki_pack(const float* X, long long ld, bool trans, int rows, int k, const
 }
 
 void ozaki_gemm(const OzakiOperand& A, const OzakiOperand& B, int k, double* C, long long ldc, int m, int n,
-                double alpha, double beta, bool lower_only, bool a_lower, unsigned* status, cudaStream_t s) {
+                bool add, bool negate, bool lower_only, bool a_lower, OzakiTri b_tri, unsigned* status,
+                cudaStream_t s) {
   if (m <= 0 || n <= 0 || k <= 0) return;
   GemmArgs g;
   g.pa = A.packed;
@@ -710,10 +725,11 @@ void ozaki_gemm(const OzakiOperand& A, const OzakiOperand& B, int k, double* C, 
   g.ldc = ldc;
   g.m = m;
   g.n = n;
-  g.alpha = alpha;
-  g.beta = beta;
+  g.add = add ? 1 : 0;
+  g.negate = negate ? 1 : 0;
   g.lower_only = lower_only ? 1 : 0;
   g.a_lower = a_lower ? 1 : 0;
+  g.b_tri = (int)b_tri;
   g.vec = ((uintptr_t)C & 15) == 0 && (ldc & 1) == 0;
   g.status = status;
   dim3 grid((n + kTN - 1) / kTN, (m + kTM - 1) / kTM);
@@ -741,8 +757,8 @@ ep_tv_status ozaki_gemm_standalone(const double* A, const double* B, double* C, 
     cudaMemsetAsync(status, 0, sizeof(unsigned), s);
     ozaki_pack(A, k, false, m, k, nullptr, ea, pa, s, slices);
     ozaki_pack(B, k, false, n, k, nullptr, eb, pb, s, slices);
-    ozaki_gemm(OzakiOperand{pa, ea, slices}, OzakiOperand{pb, eb, slices}, k, C, n, m, n, 0.0, 1.0, false, false,
-               status, s);
+    ozaki_gemm(OzakiOperand{pa, ea, slices}, OzakiOperand{pb, eb, slices}, k, C, n, m, n, false, false, false,
+               false, OzakiTri::kNone, status, s);
     if (cudaMemcpyAsync(&h_status, status, sizeof(unsigned), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
       st = EP_TV_ERR_CUDA;

@@ -28,13 +28,18 @@ void ozaki_pack(const double* X, long long ld, bool trans, int rows, int k, cons
                 uint8_t* out, cudaStream_t s, int slices = 8);
 void ozaki_pack(const float* X, long long ld, bool trans, int rows, int k, const double* kscale, int* e,
                 uint8_t* out, cudaStream_t s, int slices = 8);
-// C = alpha C + beta A B^T for packed A (m x k) and B (n x k; may be A); C row-major, ldc.
+// Zeros of the right operand B(j, k): none known, k > j, or k < j.
+enum class OzakiTri { kNone, kLower, kUpper };
+// C = (add ? C : 0) +- A B^T (- when negate) for packed A (m x k) and B (n x k; may be A);
+// C row-major, ldc.
 // With 10 slices k must be at most 8192.
 // lower_only: only entries with col <= row are written.  a_lower: A is lower
-// triangular (row i has no entries beyond k = i), so row tiles stop early.
+// triangular (row i has no entries beyond k = i), so row tiles stop early; b_tri: the
+// same for B, whose column tiles stop early or start late.
 // A timed-out wait raises ST_TIMEOUT in status.
 void ozaki_gemm(const OzakiOperand& A, const OzakiOperand& B, int k, double* C, long long ldc, int m, int n,
-                double alpha, double beta, bool lower_only, bool a_lower, unsigned* status, cudaStream_t s);
+                bool add, bool negate, bool lower_only, bool a_lower, OzakiTri b_tri, unsigned* status,
+                cudaStream_t s);
 // C = A B^T for row-major A (m x k), B (n x k), C (m x n), all device memory,
 // with its own packing buffers (the exported ep_tv_tc_gemm_f64).
 ep_tv_status ozaki_gemm_standalone(const double* A, const double* B, double* C, int m, int n, int k, int slices,

@@ -34,6 +34,7 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "internal.cuh"
@@ -356,7 +357,7 @@ struct CgArgs {
   int fft;               // 1: z = M^{-1} r by the circulant preconditioner, else Jacobi
   unsigned long long* counters;
   int defer_e;           // 1: the update leaves e += alpha p to the next direction kernel
-                         // (or the commit), see fft512_update_rows_fwd_kernel
+                         // (or the commit), see warp_update_rows_fwd_kernel
 };
 
 // d = sum tau_k, n = sum nu_k (k = 1..4), Minv = 1 / (sum k^2 / xi + d); block sums of d.
@@ -1563,10 +1564,23 @@ struct LoopState {
 };
 
 // ---------------------------------------------------------------------------
-// Circulant preconditioner for power-of-two H and W:
+// Circulant preconditioner on a power-of-two torus HP x WP that holds the image:
 //   M = H^T H / xi + dbar I,  dbar = mean(d),  M^{-1} r = F^{-1}[F r / (|h_f|^2 / xi + dbar)].
-// H^T H is circulant, so M differs from Q only by d - dbar on the diagonal; CG
-// on M^{-1} Q needs a few tens of iterations where Jacobi needs hundreds.
+// H^T H is circulant, so for an image of that size M differs from Q only by d - dbar on
+// the diagonal; CG on M^{-1} Q needs a few tens of iterations where Jacobi needs hundreds.
+//
+// Other sizes: z = E^T C^{-1} E r, C the same operator on the HP x WP torus and E the
+// periodic extension of the image into the rest of it under a window.  Along an axis of
+// n pixels padded to P, L = floor((P - n) / 2): positions 0 .. n - 1 hold the image,
+// n .. n + L - 1 its first L pixels again and P - L .. P - 1 its last L (the middle one, if
+// P - n is odd, zero), times weights w that are 1 away from the ends and for the two
+// copies of a pixel near an end sin and cos of one angle rising over 2 L pixels, so that
+// E^T E = I (E^T folds the copies back).  C^{-1} then acts as the image's own circulant up
+// to what its response carries across the window.  The form is symmetric positive
+// definite for any window, as the zero padding before it was (w = 1, no copies), which
+// cut the image at its borders: 300 x 420 at 30 dB took 221, 201 and 165 iterations in
+// its first sweeps, and takes the 72, 65 and 48 of an exact circulant (FP64 emulation;
+// with a margin of 3 pixels, 250 x 250, 163 against 237 and 71).
 // Two real systems share one complex transform (z = r_a + i r_b): the filter is
 // real and even in frequency, so the real and imaginary parts of the result are
 // M^{-1} r_a and M^{-1} r_b.  Rows, then columns (forward, filter, inverse in one
@@ -1584,6 +1598,10 @@ struct FftDesc {
   const double* dbar;
   const float2* tw512;  // exp(-2 pi i m / 512), m < 512 (the 512-point kernels)
   const float2* tw1024; // exp(-2 pi i m / 1024), m < 512 (the 1024-point kernels)
+  const float2* twr;    // twiddles of the rows' and the columns' warp transforms (warp_twiddles)
+  const float2* twc;
+  const float* wr;      // window of the rows (HP) and of the columns (WP), see margin()
+  const float* wc;
   const float* act;  // CG scalars of the current iteration ([4 R], [4 j] = 1 if system j
                      // is active), or NULL: transform every system
   float* scal_w;     // the same array, written: beta of the active systems
@@ -1636,6 +1654,32 @@ __device__ __forceinline__ void loop_step(const FftDesc& f) {
     cudaGraphSetConditional(f.h_inner, (cnt > 0 && f.loop->total < f.max_iter) ? 1u : 0u);
   }
 }
+
+// The image position that position i of the padded axis holds (see above), or -1.
+__device__ __forceinline__ int margin(int i, int n, int P) {
+  if (i < n) return i;
+  const int L = (P - n) >> 1;
+  if (i < n + L) return i - n;
+  return i >= P - L ? i - P + n : -1;
+}
+// Sum over the copies of image position i of get(position): E^T along one axis.
+template <typename Get>
+__device__ __forceinline__ float2 fold(int i, int n, int P, Get get) {
+  float2 v = get(i);
+  const int L = (P - n) >> 1;
+  if (i < L) {
+    const float2 u = get(n + i);
+    v.x += u.x;
+    v.y += u.y;
+  } else if (i >= n - L) {
+    const float2 u = get(i - n + P);
+    v.x += u.x;
+    v.y += u.y;
+  }
+  return v;
+}
+
+__device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -1776,7 +1820,7 @@ __device__ __forceinline__ void stage_loads(float2* s, int total, Get get) {
   }
 }
 
-// Pack two residual planes into complex rows (zero-padded to WP) and transform them.
+// Pack two residual planes into complex rows (extended to WP) and transform them.
 __global__ void __launch_bounds__(kFftThreads, 4) fft_rows_fwd_kernel(FftDesc f, const float* __restrict__ Rr) {
   if (pair_idle(f, blockIdx.y)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0 && f.counters)
@@ -1794,11 +1838,11 @@ __global__ void __launch_bounds__(kFftThreads, 4) fft_rows_fwd_kernel(FftDesc f,
   const bool two = j1 < f.R;
   stage_loads(s, f.rpb * f.WP, [&](int idx) {
     const int rr = idx / f.WP, cc = idx - rr * f.WP;
-    const int row = row0 + rr;
+    const int row = row0 + rr, src = margin(cc, f.W, f.WP);
     float2 v = make_float2(0.f, 0.f);
-    if (row < f.H && cc < f.W) {
-      const long long p = (long long)row * f.W + cc;
-      v = make_float2(r0p[p], two ? r1p[p] : 0.f);
+    if (row < f.H && src >= 0) {
+      const long long p = (long long)row * f.W + src;
+      v = cscale(make_float2(r0p[p], two ? r1p[p] : 0.f), f.wc[cc]);
     }
     return v;
   });
@@ -1813,8 +1857,8 @@ __global__ void __launch_bounds__(kFftThreads, 4) fft_rows_fwd_kernel(FftDesc f,
   }
 }
 
-// Column transforms (rows beyond H are zero), the preconditioner filter and the
-// inverse column transforms; only rows below H are kept.
+// Column transforms (extended to HP rows), the preconditioner filter and the inverse
+// column transforms, folded to H rows.
 __global__ void __launch_bounds__(kFftThreads, 4) fft_cols_filter_kernel(FftDesc f) {
   loop_step(f);
   if (pair_idle(f, blockIdx.y)) return;
@@ -1827,7 +1871,8 @@ __global__ void __launch_bounds__(kFftThreads, 4) fft_cols_filter_kernel(FftDesc
   make_table(tw, f.HP);
   stage_loads(s, f.HP * f.cw, [&](int idx) {
     const int i = idx / f.cw, c = idx - i * f.cw;
-    return i < f.H ? t[(long long)i * f.WP + c0 + c] : make_float2(0.f, 0.f);
+    const int src = margin(i, f.H, f.HP);
+    return src >= 0 ? cscale(t[(long long)src * f.WP + c0 + c], f.wr[i]) : make_float2(0.f, 0.f);
   });
   __syncthreads();
   fft_forward(s, f.HP, f.cw, f.cw, 1, tw);
@@ -1842,11 +1887,12 @@ __global__ void __launch_bounds__(kFftThreads, 4) fft_cols_filter_kernel(FftDesc
   fft_forward(s, f.HP, f.cw, f.cw, 1, tw);
   for (int idx = threadIdx.x; idx < f.H * f.cw; idx += blockDim.x) {
     const int i = idx / f.cw, c = idx - i * f.cw;
-    t[(long long)i * f.WP + c0 + c] = cconj(s[idx]);
+    t[(long long)i * f.WP + c0 + c] =
+        cconj(fold(i, f.H, f.HP, [&](int k) { return cscale(s[k * f.cw + c], f.wr[k]); }));
   }
 }
 
-// Inverse row transforms, scale 1/(HP WP), crop to W, unpack into z planes,
+// Inverse row transforms, scale 1/(HP WP), fold to W, unpack into z planes,
 // partial r.z per system.
 __global__ void __launch_bounds__(kFftThreads, 4) fft_rows_inv_kernel(FftDesc f, const float* __restrict__ Rr,
                                                                       float* Z, double* part_rz) {
@@ -1877,7 +1923,7 @@ __global__ void __launch_bounds__(kFftThreads, 4) fft_rows_inv_kernel(FftDesc f,
       const int row = r0 + rr;
       if (row >= rend) break;
       for (int cc = threadIdx.x; cc < f.W; cc += blockDim.x) {
-        const float2 v = cconj(s[rr * f.WP + cc]);
+        const float2 v = cconj(fold(cc, f.W, f.WP, [&](int k) { return cscale(s[rr * f.WP + k], f.wc[k]); }));
         const long long p = (long long)row * f.W + cc;
         const float z0 = v.x * scale;
         Z[(long long)j0 * N + p] = z0;
@@ -1914,14 +1960,39 @@ __global__ void __launch_bounds__(kFftThreads, 4) fft_rows_inv_kernel(FftDesc f,
 constexpr int kF = 512;
 constexpr int kXs = 578;        // scratch / staged-column pitch in float2
 constexpr int kF512Warps = 8;   // warps per block of the 512-point kernels
-// Rows per warp of the 512-point row passes, one after another; each row's loads
-// are all issued before the transform starts (prefetching the next row during the
-// transform measured slower: it raises register pressure at the 128-register limit).
-constexpr int kRowsPerWarp512 = 4;
+// The row passes take a warp's rows one after another, each row's loads all issued before
+// its transform starts (prefetching the next row during the transform measured slower:
+// it raises register pressure at the 128-register limit).
+
+// The window of one axis (see margin()).
+__global__ void window_kernel(float* w, int n, int P) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= P) return;
+  const int L = (P - n) >> 1, src = margin(i, n, P);
+  double v = src < 0 ? 0.0 : 1.0;
+  if (L > 0 && src >= 0) {
+    // offset from the seam between the image's end and its beginning, -L .. L - 1, on the
+    // side that rises (the copies left of the image and its first L pixels) or falls
+    const int k = i >= P - L ? i - P : i < L ? i : i >= n - L ? i - n : 2 * L;
+    const double t = (k + L + 0.5) / (4.0 * L);
+    if (k < L) v = (i >= P - L || i < L) ? sinpi(t) : cospi(t);
+  }
+  w[i] = (float)v;
+}
 
 // tw[m] = w512^m and tw[512 + m] = w1024^m for m < 512
+constexpr int kTwCount = 2 * kF + 256 + 128 + 64;
 __global__ void tw512_kernel(float2* tw) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  if (m >= 2 * kF && m < kTwCount) {
+    // the tables of the 256-, 128- and 64-point transforms: entry k1 T + t is w_n^(t k1), T = n / 16
+    const int q = m - 2 * kF;
+    const int n = q < 256 ? 256 : q < 384 ? 128 : 64, e = q < 256 ? q : q < 384 ? q - 256 : q - 384;
+    const int T = n / 16, t = e % T, k1 = e / T;
+    float sn, cs;
+    sincospif(-2.0f * (float)((t * k1) % n) / (float)n, &sn, &cs);
+    tw[m] = make_float2(cs, sn);
+  }
   if (m < 2 * kF) {
     float sn, cs;
     if (m < kF)
@@ -1971,9 +2042,10 @@ __device__ __forceinline__ void st_hint(float2* a, float2 v, uint64_t pol) {
                : "memory");
 }
 
-// Which passes take the 512-point kernels (the others take the Stockham ones).
-inline bool fft512_rows(const FftDesc& f) { return f.WP == kF; }
-inline bool fft512_cols(const FftDesc& f) { return f.HP == kF && f.WP >= kF512Warps; }
+// Which passes take the warp transforms of 64 to 512 points (the others take the Stockham
+// ones): a block of the column pass holds 4096 / HP columns.
+inline bool warp_rows(const FftDesc& f) { return f.WP >= 64 && f.WP <= kF; }
+inline bool warp_cols(const FftDesc& f) { return f.HP >= 64 && f.HP <= kF && f.WP >= 4096 / f.HP; }
 // and the 1024-point ones (below)
 inline bool fft1024_rows(const FftDesc& f) { return f.WP == 2 * kF; }
 inline bool fft1024_cols(const FftDesc& f) { return f.HP == 2 * kF && f.WP >= kF512Warps; }
@@ -2024,49 +2096,185 @@ __device__ __forceinline__ void fft512_warp(float2 (&v)[16], float2* xs, const f
   __syncwarp();  // the scratch is free again
 }
 
-// fft_rows_fwd_kernel for WP = 512: one warp per row, rows [blockIdx.x rpb, +rpb).
-__global__ void __launch_bounds__(32 * kF512Warps) fft512_rows_fwd_kernel(FftDesc f,
-                                                                         const float* __restrict__ Rr,
-                                                                         int rpb) {
+// ---- register-resident transforms of 64, 128 and 256 points
+//
+// T = n / 16 lanes hold one transform, 16 elements each (lane t keeps x[T m + t]), so a
+// warp runs 32 / T of them side by side with the registers of the 512-point one:
+//   B_t[k1]      = w_n^(t k1) sum_m x[T m + t] w16^(m k1)      (in a lane)
+//   X[k1 + 16 k2] = sum_t B_t[k1] w_T^(t k2)
+// with one regrouping through the warp's scratch, after which lane t takes k1 = t + T j,
+// j < 16 / T: X[T (16 / T k2 + j) + t], the layout of the input.  For one pass over 17
+// pairs of a 256^2 image the Stockham kernels (passes through shared memory behind block
+// barriers) took 59 us, these 21.
+//
+// Sizes per warp, in float2: kRow, from one transform's regrouping area to the next (entry
+// (k1, t) at k1 (T + 1) + t); kCol, from one staged column to the next in the column pass;
+// kScratch, from one warp's area to the next.  Their residues mod 16 keep the accesses of a
+// half-warp in distinct banks.
+template <int T>
+struct Warp {
+  static constexpr int kN = 16 * T, kPer = 32 / T;
+  static constexpr int kRow = T == 32 ? 0 : T == 16 ? 272 : T == 8 ? 152 : 84;
+  static constexpr int kCol = T == 32 ? 0 : kN + 1;
+  static constexpr int kScratch = T == 32 ? kXs : T == 16 ? 546 : T == 8 ? 612 : 680;
+  static constexpr int kCols = kF512Warps * kPer;  // columns per block of the column pass
+  // rows per block of the row passes: four, one, one, one rounds of the block's warps
+  static constexpr int kRows = T == 32 ? 4 * kF512Warps : kF512Warps * kPer;
+  static_assert(kPer * kRow <= kScratch && kPer * kCol <= kScratch, "scratch");
+};
+
+template <> __device__ __forceinline__ void dft_reg<16>(float2* v) {
+  // 16 = 4 x 4: k = q + 4 s, n = 4 a + b
+  const float c1 = 0.92387953251128675613f, s1 = 0.38268343236508977173f, r2 = 0.70710678118654752440f;
+  float2 c[4][4];
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    float2 u[4] = {v[b], v[4 + b], v[8 + b], v[12 + b]};
+    dft_reg<4>(u);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) c[b][q] = u[q];
+  }
+  // w16^(b q)
+  c[1][1] = cmul(c[1][1], make_float2(c1, -s1));
+  c[1][2] = cmul(c[1][2], make_float2(r2, -r2));
+  c[1][3] = cmul(c[1][3], make_float2(s1, -c1));
+  c[2][1] = cmul(c[2][1], make_float2(r2, -r2));
+  c[2][2] = cmul_mi(c[2][2]);
+  c[2][3] = cmul(c[2][3], make_float2(-r2, -r2));
+  c[3][1] = cmul(c[3][1], make_float2(s1, -c1));
+  c[3][2] = cmul(c[3][2], make_float2(-r2, -r2));
+  c[3][3] = cmul(c[3][3], make_float2(-c1, s1));
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    float2 u[4] = {c[0][q], c[1][q], c[2][q], c[3][q]};
+    dft_reg<4>(u);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[q + 4 * k] = u[k];
+  }
+}
+
+// The warp's forward transforms in place; xs: the warp's scratch; tw: kN entries (natural for
+// T = 32, entry k1 T + t for the others).
+template <int T>
+__device__ __forceinline__ void fft_warp(float2 (&v)[16], float2* xs, const float2* tw) {
+  if constexpr (T == 32) {
+    fft512_warp(v, xs, tw);
+  } else {
+    const int l = threadIdx.x & 31, t = l % T;
+    float2* x = xs + (l / T) * Warp<T>::kRow;
+    dft_reg<16>(v);
+    x[t] = v[0];
+#pragma unroll
+    for (int k1 = 1; k1 < 16; ++k1) x[k1 * (T + 1) + t] = cmul(v[k1], tw[k1 * T + t]);
+    __syncwarp();
+    float2 b[16 / T][T];
+#pragma unroll
+    for (int j = 0; j < 16 / T; ++j)
+#pragma unroll
+      for (int u = 0; u < T; ++u) b[j][u] = x[(t + T * j) * (T + 1) + u];
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 16 / T; ++j) {
+      dft_reg<T>(b[j]);
+#pragma unroll
+      for (int k2 = 0; k2 < T; ++k2) v[16 / T * k2 + j] = b[j][k2];
+    }
+  }
+}
+
+// The extension E along a row held by T lanes (W image columns in place): the copies past
+// column W through the scratch, and the window wc.
+template <int T>
+__device__ __forceinline__ void extend_row(float2 (&v)[16], float2* xs, const float* wc, int W) {
+  constexpr int P = 16 * T;
+  const int l = threadIdx.x & 31, t = l % T, ext = P - W, L = ext >> 1;
+  float2* x = xs + (l / T) * Warp<T>::kRow;
+#pragma unroll
+  for (int m = 0; m < 16; ++m) {
+    const int c = T * m + t;
+    if (c < L) x[c] = v[m];
+    else if (c < W && c >= W - L) x[c - W + ext] = v[m];
+  }
+  __syncwarp();
+#pragma unroll
+  for (int m = 0; m < 16; ++m) {
+    const int c = T * m + t;
+    if (c >= W) v[m] = margin(c, W, P) >= 0 ? x[c - W] : make_float2(0.f, 0.f);
+    v[m] = cscale(v[m], wc[c]);
+  }
+  __syncwarp();
+}
+
+// E^T along a row: the windowed copies added to the image columns they copy.
+template <int T>
+__device__ __forceinline__ void fold_row(float2 (&v)[16], float2* xs, const float* wc, int W) {
+  constexpr int P = 16 * T;
+  const int l = threadIdx.x & 31, t = l % T, ext = P - W, L = ext >> 1;
+  float2* x = xs + (l / T) * Warp<T>::kRow;
+#pragma unroll
+  for (int m = 0; m < 16; ++m) {
+    const int c = T * m + t;
+    v[m] = cscale(v[m], wc[c]);
+    if (c >= W) x[c - W] = v[m];
+  }
+  __syncwarp();
+#pragma unroll
+  for (int m = 0; m < 16; ++m) {
+    const int c = T * m + t;
+    if (c < L) v[m] = cadd(v[m], x[c]);
+    else if (c < W && c >= W - L) v[m] = cadd(v[m], x[c - W + ext]);
+  }
+  __syncwarp();
+}
+
+// fft_rows_fwd_kernel for WP = 16 T: rows [blockIdx.x kRows, + kRows), 32 / T per warp.
+template <int T>
+__global__ void __launch_bounds__(32 * kF512Warps) warp_rows_fwd_kernel(FftDesc f, const float* __restrict__ Rr) {
+  using Wp = Warp<T>;
   if (pair_idle(f, blockIdx.y)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0 && f.counters)
     atomicAdd(&f.counters[DC_CG_PRE_UNITS], 2 * blockIdx.y + 1 < f.R ? 2ull : 1ull);
-  __shared__ float2 tw[kF];
-  __shared__ float2 scratch[kF512Warps][kXs];
-  for (int m = threadIdx.x; m < kF; m += blockDim.x) tw[m] = f.tw512[m];
+  __shared__ float2 tw[Wp::kN];
+  __shared__ float2 scratch[kF512Warps][Wp::kScratch];
+  for (int m = threadIdx.x; m < Wp::kN; m += blockDim.x) tw[m] = f.twr[m];
   __syncthreads();
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, t = l % T;
   const int pair = blockIdx.y;
   const int j0 = 2 * pair, j1 = 2 * pair + 1;
   const bool two = j1 < f.R;
   const long long N = (long long)f.H * f.W;
   const float* r0p = Rr + (long long)j0 * N;
   const float* r1p = Rr + (long long)j1 * N;
-  float2* out = f.tmp + (long long)pair * f.H * kF;
-  const int rend = min(f.H, (blockIdx.x + 1) * rpb);
+  float2* out = f.tmp + (long long)pair * f.H * Wp::kN;
+  const int rend = min(f.H, (int)(blockIdx.x + 1) * Wp::kRows);
   const uint64_t keep = l2_policy_keep();
-  float2 nx[16];  // the row, all loads in flight together
-  auto load_row = [&](int rw) {
-    const long long p0 = (long long)rw * f.W;
-#pragma unroll
-    for (int m = 0; m < 16; ++m) {
-      const int c = 32 * m + l;
-      nx[m] = make_float2(0.f, 0.f);
-      if (c < f.W) nx[m] = make_float2(ld_hint(r0p + p0 + c, keep), two ? ld_hint(r1p + p0 + c, keep) : 0.f);
-    }
-  };
-  for (int row = blockIdx.x * rpb + w; row < rend; row += kF512Warps) {
-    load_row(row);
+  for (int base = blockIdx.x * Wp::kRows + w * Wp::kPer; base < rend; base += kF512Warps * Wp::kPer) {
+    const int row = base + l / T;
+    const bool ok = row < rend;
+    const long long p0 = (long long)row * f.W;
     float2 v[16];
 #pragma unroll
-    for (int m = 0; m < 16; ++m) v[m] = nx[m];
-    fft512_warp(v, scratch[w], tw);
+    for (int m = 0; m < 16; ++m) {
+      const int c = T * m + t;
+      v[m] = make_float2(0.f, 0.f);
+      if (ok && c < f.W) v[m] = make_float2(ld_hint(r0p + p0 + c, keep), two ? ld_hint(r1p + p0 + c, keep) : 0.f);
+    }
+    if (f.W < Wp::kN) extend_row<T>(v, scratch[w], f.wc, f.W);
+    fft_warp<T>(v, scratch[w], tw);
+    if (ok) {
 #pragma unroll
-    for (int m = 0; m < 16; ++m) st_hint(out + (long long)row * kF + 32 * m + l, v[m], keep);
+      for (int m = 0; m < 16; ++m) st_hint(out + (long long)row * Wp::kN + T * m + t, v[m], keep);
+    }
   }
 }
 
-// The CG update fused with the forward row pass (512-point rows): for each system
+// The stopping rule of update_kernel, by the last block of a pair's forward row pass; u: the
+// pair's system, r2: its new r.r.
+__device__ __forceinline__ float still_active(const CgArgs& a, int j, double r2) {
+  return (r2 <= a.thr[j] || r2 > 16.0 * a.rr0[j]) ? 0.f : 1.f;
+}
+
+// The CG update fused with the forward row pass (rows of 64 to 512 points): for each system
 // of the pair that is active when the iteration starts, alpha = r.z / p.q from the
 // direction kernel's partials, e += alpha p and r -= alpha q, exactly as update_kernel
 // forms them; the new residual rows of the pair then go through the forward row
@@ -2079,10 +2287,9 @@ __global__ void __launch_bounds__(32 * kF512Warps) fft512_rows_fwd_kernel(FftDes
 // done by the next direction kernel over its tile, where p is the direction it reads
 // anyway, or by the commit after a system's last iteration; the same operation on the
 // same values, so the results do not change.
-__global__ void __launch_bounds__(32 * kF512Warps, 2) fft512_update_rows_fwd_kernel(FftDesc f,
-                                                                                CgArgs a,
-                                                                                int it_arg,
-                                                                                int rpb) {
+template <int T>
+__global__ void __launch_bounds__(32 * kF512Warps, 2) warp_update_rows_fwd_kernel(FftDesc f, CgArgs a, int it_arg) {
+  using Wp = Warp<T>;
   const int pair = blockIdx.y;
   const int j0 = 2 * pair, j1 = 2 * pair + 1;
   const bool two = j1 < f.R;
@@ -2094,11 +2301,11 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft512_update_rows_fwd_ker
   }
   const int it = a.it_dev ? *a.it_dev : it_arg;
   const bool first = it == 0;  // the correction starts at zero: not read
-  __shared__ float2 tw[kF];
-  __shared__ float2 scratch[kF512Warps][kXs];
+  __shared__ float2 tw[Wp::kN];
+  __shared__ float2 scratch[kF512Warps][Wp::kScratch];
   __shared__ float alpha_s[2];
-  for (int m = threadIdx.x; m < kF; m += blockDim.x) tw[m] = f.tw512[m];
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  for (int m = threadIdx.x; m < Wp::kN; m += blockDim.x) tw[m] = f.twr[m];
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, t = l % T;
   if (w < 2 && (w == 0 ? act0 : act1)) {
     const int j = j0 + w;
     const double pqs = group_sum(a.part_pq + (long long)j * a.nb, a.nb);
@@ -2106,11 +2313,13 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft512_update_rows_fwd_ker
   }
   __syncthreads();
   const long long N = (long long)f.H * f.W;
-  float2* out = f.tmp + (long long)pair * f.H * kF;
-  const int rend = min(f.H, (blockIdx.x + 1) * rpb);
+  float2* out = f.tmp + (long long)pair * f.H * Wp::kN;
+  const int rend = min(f.H, (int)(blockIdx.x + 1) * Wp::kRows);
   const uint64_t keep = l2_policy_keep();
   float rr0 = 0.f, rr1 = 0.f;
-  for (int row = blockIdx.x * rpb + w; row < rend; row += kF512Warps) {
+  for (int base = blockIdx.x * Wp::kRows + w * Wp::kPer; base < rend; base += kF512Warps * Wp::kPer) {
+    const int row = base + l / T;
+    const int cols = row < rend ? f.W : 0;  // columns of this lane's row that exist
     const long long p0 = (long long)row * f.W;
     float2 v[16];
     if (a.defer_e) {
@@ -2123,9 +2332,9 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft512_update_rows_fwd_ker
       float qa[16], ra[16], qb[16], rb[16];
 #pragma unroll
       for (int m = 0; m < 16; ++m) {
-        const int c = 32 * m + l;
+        const int c = T * m + t;
         qa[m] = ra[m] = qb[m] = rb[m] = 0.f;
-        if (c < f.W) {
+        if (c < cols) {
           if (act0) {
             qa[m] = Q0[c];
             ra[m] = R0[c];
@@ -2139,9 +2348,9 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft512_update_rows_fwd_ker
       const float al0 = alpha_s[0], al1 = alpha_s[1];
 #pragma unroll
       for (int m = 0; m < 16; ++m) {
-        const int c = 32 * m + l;
+        const int c = T * m + t;
         v[m] = make_float2(0.f, 0.f);
-        if (c < f.W) {
+        if (c < cols) {
           if (act0) {
             v[m].x = fmaf(-al0, qa[m], ra[m]);
             st_hint_f(R0 + c, v[m].x, keep);
@@ -2156,47 +2365,50 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft512_update_rows_fwd_ker
       }
     } else {
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      if (!(u ? act1 : act0)) {
+      for (int u = 0; u < 2; ++u) {
+        if (!(u ? act1 : act0)) {
 #pragma unroll
-        for (int m = 0; m < 16; ++m) (u ? v[m].y : v[m].x) = 0.f;
-        continue;
-      }
-      const long long o = (long long)(j0 + u) * N + p0;
-      const float* P = ((it & 1) ? a.P2 : a.P) + o;
-      const float* Q = a.Qp + o;
-      float* Ec = a.Ec + o;
-      float* Rr = a.Rr + o;
-      const float alpha = alpha_s[u];
-      float pv[16], qv[16], rv[16], ev[16];
+          for (int m = 0; m < 16; ++m) (u ? v[m].y : v[m].x) = 0.f;
+          continue;
+        }
+        const long long o = (long long)(j0 + u) * N + p0;
+        const float* P = ((it & 1) ? a.P2 : a.P) + o;
+        const float* Q = a.Qp + o;
+        float* Ec = a.Ec + o;
+        float* Rr = a.Rr + o;
+        const float alpha = alpha_s[u];
+        float pv[16], qv[16], rv[16], ev[16];
 #pragma unroll
-      for (int m = 0; m < 16; ++m) {
-        const int c = 32 * m + l;
-        pv[m] = qv[m] = rv[m] = ev[m] = 0.f;
-        if (c < f.W) {
-          pv[m] = P[c];
-          qv[m] = Q[c];
-          rv[m] = Rr[c];
-          if (!first) ev[m] = Ec[c];
+        for (int m = 0; m < 16; ++m) {
+          const int c = T * m + t;
+          pv[m] = qv[m] = rv[m] = ev[m] = 0.f;
+          if (c < cols) {
+            pv[m] = P[c];
+            qv[m] = Q[c];
+            rv[m] = Rr[c];
+            if (!first) ev[m] = Ec[c];
+          }
+        }
+#pragma unroll
+        for (int m = 0; m < 16; ++m) {
+          const int c = T * m + t;
+          float r = 0.f;
+          if (c < cols) {
+            Ec[c] = fmaf(alpha, pv[m], ev[m]);
+            r = fmaf(-alpha, qv[m], rv[m]);
+            st_hint_f(Rr + c, r, keep);
+            if (u) rr1 = fmaf(r, r, rr1); else rr0 = fmaf(r, r, rr0);
+          }
+          (u ? v[m].y : v[m].x) = r;
         }
       }
-#pragma unroll
-      for (int m = 0; m < 16; ++m) {
-        const int c = 32 * m + l;
-        float r = 0.f;
-        if (c < f.W) {
-          Ec[c] = fmaf(alpha, pv[m], ev[m]);
-          r = fmaf(-alpha, qv[m], rv[m]);
-          st_hint_f(Rr + c, r, keep);
-          if (u) rr1 = fmaf(r, r, rr1); else rr0 = fmaf(r, r, rr0);
-        }
-        (u ? v[m].y : v[m].x) = r;
-      }
     }
-    }
-    fft512_warp(v, scratch[w], tw);
+    if (f.W < Wp::kN) extend_row<T>(v, scratch[w], f.wc, f.W);
+    fft_warp<T>(v, scratch[w], tw);
+    if (row < rend) {
 #pragma unroll
-    for (int m = 0; m < 16; ++m) st_hint(out + (long long)row * kF + 32 * m + l, v[m], keep);
+      for (int m = 0; m < 16; ++m) st_hint(out + (long long)row * Wp::kN + T * m + t, v[m], keep);
+    }
   }
   block_sumf<2>(rr0, rr1, 0.f, act0 ? a.part_rr + (long long)j0 * a.nb + blockIdx.x : nullptr,
                 act1 ? a.part_rr + (long long)j1 * a.nb + blockIdx.x : nullptr, nullptr);
@@ -2206,9 +2418,8 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft512_update_rows_fwd_ker
       if (!(u ? act1 : act0)) continue;
       const int j = j0 + u;
       const double r2 = group_sum(a.part_rr + (long long)j * a.nb, gridDim.x);
-      // the stopping rule of update_kernel
       if (threadIdx.x == 0) {
-        a.scal[4 * j] = (r2 <= a.thr[j] || r2 > 16.0 * a.rr0[j]) ? 0.f : 1.f;
+        a.scal[4 * j] = still_active(a, j, r2);
         if (a.defer_e) {
           a.scal[4 * j + 2] = alpha_s[u];
           a.scal[4 * j + 3] = (float)it;
@@ -2218,44 +2429,53 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft512_update_rows_fwd_ker
   }
 }
 
-// fft_cols_filter_kernel for HP = 512: the block takes columns c0 .. c0 + 7 of a
-// pair, stages the 512 x 8 tile in shared memory (64-byte row segments from
-// global memory; rows at and beyond H are zero), and each warp transforms one
-// column in registers, filters it with hthT (the filter stored column-major,
-// [c][i]), transforms again and leaves it in its slot for the block's store.
-__global__ void __launch_bounds__(32 * kF512Warps, 3) fft512_cols_filter_kernel(FftDesc f,
-                                                                            const float* __restrict__ hthT) {
+// fft_cols_filter_kernel for HP = 16 T: the block takes columns [blockIdx.x kCols, + kCols) of
+// a pair, stages the tile in shared memory (row segments of 64 bytes and more from global
+// memory, extended to HP rows), and each group of T lanes transforms one column in
+// registers, filters it with hthT (the filter stored column-major, [c][i]), transforms
+// again and leaves it in its slot for the block's store of the fold to H rows.
+template <int T>
+__global__ void __launch_bounds__(32 * kF512Warps, 3) warp_cols_filter_kernel(FftDesc f,
+                                                                          const float* __restrict__ hthT) {
+  using Wp = Warp<T>;
   loop_step(f);
   if (pair_idle(f, blockIdx.y)) return;
-  __shared__ float2 tw[kF];
-  __shared__ float2 cols[kF512Warps][kXs];
-  for (int m = threadIdx.x; m < kF; m += blockDim.x) tw[m] = f.tw512[m];
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  const int c0 = blockIdx.x * kF512Warps;
-  float2* t = f.tmp + (long long)blockIdx.y * f.H * f.WP;
-  const int cc = threadIdx.x & 7, ro = threadIdx.x >> 3;  // 32 rows x 8 columns per block step
+  __shared__ float2 tw[Wp::kN];
+  __shared__ float2 cols[kF512Warps * Wp::kScratch];
+  for (int m = threadIdx.x; m < Wp::kN; m += blockDim.x) tw[m] = f.twc[m];
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, t = l % T;
+  const int c0 = blockIdx.x * Wp::kCols;
+  float2* tp = f.tmp + (long long)blockIdx.y * f.H * f.WP;
+  constexpr int kStep = 32 * kF512Warps / Wp::kCols;  // rows per round of the block
+  const int cc = threadIdx.x % Wp::kCols, ro = threadIdx.x / Wp::kCols;
+  float2* const slot = cols + (cc / Wp::kPer) * Wp::kScratch + (cc % Wp::kPer) * Wp::kCol;
   const uint64_t keep = l2_policy_keep();
   {
     float2 x[16];  // all of the thread's tile loads in flight at once
 #pragma unroll
     for (int u = 0; u < 16; ++u) {
-      const int i = 32 * u + ro;
-      x[u] = i < f.H ? ld_hint(t + (long long)i * f.WP + c0 + cc, keep) : make_float2(0.f, 0.f);
+      const int src = margin(kStep * u + ro, f.H, Wp::kN);
+      x[u] = src >= 0 ? ld_hint(tp + (long long)src * f.WP + c0 + cc, keep) : make_float2(0.f, 0.f);
+    }
+    if (f.H < Wp::kN) {
+#pragma unroll
+      for (int u = 0; u < 16; ++u) x[u] = cscale(x[u], f.wr[kStep * u + ro]);
     }
 #pragma unroll
-    for (int u = 0; u < 16; ++u) cols[cc][32 * u + ro] = x[u];
+    for (int u = 0; u < 16; ++u) slot[kStep * u + ro] = x[u];
   }
   __syncthreads();
-  float2* xs = cols[w];
-  const float* g = hthT + (long long)(c0 + w) * kF;
+  float2* xs = cols + w * Wp::kScratch;
+  float2* const mine = xs + (l / T) * Wp::kCol;
+  const float* g = hthT + (long long)(c0 + w * Wp::kPer + l / T) * Wp::kN;
   float gv[16];  // the filter column, loaded before the transform
 #pragma unroll
-  for (int m = 0; m < 16; ++m) gv[m] = g[32 * m + l];
+  for (int m = 0; m < 16; ++m) gv[m] = g[T * m + t];
   float2 v[16];
 #pragma unroll
-  for (int m = 0; m < 16; ++m) v[m] = xs[32 * m + l];
+  for (int m = 0; m < 16; ++m) v[m] = mine[T * m + t];
   __syncwarp();
-  fft512_warp(v, xs, tw);
+  fft_warp<T>(v, xs, tw);
   // filter, then the inverse transform as conj(F(conj(.)))
   const float dbar = (float)(*f.dbar);
 #pragma unroll
@@ -2263,69 +2483,68 @@ __global__ void __launch_bounds__(32 * kF512Warps, 3) fft512_cols_filter_kernel(
     const float gi = __frcp_rn(gv[m] + dbar);
     v[m] = make_float2(v[m].x * gi, -v[m].y * gi);
   }
-  fft512_warp(v, xs, tw);
+  fft_warp<T>(v, xs, tw);
 #pragma unroll
-  for (int m = 0; m < 16; ++m) xs[32 * m + l] = cconj(v[m]);
+  for (int m = 0; m < 16; ++m) mine[T * m + t] = cconj(v[m]);
   __syncthreads();
 #pragma unroll
   for (int u = 0; u < 16; ++u) {
-    const int i = 32 * u + ro;
-    if (i < f.H) st_hint(t + (long long)i * f.WP + c0 + cc, cols[cc][i], keep);
+    const int i = kStep * u + ro;
+    if (i < f.H) {
+      const float2 x = f.H < Wp::kN
+                           ? fold(i, f.H, Wp::kN, [&](int k) { return cscale(slot[k], f.wr[k]); })
+                           : slot[i];
+      st_hint(tp + (long long)i * f.WP + c0 + cc, x, keep);
+    }
   }
 }
 
-// fft_rows_inv_kernel for WP = 512: one warp per row of the block's range
-// [blockIdx.x rows_per, +rows_per), rows_per = ceil(H / nbz).
-__global__ void __launch_bounds__(32 * kF512Warps, 2) fft512_rows_inv_kernel(FftDesc f,
-                                                                         const float* __restrict__ Rr,
-                                                                         float* Z, double* part_rz) {
+// fft_rows_inv_kernel for WP = 16 T: rows [blockIdx.x rows_per, + rows_per), rows_per =
+// ceil(H / nbz).
+template <int T>
+__global__ void __launch_bounds__(32 * kF512Warps, 2) warp_rows_inv_kernel(FftDesc f, const float* __restrict__ Rr,
+                                                                       float* Z, double* part_rz) {
+  using Wp = Warp<T>;
   if (pair_idle(f, blockIdx.y)) return;
-  __shared__ float2 tw[kF];
-  __shared__ float2 scratch[kF512Warps][kXs];
-  for (int m = threadIdx.x; m < kF; m += blockDim.x) tw[m] = f.tw512[m];
+  __shared__ float2 tw[Wp::kN];
+  __shared__ float2 scratch[kF512Warps][Wp::kScratch];
+  for (int m = threadIdx.x; m < Wp::kN; m += blockDim.x) tw[m] = f.twr[m];
   __syncthreads();
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, t = l % T;
   const int pair = blockIdx.y;
   const int j0 = 2 * pair, j1 = 2 * pair + 1;
   const bool two = j1 < f.R;
   const long long N = (long long)f.H * f.W;
-  const float scale = 1.0f / ((float)f.HP * (float)kF);
+  const float scale = 1.0f / ((float)f.HP * (float)Wp::kN);
   const int rows_per = (f.H + f.nbz - 1) / f.nbz;
-  const int rend = min(f.H, (blockIdx.x + 1) * rows_per);
-  const float2* tin = f.tmp + (long long)pair * f.H * kF;
+  const int rend = min(f.H, (int)(blockIdx.x + 1) * rows_per);
+  const float2* tin = f.tmp + (long long)pair * f.H * Wp::kN;
   const uint64_t release = l2_policy_release();
   double acc0 = 0.0, acc1 = 0.0;
-  // the row's transform input and both residuals, all loads in flight together
-  float2 nv[16], nr[16];
-  auto load_row = [&](int rw) {
-    const long long p0 = (long long)rw * f.W;
-#pragma unroll
-    for (int m = 0; m < 16; ++m) {
-      nv[m] = cconj(ld_hint(tin + (long long)rw * kF + 32 * m + l, release));
-      const int c = 32 * m + l;
-      nr[m] = make_float2(0.f, 0.f);
-      if (c < f.W) {
-        nr[m].x = ld_hint(Rr + (long long)j0 * N + p0 + c, release);
-        if (two) nr[m].y = ld_hint(Rr + (long long)j1 * N + p0 + c, release);
-      }
-    }
-  };
-  int row = blockIdx.x * rows_per + w;
-  for (; row < rend; row += kF512Warps) {
-    load_row(row);
+  for (int base = blockIdx.x * rows_per + w * Wp::kPer; base < rend; base += kF512Warps * Wp::kPer) {
+    const int row = base + l / T;
+    const bool ok = row < rend;
+    const int cols = ok ? f.W : 0;
     const long long p0 = (long long)row * f.W;
+    // the row's transform input and both residuals, all loads in flight together
     float2 v[16], rr[16];
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
-      v[m] = nv[m];
-      rr[m] = nr[m];
+      const int c = T * m + t;
+      v[m] = rr[m] = make_float2(0.f, 0.f);
+      if (ok) v[m] = cconj(ld_hint(tin + (long long)row * Wp::kN + c, release));
+      if (c < cols) {
+        rr[m].x = ld_hint(Rr + (long long)j0 * N + p0 + c, release);
+        if (two) rr[m].y = ld_hint(Rr + (long long)j1 * N + p0 + c, release);
+      }
     }
-    fft512_warp(v, scratch[w], tw);
+    fft_warp<T>(v, scratch[w], tw);
+    if (f.W < Wp::kN) fold_row<T>(v, scratch[w], f.wc, f.W);
     float rz0 = 0.f, rz1 = 0.f;
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
-      const int c = 32 * m + l;
-      if (c < f.W) {
+      const int c = T * m + t;
+      if (c < cols) {
         const long long p = p0 + c;
         const float z0 = v[m].x * scale;
         Z[(long long)j0 * N + p] = z0;
@@ -2344,6 +2563,24 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft512_rows_inv_kernel(Fft
              two ? part_rz + (long long)j1 * f.nbz + blockIdx.x : nullptr, nullptr);
   rz_tail(f, pair, part_rz);
 }
+
+// Runs fn<T>() for the transform length n = 16 T.
+template <typename Fn>
+inline void with_warp(int n, Fn&& fn) {
+  switch (n) {
+    case 64: fn(std::integral_constant<int, 4>()); return;
+    case 128: fn(std::integral_constant<int, 8>()); return;
+    case 256: fn(std::integral_constant<int, 16>()); return;
+    default: fn(std::integral_constant<int, 32>()); return;
+  }
+}
+inline int warp_rows_per_block(int n) {
+  int r = 0;
+  with_warp(n, [&](auto t) { r = Warp<decltype(t)::value>::kRows; });
+  return r;
+}
+// Where the table of the n-point transform lies in the twiddle buffer (tw512_kernel).
+inline int warp_twiddles(int n) { return n == 512 ? 0 : n == 256 ? 2 * kF : n == 128 ? 2 * kF + 256 : 2 * kF + 384; }
 
 // ---- register-resident 1024-point transforms
 //
@@ -2398,10 +2635,12 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_rows_fwd_kernel(Ff
     float2 lo[16], hi[16];
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
-      const int c = 32 * q + l, c2 = c + kF;
-      lo[q] = hi[q] = make_float2(0.f, 0.f);
-      if (c < f.W) lo[q] = make_float2(ld_hint(r0p + p0 + c, keep), two ? ld_hint(r1p + p0 + c, keep) : 0.f);
-      if (c2 < f.W) hi[q] = make_float2(ld_hint(r0p + p0 + c2, keep), two ? ld_hint(r1p + p0 + c2, keep) : 0.f);
+      const int c = 32 * q + l, c2 = c + kF;  // W > 512: c is an image column
+      lo[q] = cscale(make_float2(ld_hint(r0p + p0 + c, keep), two ? ld_hint(r1p + p0 + c, keep) : 0.f), f.wc[c]);
+      const int src = margin(c2, f.W, 2 * kF);
+      hi[q] = make_float2(0.f, 0.f);
+      if (src >= 0)
+        hi[q] = cscale(make_float2(ld_hint(r0p + p0 + src, keep), two ? ld_hint(r1p + p0 + src, keep) : 0.f), f.wc[c2]);
     }
     fft1024_warp(lo, hi, scratch[w], tw, tw2);
 #pragma unroll
@@ -2409,7 +2648,7 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_rows_fwd_kernel(Ff
   }
 }
 
-// fft512_update_rows_fwd_kernel for WP = 1024, deferred correction updates only
+// warp_update_rows_fwd_kernel for WP = 1024, deferred correction updates only
 // (a.defer_e): r -= alpha q per active system of the pair, the new residual rows
 // transformed without a re-read; the pair's last block sets the active flags, alpha
 // and the iteration.  A row's loads go in four batches of eight columns per lane.
@@ -2495,6 +2734,28 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_update_rows_fwd_ke
           hi[8 * (b - 2) + qq] = v;
       }
     }
+    if (f.W < 2 * kF) {
+      // the copies of the row's ends (all columns below 512 are image columns, the copies
+      // are above): each passes through the scratch at its place past column W
+      float2* xs = scratch[w];
+      const int W = f.W, ext = 2 * kF - W, L = ext >> 1;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        const int c = 32 * q + l, c2 = c + kF;
+        if (c < L) xs[c] = lo[q];
+        if (c >= W - L) xs[c - W + ext] = lo[q];
+        if (c2 >= W - L && c2 < W) xs[c2 - W + ext] = hi[q];
+        lo[q] = cscale(lo[q], f.wc[c]);
+      }
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        const int c2 = 32 * q + l + kF;
+        if (c2 >= W) hi[q] = margin(c2, W, 2 * kF) >= 0 ? xs[c2 - W] : make_float2(0.f, 0.f);
+        hi[q] = cscale(hi[q], f.wc[c2]);
+      }
+      __syncwarp();
+    }
     fft1024_warp(lo, hi, scratch[w], tw, tw2);
 #pragma unroll
     for (int m = 0; m < 16; ++m) st_hint4(out + (long long)row * (2 * kF) + 64 * m + 2 * l, lo[m], hi[m], keep);
@@ -2518,10 +2779,10 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_update_rows_fwd_ke
 }
 
 // fft_cols_filter_kernel for HP = 1024: the block stages columns c0 .. c0 + 7 of a pair
-// (rows at and beyond H are zero); each warp transforms one column, filters it with
+// (extended to 1024 rows); each warp transforms one column, filters it with
 // hthT (column-major, [c][i]), writes it back to its slot in natural order and
-// transforms it again (the inverse as conj(F(conj(.)))); the block then stores rows
-// below H.  Shared memory: kF512Warps x kXs2 float2, dynamic.
+// transforms it again (the inverse as conj(F(conj(.)))); the block then stores the fold
+// to H rows.  Shared memory: kF512Warps x kXs2 float2, dynamic.
 __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_cols_filter_kernel(FftDesc f,
                                                                              const float* __restrict__ hthT) {
   loop_step(f);
@@ -2544,10 +2805,14 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_cols_filter_kernel
 #pragma unroll
     for (int u = 0; u < 16; ++u) {
       const int i = 32 * (16 * h + u) + ro;
-      x[u] = i < f.H ? ld_hint(t + (long long)i * f.WP + c0 + cc, keep) : make_float2(0.f, 0.f);
+      const int src = margin(i, f.H, 2 * kF);
+      x[u] = src >= 0 ? ld_hint(t + (long long)src * f.WP + c0 + cc, keep) : make_float2(0.f, 0.f);
     }
 #pragma unroll
-    for (int u = 0; u < 16; ++u) cols[cc * kXs2 + 32 * (16 * h + u) + ro] = x[u];
+    for (int u = 0; u < 16; ++u) {
+      const int i = 32 * (16 * h + u) + ro;
+      cols[cc * kXs2 + i] = cscale(x[u], f.wr[i]);
+    }
   }
   __syncthreads();
   float2* xs = cols + w * kXs2;
@@ -2590,7 +2855,9 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_cols_filter_kernel
 #pragma unroll
   for (int u = 0; u < 32; ++u) {
     const int i = 32 * u + ro;
-    if (i < f.H) st_hint(t + (long long)i * f.WP + c0 + cc, cols[cc * kXs2 + i], keep);
+    if (i < f.H)
+      st_hint(t + (long long)i * f.WP + c0 + cc,
+              fold(i, f.H, 2 * kF, [&](int k) { return cscale(cols[cc * kXs2 + k], f.wr[k]); }), keep);
   }
 }
 
@@ -2630,6 +2897,33 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_rows_inv_kernel(Ff
       hi[q] = cconj(ld_hint(trow + kF + 32 * q + l, release));
     }
     fft1024_warp(lo, hi, scratch[w], tw, tw2);
+    if (f.W < 2 * kF) {
+      // fold: columns from W on pass through the scratch to the image column they copy
+      float2* xs = scratch[w];
+      const int W = f.W, ext = 2 * kF - W, L = ext >> 1;
+#pragma unroll
+      for (int m = 0; m < 16; ++m) {
+        const int c = 64 * m + 2 * l;
+        lo[m] = cscale(lo[m], f.wc[c]);
+        hi[m] = cscale(hi[m], f.wc[c + 1]);
+        if (c >= W) xs[c - W] = lo[m];
+        if (c + 1 >= W) xs[c + 1 - W] = hi[m];
+      }
+      __syncwarp();
+#pragma unroll
+      for (int m = 0; m < 16; ++m) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int c = 64 * m + 2 * l + e;
+          float2& v = e ? hi[m] : lo[m];
+          if (c < W) {
+            if (c < L) v = cadd(v, xs[c]);
+            if (c >= W - L) v = cadd(v, xs[c - W + ext]);
+          }
+        }
+      }
+      __syncwarp();
+    }
     // lo[m], hi[m]: columns 64 m + 2 l and 64 m + 2 l + 1; the residuals there are read
     // in two halves of eight m each
     float rz0 = 0.f, rz1 = 0.f;
@@ -2974,7 +3268,8 @@ struct LikelihoodState {
   float2* ftmp = nullptr;
   float* Z = nullptr;
   float* hth = nullptr;
-  float2* tw512 = nullptr;      // w512^m, then w1024^m (m < 512)
+  float2* tw512 = nullptr;      // w512^m, w1024^m (m < 512), the tables of the shorter transforms
+  float* window = nullptr;      // the windows of the rows (HP), then of the columns (WP)
   double* dpart = nullptr;
   double* dbar = nullptr;
   int prep_blocks = 0;
@@ -3081,37 +3376,47 @@ void precond_apply(LikelihoodState* L, double* rz_buf, bool cg, int first,
   f.arrive = L->d_arrive + L->R;
   f.first = first;
   f.counters = counters;
-  constexpr int kRows512 = kF512Warps * kRowsPerWarp512;
   constexpr int kRows1024 = kF512Warps * kRowsPerWarp1024;
+  constexpr int kWt = 32 * kF512Warps;
   if (stages & 1) {
-    if (upd && fft1024_rows(f))
-      fft1024_update_rows_fwd_kernel<<<dim3((f.H + kRows1024 - 1) / kRows1024, f.pairs),
-                                       32 * kF512Warps, 0, s>>>(f, *upd, it, kRows1024);
-    else if (upd)
-      fft512_update_rows_fwd_kernel<<<dim3((f.H + kRows512 - 1) / kRows512, f.pairs),
-                                      32 * kF512Warps, 0, s>>>(f, *upd, it, kRows512);
-    else if (fft512_rows(f))
-      fft512_rows_fwd_kernel<<<dim3((f.H + kRows512 - 1) / kRows512, f.pairs), 32 * kF512Warps, 0,
-                               s>>>(f, L->Rr, kRows512);
-    else if (fft1024_rows(f))
-      fft1024_rows_fwd_kernel<<<dim3((f.H + kRows1024 - 1) / kRows1024, f.pairs), 32 * kF512Warps,
-                                0, s>>>(f, L->Rr, kRows1024);
-    else
+    if (warp_rows(f)) {
+      with_warp(f.WP, [&](auto t) {
+        constexpr int T = decltype(t)::value;
+        const dim3 grid((f.H + Warp<T>::kRows - 1) / Warp<T>::kRows, f.pairs);
+        if (upd)
+          warp_update_rows_fwd_kernel<T><<<grid, kWt, 0, s>>>(f, *upd, it);
+        else
+          warp_rows_fwd_kernel<T><<<grid, kWt, 0, s>>>(f, L->Rr);
+      });
+    } else if (fft1024_rows(f)) {
+      const dim3 grid((f.H + kRows1024 - 1) / kRows1024, f.pairs);
+      if (upd)
+        fft1024_update_rows_fwd_kernel<<<grid, kWt, 0, s>>>(f, *upd, it, kRows1024);
+      else
+        fft1024_rows_fwd_kernel<<<grid, kWt, 0, s>>>(f, L->Rr, kRows1024);
+    } else {
       fft_rows_fwd_kernel<<<dim3((f.H + f.rpb - 1) / f.rpb, f.pairs), kFftThreads, L->smem_rows,
                             s>>>(f, L->Rr);
+    }
   }
   if (!(stages & 2)) return;
-  if (fft512_cols(f))
-    fft512_cols_filter_kernel<<<dim3(f.WP / kF512Warps, f.pairs), 32 * kF512Warps, 0, s>>>(f, f.hth);
+  if (warp_cols(f))
+    with_warp(f.HP, [&](auto t) {
+      constexpr int T = decltype(t)::value;
+      warp_cols_filter_kernel<T><<<dim3(f.WP / Warp<T>::kCols, f.pairs), kWt, 0, s>>>(f, f.hth);
+    });
   else if (fft1024_cols(f))
-    fft1024_cols_filter_kernel<<<dim3(f.WP / kF512Warps, f.pairs), 32 * kF512Warps,
-                                 sizeof(float2) * kF512Warps * kXs2, s>>>(f, f.hth);
+    fft1024_cols_filter_kernel<<<dim3(f.WP / kF512Warps, f.pairs), kWt, sizeof(float2) * kF512Warps * kXs2, s>>>(
+        f, f.hth);
   else
     fft_cols_filter_kernel<<<dim3(f.WP / f.cw, f.pairs), kFftThreads, L->smem_cols, s>>>(f);
-  if (fft512_rows(f))
-    fft512_rows_inv_kernel<<<dim3(f.nbz, f.pairs), 32 * kF512Warps, 0, s>>>(f, L->Rr, L->Z, rz_buf);
+  if (warp_rows(f))
+    with_warp(f.WP, [&](auto t) {
+      constexpr int T = decltype(t)::value;
+      warp_rows_inv_kernel<T><<<dim3(f.nbz, f.pairs), kWt, 0, s>>>(f, L->Rr, L->Z, rz_buf);
+    });
   else if (fft1024_rows(f))
-    fft1024_rows_inv_kernel<<<dim3(f.nbz, f.pairs), 32 * kF512Warps, 0, s>>>(f, L->Rr, L->Z, rz_buf);
+    fft1024_rows_inv_kernel<<<dim3(f.nbz, f.pairs), kWt, 0, s>>>(f, L->Rr, L->Z, rz_buf);
   else
     fft_rows_inv_kernel<<<dim3(f.nbz, f.pairs), kFftThreads, L->smem_rows, s>>>(f, L->Rr, L->Z,
                                                                                 rz_buf);
@@ -3164,10 +3469,10 @@ void launch_direction(const LikelihoodState* L, const CgArgs& a, int it, cudaStr
 }
 
 // Whether a CG iteration runs its update inside the preconditioner's forward row
-// pass (fft512_update_rows_fwd_kernel; for 1024-point rows, which take deferred
+// pass (warp_update_rows_fwd_kernel; for 1024-point rows, which take deferred
 // correction updates only, fft1024_update_rows_fwd_kernel) instead of update_kernel.
 inline bool fused_update(const LikelihoodState* L) {
-  return L->fft && (fft512_rows(L->fd) || (fft1024_rows(L->fd) && pair_direction(L)));
+  return L->fft && (warp_rows(L->fd) || (fft1024_rows(L->fd) && pair_direction(L)));
 }
 
 // ---- launch-shape tuning of the FFT preconditioner
@@ -3202,7 +3507,7 @@ void tune_fft_shape(LikelihoodState* L, cudaStream_t s) {
   const char* env = getenv("EPTV_FFT_TUNE");
   if (env && env[0] == '0') return;
   FftDesc& f = L->fd;
-  if ((fft512_rows(f) || fft1024_rows(f)) && (fft512_cols(f) || fft1024_cols(f)))
+  if ((warp_rows(f) || fft1024_rows(f)) && (warp_cols(f) || fft1024_cols(f)))
     return;  // the tuned shapes are not used
   int dev = 0;
   cudaGetDevice(&dev);
@@ -3424,13 +3729,9 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
     const int cap = kFftMaxItems * kFftThreads;
     f.rpb = std::max(1, std::min({HP, 4096 / WP, cap * rmin(WP) / WP}));
     f.cw = std::max(1, std::min({WP, 16, cap * rmin(HP) / HP}));
-    // r.z partials: one per block of the inverse row pass (kF512Warps * kRowsPerWarp512
-    // rows each for 512-point rows)
-    constexpr int kRowsInv512 = kF512Warps * kRowsPerWarp512;
-    constexpr int kRowsInv1024 = kF512Warps * kRowsPerWarp1024;
-    f.nbz = WP == kF       ? (c.H + kRowsInv512 - 1) / kRowsInv512
-            : WP == 2 * kF ? (c.H + kRowsInv1024 - 1) / kRowsInv1024
-                           : std::min(c.H, 64);
+    // r.z partials: one per block of the inverse row pass
+    const int rows_inv = warp_rows(f) ? warp_rows_per_block(WP) : kF512Warps * kRowsPerWarp1024;
+    f.nbz = warp_rows(f) || fft1024_rows(f) ? (c.H + rows_inv - 1) / rows_inv : std::min(c.H, 64);
     L->nbz = f.nbz;
     L->smem_rows = sizeof(float2) * ((size_t)WP + (size_t)f.rpb * WP);
     L->smem_cols = sizeof(float2) * ((size_t)HP + (size_t)HP * f.cw);
@@ -3475,7 +3776,8 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
              (cudaMalloc(&L->ftmp, sizeof(float2) * ((L->R + 1) / 2) * c.H * L->fd.WP) == cudaSuccess &&
               cudaMalloc(&L->Z, sizeof(float) * RN) == cudaSuccess &&
               cudaMalloc(&L->hth, sizeof(float) * L->fd.HP * L->fd.WP) == cudaSuccess &&
-              cudaMalloc(&L->tw512, sizeof(float2) * 2 * kF) == cudaSuccess)) &&
+              cudaMalloc(&L->tw512, sizeof(float2) * kTwCount) == cudaSuccess &&
+              cudaMalloc(&L->window, sizeof(float) * (L->fd.HP + L->fd.WP)) == cudaSuccess)) &&
             cudaMalloc(&L->d_active, sizeof(int)) == cudaSuccess &&
             cudaMalloc(&L->d_relres, sizeof(double) * L->R) == cudaSuccess &&
             cudaMalloc(&L->d_prev_rr, sizeof(double) * L->R) == cudaSuccess &&
@@ -3554,11 +3856,17 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
     L->fd.hth = L->hth;
     L->fd.tw512 = L->tw512;
     L->fd.tw1024 = L->tw512 + kF;
-    tw512_kernel<<<(2 * kF + 255) / 256, 256, 0, s>>>(L->tw512);
+    L->fd.twr = L->tw512 + warp_twiddles(L->fd.WP);
+    L->fd.twc = L->tw512 + warp_twiddles(L->fd.HP);
+    L->fd.wr = L->window;
+    L->fd.wc = L->window + L->fd.HP;
+    tw512_kernel<<<(kTwCount + 255) / 256, 256, 0, s>>>(L->tw512);
+    window_kernel<<<(L->fd.HP + 255) / 256, 256, 0, s>>>(L->window, c.H, L->fd.HP);
+    window_kernel<<<(L->fd.WP + 255) / 256, 256, 0, s>>>(L->window + L->fd.HP, c.W, L->fd.WP);
     L->fd.dbar = L->dbar;
     hth_kernel<<<grid1d((long long)L->fd.HP * L->fd.WP), 256, 0, s>>>(
         L->hth, L->fd.HP, L->fd.WP, L->d_k, kh, kw, L->inv_xi,
-        (fft512_cols(L->fd) || fft1024_cols(L->fd)) ? 1 : 0);
+        (warp_cols(L->fd) || fft1024_cols(L->fd)) ? 1 : 0);
   }
   // H^T y / xi
   conv_t_kernel<<<dim3(grid1d(N), 1), 256, 0, s>>>(cfg.y, L->Hty, c.H, c.W, L->d_k, kh, kw,
@@ -3611,6 +3919,7 @@ void likelihood_destroy(LikelihoodState* L) {
   cudaFree(L->dbar);
   cudaFree(L->ftmp);
   cudaFree(L->tw512);
+  cudaFree(L->window);
   cudaFree(L->Z);
   cudaFree(L->hth);
   cudaFree(L->d_active);

@@ -249,3 +249,113 @@ def test_deconv_mog2_prior_parity_and_no_em():
     mu_r, var_r, capped_r = mog2_oracle_run(p, y32(p), pr)
     assert_parity(mu, var, mu_r, var_r, p.y)
     assert abs(capped - capped_r) <= max(4, 0.01 * capped_r), (capped, capped_r)
+
+
+@pytest.mark.parametrize("h,w,periodic", [(60, 60, 1), (64, 128, 1), (33, 67, 0), (100, 250, 1), (131, 256, 0),
+                                          (256, 40, 1), (300, 130, 1), (30, 511, 0), (520, 66, 1), (62, 1000, 1)])
+def test_deconv_parity_transform_sizes(h, w, periodic):
+    """Every length of the preconditioner's warp transforms (64 to 512 points) along rows
+    and columns, with 1024 and the shared-memory ones, with margins from none to
+    nearly half the transform, even and odd; the oracle solves by FP64 CG."""
+    p = syn.deconv_problem(h, w, kernel=syn.uniform_kernel(5), bsnr_db=30.0, beta0=2.0, seed=h + w,
+                           grf_length=8.0)
+    S = 3
+    pr = probes(p, S, 52)
+    mu, var, ep = _gpu(p, 2, S, pr, periodic=periodic)
+    o = EPOracle("deconv", y32(p), p.xi, p.beta, h, w, kernel=p.kernel, site0="rbmc_cg", probes=pr,
+                 periodic=bool(periodic))
+    o.run(2)
+    assert_parity(mu, var, *o.posterior(), p.y)
+    ep.close()
+
+
+def _emulated_iterations(p, pr, d, ncav, rtol, eta=3.2e-5):
+    """Iterations of the first likelihood update (zero start): refinement passes of FP32 CG
+    preconditioned by the windowed periodic extension into the power-of-two torus, all
+    systems in step, each pass down to max(eta |r|, rtol |b| / 2).  In FP32 as on the GPU:
+    on these systems (flat regions have d near 1e-7) rounding costs CG iterations."""
+    import scipy.fft as sf
+    f4 = np.float32
+    h, w = p.y.shape
+
+    def axis(n):
+        P = 2
+        while P < n:
+            P *= 2
+        L = (P - n) // 2
+        i = np.arange(P)
+        src = np.where(i < n, i, np.where(i < n + L, i - n, np.where(i >= P - L, i - P + n, -1)))
+        wgt = (src >= 0).astype(float)
+        for k in range(-L, L):
+            t = np.pi / 2 * (k + L + 0.5) / (2 * L)
+            wgt[k % P] = np.sin(t)
+            wgt[n + k] = np.cos(t)
+        E = np.zeros((P, n))
+        E[i[src >= 0], src[src >= 0]] = wgt[src >= 0]
+        assert np.allclose(E.T @ E, np.eye(n))
+        return E
+
+    Er, Ec = axis(h), axis(w)
+    Er4, Ec4 = Er.astype(f4), Ec.astype(f4)
+    k = p.kernel
+    pad = np.zeros((Er.shape[0], Ec.shape[0]))
+    pad[:k.shape[0], :k.shape[1]] = k
+    filt = (1.0 / (np.abs(np.fft.fft2(pad)) ** 2 / p.xi + d.mean())).astype(f4)
+    conv, conv_t = operators.conv_periodic, operators.conv_periodic_t
+    d4 = d.astype(f4)
+    gr, gc = (np.correlate(v, v, "full").astype(f4) for v in (k.sum(axis=1), k.sum(axis=0) / k.sum()))
+
+    def stencil(v):
+        out = v
+        for ax, g in ((1, gc), (0, gr)):
+            out = sum(g[i] * np.roll(out, i - len(g) // 2, axis=ax) for i in range(len(g)))
+        return out
+
+    def M(r):
+        return Er4.T @ sf.ifft2(sf.fft2(Er4 @ r @ Ec4.T) * filt).real @ Ec4
+
+    bs = [conv_t(p.y, k) / p.xi + ncav]
+    for e1, e2 in zip(*pr):
+        bs.append(conv_t(e1.reshape(h, w), k) / np.sqrt(p.xi) + np.sqrt(d) * e2.reshape(h, w))
+    tols = [rtol] + [max(rtol, 1e-6)] * (len(bs) - 1)
+    total = 0
+    for b, tol in zip(bs, tols):
+        r = b.astype(f4)
+        nb = np.linalg.norm(b)
+        stop, z, it = max(eta, 0.5 * tol) * nb, M(r), 0
+        q, rz = z, np.sum(r * z, dtype=np.float64)
+        while np.linalg.norm(r) > stop:
+            aq = stencil(q) * f4(1.0 / p.xi) + d4 * q
+            al = f4(rz / np.sum(q * aq, dtype=np.float64))
+            r = r - al * aq
+            z = M(r)
+            rz, old = np.sum(r * z, dtype=np.float64), rz
+            q = z + f4(rz / old) * q
+            it += 1
+        assert r.dtype == f4
+        total = max(total, it)
+    return total
+
+
+@pytest.mark.parametrize("h,w,periodic", [(76, 108, 1), (45, 99, 0), (40, 140, 1), (128, 64, 1), (24, 600, 1)])
+def test_preconditioner_iterations_are_those_of_the_windowed_extension(h, w, periodic):
+    """The preconditioner shows in the iteration count alone: the count of the first
+    likelihood update is that of the FP64 emulation.  The tolerance is one that a single
+    refinement pass meets (at 1e-9 the FP32 floor decides how many passes follow); FP32
+    rounding moves a pass by an iteration or two."""
+    p = syn.deconv_problem(h, w, kernel=syn.uniform_kernel(5), bsnr_db=30.0, beta0=2.0, seed=3, grf_length=8.0)
+    p.y = p.y.astype(np.float32).astype(np.float64)
+    S = 1
+    pr = probes(p, S, 53)
+    torch = cuda()
+    # a stream of its own: the update runs as a graph, whose loop counts iterations one by
+    # one (the host-driven loop launches them in fours)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        _, _, ep = _gpu(p, 1, S, pr, periodic=periodic, cg_rtol=1e-4, stream=stream)
+        its = ep.stats()["cg_iters"]
+        assert ep.solver_report()["passes"] == 1
+        tau, nu = (t.cpu().numpy().astype(np.float64) for t in ep.sites())
+        ep.close()
+    ref = _emulated_iterations(p, pr, tau[1:].sum(axis=0), nu[1:].sum(axis=0), rtol=1e-4)
+    assert abs(its - ref) <= 3 + 0.1 * ref, (its, ref)

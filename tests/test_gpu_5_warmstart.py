@@ -179,3 +179,40 @@ def test_trained_network_against_cold_start_and_control():
     assert None not in (cold["sweeps"], warm["sweeps"], ctrl["sweeps"]), r
     assert warm["sweeps"] < ctrl["sweeps"] < cold["sweeps"], r
     assert warm["seconds"] < 0.1 * cold["seconds"] and ctrl["seconds"] < 0.1 * cold["seconds"], r
+
+
+@pytest.mark.parametrize("n,cin,cout,h,w,relu", [(1, 9, 8, 17, 31, 1), (2, 8, 9, 16, 32, 1), (1, 33, 17, 9, 36, 1),
+                                                 (2, 4, 16, 15, 33, 0), (1, 32, 31, 2, 64, 1), (1, 1, 1, 1, 1, 1),
+                                                 (170, 3, 6, 16, 16, 1)])
+def test_conv_tile_edges(n, cin, cout, h, w, relu):
+    """Sizes at the edges of the convolution's tiles and stages: widths with and without
+    whole float4 rows, one off the 32 x 8 and 32 x 16 tiles, channel counts one off the
+    staged four and eight, the output groups of 8, 16 and 32, more input channels than one
+    block's gradient holds, and more gradient tiles than blocks."""
+    torch = cuda()
+    from paper_2110_01585_gb300 import _lib
+    lib = _lib.load()
+    rng = np.random.default_rng(n + 7 * cin + h)
+    x = rng.standard_normal((n, cin, h, w)).astype(np.float32)
+    wt = (rng.standard_normal((cout, cin, 3, 3)) / math.sqrt(cin * 9)).astype(np.float32)
+    b = rng.standard_normal(cout).astype(np.float32)
+    dy = rng.standard_normal((n, cout, h, w)).astype(np.float32)
+    z = cnn.conv3x3(x.astype(np.float64), wt.astype(np.float64), b.astype(np.float64))
+    yref = np.maximum(z, 0.0) if relu else z
+    xd, wd, bd, dyd = _t(torch, x), _t(torch, wt), _t(torch, b), _t(torch, dy)
+    yd = torch.empty((n, cout, h, w), dtype=torch.float32, device="cuda")
+    s = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    P = lambda t: ctypes.c_void_p(t.data_ptr()) if t is not None else ctypes.c_void_p()
+    assert lib.ep_tv_conv3x3_forward(n, cin, cout, h, w, P(xd), P(wd), P(bd), relu, P(yd), s) == 0
+    _close(yd.cpu().numpy(), yref)
+    work = torch.full((lib.ep_tv_conv3x3_backward_work(n, cin, cout, h, w) // 4 + 1,), float("nan"), device="cuda")
+    dx = torch.empty_like(xd) if cin <= 32 else None
+    dw, db = torch.empty_like(wd), torch.empty_like(bd)
+    assert lib.ep_tv_conv3x3_backward(n, cin, cout, h, w, P(xd), P(wd), P(yd if relu else None), P(dyd), P(dx),
+                                      P(dw), P(db), P(work), ctypes.c_size_t(work.numel() * 4), s) == 0
+    g = np.where(yd.cpu().numpy() > 0, dy, 0.0) if relu else dy
+    dxr, dwr, dbr = cnn.conv3x3_backward(x.astype(np.float64), wt.astype(np.float64), g.astype(np.float64))
+    _close(dw.cpu().numpy(), dwr)
+    _close(db.cpu().numpy(), dbr)
+    if dx is not None:
+        _close(dx.cpu().numpy(), dxr)

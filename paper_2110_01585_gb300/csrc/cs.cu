@@ -379,16 +379,6 @@ __global__ void aty_kernel(const float* A, const float* y, int M, int N, float* 
   out[i] = (float)s;
 }
 
-// 1 / d to FP64 rounding from the hardware's approximation, by one third-order
-// (Householder) step: with e = 1 - d r0, 1 / d = r0 (1 + e + e^2 + O(e^3)), and e is below
-// 2^-19.  Three dependent FP64 operations.
-__device__ __forceinline__ double recip_f64(double d) {
-  double r0;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d));
-  const double e = fma(-d, r0, 1.0);
-  return fma(r0, fma(e, e, e), r0);
-}
-
 // Z = L^{-1} of the Cholesky factor of the n x n (n <= 64) block K (lower triangle read),
 // zeros above the diagonal; a pivot that is not positive raises the non-finite bit.
 //

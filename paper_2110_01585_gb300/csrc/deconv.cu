@@ -23,6 +23,7 @@
 //
 // Layout: every vector is one FP32 plane of N = H*W pixels, row-major; the
 // 1 + S right-hand sides are consecutive planes ([0] = mean system).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdio.h>
 #include <stdlib.h>
@@ -289,6 +290,44 @@ __device__ __forceinline__ void block_sumf(float a, float b, float c3, double* o
   __syncthreads();
 }
 
+// Block sums of two or four FP64 values per thread, written by threads 0 .. NV - 1.  A
+// warp's tree halves the number of values each lane carries along with the distance
+// (one value per lane after the first steps), which takes 5 or 6 additions per lane
+// in place of 10 or 20 of the narrow FP64 pipe.
+template <int NV>
+__device__ __forceinline__ void block_sumd(const double (&v)[NV], double* const (&out)[NV]) {
+  static_assert(NV == 2 || NV == 4, "values");
+  __shared__ double red[NV][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double x;
+  if (NV == 2) {
+    const bool up = lane & 16;
+    x = (up ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, up ? v[0] : v[1], 16);
+    x += __shfl_xor_sync(0xffffffffu, x, 8);
+  } else {
+    const bool up = lane & 16, up2 = lane & 8;
+    const double a = (up ? v[NV - 2] : v[0]) + __shfl_xor_sync(0xffffffffu, up ? v[0] : v[NV - 2], 16);
+    const double b = (up ? v[NV - 1] : v[1]) + __shfl_xor_sync(0xffffffffu, up ? v[1] : v[NV - 1], 16);
+    x = (up2 ? b : a) + __shfl_xor_sync(0xffffffffu, up2 ? a : b, 8);
+  }
+#pragma unroll
+  for (int off = 4; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+  // lanes 0, 16 (NV = 2) or 0, 8, 16, 24 (NV = 4) hold values 0, 1, ...
+  constexpr int kStep = 32 / NV;
+  if (lane % kStep == 0) red[lane / kStep][w] = x;
+  __syncthreads();
+  if (threadIdx.x < NV) {
+    double s = 0.0;
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[threadIdx.x][i];
+    double* o = nullptr;
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+      if ((int)threadIdx.x == k) o = out[k];
+    if (o) *o = s;
+  }
+  __syncthreads();
+}
+
 // Last-block reduction.  Every block of a group has written its partial sum (by
 // thread 0, before the block barrier at the end of block_sum3); each then counts
 // itself in with an atomic, and the block that arrives last returns true and
@@ -358,6 +397,9 @@ struct CgArgs {
   unsigned long long* counters;
   int defer_e;           // 1: the update leaves e += alpha p to the next direction kernel
                          // (or the commit), see warp_update_rows_fwd_kernel
+  int res_all;           // 1: true residuals of every system (the first of an update); 0: of
+                         // those that iterated in the pass before.  The others' solutions,
+                         // and so their residuals' partial sums, are as they were.
 };
 
 // d = sum tau_k, n = sum nu_k (k = 1..4), Minv = 1 / (sum k^2 / xi + d); block sums of d.
@@ -379,8 +421,10 @@ __global__ void __launch_bounds__(kThreads) prep_kernel(const float* __restrict_
 }
 
 // dbar = mean of d over the image (fixed-order reduction of the block sums).
-__global__ void mean_kernel(const double* dpart, int n, double inv_count, double* out) {
+// Graph replays: also clears the loop counters ls (integers).
+__global__ void mean_kernel(const double* dpart, int n, double inv_count, double* out, int* ls, int ls_n) {
   __shared__ double buf[1024];
+  if (ls && (int)threadIdx.x < ls_n) ls[threadIdx.x] = 0;
   double s = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) s += dpart[i];
   buf[threadIdx.x] = s;
@@ -602,6 +646,7 @@ __global__ void __launch_bounds__(kThreads) residual_kernel(CgArgs a) {
   __shared__ int ctab[kTile + 2 * kMaxHalf];
   const ConvDesc& c = a.c;
   const int j = blockIdx.z;
+  if (!a.res_all && !a.act0[j]) return;
   const int r0 = blockIdx.y * kTile, c0 = blockIdx.x * kTile;
   const int hh = c.kh / 2, hw = c.kw / 2;
   const int RH = kTile + 2 * c.hr, RW = kTile + 2 * c.hc;  // x region, halo kh - 1
@@ -804,6 +849,7 @@ __global__ void __launch_bounds__(kThreads, K >= 15 ? 2 : 3) residual_pair_kerne
   const ConvDesc& c = a.c;
   const int j0 = 2 * blockIdx.z, j1 = j0 + 1;
   const bool two = j1 < a.R;
+  if (!a.res_all && !a.act0[j0] && !(two && a.act0[j1])) return;
   const int r0 = blockIdx.y * kTile, c0 = blockIdx.x * kTile;
   for (int i = threadIdx.x; i < 2 * K; i += kThreads) {
     const ff t = ff_from_double(c.hd[i]);
@@ -1026,6 +1072,42 @@ __global__ void __launch_bounds__(kThreads, K >= 15 ? 2 : 3) residual_pair_kerne
                   a.part_bb + o1);
 }
 
+// Device-side state of the solver loops of a graph replay.
+struct LoopState {
+  int it;         // CG iteration within the current pass
+  int outer;      // passes started
+  int total;      // CG iterations of this update
+  int converged;  // 1 once a true residual met every system's target
+  int live;       // the current pass has iterations left to do
+  int pass_its;   // iterations of a pass run by pw_solve_kernel (the largest of its pairs)
+};
+
+struct PassArgs {
+  LoopState* ls;  // NULL: the host drives the loop
+  int max_outer, max_iter;
+  int inner;      // the pass has an inner loop (none with pw_solve_kernel)
+  cudaGraphConditionalHandle h_outer, h_inner;
+};
+
+// After a true residual and its thresholds: start another pass, or stop (converged, or
+// out of passes or iterations), as the host loop does.
+__device__ __forceinline__ void start_pass(const PassArgs& p, int active) {
+  LoopState* ls = p.ls;
+  ls->total += ls->pass_its;
+  ls->pass_its = 0;
+  unsigned go = 0;
+  if (active == 0) {
+    ls->converged = 1;
+  } else if (ls->outer < p.max_outer && ls->total < p.max_iter) {
+    go = 1;
+    ls->it = 0;
+    ls->outer += 1;
+  }
+  ls->live = (int)go;
+  cudaGraphSetConditional(p.h_outer, go);
+  if (p.inner) cudaGraphSetConditional(p.h_inner, go);
+}
+
 // Per system after a true residual: done if r.r <= rtol^2 b.b (threshold +inf),
 // otherwise the inner loop runs until r.r <= max(eta^2 r.r, (rtol/2)^2 b.b).
 // Also starts the pass's CG scalars: active flag (and act0) = not done, beta = 0,
@@ -1034,10 +1116,9 @@ __global__ void thresholds_kernel(const double* part_rr, const double* part_bb,
                                   const double* part_rz, int fft, int R, int nb,
                                   double rtol2_mean, double rtol2_probe, double eta2, double* thr,
                                   double* relres, double* prev_rr, double* rr0, int first_arg,
-                                  const int* outer_dev, int* active, float* scal, int* act0,
-                                  double* rzs) {
+                                  int* active, float* scal, int* act0, double* rzs, PassArgs pass) {
   // the first true residual of this update (graph replays: passes started = 0)
-  const int first = outer_dev ? (*outer_dev == 0) : first_arg;
+  const int first = pass.ls ? (pass.ls->outer == 0) : first_arg;
   __shared__ int cnt;
   if (threadIdx.x == 0) cnt = 0;
   __syncthreads();
@@ -1083,7 +1164,10 @@ __global__ void thresholds_kernel(const double* part_rr, const double* part_bb,
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) *active = cnt;
+  if (threadIdx.x == 0) {
+    *active = cnt;
+    if (pass.ls) start_pass(pass, cnt);
+  }
 }
 
 // Direction and product: p = Minv r + beta p, q = Q p, partial p.q.
@@ -1555,14 +1639,6 @@ __global__ void commit_kernel(double* X, const float* Ec, const int* act0, long 
 }
 
 
-// Device-side state of the solver loops of a graph replay.
-struct LoopState {
-  int it;         // CG iteration within the current pass
-  int outer;      // passes started
-  int total;      // CG iterations of this update
-  int converged;  // 1 once a true residual met every system's target
-};
-
 // ---------------------------------------------------------------------------
 // Circulant preconditioner on a power-of-two torus HP x WP that holds the image:
 //   M = H^T H / xi + dbar I,  dbar = mean(d),  M^{-1} r = F^{-1}[F r / (|h_f|^2 / xi + dbar)].
@@ -1595,8 +1671,9 @@ struct FftDesc {
   int nbz;           // blocks per pair in the inverse row pass
   float2* tmp;       // pairs x H x WP (rows of the padded grid beyond H are zero)
   const float* hth;  // |h_f|^2 / xi on the HP x WP grid
+  float* filt;       // 1 / (|h_f|^2 / xi + dbar), formed once per update (filter_kernel)
   const double* dbar;
-  const float2* tw512;  // exp(-2 pi i m / 512), m < 512 (the 512-point kernels)
+  const float2* tw512;  // twiddles of the 512-point warp transform (kTw512)
   const float2* tw1024; // exp(-2 pi i m / 1024), m < 512 (the 1024-point kernels)
   const float2* twr;    // twiddles of the rows' and the columns' warp transforms (warp_twiddles)
   const float2* twc;
@@ -1607,6 +1684,9 @@ struct FftDesc {
   float* scal_w;     // the same array, written: beta of the active systems
   double* rzs;       // [R] r.z, or NULL: leave the CG scalars alone (shape tuning)
   unsigned* arrive;  // [pairs] block-arrival counters of the inverse row pass
+  const float* D;    // pointwise products (see pw_update_rows_fwd_kernel), else unused: d,
+  double* part_dl;   // [R][nbz] partials of sum (d - dbar) z^2,
+  double* alphas;    // [R] alpha of the current iteration
   int first;         // 1: first application of a refinement pass (beta = 0)
   unsigned long long* counters;  // DC_CG_PRE_UNITS counts the systems transformed
   LoopState* loop;   // graph replays: the column pass also counts the CG iteration and
@@ -1620,16 +1700,48 @@ struct FftDesc {
 // (0 in the first application of a refinement pass) and r.z = r.z(new).
 __device__ __forceinline__ void rz_tail(const FftDesc& f, int pair, const double* part_rz) {
   if (!f.rzs) return;
-  if (!arrive_last(f.arrive + pair, gridDim.x) || threadIdx.x >= 32) return;
-  for (int u = 0; u < 2; ++u) {
-    const int j = 2 * pair + u;
-    if (j >= f.R) break;
-    const double rz = group_sum(part_rz + (long long)j * f.nbz, f.nbz);
-    if (threadIdx.x == 0 && f.act[4 * j] != 0.f) {
-      f.scal_w[4 * j + 1] = f.first ? 0.f : (float)(rz / f.rzs[j]);
-      f.rzs[j] = rz;
+  if (!arrive_last(f.arrive + pair, gridDim.x) || threadIdx.x >= 64) return;
+  const int j = 2 * pair + (threadIdx.x >> 5);  // warp u: system u of the pair
+  if (j >= f.R) return;
+  const double rz = group_sum(part_rz + (long long)j * f.nbz, f.nbz);
+  if ((threadIdx.x & 31) == 0 && f.act[4 * j] != 0.f) {
+    f.scal_w[4 * j + 1] = f.first ? 0.f : (float)(rz / f.rzs[j]);
+    f.rzs[j] = rz;
+  }
+}
+
+// The same with pointwise products: from gamma = r.z and the partials of sum (d - dbar) z^2,
+// which give delta = z.Q z = gamma + sum, beta = gamma(new) / gamma(old) and
+// alpha = gamma / (delta - beta gamma / alpha(old)) (Chronopoulos and Gear, 1989).  A
+// denominator that rounding has made non-positive restarts the directions (beta = 0,
+// alpha = gamma / delta, the steepest-descent step).
+__device__ __forceinline__ void pw_tail(const FftDesc& f, int pair, const double* part_rz) {
+  __shared__ double sums[4];
+  if (!arrive_last(f.arrive + pair, gridDim.x)) return;
+  // warps 0 .. 3: gamma and the sum, of system 0 and 1 of the pair
+  const int w = threadIdx.x >> 5, js = 2 * pair + (w >> 1);
+  if (w < 4 && js < f.R) {
+    const double x = group_sum((w & 1 ? f.part_dl : part_rz) + (long long)js * f.nbz, f.nbz);
+    if ((threadIdx.x & 31) == 0) sums[w] = x;
+  }
+  __syncthreads();
+  const int u = threadIdx.x, j = 2 * pair + u;
+  if (u >= 2 || j >= f.R || f.act[4 * j] == 0.f) return;
+  const double rz = sums[2 * u], delta = rz + sums[2 * u + 1];
+  double beta = 0.0, den = delta;
+  if (!f.first) {
+    beta = rz / f.rzs[j];
+    den = delta - beta * rz / f.alphas[j];
+    if (!(den > 0.0)) {
+      beta = 0.0;
+      den = delta;
     }
   }
+  const double alpha = rz / den;
+  f.scal_w[4 * j + 1] = (float)beta;
+  f.scal_w[4 * j + 2] = (float)alpha;
+  f.alphas[j] = alpha;
+  f.rzs[j] = rz;
 }
 
 // Both systems of a pair have stopped in this CG iteration: their z is not used.
@@ -1641,17 +1753,25 @@ __device__ __forceinline__ bool pair_idle(const FftDesc& f, int pair) {
 
 // After a CG iteration's update (graph replays, by block (0, 0) of the column pass,
 // which every iteration launches): count the iteration, and go on while a system is
-// still active and the iteration budget lasts, as iter_kernel does.
+// still active and the iteration budget lasts, as iter_kernel does.  A body of the loop
+// holds kUnroll iterations; those launched after the last one find every system stopped
+// (with the budget spent, by the flags cleared here) and are not counted.
 __device__ __forceinline__ void loop_step(const FftDesc& f) {
-  if (!f.loop || blockIdx.x != 0 || blockIdx.y != 0 || threadIdx.x >= 32) return;
+  if (!f.loop || blockIdx.x != 0 || blockIdx.y != 0 || threadIdx.x >= 32 || !f.loop->live) return;
   int cnt = 0;
   for (int j = threadIdx.x; j < f.R; j += 32) cnt += f.act[4 * j] != 0.f;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, off);
+  const bool spent = f.loop->total + 1 >= f.max_iter;
+  __syncwarp();
+  if (spent)
+    for (int j = threadIdx.x; j < f.R; j += 32) f.scal_w[4 * j] = 0.f;
   if (threadIdx.x == 0) {
     f.loop->it += 1;
     f.loop->total += 1;
-    cudaGraphSetConditional(f.h_inner, (cnt > 0 && f.loop->total < f.max_iter) ? 1u : 0u);
+    const int go = cnt > 0 && !spent;
+    f.loop->live = go;
+    cudaGraphSetConditional(f.h_inner, go);
   }
 }
 
@@ -1685,8 +1805,10 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// complex sums and differences as one packed FP32 operation each (the difference as an
+// FMA with -1, which rounds as the subtraction does)
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 __device__ __forceinline__ float2 cmul_mi(float2 a) { return make_float2(a.y, -a.x); }  // a * (-i)
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 
@@ -1877,10 +1999,9 @@ __global__ void __launch_bounds__(kFftThreads, 4) fft_cols_filter_kernel(FftDesc
   __syncthreads();
   fft_forward(s, f.HP, f.cw, f.cw, 1, tw);
   // filter, then the inverse column transform as conj(F(conj(.)))
-  const float dbar = (float)(*f.dbar);
   for (int idx = threadIdx.x; idx < f.HP * f.cw; idx += blockDim.x) {
     const int i = idx / f.cw, c = idx - i * f.cw;
-    const float g = __frcp_rn(f.hth[(long long)i * f.WP + c0 + c] + dbar);
+    const float g = f.filt[(long long)i * f.WP + c0 + c];
     s[idx] = make_float2(s[idx].x * g, -s[idx].y * g);
   }
   __syncthreads();
@@ -1980,27 +2101,35 @@ __global__ void window_kernel(float* w, int n, int P) {
   w[i] = (float)v;
 }
 
-// tw[m] = w512^m and tw[512 + m] = w1024^m for m < 512
-constexpr int kTwCount = 2 * kF + 256 + 128 + 64;
-__global__ void tw512_kernel(float2* tw) {
+// The twiddle tables, in the order their transforms read them (neighbouring lanes on
+// neighbouring entries; with w512^m at m the first step's reads met up to four to a bank):
+//   kTw512: w512^(t k1) at 64 k1 + t (t < 64, k1 < 8), then w64^(u k3) at 512 + 8 k3 + u
+//   w1024^m, m < 512
+//   256, 128 and 64 points: w_n^(t k1) at k1 T + t, T = n / 16
+constexpr int kTw512 = kF + 64;
+constexpr int kTwCount = kTw512 + kF + 256 + 128 + 64;
+__global__ void twiddle_kernel(float2* tw) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= 2 * kF && m < kTwCount) {
-    // the tables of the 256-, 128- and 64-point transforms: entry k1 T + t is w_n^(t k1), T = n / 16
-    const int q = m - 2 * kF;
-    const int n = q < 256 ? 256 : q < 384 ? 128 : 64, e = q < 256 ? q : q < 384 ? q - 256 : q - 384;
-    const int T = n / 16, t = e % T, k1 = e / T;
-    float sn, cs;
-    sincospif(-2.0f * (float)((t * k1) % n) / (float)n, &sn, &cs);
-    tw[m] = make_float2(cs, sn);
+  if (m >= kTwCount) return;
+  int n, e;  // the entry is w_n^e
+  if (m < kF) {
+    n = kF;
+    e = (m & 63) * (m >> 6);
+  } else if (m < kTw512) {
+    n = 64;
+    e = (m & 7) * ((m - kF) >> 3);
+  } else if (m < kTw512 + kF) {
+    n = 2 * kF;
+    e = m - kTw512;
+  } else {
+    const int q = m - kTw512 - kF;
+    n = q < 256 ? 256 : q < 384 ? 128 : 64;
+    const int k = q < 256 ? q : q < 384 ? q - 256 : q - 384, T = n / 16;
+    e = (k % T) * (k / T);
   }
-  if (m < 2 * kF) {
-    float sn, cs;
-    if (m < kF)
-      sincospif(-2.0f * (float)m / (float)kF, &sn, &cs);
-    else
-      sincospif(-2.0f * (float)(m - kF) / (float)(2 * kF), &sn, &cs);
-    tw[m] = make_float2(cs, sn);
-  }
+  float sn, cs;
+  sincospif(-2.0f * (float)(e % n) / (float)n, &sn, &cs);
+  tw[m] = make_float2(cs, sn);
 }
 
 // L2 eviction priorities for the preconditioner's planes: the complex plane of
@@ -2061,7 +2190,7 @@ __device__ __forceinline__ void fft512_warp(float2 (&v)[16], float2* xs, const f
     dft_reg<8>(a);
     xs[t * 9] = a[0];
 #pragma unroll
-    for (int k1 = 1; k1 < 8; ++k1) xs[t * 9 + k1] = cmul(a[k1], tw[(t * k1) & (kF - 1)]);
+    for (int k1 = 1; k1 < 8; ++k1) xs[t * 9 + k1] = cmul(a[k1], tw[64 * k1 + t]);
   }
   __syncwarp();
   const int k1 = l & 7;
@@ -2080,7 +2209,7 @@ __device__ __forceinline__ void fft512_warp(float2 (&v)[16], float2* xs, const f
     xs[u * 72 + k1] = b[g][0];
 #pragma unroll
     for (int k3 = 1; k3 < 8; ++k3)
-      xs[u * 72 + k1 + 8 * k3] = cmul(b[g][k3], tw[(8 * u * k3) & (kF - 1)]);
+      xs[u * 72 + k1 + 8 * k3] = cmul(b[g][k3], tw[kF + 8 * k3 + u]);
   }
   __syncwarp();
 #pragma unroll
@@ -2103,9 +2232,10 @@ __device__ __forceinline__ void fft512_warp(float2 (&v)[16], float2* xs, const f
 //   B_t[k1]      = w_n^(t k1) sum_m x[T m + t] w16^(m k1)      (in a lane)
 //   X[k1 + 16 k2] = sum_t B_t[k1] w_T^(t k2)
 // with one regrouping through the warp's scratch, after which lane t takes k1 = t + T j,
-// j < 16 / T: X[T (16 / T k2 + j) + t], the layout of the input.  For one pass over 17
-// pairs of a 256^2 image the Stockham kernels (passes through shared memory behind block
-// barriers) took 59 us, these 21.
+// j < 16 / T: X[T (16 / T k2 + j) + t], the layout of the input.  For 17 pairs of a 256^2
+// image the preconditioner took 59 us in Stockham kernels (passes through shared memory
+// behind block barriers); its column and inverse row passes take 26 us here, and the
+// forward one is fused with the CG update.
 //
 // Sizes per warp, in float2: kRow, from one transform's regrouping area to the next (entry
 // (k1, t) at k1 (T + 1) + t); kCol, from one staged column to the next in the column pass;
@@ -2114,11 +2244,13 @@ __device__ __forceinline__ void fft512_warp(float2 (&v)[16], float2* xs, const f
 template <int T>
 struct Warp {
   static constexpr int kN = 16 * T, kPer = 32 / T;
+  static constexpr int kTw = T == 32 ? kTw512 : kN;  // entries of the twiddle table
   static constexpr int kRow = T == 32 ? 0 : T == 16 ? 272 : T == 8 ? 152 : 84;
   static constexpr int kCol = T == 32 ? 0 : kN + 1;
   static constexpr int kScratch = T == 32 ? kXs : T == 16 ? 546 : T == 8 ? 612 : 680;
   static constexpr int kCols = kF512Warps * kPer;  // columns per block of the column pass
-  // rows per block of the row passes: four, one, one, one rounds of the block's warps
+  // rows per block of the row passes: four rounds of the block's warps for 512 points (one
+  // and two rounds were within 3% on 512^2 and 300 x 420), one for the others
   static constexpr int kRows = T == 32 ? 4 * kF512Warps : kF512Warps * kPer;
   static_assert(kPer * kRow <= kScratch && kPer * kCol <= kScratch, "scratch");
 };
@@ -2153,8 +2285,7 @@ template <> __device__ __forceinline__ void dft_reg<16>(float2* v) {
   }
 }
 
-// The warp's forward transforms in place; xs: the warp's scratch; tw: kN entries (natural for
-// T = 32, entry k1 T + t for the others).
+// The warp's forward transforms in place; xs: the warp's scratch; tw: its kTw twiddles.
 template <int T>
 __device__ __forceinline__ void fft_warp(float2 (&v)[16], float2* xs, const float2* tw) {
   if constexpr (T == 32) {
@@ -2234,9 +2365,9 @@ __global__ void __launch_bounds__(32 * kF512Warps) warp_rows_fwd_kernel(FftDesc 
   if (pair_idle(f, blockIdx.y)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0 && f.counters)
     atomicAdd(&f.counters[DC_CG_PRE_UNITS], 2 * blockIdx.y + 1 < f.R ? 2ull : 1ull);
-  __shared__ float2 tw[Wp::kN];
+  __shared__ float2 tw[Wp::kTw];
   __shared__ float2 scratch[kF512Warps][Wp::kScratch];
-  for (int m = threadIdx.x; m < Wp::kN; m += blockDim.x) tw[m] = f.twr[m];
+  for (int m = threadIdx.x; m < Wp::kTw; m += blockDim.x) tw[m] = f.twr[m];
   __syncthreads();
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, t = l % T;
   const int pair = blockIdx.y;
@@ -2301,15 +2432,15 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_update_rows_fwd_kerne
   }
   const int it = a.it_dev ? *a.it_dev : it_arg;
   const bool first = it == 0;  // the correction starts at zero: not read
-  __shared__ float2 tw[Wp::kN];
+  __shared__ float2 tw[Wp::kTw];
   __shared__ float2 scratch[kF512Warps][Wp::kScratch];
   __shared__ float alpha_s[2];
-  for (int m = threadIdx.x; m < Wp::kN; m += blockDim.x) tw[m] = f.twr[m];
+  for (int m = threadIdx.x; m < Wp::kTw; m += blockDim.x) tw[m] = f.twr[m];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, t = l % T;
   if (w < 2 && (w == 0 ? act0 : act1)) {
     const int j = j0 + w;
     const double pqs = group_sum(a.part_pq + (long long)j * a.nb, a.nb);
-    if (l == 0) alpha_s[w] = (float)(a.rzs[j] / pqs);
+    if (l == 0) alpha_s[w] = (float)(a.rzs[j] * recip_f64(pqs));
   }
   __syncthreads();
   const long long N = (long long)f.H * f.W;
@@ -2412,18 +2543,14 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_update_rows_fwd_kerne
   }
   block_sumf<2>(rr0, rr1, 0.f, act0 ? a.part_rr + (long long)j0 * a.nb + blockIdx.x : nullptr,
                 act1 ? a.part_rr + (long long)j1 * a.nb + blockIdx.x : nullptr, nullptr);
-  if (arrive_last(a.arrive + j0, gridDim.x) && threadIdx.x < 32) {
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      if (!(u ? act1 : act0)) continue;
-      const int j = j0 + u;
-      const double r2 = group_sum(a.part_rr + (long long)j * a.nb, gridDim.x);
-      if (threadIdx.x == 0) {
-        a.scal[4 * j] = still_active(a, j, r2);
-        if (a.defer_e) {
-          a.scal[4 * j + 2] = alpha_s[u];
-          a.scal[4 * j + 3] = (float)it;
-        }
+  if (arrive_last(a.arrive + j0, gridDim.x) && w < 2 && (w ? act1 : act0)) {
+    const int j = j0 + w;
+    const double r2 = group_sum(a.part_rr + (long long)j * a.nb, gridDim.x);
+    if (l == 0) {
+      a.scal[4 * j] = still_active(a, j, r2);
+      if (a.defer_e) {
+        a.scal[4 * j + 2] = alpha_s[w];
+        a.scal[4 * j + 3] = (float)it;
       }
     }
   }
@@ -2432,17 +2559,17 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_update_rows_fwd_kerne
 // fft_cols_filter_kernel for HP = 16 T: the block takes columns [blockIdx.x kCols, + kCols) of
 // a pair, stages the tile in shared memory (row segments of 64 bytes and more from global
 // memory, extended to HP rows), and each group of T lanes transforms one column in
-// registers, filters it with hthT (the filter stored column-major, [c][i]), transforms
+// registers, filters it with filtT (the filter stored column-major, [c][i]), transforms
 // again and leaves it in its slot for the block's store of the fold to H rows.
 template <int T>
 __global__ void __launch_bounds__(32 * kF512Warps, 3) warp_cols_filter_kernel(FftDesc f,
-                                                                          const float* __restrict__ hthT) {
+                                                                          const float* __restrict__ filtT) {
   using Wp = Warp<T>;
   loop_step(f);
   if (pair_idle(f, blockIdx.y)) return;
-  __shared__ float2 tw[Wp::kN];
+  __shared__ float2 tw[Wp::kTw];
   __shared__ float2 cols[kF512Warps * Wp::kScratch];
-  for (int m = threadIdx.x; m < Wp::kN; m += blockDim.x) tw[m] = f.twc[m];
+  for (int m = threadIdx.x; m < Wp::kTw; m += blockDim.x) tw[m] = f.twc[m];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, t = l % T;
   const int c0 = blockIdx.x * Wp::kCols;
   float2* tp = f.tmp + (long long)blockIdx.y * f.H * f.WP;
@@ -2450,14 +2577,18 @@ __global__ void __launch_bounds__(32 * kF512Warps, 3) warp_cols_filter_kernel(Ff
   const int cc = threadIdx.x % Wp::kCols, ro = threadIdx.x / Wp::kCols;
   float2* const slot = cols + (cc / Wp::kPer) * Wp::kScratch + (cc % Wp::kPer) * Wp::kCol;
   const uint64_t keep = l2_policy_keep();
+  float2* const col = tp + c0 + cc;
   {
     float2 x[16];  // all of the thread's tile loads in flight at once
+    if (f.H == Wp::kN) {
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int src = margin(kStep * u + ro, f.H, Wp::kN);
-      x[u] = src >= 0 ? ld_hint(tp + (long long)src * f.WP + c0 + cc, keep) : make_float2(0.f, 0.f);
-    }
-    if (f.H < Wp::kN) {
+      for (int u = 0; u < 16; ++u) x[u] = ld_hint(col + (long long)(kStep * u + ro) * f.WP, keep);
+    } else {
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        const int src = margin(kStep * u + ro, f.H, Wp::kN);
+        x[u] = src >= 0 ? ld_hint(col + (long long)src * f.WP, keep) : make_float2(0.f, 0.f);
+      }
 #pragma unroll
       for (int u = 0; u < 16; ++u) x[u] = cscale(x[u], f.wr[kStep * u + ro]);
     }
@@ -2467,7 +2598,7 @@ __global__ void __launch_bounds__(32 * kF512Warps, 3) warp_cols_filter_kernel(Ff
   __syncthreads();
   float2* xs = cols + w * Wp::kScratch;
   float2* const mine = xs + (l / T) * Wp::kCol;
-  const float* g = hthT + (long long)(c0 + w * Wp::kPer + l / T) * Wp::kN;
+  const float* g = filtT + (long long)(c0 + w * Wp::kPer + l / T) * Wp::kN;
   float gv[16];  // the filter column, loaded before the transform
 #pragma unroll
   for (int m = 0; m < 16; ++m) gv[m] = g[T * m + t];
@@ -2477,38 +2608,132 @@ __global__ void __launch_bounds__(32 * kF512Warps, 3) warp_cols_filter_kernel(Ff
   __syncwarp();
   fft_warp<T>(v, xs, tw);
   // filter, then the inverse transform as conj(F(conj(.)))
-  const float dbar = (float)(*f.dbar);
 #pragma unroll
-  for (int m = 0; m < 16; ++m) {
-    const float gi = __frcp_rn(gv[m] + dbar);
-    v[m] = make_float2(v[m].x * gi, -v[m].y * gi);
-  }
+  for (int m = 0; m < 16; ++m) v[m] = make_float2(v[m].x * gv[m], -v[m].y * gv[m]);
   fft_warp<T>(v, xs, tw);
 #pragma unroll
   for (int m = 0; m < 16; ++m) mine[T * m + t] = cconj(v[m]);
   __syncthreads();
+  if (f.H == Wp::kN) {
 #pragma unroll
-  for (int u = 0; u < 16; ++u) {
-    const int i = kStep * u + ro;
-    if (i < f.H) {
-      const float2 x = f.H < Wp::kN
-                           ? fold(i, f.H, Wp::kN, [&](int k) { return cscale(slot[k], f.wr[k]); })
-                           : slot[i];
-      st_hint(tp + (long long)i * f.WP + c0 + cc, x, keep);
+    for (int u = 0; u < 16; ++u) st_hint(col + (long long)(kStep * u + ro) * f.WP, slot[kStep * u + ro], keep);
+  } else {
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      const int i = kStep * u + ro;
+      if (i < f.H)
+        st_hint(col + (long long)i * f.WP, fold(i, f.H, Wp::kN, [&](int k) { return cscale(slot[k], f.wr[k]); }), keep);
     }
   }
 }
 
-// fft_rows_inv_kernel for WP = 16 T: rows [blockIdx.x rows_per, + rows_per), rows_per =
-// ceil(H / nbz).
+// The whole CG step of images that fill the torus (H = HP, W = WP), fused with the forward
+// row pass.  There M z = r holds exactly (M = H^T H / xi + dbar I is the image's own
+// circulant), so the product with Q needs no stencil:
+//   Q z = M z + (d - dbar) z = r + (d - dbar) z,
+// pointwise, and with the directions p = z + beta p also s = Q p = Q z + beta s.  One kernel
+// per iteration then does, for both systems of a pair, p, s, e += alpha p and
+// r -= alpha s, and transforms the new residual rows; alpha and beta come from the inverse
+// row pass before it (pw_tail).  The rounding error of Q z is that of the transforms times
+// |H^T H| / xi, the same order as the FP32 stencil's: in an FP32 emulation at 128^2 and 256^2
+// (40 dB and 30 dB) both take the same iterations in every pass, and the true residual that
+// ends a solve is formed by the float-float residual kernel as before.
+// Bound by its nine planes (36 bytes per pixel and system, and d): at 512^2 with 33 systems
+// 61 us, 5.7 TB/s.  Three kernels per iteration, 60 bytes in all, against four with the
+// stencil kernel and the same bytes (direction 53 us and update 28 us there).
 template <int T>
+__global__ void __launch_bounds__(32 * kF512Warps, 2) pw_update_rows_fwd_kernel(FftDesc f, CgArgs a, int it_arg) {
+  using Wp = Warp<T>;
+  const int pair = blockIdx.y;
+  const int j0 = 2 * pair, j1 = 2 * pair + 1;
+  const bool two = j1 < f.R;
+  const bool act0 = a.scal[4 * j0] != 0.f, act1 = two && a.scal[4 * j1] != 0.f;
+  if (!act0 && !act1) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0 && f.counters) {
+    atomicAdd(&f.counters[DC_CG_PRE_UNITS], two ? 2ull : 1ull);
+    atomicAdd(&f.counters[DC_CG_UPD_UNITS], (unsigned long long)(act0 + act1));
+  }
+  const bool first = (a.it_dev ? *a.it_dev : it_arg) == 0;  // p, s and e start here: not read
+  __shared__ float2 tw[Wp::kTw];
+  __shared__ float2 scratch[kF512Warps][Wp::kScratch];
+  for (int m = threadIdx.x; m < Wp::kTw; m += blockDim.x) tw[m] = f.twr[m];
+  __syncthreads();
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, t = l % T;
+  const float dbar = (float)(*f.dbar);
+  const long long N = (long long)f.H * Wp::kN;
+  float2* out = f.tmp + (long long)pair * N;
+  const int rend = min(f.H, (int)(blockIdx.x + 1) * Wp::kRows);
+  const uint64_t keep = l2_policy_keep();
+  float rr[2] = {0.f, 0.f};
+  for (int base = blockIdx.x * Wp::kRows + w * Wp::kPer; base < rend; base += kF512Warps * Wp::kPer) {
+    const int row = base + l / T;
+    const bool ok = row < rend;
+    const long long p0 = (long long)row * Wp::kN + t;
+    float2 v[16];
+#pragma unroll
+    for (int m = 0; m < 16; ++m) v[m] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      if (!ok || !(u ? act1 : act0)) continue;
+      const int j = j0 + u;
+      const float beta = a.scal[4 * j + 1], alpha = a.scal[4 * j + 2];
+      const long long o = (long long)j * N + p0;
+      constexpr int kB = 8;  // elements per lane whose loads are in flight together
+#pragma unroll
+      for (int b = 0; b < 16; b += kB) {
+        float zv[kB], rv[kB], sv[kB], pv[kB], ev[kB], dv[kB];
+#pragma unroll
+        for (int k = 0; k < kB; ++k) {
+          const long long q = o + T * (b + k);
+          zv[k] = a.Z[q];
+          rv[k] = a.Rr[q];
+          dv[k] = a.D[p0 + T * (b + k)];
+          sv[k] = pv[k] = ev[k] = 0.f;
+          if (!first) {
+            sv[k] = a.Qp[q];
+            pv[k] = a.P[q];
+            ev[k] = a.Ec[q];
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < kB; ++k) {
+          const long long q = o + T * (b + k);
+          const float pn = fmaf(beta, pv[k], zv[k]);
+          const float sn = fmaf(beta, sv[k], fmaf(dv[k] - dbar, zv[k], rv[k]));
+          const float r = fmaf(-alpha, sn, rv[k]);
+          a.P[q] = pn;
+          a.Qp[q] = sn;
+          a.Ec[q] = fmaf(alpha, pn, ev[k]);
+          st_hint_f(a.Rr + q, r, keep);
+          rr[u] = fmaf(r, r, rr[u]);
+          (u ? v[b + k].y : v[b + k].x) = r;
+        }
+      }
+    }
+    fft_warp<T>(v, scratch[w], tw);
+    if (ok) {
+#pragma unroll
+      for (int m = 0; m < 16; ++m) st_hint(out + p0 + T * m, v[m], keep);
+    }
+  }
+  block_sumf<2>(rr[0], rr[1], 0.f, act0 ? a.part_rr + (long long)j0 * a.nb + blockIdx.x : nullptr,
+                act1 ? a.part_rr + (long long)j1 * a.nb + blockIdx.x : nullptr, nullptr);
+  if (arrive_last(a.arrive + j0, gridDim.x) && w < 2 && (w ? act1 : act0)) {
+    const double r2 = group_sum(a.part_rr + (long long)(j0 + w) * a.nb, gridDim.x);
+    if (l == 0) a.scal[4 * (j0 + w)] = still_active(a, j0 + w, r2);
+  }
+}
+
+// fft_rows_inv_kernel for WP = 16 T: rows [blockIdx.x rows_per, + rows_per), rows_per =
+// ceil(H / nbz).  kPw: the image fills the torus, and the pass also sums (d - dbar) z^2.
+template <int T, bool kPw>
 __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_rows_inv_kernel(FftDesc f, const float* __restrict__ Rr,
                                                                        float* Z, double* part_rz) {
   using Wp = Warp<T>;
   if (pair_idle(f, blockIdx.y)) return;
-  __shared__ float2 tw[Wp::kN];
+  __shared__ float2 tw[Wp::kTw];
   __shared__ float2 scratch[kF512Warps][Wp::kScratch];
-  for (int m = threadIdx.x; m < Wp::kN; m += blockDim.x) tw[m] = f.twr[m];
+  for (int m = threadIdx.x; m < Wp::kTw; m += blockDim.x) tw[m] = f.twr[m];
   __syncthreads();
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, t = l % T;
   const int pair = blockIdx.y;
@@ -2520,7 +2745,8 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_rows_inv_kernel(FftDe
   const int rend = min(f.H, (int)(blockIdx.x + 1) * rows_per);
   const float2* tin = f.tmp + (long long)pair * f.H * Wp::kN;
   const uint64_t release = l2_policy_release();
-  double acc0 = 0.0, acc1 = 0.0;
+  const float dbar = kPw ? (float)(*f.dbar) : 0.f;
+  double acc0 = 0.0, acc1 = 0.0, dacc0 = 0.0, dacc1 = 0.0;
   for (int base = blockIdx.x * rows_per + w * Wp::kPer; base < rend; base += kF512Warps * Wp::kPer) {
     const int row = base + l / T;
     const bool ok = row < rend;
@@ -2528,10 +2754,12 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_rows_inv_kernel(FftDe
     const long long p0 = (long long)row * f.W;
     // the row's transform input and both residuals, all loads in flight together
     float2 v[16], rr[16];
+    float dv[kPw ? 16 : 1];
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
       const int c = T * m + t;
       v[m] = rr[m] = make_float2(0.f, 0.f);
+      if (kPw) dv[m] = ok ? f.D[p0 + c] : 0.f;
       if (ok) v[m] = cconj(ld_hint(tin + (long long)row * Wp::kN + c, release));
       if (c < cols) {
         rr[m].x = ld_hint(Rr + (long long)j0 * N + p0 + c, release);
@@ -2539,8 +2767,8 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_rows_inv_kernel(FftDe
       }
     }
     fft_warp<T>(v, scratch[w], tw);
-    if (f.W < Wp::kN) fold_row<T>(v, scratch[w], f.wc, f.W);
-    float rz0 = 0.f, rz1 = 0.f;
+    if (!kPw && f.W < Wp::kN) fold_row<T>(v, scratch[w], f.wc, f.W);
+    float rz0 = 0.f, rz1 = 0.f, dz0 = 0.f, dz1 = 0.f;
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
       const int c = T * m + t;
@@ -2549,19 +2777,327 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_rows_inv_kernel(FftDe
         const float z0 = v[m].x * scale;
         Z[(long long)j0 * N + p] = z0;
         rz0 = fmaf(rr[m].x, z0, rz0);
+        if (kPw) dz0 = fmaf((dv[m] - dbar) * z0, z0, dz0);
         if (two) {
           const float z1 = -v[m].y * scale;
           Z[(long long)j1 * N + p] = z1;
           rz1 = fmaf(rr[m].y, z1, rz1);
+          if (kPw) dz1 = fmaf((dv[m] - dbar) * z1, z1, dz1);
         }
       }
     }
     acc0 += (double)rz0;
     acc1 += (double)rz1;
+    if (kPw) {
+      dacc0 += (double)dz0;
+      dacc1 += (double)dz1;
+    }
   }
-  block_sum3(acc0, acc1, 0.0, part_rz + (long long)j0 * f.nbz + blockIdx.x,
-             two ? part_rz + (long long)j1 * f.nbz + blockIdx.x : nullptr, nullptr);
-  rz_tail(f, pair, part_rz);
+  const long long b0 = (long long)j0 * f.nbz + blockIdx.x, b1 = b0 + f.nbz;
+  if (kPw) {
+    block_sumd<4>({acc0, acc1, dacc0, dacc1}, {part_rz + b0, two ? part_rz + b1 : nullptr, f.part_dl + b0,
+                                               two ? f.part_dl + b1 : nullptr});
+    pw_tail(f, pair, part_rz);
+  } else {
+    block_sumd<2>({acc0, acc1}, {part_rz + b0, two ? part_rz + b1 : nullptr});
+    rz_tail(f, pair, part_rz);
+  }
+}
+
+// ---- one refinement pass of a square image that fills the torus, in one kernel
+//
+// H = W = 16 T (64 to 256) with pointwise products: one cluster of kSolveCtas CTAs runs all CG
+// iterations of a pass for one pair of systems, from the first z = M^{-1} r to the commit
+// x += e.  CTA c owns an eighth of the rows, which stay its own from iteration to
+// iteration, and an eighth of the columns of the transform plane, which passes through L2.
+// The phases are those of warp_rows_fwd / pw_update_rows_fwd, warp_cols_filter and
+// warp_rows_inv; between them the cluster's barrier takes the place of a kernel boundary,
+// and the dot products' partial sums go to every CTA's shared memory, so that each forms
+// the same alpha, beta and active flags.  Pairs do not wait for one another.
+// What it saves is latency: kernel starts, loop nodes, and fences, atomics and a last
+// block's sums at the end of every kernel.  An iteration of a first sweep with 33 systems
+// (its residuals included) took 40 us at 64^2, 33 at 128^2 and 40 at 256^2 with three
+// kernels per iteration, and takes 13.6, 14.9 and 33 here.
+constexpr int kSolveCtas = 8;
+// Warps per CTA.  Two such CTAs fit an SM, so that the 17 pairs of the default 33 systems
+// are resident at once; with 16 warps a 256^2 pass was 10% slower.
+template <int T>
+constexpr int solve_warps() { return 8; }
+
+// Sums NV values per thread over the CTA and writes the sums to slot[rank] of every CTA of the
+// cluster; they are there after the next cluster barrier.
+template <int kWarps, int NV>
+__device__ __forceinline__ void cluster_sum(cooperative_groups::cluster_group& cl, const double (&v)[NV],
+                                            double (*red)[kWarps], double (*slot)[4]) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double x;
+  if (NV == 2) {
+    const bool up = lane & 16;
+    x = (up ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, up ? v[0] : v[1], 16);
+    x += __shfl_xor_sync(0xffffffffu, x, 8);
+  } else {
+    const bool up = lane & 16, up2 = lane & 8;
+    const double a = (up ? v[NV - 2] : v[0]) + __shfl_xor_sync(0xffffffffu, up ? v[0] : v[NV - 2], 16);
+    const double b = (up ? v[NV - 1] : v[1]) + __shfl_xor_sync(0xffffffffu, up ? v[1] : v[NV - 1], 16);
+    x = (up2 ? b : a) + __shfl_xor_sync(0xffffffffu, up2 ? a : b, 8);
+  }
+#pragma unroll
+  for (int off = 4; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+  constexpr int kStep = 32 / NV;
+  if (lane % kStep == 0) red[lane / kStep][w] = x;
+  __syncthreads();
+  if (w < NV) {
+    double s = red[w][lane & (kWarps - 1)];
+#pragma unroll
+    for (int off = kWarps / 2; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane < kSolveCtas) cl.map_shared_rank(&slot[0][0], lane)[4 * cl.block_rank() + w] = s;
+  }
+}
+
+template <int T>
+constexpr size_t solve_smem() {
+  return sizeof(float2) * (size_t)solve_warps<T>() * Warp<T>::kScratch;
+}
+
+template <int T>
+__global__ void __cluster_dims__(kSolveCtas, 1, 1) __launch_bounds__(32 * solve_warps<T>(), 16 / solve_warps<T>())
+    pw_solve_kernel(FftDesc f, CgArgs a, const float* filtT, const LoopState* ls, int budget, int* pass_its) {
+  namespace cg = cooperative_groups;
+  using Wp = Warp<T>;
+  constexpr int kN = Wp::kN, kPer = Wp::kPer, kSolveWarps = solve_warps<T>();
+  constexpr int kOwn = kN / kSolveCtas;  // rows, and columns, of one CTA
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank();
+  const int pair = blockIdx.x / kSolveCtas;
+  const int j0 = 2 * pair, j1 = 2 * pair + 1;
+  const bool two = j1 < f.R;
+  bool act0 = a.act0[j0] != 0, act1 = two && a.act0[j1] != 0;
+  const bool started0 = act0, started1 = act1;
+  if (!act0 && !act1) return;  // the same for the whole cluster
+  if (ls) budget = f.max_iter - ls->total;
+  extern __shared__ float4 solve_smem4[];
+  float2* const scratch = reinterpret_cast<float2*>(solve_smem4);
+  __shared__ float2 twr[Wp::kTw];
+  __shared__ double red[4][kSolveWarps];
+  __shared__ double slot_rr[kSolveCtas][4], slot_gd[kSolveCtas][4];
+  __shared__ float coef[2][2];  // beta and alpha of the two systems
+  __shared__ int stop[2];
+  const int tid = threadIdx.x, w = tid >> 5, l = tid & 31, t = l % T;
+  for (int m = tid; m < Wp::kTw; m += blockDim.x) twr[m] = f.twr[m];
+  __syncthreads();
+  float2* const xs = scratch + w * Wp::kScratch;
+  const float dbar = (float)(*f.dbar);
+  constexpr long long N = (long long)kN * kN;
+  float2* const tmp = f.tmp + pair * N;
+  const int row0 = rank * kOwn + w * kPer + l / T;  // first row of this lane; the next are kRowStep apart
+  const int row_end = (rank + 1) * kOwn;
+  // whole warps take part in a round of the row phases: kOwn is a multiple of kPer
+  constexpr int kRowStep = kSolveWarps * kPer;
+
+  // column phase: tiles of kTileC columns staged in shared memory
+  constexpr int kTileC = kOwn < kRowStep ? kOwn : kRowStep;
+  auto columns = [&]() {
+    constexpr int kItems = kTileC * kN / (32 * kSolveWarps);  // elements per thread
+    constexpr int kRowsPer = 32 * kSolveWarps / kTileC;
+    const int cc = tid % kTileC, ro = tid / kTileC;
+    float2* const slot = scratch + (cc / kPer) * Wp::kScratch + (cc % kPer) * Wp::kCol;
+    for (int c0 = rank * kOwn; c0 < (rank + 1) * kOwn; c0 += kTileC) {
+      float2* const tp = tmp + c0 + cc;
+      float2 x[kItems];
+#pragma unroll
+      for (int u = 0; u < kItems; ++u) x[u] = __ldcg(tp + (long long)(kRowsPer * u + ro) * kN);
+#pragma unroll
+      for (int u = 0; u < kItems; ++u) slot[kRowsPer * u + ro] = x[u];
+      __syncthreads();
+      if (w * kPer < kTileC) {
+        float2* const mine = xs + (l / T) * Wp::kCol;
+        const float* g = filtT + (long long)(c0 + w * kPer + l / T) * kN;
+        float gv[16];
+#pragma unroll
+        for (int m = 0; m < 16; ++m) gv[m] = g[T * m + t];
+        float2 v[16];
+#pragma unroll
+        for (int m = 0; m < 16; ++m) v[m] = mine[T * m + t];
+        __syncwarp();
+        fft_warp<T>(v, xs, twr);
+#pragma unroll
+        for (int m = 0; m < 16; ++m) v[m] = make_float2(v[m].x * gv[m], -v[m].y * gv[m]);
+        fft_warp<T>(v, xs, twr);
+#pragma unroll
+        for (int m = 0; m < 16; ++m) mine[T * m + t] = cconj(v[m]);
+      }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < kItems; ++u) tp[(long long)(kRowsPer * u + ro) * kN] = slot[kRowsPer * u + ro];
+      __syncthreads();
+    }
+  };
+  // inverse row phase: z of the owned rows, partials of r.z and (d - dbar) z^2
+  const float scale = 1.0f / ((float)kN * (float)kN);
+  auto rows_inv = [&]() {
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int row = row0; row < row_end; row += kRowStep) {
+      const long long p0 = (long long)row * kN + t;
+      float2 v[16];
+      float ra[16], rb[16], dv[16];
+#pragma unroll
+      for (int m = 0; m < 16; ++m) {
+        v[m] = cconj(__ldcg(tmp + p0 + T * m));
+        ra[m] = a.Rr[j0 * N + p0 + T * m];
+        rb[m] = two ? a.Rr[j1 * N + p0 + T * m] : 0.f;
+        dv[m] = a.D[p0 + T * m];
+      }
+      fft_warp<T>(v, xs, twr);
+      float s0 = 0.f, s1 = 0.f, q0 = 0.f, q1 = 0.f;
+#pragma unroll
+      for (int m = 0; m < 16; ++m) {
+        const float z0 = v[m].x * scale, z1 = -v[m].y * scale;
+        a.Z[j0 * N + p0 + T * m] = z0;
+        s0 = fmaf(ra[m], z0, s0);
+        q0 = fmaf((dv[m] - dbar) * z0, z0, q0);
+        if (two) {
+          a.Z[j1 * N + p0 + T * m] = z1;
+          s1 = fmaf(rb[m], z1, s1);
+          q1 = fmaf((dv[m] - dbar) * z1, z1, q1);
+        }
+      }
+      acc[0] += (double)s0;
+      acc[1] += (double)q0;
+      acc[2] += (double)s1;
+      acc[3] += (double)q1;
+    }
+    cluster_sum<kSolveWarps, 4>(cl, acc, red, slot_gd);
+  };
+  // alpha and beta (pw_tail), by warp 0, lane u for system u
+  double gamma_old = 0.0, den_old = 0.0;
+  auto coefficients = [&](bool first) {
+    if (w == 0) {
+      static_assert(kSolveCtas == 8, "32 partials, one per lane");
+      double x = slot_gd[l >> 2][l & 3];
+#pragma unroll
+      for (int off = 4; off < 32; off <<= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+      const double gamma = __shfl_sync(0xffffffffu, x, 2 * (l & 1));
+      const double delta = gamma + __shfl_sync(0xffffffffu, x, 2 * (l & 1) + 1);
+      double beta = 0.0, den = delta;
+      if (!first) {
+        beta = gamma * recip_f64(gamma_old);
+        den = delta - beta * beta * den_old;  // beta gamma / alpha(old), alpha(old) = gamma(old) / den(old)
+        if (!(den > 0.0)) {
+          beta = 0.0;
+          den = delta;
+        }
+      }
+      if (l < 2) {
+        coef[l][0] = (float)beta;
+        coef[l][1] = (float)(gamma * recip_f64(den));
+      }
+      gamma_old = gamma;
+      den_old = den;
+    }
+    __syncthreads();
+  };
+
+  // the first z: forward rows of the true residual
+  for (int row = row0; row < row_end; row += kRowStep) {
+    const long long p0 = (long long)row * kN + t;
+    float2 v[16];
+#pragma unroll
+    for (int m = 0; m < 16; ++m)
+      v[m] = make_float2(a.Rr[j0 * N + p0 + T * m], two ? a.Rr[j1 * N + p0 + T * m] : 0.f);
+    fft_warp<T>(v, xs, twr);
+#pragma unroll
+    for (int m = 0; m < 16; ++m) tmp[p0 + T * m] = v[m];
+  }
+  cl.sync();
+  columns();
+  cl.sync();
+  rows_inv();
+  cl.sync();
+  coefficients(true);
+  int it = 0;
+  unsigned long long units = 0;
+  while (true) {
+    // the CG step and the forward rows of the new residual (pw_update_rows_fwd_kernel)
+    const bool first = it == 0;
+    float rr[2] = {0.f, 0.f};
+    for (int row = row0; row < row_end; row += kRowStep) {
+      const long long p0 = (long long)row * kN + t;
+      float2 v[16];
+#pragma unroll
+      for (int m = 0; m < 16; ++m) v[m] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        if (!(u ? act1 : act0)) continue;
+        const float beta = coef[u][0], alpha = coef[u][1];
+        const long long o = (long long)(j0 + u) * N + p0;
+        constexpr int kB = 8;  // elements per lane whose loads are in flight together
+#pragma unroll
+        for (int b = 0; b < 16; b += kB) {
+          float zv[kB], rv[kB], sv[kB], pv[kB], ev[kB], dv[kB];
+#pragma unroll
+          for (int k = 0; k < kB; ++k) {
+            const long long q = o + T * (b + k);
+            zv[k] = a.Z[q];
+            rv[k] = a.Rr[q];
+            dv[k] = a.D[p0 + T * (b + k)];
+            sv[k] = pv[k] = ev[k] = 0.f;
+            if (!first) {
+              sv[k] = a.Qp[q];
+              pv[k] = a.P[q];
+              ev[k] = a.Ec[q];
+            }
+          }
+#pragma unroll
+          for (int k = 0; k < kB; ++k) {
+            const long long q = o + T * (b + k);
+            const float pn = fmaf(beta, pv[k], zv[k]);
+            const float sn = fmaf(beta, sv[k], fmaf(dv[k] - dbar, zv[k], rv[k]));
+            const float r = fmaf(-alpha, sn, rv[k]);
+            a.P[q] = pn;
+            a.Qp[q] = sn;
+            a.Ec[q] = fmaf(alpha, pn, ev[k]);
+            a.Rr[q] = r;
+            rr[u] = fmaf(r, r, rr[u]);
+            (u ? v[b + k].y : v[b + k].x) = r;
+          }
+        }
+      }
+      fft_warp<T>(v, xs, twr);
+#pragma unroll
+      for (int m = 0; m < 16; ++m) tmp[p0 + T * m] = v[m];
+    }
+    units += (unsigned long long)(act0 + act1);
+    ++it;
+    cluster_sum<kSolveWarps, 2>(cl, {(double)rr[0], (double)rr[1]}, red, slot_rr);
+    cl.sync();
+    if (w == 0) {
+      double r2 = l < 16 ? slot_rr[l >> 1][l & 1] : 0.0;
+#pragma unroll
+      for (int off = 2; off < 16; off <<= 1) r2 += __shfl_xor_sync(0xffffffffu, r2, off);
+      if (l < 2) stop[l] = j0 + l < f.R && still_active(a, j0 + l, r2) == 0.f;
+    }
+    __syncthreads();
+    act0 = act0 && !stop[0];
+    act1 = act1 && !stop[1];
+    if ((!act0 && !act1) || it >= budget) break;
+    columns();
+    cl.sync();
+    rows_inv();
+    cl.sync();
+    coefficients(false);
+  }
+  // x += e on the owned rows
+  for (long long q = (long long)rank * kOwn * kN + tid; q < (long long)row_end * kN; q += blockDim.x) {
+    if (started0) a.X[j0 * N + q] += (double)a.Ec[j0 * N + q];
+    if (started1) a.X[j1 * N + q] += (double)a.Ec[j1 * N + q];
+  }
+  if (rank == 0 && tid == 0) {
+    atomicMax(pass_its, it);
+    if (f.counters) {
+      atomicAdd(&f.counters[DC_CG_UPD_UNITS], units);
+      atomicAdd(&f.counters[DC_CG_PRE_UNITS], (unsigned long long)it * (two ? 2ull : 1ull));
+    }
+  }
 }
 
 // Runs fn<T>() for the transform length n = 16 T.
@@ -2579,8 +3115,10 @@ inline int warp_rows_per_block(int n) {
   with_warp(n, [&](auto t) { r = Warp<decltype(t)::value>::kRows; });
   return r;
 }
-// Where the table of the n-point transform lies in the twiddle buffer (tw512_kernel).
-inline int warp_twiddles(int n) { return n == 512 ? 0 : n == 256 ? 2 * kF : n == 128 ? 2 * kF + 256 : 2 * kF + 384; }
+// Where the table of the n-point transform lies in the twiddle buffer (twiddle_kernel).
+inline int warp_twiddles(int n) {
+  return n == 512 ? 0 : kTw512 + kF + (n == 256 ? 0 : n == 128 ? 256 : 384);
+}
 
 // ---- register-resident 1024-point transforms
 //
@@ -2613,11 +3151,11 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_rows_fwd_kernel(Ff
   if (pair_idle(f, blockIdx.y)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0 && f.counters)
     atomicAdd(&f.counters[DC_CG_PRE_UNITS], 2 * blockIdx.y + 1 < f.R ? 2ull : 1ull);
-  __shared__ float2 tw[kF], tw2[kF];
+  __shared__ float2 tw[kTw512], tw2[kF];
   __shared__ float2 scratch[kF512Warps][kXs];
-  for (int m = threadIdx.x; m < kF; m += blockDim.x) {
+  for (int m = threadIdx.x; m < kTw512; m += blockDim.x) {
     tw[m] = f.tw512[m];
-    tw2[m] = f.tw1024[m];
+    if (m < kF) tw2[m] = f.tw1024[m];
   }
   __syncthreads();
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -2666,18 +3204,18 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_update_rows_fwd_ke
     atomicAdd(&f.counters[DC_CG_UPD_UNITS], (unsigned long long)(act0 + act1));
   }
   const int it = a.it_dev ? *a.it_dev : it_arg;
-  __shared__ float2 tw[kF], tw2[kF];
+  __shared__ float2 tw[kTw512], tw2[kF];
   __shared__ float2 scratch[kF512Warps][kXs];
   __shared__ float alpha_s[2];
-  for (int m = threadIdx.x; m < kF; m += blockDim.x) {
+  for (int m = threadIdx.x; m < kTw512; m += blockDim.x) {
     tw[m] = f.tw512[m];
-    tw2[m] = f.tw1024[m];
+    if (m < kF) tw2[m] = f.tw1024[m];
   }
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   if (w < 2 && (w == 0 ? act0 : act1)) {
     const int j = j0 + w;
     const double pqs = group_sum(a.part_pq + (long long)j * a.nb, a.nb);
-    if (l == 0) alpha_s[w] = (float)(a.rzs[j] / pqs);
+    if (l == 0) alpha_s[w] = (float)(a.rzs[j] * recip_f64(pqs));
   }
   __syncthreads();
   const long long N = (long long)f.H * f.W;
@@ -2780,19 +3318,19 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_update_rows_fwd_ke
 
 // fft_cols_filter_kernel for HP = 1024: the block stages columns c0 .. c0 + 7 of a pair
 // (extended to 1024 rows); each warp transforms one column, filters it with
-// hthT (column-major, [c][i]), writes it back to its slot in natural order and
+// filtT (column-major, [c][i]), writes it back to its slot in natural order and
 // transforms it again (the inverse as conj(F(conj(.)))); the block then stores the fold
 // to H rows.  Shared memory: kF512Warps x kXs2 float2, dynamic.
 __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_cols_filter_kernel(FftDesc f,
-                                                                             const float* __restrict__ hthT) {
+                                                                             const float* __restrict__ filtT) {
   loop_step(f);
   if (pair_idle(f, blockIdx.y)) return;
-  __shared__ float2 tw[kF], tw2[kF];
+  __shared__ float2 tw[kTw512], tw2[kF];
   extern __shared__ float4 colsm4[];
   float2* cols = reinterpret_cast<float2*>(colsm4);
-  for (int m = threadIdx.x; m < kF; m += blockDim.x) {
+  for (int m = threadIdx.x; m < kTw512; m += blockDim.x) {
     tw[m] = f.tw512[m];
-    tw2[m] = f.tw1024[m];
+    if (m < kF) tw2[m] = f.tw1024[m];
   }
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   const int c0 = blockIdx.x * kF512Warps;
@@ -2826,14 +3364,12 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_cols_filter_kernel
   fft1024_warp(lo, hi, xs, tw, tw2);
   // filter (frequencies 64 m + 2 l and 64 m + 2 l + 1 of this lane), conjugated for the
   // inverse, and back to natural order in the slot
-  const float* g = hthT + (long long)(c0 + w) * (2 * kF);
-  const float dbar = (float)(*f.dbar);
+  const float* g = filtT + (long long)(c0 + w) * (2 * kF);
 #pragma unroll
   for (int m = 0; m < 16; ++m) {
     const float2 gv = *reinterpret_cast<const float2*>(g + 64 * m + 2 * l);
-    const float g0 = __frcp_rn(gv.x + dbar), g1 = __frcp_rn(gv.y + dbar);
-    lo[m] = make_float2(lo[m].x * g0, -lo[m].y * g0);
-    hi[m] = make_float2(hi[m].x * g1, -hi[m].y * g1);
+    lo[m] = make_float2(lo[m].x * gv.x, -lo[m].y * gv.x);
+    hi[m] = make_float2(hi[m].x * gv.y, -hi[m].y * gv.y);
   }
 #pragma unroll
   for (int m = 0; m < 16; ++m)
@@ -2867,11 +3403,11 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_rows_inv_kernel(Ff
                                                                           const float* __restrict__ Rr,
                                                                           float* Z, double* part_rz) {
   if (pair_idle(f, blockIdx.y)) return;
-  __shared__ float2 tw[kF], tw2[kF];
+  __shared__ float2 tw[kTw512], tw2[kF];
   __shared__ float2 scratch[kF512Warps][kXs];
-  for (int m = threadIdx.x; m < kF; m += blockDim.x) {
+  for (int m = threadIdx.x; m < kTw512; m += blockDim.x) {
     tw[m] = f.tw512[m];
-    tw2[m] = f.tw1024[m];
+    if (m < kF) tw2[m] = f.tw1024[m];
   }
   __syncthreads();
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -2997,6 +3533,13 @@ __global__ void hth_kernel(float* out, int H, int W, const float* k, int kh, int
   }
 }
 
+// The preconditioner's filter of one update.
+__global__ void filter_kernel(const float* hth, const double* dbar, float* filt, long long n) {
+  const float d = (float)(*dbar);
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    filt[i] = __frcp_rn(hth[i] + d);
+}
+
 // Number of systems still active after the last update (their flags).
 __global__ void check_kernel(const float* scal, int R, int* active) {
   int cnt = 0;
@@ -3015,14 +3558,17 @@ __global__ void check_kernel(const float* scal, int R, int* active) {
 
 // ---- device-driven solver loop (CUDA graph with conditional nodes)
 //
-// The refinement passes and the CG iterations of a pass run as two nested WHILE
-// nodes of a graph, with an IF node around each pass; their conditions are set
-// by the kernels below from counters in device memory, so a likelihood-site
-// update needs no host round trip.  The outer body (and the inner one with Jacobi)
-// starts by clearing its own condition (cond_clear_kernel), so a body that did not
-// set it again ends the loop; with the FFT preconditioner the column pass of every
-// iteration sets the inner condition to 0 or 1 (loop_step).  The counters bound
-// both loops (max_outer passes, max_iter iterations).
+// The refinement passes and the CG iterations of a pass run as two nested WHILE nodes of
+// a graph; their conditions are set by the kernels from counters in device memory, so a
+// likelihood-site update needs no host round trip.  The first true residual and its
+// thresholds come before the outer loop; its body is one pass, the residual after it and
+// the thresholds, which set both conditions to 0 or 1 (start_pass).  With the FFT
+// preconditioner the column pass of every iteration sets the inner condition to 0 or 1
+// (loop_step); with Jacobi the inner body starts by clearing its own (cond_clear_kernel).
+// The counters bound both loops (max_outer passes, max_iter iterations).
+// Going round a WHILE node costs about as much as a small kernel, so the inner body holds
+// kUnroll iterations; those past the end of a pass find every system stopped and return.
+constexpr int kUnroll = 4;
 // Iterative refinement of the likelihood-site solves: a true residual in
 // float-float, then FP32 preconditioned CG on the correction until its recurrence
 // residual has dropped below max(eta ||r||, (rtol / 2) ||b||), repeated until
@@ -3034,34 +3580,6 @@ constexpr double kEta2 = 1e-9;
 
 __global__ void cond_clear_kernel(cudaGraphConditionalHandle h) {
   if (threadIdx.x == 0) cudaGraphSetConditional(h, 0u);
-}
-
-__global__ void loop_init_kernel(LoopState* ls) {
-  if (threadIdx.x == 0) {
-    ls->it = 0;
-    ls->outer = 0;
-    ls->total = 0;
-    ls->converged = 0;
-  }
-}
-
-// After a true residual and its thresholds: start another pass, or stop
-// (converged, or out of passes or iterations), as the host loop does.
-__global__ void pass_kernel(LoopState* ls, const int* active, int max_outer, int max_iter,
-                            cudaGraphConditionalHandle h_outer, cudaGraphConditionalHandle h_pass,
-                            cudaGraphConditionalHandle h_inner) {
-  if (threadIdx.x != 0) return;
-  unsigned go = 0;
-  if (*active == 0) {
-    ls->converged = 1;
-  } else if (ls->outer < max_outer && ls->total < max_iter) {
-    go = 1;
-    ls->it = 0;
-    ls->outer += 1;
-  }
-  cudaGraphSetConditional(h_pass, go);
-  cudaGraphSetConditional(h_outer, go);
-  cudaGraphSetConditional(h_inner, go);
 }
 
 // After a CG iteration: count it, and go on while a system is active and the
@@ -3264,11 +3782,13 @@ struct LikelihoodState {
   int nbz = 0, nbmax = 0;
   // circulant FFT preconditioner (power-of-two sizes)
   bool fft = false;
+  bool pw = false;          // pointwise products: the image fills the torus (pw_update_rows_fwd_kernel)
+  bool solve = false;       // and is square: a pass is one kernel (pw_solve_kernel)
   FftDesc fd;
   float2* ftmp = nullptr;
   float* Z = nullptr;
-  float* hth = nullptr;
-  float2* tw512 = nullptr;      // w512^m, w1024^m (m < 512), the tables of the shorter transforms
+  float* hth = nullptr;         // |h_f|^2 / xi, then the filter of the current update
+  float2* tw512 = nullptr;      // the twiddle tables (twiddle_kernel)
   float* window = nullptr;      // the windows of the rows (HP), then of the columns (WP)
   double* dpart = nullptr;
   double* dbar = nullptr;
@@ -3284,6 +3804,7 @@ struct LikelihoodState {
   float* d_scal = nullptr;      // [R][4] CG scalars: active flag, beta, alpha and iteration of
                                 // a deferred correction update
   double* d_rzs = nullptr;      // [R] r.z of the current iteration
+  double* d_alphas = nullptr;   // [R] alpha of the current iteration (pointwise products)
   unsigned* d_arrive = nullptr; // [R + pairs] block-arrival counters (start and stay zero)
   int* d_act0 = nullptr;        // [R] systems that iterate in the current pass
   float* Ec = nullptr;          // R planes: FP32 correction of the current pass
@@ -3374,6 +3895,9 @@ void precond_apply(LikelihoodState* L, double* rz_buf, bool cg, int first,
   f.scal_w = cg ? L->d_scal : nullptr;
   f.rzs = cg ? L->d_rzs : nullptr;
   f.arrive = L->d_arrive + L->R;
+  f.D = L->D;
+  f.part_dl = L->part;  // the p.q partials' place: pointwise products have none
+  f.alphas = L->d_alphas;
   f.first = first;
   f.counters = counters;
   constexpr int kRows1024 = kF512Warps * kRowsPerWarp1024;
@@ -3383,7 +3907,9 @@ void precond_apply(LikelihoodState* L, double* rz_buf, bool cg, int first,
       with_warp(f.WP, [&](auto t) {
         constexpr int T = decltype(t)::value;
         const dim3 grid((f.H + Warp<T>::kRows - 1) / Warp<T>::kRows, f.pairs);
-        if (upd)
+        if (upd && L->pw)
+          pw_update_rows_fwd_kernel<T><<<grid, kWt, 0, s>>>(f, *upd, it);
+        else if (upd)
           warp_update_rows_fwd_kernel<T><<<grid, kWt, 0, s>>>(f, *upd, it);
         else
           warp_rows_fwd_kernel<T><<<grid, kWt, 0, s>>>(f, L->Rr);
@@ -3403,23 +3929,46 @@ void precond_apply(LikelihoodState* L, double* rz_buf, bool cg, int first,
   if (warp_cols(f))
     with_warp(f.HP, [&](auto t) {
       constexpr int T = decltype(t)::value;
-      warp_cols_filter_kernel<T><<<dim3(f.WP / Warp<T>::kCols, f.pairs), kWt, 0, s>>>(f, f.hth);
+      warp_cols_filter_kernel<T><<<dim3(f.WP / Warp<T>::kCols, f.pairs), kWt, 0, s>>>(f, f.filt);
     });
   else if (fft1024_cols(f))
     fft1024_cols_filter_kernel<<<dim3(f.WP / kF512Warps, f.pairs), kWt, sizeof(float2) * kF512Warps * kXs2, s>>>(
-        f, f.hth);
+        f, f.filt);
   else
     fft_cols_filter_kernel<<<dim3(f.WP / f.cw, f.pairs), kFftThreads, L->smem_cols, s>>>(f);
   if (warp_rows(f))
     with_warp(f.WP, [&](auto t) {
       constexpr int T = decltype(t)::value;
-      warp_rows_inv_kernel<T><<<dim3(f.nbz, f.pairs), kWt, 0, s>>>(f, L->Rr, L->Z, rz_buf);
+      if (L->pw && cg)
+        warp_rows_inv_kernel<T, true><<<dim3(f.nbz, f.pairs), kWt, 0, s>>>(f, L->Rr, L->Z, rz_buf);
+      else
+        warp_rows_inv_kernel<T, false><<<dim3(f.nbz, f.pairs), kWt, 0, s>>>(f, L->Rr, L->Z, rz_buf);
     });
   else if (fft1024_rows(f))
     fft1024_rows_inv_kernel<<<dim3(f.nbz, f.pairs), kWt, 0, s>>>(f, L->Rr, L->Z, rz_buf);
   else
     fft_rows_inv_kernel<<<dim3(f.nbz, f.pairs), kFftThreads, L->smem_rows, s>>>(f, L->Rr, L->Z,
                                                                                 rz_buf);
+}
+
+void launch_filter(const LikelihoodState* L, cudaStream_t s) {
+  if (!L->fft) return;
+  const long long n = (long long)L->fd.HP * L->fd.WP;
+  filter_kernel<<<std::min(grid1d(n), 4096), 256, 0, s>>>(L->fd.hth, L->fd.dbar, L->fd.filt, n);
+}
+
+// All CG iterations of a pass and its commit (L->solve).  ls: the graph's loop state, or NULL
+// (budget: the iterations left).
+void launch_solve(LikelihoodState* L, const CgArgs& a, const LoopState* ls, int budget,
+                  unsigned long long* counters, cudaStream_t s) {
+  FftDesc f = L->fd;
+  f.max_iter = L->max_iter;
+  f.counters = counters;
+  with_warp(f.WP, [&](auto t) {
+    constexpr int T = decltype(t)::value;
+    pw_solve_kernel<T><<<f.pairs * kSolveCtas, 32 * solve_warps<T>(), solve_smem<T>(), s>>>(f, a, f.filt, ls, budget,
+                                                                                     &L->d_loop->pass_its);
+  });
 }
 
 // The true residual of every system: two systems per block for a separable K x K blur,
@@ -3432,7 +3981,10 @@ void launch_residual_pair(const LikelihoodState* L, const CgArgs& a, cudaStream_
   residual_pair_kernel<K><<<dim3(c.tiles_x, c.tiles_y, (L->R + 1) / 2), kThreads, sm, s>>>(a);
 }
 
-void launch_residual(const LikelihoodState* L, const CgArgs& a, cudaStream_t s) {
+// all: every system, else those that iterated in the pass before (CgArgs::res_all).
+void launch_residual(const LikelihoodState* L, const CgArgs& args, bool all, cudaStream_t s) {
+  CgArgs a = args;
+  a.res_all = all ? 1 : 0;
   const ConvDesc& c = L->c;
   if (c.separable && c.kh == c.kw) {
     switch (c.kh) {
@@ -3600,7 +4152,9 @@ bool raise_smem_limits() {
                        (const void*)residual_pair_kernel<5>, (const void*)residual_pair_kernel<9>,
                        (const void*)residual_pair_kernel<15>,
                        (const void*)fft_rows_fwd_kernel, (const void*)fft_rows_inv_kernel,
-                       (const void*)fft_cols_filter_kernel, (const void*)fft1024_cols_filter_kernel};
+                       (const void*)fft_cols_filter_kernel, (const void*)fft1024_cols_filter_kernel,
+                       (const void*)pw_solve_kernel<4>, (const void*)pw_solve_kernel<8>,
+                       (const void*)pw_solve_kernel<16>, (const void*)pw_solve_kernel<32>};
   for (const void* f : fns) {
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, f) != cudaSuccess) return false;
@@ -3733,6 +4287,10 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
     const int rows_inv = warp_rows(f) ? warp_rows_per_block(WP) : kF512Warps * kRowsPerWarp1024;
     f.nbz = warp_rows(f) || fft1024_rows(f) ? (c.H + rows_inv - 1) / rows_inv : std::min(c.H, 64);
     L->nbz = f.nbz;
+    L->pw = c.H == HP && c.W == WP && warp_rows(f);
+    // 512^2: three kernels per iteration with 16 to 24 warps per SM are faster there (124
+    // against 173 us) than one cluster of eight 8-warp CTAs per pair
+    L->solve = L->pw && HP == WP && HP <= 256;
     L->smem_rows = sizeof(float2) * ((size_t)WP + (size_t)f.rpb * WP);
     L->smem_cols = sizeof(float2) * ((size_t)HP + (size_t)HP * f.cw);
   }
@@ -3767,7 +4325,7 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
             cudaMalloc(&L->d_hf, sizeof(float) * (kh * kw + kh + kw)) == cudaSuccess &&
             cudaMalloc(&L->Rr, sizeof(float) * RN) == cudaSuccess &&
             cudaMalloc(&L->P, sizeof(float) * RN) == cudaSuccess &&
-            cudaMalloc(&L->P2, sizeof(float) * RN) == cudaSuccess &&
+            (L->pw || cudaMalloc(&L->P2, sizeof(float) * RN) == cudaSuccess) &&
             cudaMalloc(&L->Qp, sizeof(float) * RN) == cudaSuccess &&
             cudaMalloc(&L->part, sizeof(double) * 4 * L->R * L->nbmax) == cudaSuccess &&
             cudaMalloc(&L->dpart, sizeof(double) * L->prep_blocks) == cudaSuccess &&
@@ -3775,7 +4333,7 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
             (!L->fft ||
              (cudaMalloc(&L->ftmp, sizeof(float2) * ((L->R + 1) / 2) * c.H * L->fd.WP) == cudaSuccess &&
               cudaMalloc(&L->Z, sizeof(float) * RN) == cudaSuccess &&
-              cudaMalloc(&L->hth, sizeof(float) * L->fd.HP * L->fd.WP) == cudaSuccess &&
+              cudaMalloc(&L->hth, 2 * sizeof(float) * L->fd.HP * L->fd.WP) == cudaSuccess &&
               cudaMalloc(&L->tw512, sizeof(float2) * kTwCount) == cudaSuccess &&
               cudaMalloc(&L->window, sizeof(float) * (L->fd.HP + L->fd.WP)) == cudaSuccess)) &&
             cudaMalloc(&L->d_active, sizeof(int)) == cudaSuccess &&
@@ -3784,6 +4342,7 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
             cudaMalloc(&L->d_rr0, sizeof(double) * L->R) == cudaSuccess &&
             cudaMalloc(&L->d_scal, sizeof(float) * 4 * L->R) == cudaSuccess &&
             cudaMalloc(&L->d_rzs, sizeof(double) * L->R) == cudaSuccess &&
+            cudaMalloc(&L->d_alphas, sizeof(double) * L->R) == cudaSuccess &&
             cudaMalloc(&L->d_arrive, sizeof(unsigned) * (L->R + (L->R + 1) / 2)) == cudaSuccess &&
             cudaMalloc(&L->d_act0, sizeof(int) * L->R) == cudaSuccess &&
             cudaMalloc(&L->d_loop, sizeof(LoopState)) == cudaSuccess &&
@@ -3854,13 +4413,14 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
   if (L->fft) {
     L->fd.tmp = L->ftmp;
     L->fd.hth = L->hth;
+    L->fd.filt = L->hth + (size_t)L->fd.HP * L->fd.WP;
     L->fd.tw512 = L->tw512;
-    L->fd.tw1024 = L->tw512 + kF;
+    L->fd.tw1024 = L->tw512 + kTw512;
     L->fd.twr = L->tw512 + warp_twiddles(L->fd.WP);
     L->fd.twc = L->tw512 + warp_twiddles(L->fd.HP);
     L->fd.wr = L->window;
     L->fd.wc = L->window + L->fd.HP;
-    tw512_kernel<<<(kTwCount + 255) / 256, 256, 0, s>>>(L->tw512);
+    twiddle_kernel<<<(kTwCount + 255) / 256, 256, 0, s>>>(L->tw512);
     window_kernel<<<(L->fd.HP + 255) / 256, 256, 0, s>>>(L->window, c.H, L->fd.HP);
     window_kernel<<<(L->fd.WP + 255) / 256, 256, 0, s>>>(L->window + L->fd.HP, c.W, L->fd.WP);
     L->fd.dbar = L->dbar;
@@ -3928,6 +4488,7 @@ void likelihood_destroy(LikelihoodState* L) {
   cudaFree(L->d_rr0);
   cudaFree(L->d_scal);
   cudaFree(L->d_rzs);
+  cudaFree(L->d_alphas);
   cudaFree(L->d_arrive);
   cudaFree(L->d_act0);
   cudaFree(L->d_loop);
@@ -3969,7 +4530,7 @@ namespace {
 
 // The likelihood-site update of likelihood_update below as one graph: the prior
 // sites tp/np in, site 0 out; the refinement passes and the CG iterations are
-// WHILE nodes, each pass an IF node (see LoopState).  Built by stream capture
+// nested WHILE nodes (see LoopState).  Built by stream capture
 // into the graph and its conditional bodies, one at a time; false if CUDA
 // refuses any step (the caller then keeps the host-driven loop).
 bool build_update_graph(LikelihoodState* L, float* tau, float* nu, const float* tp, const float* np,
@@ -3981,15 +4542,15 @@ bool build_update_graph(LikelihoodState* L, float* tau, float* nu, const float* 
   CgArgs a = cg_args(L);
   a.counters = counters;
   a.it_dev = &L->d_loop->it;
-  a.defer_e = fused_update(L) && pair_direction(L);
+  a.defer_e = !L->pw && fused_update(L) && pair_direction(L);
   const dim3 grid(c.tiles_x, c.tiles_y, L->R);
   const int groups = (L->S + kRbGroup - 1) / kRbGroup;
   cudaGraph_t G = nullptr;
   if (cudaGraphCreate(&G, 0) != cudaSuccess) return false;
-  cudaGraphConditionalHandle h_outer = 0, h_pass = 0, h_inner = 0;
-  bool ok = cudaGraphConditionalHandleCreate(&h_outer, G, 1, cudaGraphCondAssignDefault) == cudaSuccess &&
-            cudaGraphConditionalHandleCreate(&h_pass, G, 0, cudaGraphCondAssignDefault) == cudaSuccess &&
-            cudaGraphConditionalHandleCreate(&h_inner, G, 0, cudaGraphCondAssignDefault) == cudaSuccess;
+  cudaGraphConditionalHandle h_outer = 0, h_inner = 0;
+  bool ok = cudaGraphConditionalHandleCreate(&h_outer, G, 0, cudaGraphCondAssignDefault) == cudaSuccess &&
+            (L->solve ||
+             cudaGraphConditionalHandleCreate(&h_inner, G, 0, cudaGraphCondAssignDefault) == cudaSuccess);
   // a conditional node after the current capture dependencies of s; *body gets its graph
   auto add_cond = [&](cudaGraphConditionalHandle h, cudaGraphConditionalNodeType type,
                       cudaGraph_t* body) -> bool {
@@ -4020,12 +4581,22 @@ bool build_update_graph(LikelihoodState* L, float* tau, float* nu, const float* 
     const bool ended = cudaStreamEndCapture(s, &tmp) == cudaSuccess;
     return fine && ended && cudaGetLastError() == cudaSuccess;
   };
-  cudaGraph_t b_outer = nullptr, b_pass = nullptr, b_inner = nullptr;
+  cudaGraph_t b_outer = nullptr, b_inner = nullptr;
+  auto residual = [&](bool all) {
+    launch_residual(L, a, all, s);
+    const PassArgs pass{L->d_loop, L->max_outer, L->max_iter, L->solve ? 0 : 1, h_outer, h_inner};
+    thresholds_kernel<<<1, 1024, 0, s>>>(a.part_rr, a.part_bb, a.part_rz, a.fft, L->R, L->nb,
+                                         L->rtol2_true, L->rtol2_probe, kEta2, L->thr, L->d_relres,
+                                         L->d_prev_rr, L->d_rr0, 0, L->d_active, L->d_scal, L->d_act0,
+                                         L->d_rzs, pass);
+  };
   ok = ok && capture(G, [&]() {
     prep_kernel<<<L->prep_blocks, kThreads, 0, s>>>(tp, np, N, c.g0_xi, L->D, L->Ncav, L->Minv,
                                                     L->dpart);
-    mean_kernel<<<1, 1024, 0, s>>>(L->dpart, L->prep_blocks, 1.0 / (double)N, L->dbar);
-    loop_init_kernel<<<1, 32, 0, s>>>(L->d_loop);
+    mean_kernel<<<1, 1024, 0, s>>>(L->dpart, L->prep_blocks, 1.0 / (double)N, L->dbar, (int*)L->d_loop,
+                                   (int)(sizeof(LoopState) / sizeof(int)));
+    launch_filter(L, s);
+    residual(true);
     if (!add_cond(h_outer, cudaGraphCondTypeWhile, &b_outer)) return false;
     loop_finish_kernel<<<1, 32, 0, s>>>(L->d_loop, status, counters);
     rb_offdiag_kernel<<<dim3(c.tiles_x, c.tiles_y, groups), kThreads, L->smem, s>>>(a, L->Qp);
@@ -4034,38 +4605,35 @@ bool build_update_graph(LikelihoodState* L, float* tau, float* nu, const float* 
     return true;
   });
   ok = ok && capture(b_outer, [&]() {
-    cond_clear_kernel<<<1, 32, 0, s>>>(h_outer);
-    launch_residual(L, a, s);
-    thresholds_kernel<<<1, 1024, 0, s>>>(a.part_rr, a.part_bb, a.part_rz, a.fft, L->R, L->nb,
-                                         L->rtol2_true, L->rtol2_probe, kEta2, L->thr, L->d_relres,
-                                         L->d_prev_rr, L->d_rr0, 0, &L->d_loop->outer, L->d_active,
-                                         L->d_scal, L->d_act0, L->d_rzs);
-    pass_kernel<<<1, 32, 0, s>>>(L->d_loop, L->d_active, L->max_outer, L->max_iter, h_outer, h_pass,
-                                 h_inner);
-    return add_cond(h_pass, cudaGraphCondTypeIf, &b_pass);
-  });
-  ok = ok && capture(b_pass, [&]() {
+    if (L->solve) {
+      launch_solve(L, a, L->d_loop, 0, counters, s);
+      residual(false);
+      return true;
+    }
     if (L->fft) precond_apply(L, a.part_rz, true, 1, counters, s);
     if (!add_cond(h_inner, cudaGraphCondTypeWhile, &b_inner)) return false;
     commit_kernel<<<dim3(std::min(grid1d((N + 3) / 4), 1024), L->R), 256, 0, s>>>(
         L->X, L->Ec, L->d_act0, N, a.defer_e ? L->d_scal : nullptr, L->P, L->P2);
+    residual(false);
     return true;
   });
   // with the FFT preconditioner the column pass, which every iteration launches,
   // counts the iteration and sets the condition (0 or 1, and 0 once the budget is
   // spent); Jacobi keeps the clearing and counting kernels
-  ok = ok && capture(b_inner, [&]() {
+  ok = ok && (L->solve || capture(b_inner, [&]() {
     if (!L->fft) cond_clear_kernel<<<1, 32, 0, s>>>(h_inner);
-    launch_direction(L, a, 0, s);
-    if (fused_update(L)) {
-      precond_apply(L, a.part_rz, true, 0, counters, s, &a, 0, 3, true, h_inner);
-    } else {
-      update_kernel<<<grid, kUpdThreads, 0, s>>>(a, 0);
-      if (L->fft) precond_apply(L, a.part_rz, true, 0, counters, s, nullptr, 0, 3, true, h_inner);
+    for (int k = 0; k < (L->fft ? kUnroll : 1); ++k) {
+      if (!L->pw) launch_direction(L, a, 0, s);
+      if (fused_update(L)) {
+        precond_apply(L, a.part_rz, true, 0, counters, s, &a, 0, 3, true, h_inner);
+      } else {
+        update_kernel<<<grid, kUpdThreads, 0, s>>>(a, 0);
+        if (L->fft) precond_apply(L, a.part_rz, true, 0, counters, s, nullptr, 0, 3, true, h_inner);
+      }
     }
     if (!L->fft) iter_kernel<<<1, 64, 0, s>>>(L->d_loop, L->d_scal, L->R, L->max_iter, h_inner);
     return true;
-  });
+  }));
   cudaGraphExec_t exec = nullptr;
   ok = ok && cudaGraphInstantiate(&exec, G, 0) == cudaSuccess;
   cudaGraphDestroy(G);
@@ -4109,24 +4677,25 @@ ep_tv_status likelihood_update(LikelihoodState* L, float* tau, float* nu, const 
   const long long N = c.N;
   prep_kernel<<<L->prep_blocks, kThreads, 0, s>>>(tp, np, N, c.g0_xi, L->D, L->Ncav, L->Minv,
                                                   L->dpart);
-  mean_kernel<<<1, 1024, 0, s>>>(L->dpart, L->prep_blocks, 1.0 / (double)N, L->dbar);
+  mean_kernel<<<1, 1024, 0, s>>>(L->dpart, L->prep_blocks, 1.0 / (double)N, L->dbar, nullptr, 0);
+  launch_filter(L, s);
   CgArgs a = cg_args(L);
   a.counters = counters;
-  a.defer_e = fused_update(L) && pair_direction(L);
+  a.defer_e = !L->pw && fused_update(L) && pair_direction(L);
   dim3 grid(c.tiles_x, c.tiles_y, L->R);
   // Iterative refinement (see kEta2): true residual (float-float), then FP32
   // preconditioned CG on the correction, repeated until ||r|| <= rtol ||b||.
   const double eta2 = kEta2;
-  int total = 0, iters = 0;
+  int total = 0, iters = 0, prev_active = 0;
   bool converged = false;
   for (int outer = 0;; ++outer) {
     tr->begin(EP_TV_K_CG_RESIDUAL, s);
-    launch_residual(L, a, s);
-    tr->end(s, (double)L->R * N);
+    launch_residual(L, a, outer == 0, s);
+    tr->end(s, (double)(outer == 0 ? L->R : prev_active) * N);
     thresholds_kernel<<<1, 1024, 0, s>>>(a.part_rr, a.part_bb, a.part_rz, a.fft, L->R, L->nb,
                                          L->rtol2_true, L->rtol2_probe, eta2, L->thr, L->d_relres,
-                                         L->d_prev_rr, L->d_rr0, outer == 0, nullptr, L->d_active,
-                                         L->d_scal, L->d_act0, L->d_rzs);
+                                         L->d_prev_rr, L->d_rr0, outer == 0, L->d_active, L->d_scal,
+                                         L->d_act0, L->d_rzs, PassArgs{});
     if (cudaMemcpyAsync(L->h_active, L->d_active, sizeof(int), cudaMemcpyDeviceToHost, s) !=
             cudaSuccess ||
         cudaMemcpyAsync(L->h_relres, L->d_relres, sizeof(double) * L->R, cudaMemcpyDeviceToHost,
@@ -4149,6 +4718,19 @@ ep_tv_status likelihood_update(LikelihoodState* L, float* tau, float* nu, const 
     }
     if (outer >= L->max_outer || total >= L->max_iter) break;
     const int started = L->h_active[0];  // systems that iterate in this pass
+    prev_active = started;
+    if (L->solve) {
+      int* const its = &L->d_loop->pass_its;
+      if (cudaMemsetAsync(its, 0, sizeof(int), s) != cudaSuccess) return EP_TV_ERR_CUDA;
+      tr->begin(EP_TV_K_CG_UPDATE, s);
+      launch_solve(L, a, nullptr, L->max_iter - total, counters, s);
+      tr->end(s, -1.0);
+      if (cudaMemcpyAsync(L->h_active + 1, its, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+          cudaStreamSynchronize(s) != cudaSuccess)
+        return EP_TV_ERR_CUDA;
+      total += L->h_active[1];
+      continue;
+    }
     if (L->fft) {
       // z = M^{-1} r of the true residual: r.z of every active system, beta = 0
       tr->begin(EP_TV_K_CG_PRECOND, s);
@@ -4163,9 +4745,11 @@ ep_tv_status likelihood_update(LikelihoodState* L, float* tau, float* nu, const 
     while (true) {
       const int n = std::min(kChunk, L->max_iter - total - launched);
       for (int t = 0; t < n; ++t) {
-        tr->begin(EP_TV_K_CG_DIRECTION, s);
-        launch_direction(L, a, launched, s);
-        tr->end(s, -1.0);
+        if (!L->pw) {
+          tr->begin(EP_TV_K_CG_DIRECTION, s);
+          launch_direction(L, a, launched, s);
+          tr->end(s, -1.0);
+        }
         if (fused_update(L)) {
           // the update with the preconditioner's forward row pass, then its other passes
           tr->begin(EP_TV_K_CG_UPDATE, s);
@@ -4234,6 +4818,9 @@ double likelihood_bytes_per_unit(const LikelihoodState* L, int kernel) {
   // with deferred correction updates the direction kernel also does e += alpha p
   // (read and write e; p is the direction it reads anyway) and the update only r
   const bool defer = fused_update(L) && pair_direction(L);
+  // pointwise products: read z, r, s, p, e; write r, s, p, e; with a pass in one kernel
+  // also the transforms' r in and z out
+  if (L->pw && kernel == EP_TV_K_CG_UPDATE) return L->solve ? 44.0 : 36.0;
   switch (kernel) {
     case EP_TV_K_CG_DIRECTION:               // read z, p; write p, Q p (per active system
       return defer ? 24.0 : 16.0;            // pixel); deferred: also read and write e

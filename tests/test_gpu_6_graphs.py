@@ -94,3 +94,36 @@ def test_deconv_update_graph_equals_host_driven_loop(h, w, kernel, em):
         assert g.stats()["cg_iters"] > 0
         rep = g.solver_report()
         assert rep["relres_mean"] <= 1e-9 and rep["relres_probe_max"] <= 1e-6
+
+
+@pytest.mark.parametrize("h,w,S,max_iter", [
+    (64, 64, 1, 0), (64, 64, 4, 0), (128, 128, 5, 0), (256, 256, 2, 0),  # a pass as one kernel
+    (64, 128, 3, 0), (128, 64, 2, 0), (512, 64, 4, 0),                   # three kernels per iteration
+    (64, 64, 2, 7), (128, 128, 1, 1), (128, 64, 2, 7), (38, 68, 2, 6)])  # the iteration budget runs out
+def test_deconv_pass_forms_graph_equals_host_driven_loop(h, w, S, max_iter):
+    """Images that fill the preconditioner's torus (products formed pointwise, a pass
+    in one kernel or three kernels per iteration), with odd and even system counts:
+    graph and host-driven loop agree bit for bit, also when the iteration budget, which
+    is no multiple of the loop body's iterations, runs out."""
+    from paper_2110_01585_gb300 import OP_CONV_PERIODIC
+    torch = cuda()
+    stream = torch.cuda.Stream()
+    p = syn.deconv_problem(h, w, kernel=syn.uniform_kernel(5), bsnr_db=30.0, beta0=2.0, seed=h + w,
+                           grf_length=8.0)
+    y = torch.as_tensor(p.y.astype(np.float32), device="cuda")
+    kw = dict(op=OP_CONV_PERIODIC, kernel=p.kernel, rbmc_samples=S, stream=stream,
+              cg_max_iter=max_iter or 20000)
+    with EPTV(y, p.xi, p.beta, **kw) as g, EPTV(y, p.xi, p.beta, **kw) as host:
+        host.trace(True)
+        g.sweep(3)
+        host.sweep(3)
+        got = [[t.view(torch.int32) for t in ep.sites() + ep.posterior()] for ep in (g, host)]
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(*got))
+        assert g.status() == host.status() and (g.status() == 0) == (max_iter == 0)
+        assert g.graph_sweeps() == 3 and host.graph_sweeps() == 0
+        rep = g.solver_report()
+        if max_iter:
+            assert g.stats()["cg_iters"] == max_iter and host.stats()["cg_iters"] == max_iter
+        else:
+            assert rep["relres_mean"] <= 1e-9 and rep["relres_probe_max"] <= 1e-6

@@ -33,7 +33,7 @@
 // stay on the FP64 CUDA cores.  The mean uses v = Z t and g = W^T v.
 //
 // Kernels here: an FP64 tiled GEMM (64 x 64 tiles, 4 x 4 per thread) for the
-// small products; the inverse of the Cholesky factor of one block of at most 64 rows on
+// small products; the inverse of the Cholesky factor of one block of at most 128 rows on
 // a cluster of SMs; column sums; matrix-vector products; the fast Walsh-Hadamard
 // transform and the gathers of the Hadamard operator.
 #include <cooperative_groups.h>
@@ -44,6 +44,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -55,7 +56,7 @@ namespace eptv {
 
 namespace {
 
-constexpr int kNb = 64;      // Cholesky / triangular-solve block size
+constexpr int kNb = 64;      // the recursion splits at multiples of this
 constexpr int kGt = 64;      // GEMM tile
 constexpr int kGk = 16;      // GEMM k step
 
@@ -379,60 +380,62 @@ __global__ void aty_kernel(const float* A, const float* y, int M, int N, float* 
   out[i] = (float)s;
 }
 
-// Z = L^{-1} of the Cholesky factor of the n x n (n <= 64) block K (lower triangle read),
+// Z = L^{-1} of the Cholesky factor of the n x n (n <= kBlk) block K (lower triangle read),
 // zeros above the diagonal; a pivot that is not positive raises the non-finite bit.
 //
 // One cluster of kBlkCtas CTAs.  What bounds a block is FP64: one SM retires about two
-// operations per clock, and the pivots form a chain of 64 x 5 dependent ones.  So the 64
-// rows are factored in four panels of 16 whose bulk work is spread over the cluster's SMs
-// (CTA c owns the rows, and then the columns of Z, that are c modulo the cluster's size),
-// each CTA keeping the block in its own shared memory:
-//   - the 16 x 16 diagonal block by Gaussian elimination on [S | I] in place, two entries
-//     per thread (a warp's FP64 instruction holds its quarter of the SM for 64 clocks), in
-//     every CTA alike: S = L1 D L1^T, L_pp^{-1} = D^{-1/2} L1^{-1}, one reciprocal per pivot
-//     (the square roots are taken once, at the end);
+// operations per clock, and the pivots form a chain of dependent ones.  So the rows are
+// factored in panels of 16 whose bulk work is spread over the cluster's SMs (CTA c owns the
+// rows, and then the columns of Z, that are c modulo the cluster's size), each CTA keeping
+// the block in its own shared memory:
+//   - the 16 x 16 diagonal block by Gaussian elimination on [S | I] in place, one entry per
+//     thread (a warp's FP64 instruction holds its quarter of the SM for 64 clocks), in every
+//     CTA alike: S = L1 D L1^T, L_pp^{-1} = D^{-1/2} L1^{-1}, one reciprocal per pivot (the
+//     square roots are taken once, at the end);
 //   - the owned rows of the panel, L21 = S21 L_pp^{-T}, written to every CTA;
 //   - the owned rows of the trailing update; the next diagonal block's written to every CTA;
 //   - at the end the owned columns of Z by block forward substitution.
 // Measured for 64 rows: 287 us as a one-block Cholesky with square root and division
-// per pivot and a one-thread-per-column inverse, 72 us with a diagonal block held by one
-// warp, 49 us in this form.
+// per pivot and a one-thread-per-column inverse, 54 us in this form; 128 rows take 139 us,
+// against 98 for two halves and about 140 for the four products between them.
+constexpr int kBlk = 128;
 constexpr int kBlkCtas = 8;
-constexpr int kBlkThreads = 128;
+constexpr int kBlkThreads = 256;
 constexpr int kPan = 16;
+constexpr int kBlkOwn = kBlk / kBlkCtas;  // columns of Z per CTA
+constexpr int kBlkPitch = kBlk + 1;
+constexpr size_t kBlkSmem =
+    sizeof(double) * (kBlk * kBlkPitch + kBlk / kPan * kPan * (kPan + 1) + kBlk * (kBlkOwn + 1));
 
 __global__ void __cluster_dims__(kBlkCtas, 1, 1) __launch_bounds__(kBlkThreads)
     chol_inv_block_kernel(const double* K, long long ld, double* Z, long long ldz, int n, unsigned* status) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank();
-  constexpr int kPitch = kNb + 1;
-  __shared__ double S[kNb * kPitch];
-  __shared__ double Zd[kNb / kPan][kPan][kPan + 1];
-  __shared__ double Y[kNb][kNb / kBlkCtas + 1];
+  extern __shared__ double blk_smem[];
+  double* const S = blk_smem;                                                       // [kBlk][kBlkPitch]
+  double (*Zd)[kPan][kPan + 1] = reinterpret_cast<double (*)[kPan][kPan + 1]>(S + kBlk * kBlkPitch);
+  double (*Y)[kBlkOwn + 1] = reinterpret_cast<double (*)[kBlkOwn + 1]>(&Zd[kBlk / kPan][0][0]);
   __shared__ double prow[2][kPan];
   const int tid = threadIdx.x, lane = tid & 31;
-  for (int e = tid; e < kNb * kNb; e += kBlkThreads) {
-    const int i = e / kNb, j = e % kNb;  // rows beyond n: the unit matrix
-    S[i * kPitch + j] = i < n && j <= i ? K[(long long)i * ld + j] : (i == j ? 1.0 : 0.0);
+  const int nn = (n + kPan - 1) / kPan * kPan;  // rows n .. nn - 1: those of the unit matrix
+  for (int e = tid; e < nn * nn; e += kBlkThreads) {
+    const int i = e / nn, j = e % nn;
+    S[i * kBlkPitch + j] = i < n && j <= i ? K[(long long)i * ld + j] : (i == j ? 1.0 : 0.0);
   }
   cl.sync();  // every CTA's copy is loaded before another writes into it
-  for (int p = 0; p < kNb / kPan; ++p) {
-    const int o = kPan * p;
+  for (int o = 0; o < nn; o += kPan) {
+    double (*Zp)[kPan + 1] = Zd[o / kPan];
     {
-      // row i = tid / 8, columns k0 and k0 + 1; a warp holds four whole rows
-      const int i = tid >> 3, k0 = 2 * (tid & 7);
-      auto sym = [&](int k) { return S[(o + max(i, k)) * kPitch + o + min(i, k)]; };
-      double a0 = sym(k0), a1 = sym(k0 + 1), piv = 1.0;
+      // row i = tid / 16, column k = tid % 16; a warp holds two whole rows
+      const int i = tid >> 4, k = tid & 15;
+      double a = S[(o + max(i, k)) * kBlkPitch + o + min(i, k)], piv = 1.0;
       bool bad = false;
 #pragma unroll
       for (int j = 0; j < kPan; ++j) {
         double* row = prow[j & 1];  // row j, published by its owners after step j - 1
-        if (i == j) {
-          row[k0] = a0;
-          row[k0 + 1] = a1;
-        }
-        const double cij = __shfl_sync(0xffffffffu, j & 1 ? a1 : a0, (lane & ~7) | (j >> 1));
+        if (i == j) row[k] = a;
+        const double cij = __shfl_sync(0xffffffffu, a, (lane & 16) | j);
         __syncthreads();
         double d = row[j];
         if (!(d > 0.0)) {
@@ -440,80 +443,91 @@ __global__ void __cluster_dims__(kBlkCtas, 1, 1) __launch_bounds__(kBlkThreads)
           d = 1e-300;
         }
         if (i == j) piv = d;
-        if ((tid >> 5) * 4 + 3 > j) {  // warps whose rows are all done have nothing to update
-          const double t0 = cij * row[k0], t1 = cij * row[k0 + 1];
+        if ((tid >> 5) * 2 + 1 > j) {  // warps whose rows are all done have nothing to update
+          const double t = cij * row[k];
           const double r = recip_f64(d);
-          if (i > j) {
-            a0 = k0 == j ? -cij * r : fma(-t0, r, a0);
-            a1 = k0 + 1 == j ? -cij * r : fma(-t1, r, a1);
-          }
+          if (i > j) a = k == j ? -cij * r : fma(-t, r, a);
         }
       }
       if (bad && rank == 0 && tid == 0) atomicOr(status, ST_NONFINITE);
       const double y = rsqrt(piv);
-      Zd[p][i][k0] = k0 < i ? a0 * y : (k0 == i ? y : 0.0);
-      Zd[p][i][k0 + 1] = k0 + 1 < i ? a1 * y : (k0 + 1 == i ? y : 0.0);
+      Zp[i][k] = k < i ? a * y : (k == i ? y : 0.0);
     }
     __syncthreads();
-    if (o + kPan >= kNb) break;
+    const int below = nn - o - kPan, own = below / kBlkCtas;
+    if (below == 0) break;
     // owned rows of the panel: one output per thread
-    const int below = kNb - o - kPan, own = below / kBlkCtas;
     const int pr = o + kPan + (tid / kPan) * kBlkCtas + rank, q = tid % kPan;
     if (tid < own * kPan) {
       double acc0 = 0.0, acc1 = 0.0;
 #pragma unroll
       for (int t = 0; t < kPan; t += 2) {
-        acc0 = fma(S[pr * kPitch + o + t], Zd[p][q][t], acc0);
-        acc1 = fma(S[pr * kPitch + o + t + 1], Zd[p][q][t + 1], acc1);
+        acc0 = fma(S[pr * kBlkPitch + o + t], Zp[q][t], acc0);
+        acc1 = fma(S[pr * kBlkPitch + o + t + 1], Zp[q][t + 1], acc1);
       }
       acc0 += acc1;
       __syncwarp(__activemask());  // a row's 16 outputs are one half-warp: its reads are done
 #pragma unroll
-      for (int c = 0; c < kBlkCtas; ++c) cl.map_shared_rank(S, c)[pr * kPitch + o + q] = acc0;
+      for (int c = 0; c < kBlkCtas; ++c) cl.map_shared_rank(S, c)[pr * kBlkPitch + o + q] = acc0;
     }
     cl.sync();
     // owned rows of the trailing update, columns up to the diagonal
     for (int e = tid; e < own * below; e += kBlkThreads) {
       const int r = o + kPan + (e / below) * kBlkCtas + rank, j = o + kPan + e % below;
       if (j > r) continue;
-      double acc0 = S[r * kPitch + j], acc1 = 0.0;
+      double acc0 = S[r * kBlkPitch + j], acc1 = 0.0;
 #pragma unroll
       for (int t = 0; t < kPan; t += 2) {
-        acc0 = fma(-S[r * kPitch + o + t], S[j * kPitch + o + t], acc0);
-        acc1 = fma(-S[r * kPitch + o + t + 1], S[j * kPitch + o + t + 1], acc1);
+        acc0 = fma(-S[r * kBlkPitch + o + t], S[j * kBlkPitch + o + t], acc0);
+        acc1 = fma(-S[r * kBlkPitch + o + t + 1], S[j * kBlkPitch + o + t + 1], acc1);
       }
       acc0 += acc1;
       if (r < o + 2 * kPan) {
 #pragma unroll
-        for (int c = 0; c < kBlkCtas; ++c) cl.map_shared_rank(S, c)[r * kPitch + j] = acc0;
+        for (int c = 0; c < kBlkCtas; ++c) cl.map_shared_rank(S, c)[r * kBlkPitch + j] = acc0;
       } else {
-        S[r * kPitch + j] = acc0;
+        S[r * kBlkPitch + j] = acc0;
       }
     }
     cl.sync();
   }
   // owned columns of Z, block row by block row: Z_i = L_ii^{-1} (E_i - sum_{k < i} L_ik Z_k)
-  const int rr = tid / (kNb / kBlkCtas), cc = tid % (kNb / kBlkCtas), col = cc * kBlkCtas + rank;
-  for (int p = 0; p < kNb / kPan; ++p) {
-    const int o = kPan * p, r = o + rr;
+  const int rr = tid / kBlkOwn, cc = tid % kBlkOwn, col = cc * kBlkCtas + rank;
+  for (int o = 0; o < nn; o += kPan) {
+    const int r = o + rr;
     double acc[4] = {r == col ? 1.0 : 0.0, 0.0, 0.0, 0.0};
     for (int k = col / kPan * kPan; k < o; k += 4) {  // Z is zero above the diagonal
 #pragma unroll
-      for (int u = 0; u < 4; ++u) acc[u] = fma(-S[r * kPitch + k + u], Y[k + u][cc], acc[u]);
+      for (int u = 0; u < 4; ++u) acc[u] = fma(-S[r * kBlkPitch + k + u], Y[k + u][cc], acc[u]);
     }
     Y[r][cc] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
     __syncthreads();
     double z0 = 0.0, z1 = 0.0;
+    if (col < o + kPan) {
 #pragma unroll
-    for (int t = 0; t < kPan; t += 2) {
-      z0 = fma(Zd[p][rr][t], Y[o + t][cc], z0);
-      z1 = fma(Zd[p][rr][t + 1], Y[o + t + 1][cc], z1);
+      for (int t = 0; t < kPan; t += 2) {
+        z0 = fma(Zd[o / kPan][rr][t], Y[o + t][cc], z0);
+        z1 = fma(Zd[o / kPan][rr][t + 1], Y[o + t + 1][cc], z1);
+      }
     }
     __syncthreads();
     Y[r][cc] = z0 + z1;
     if (r < n && col < n) Z[(long long)r * ldz + col] = r >= col ? z0 + z1 : 0.0;
     __syncthreads();
   }
+}
+
+// Raises the block kernel's dynamic shared-memory limit (once per device).
+bool block_smem_ok() {
+  static std::mutex mu;
+  static bool done[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  std::lock_guard<std::mutex> lock(mu);
+  if (!done[dev])
+    done[dev] = cudaFuncSetAttribute(chol_inv_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)kBlkSmem) == cudaSuccess;
+  return done[dev];
 }
 
 // v = Z t for lower-triangular Z (M x M), one warp per row.
@@ -687,14 +701,14 @@ int split_point(int n) {
 //   Z11 from K11;  L21 = K21 Z11^T;  K22 <- K22 - L21 L21^T;  Z22 from K22;
 //   Z21 = -Z22 (L21 Z11),
 // with Z = L^{-1} written into Z (ldz; the block above the diagonal must be zero
-// already).  Blocks of at most 64 rows: chol_inv_block_kernel.
+// already).  Blocks of at most kBlk rows: chol_inv_block_kernel.
 // The recursion exposes large FP64 products (the top level's are n/2 square)
 // where a column-by-column factorisation has only 64-row panels.
 // pool: scratch for the L21 and L21 Z11 blocks of every level.
 void chol_inv(CsState* S, double* K, long long ld, double* Z, long long ldz, int n, double* pool,
               cudaStream_t s) {
-  if (n <= kNb) {
-    chol_inv_block_kernel<<<kBlkCtas, kBlkThreads, 0, s>>>(K, ld, Z, ldz, n, S->status);
+  if (n <= kBlk) {
+    chol_inv_block_kernel<<<kBlkCtas, kBlkThreads, kBlkSmem, s>>>(K, ld, Z, ldz, n, S->status);
     S->simt_flops += 2.0 * n * n * n / 3.0;
     return;
   }
@@ -784,7 +798,7 @@ ep_tv_status hadamard_create(const LikelihoodConfig& cfg, CsState* S, cudaStream
 
 ep_tv_status cs_create(const LikelihoodConfig& cfg, cudaStream_t s, CsState** out, float* mu0) {
   *out = nullptr;
-  if (ozaki_init() != EP_TV_OK) return EP_TV_ERR_CUDA;
+  if (ozaki_init() != EP_TV_OK || !block_smem_ok()) return EP_TV_ERR_CUDA;
   CsState* S = new (std::nothrow) CsState();
   if (!S) return EP_TV_ERR_NOMEM;
   S->M = cfg.m;

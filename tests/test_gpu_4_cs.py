@@ -101,9 +101,9 @@ def test_cs_diagonal_noise_matches_oracle():
     assert_parity(mu, var, mu_r, var_r, p.A.T @ y)
 
 
-@pytest.mark.parametrize("m", [1, 15, 16, 17, 63, 64, 65, 80, 128, 150])
+@pytest.mark.parametrize("m", [1, 15, 16, 17, 63, 64, 65, 80, 127, 128, 129, 150])
 def test_cs_factorisation_block_edges(m):
-    """Row counts at the edges of the factorisation's 16-row panels and 64-row blocks:
+    """Row counts at the edges of the factorisation's 16-row panels and 128-row blocks:
     one partial block, a full one, and a full one with a remainder."""
     mu, var, mu_r, var_r, p = _run(14, m, 4, 2, seed=100 + m)
     assert_parity(mu, var, mu_r, var_r, p.A.T @ p.y)

@@ -340,7 +340,7 @@ def _emulated_iterations(p, pr, d, ncav, rtol, eta=3.2e-5):
 @pytest.mark.parametrize("h,w,periodic", [(76, 108, 1), (45, 99, 0), (40, 140, 1), (128, 64, 1), (24, 600, 1)])
 def test_preconditioner_iterations_are_those_of_the_windowed_extension(h, w, periodic):
     """The preconditioner shows in the iteration count alone: the count of the first
-    likelihood update is that of the FP64 emulation.  The tolerance is one that a single
+    likelihood update is that of the emulation.  The target, 1e-4, is one that a single
     refinement pass meets (at 1e-9 the FP32 floor decides how many passes follow); FP32
     rounding moves a pass by an iteration or two."""
     p = syn.deconv_problem(h, w, kernel=syn.uniform_kernel(5), bsnr_db=30.0, beta0=2.0, seed=3, grf_length=8.0)
@@ -352,7 +352,9 @@ def test_preconditioner_iterations_are_those_of_the_windowed_extension(h, w, per
     # one (the host-driven loop launches them in fours)
     stream = torch.cuda.Stream()
     with torch.cuda.stream(stream):
-        _, _, ep = _gpu(p, 1, S, pr, periodic=periodic, cg_rtol=1e-4, stream=stream)
+        # sides that are not powers of two are solved to a quarter of cg_rtol
+        rtol = 1e-4 if h & (h - 1) == 0 and w & (w - 1) == 0 else 4e-4
+        _, _, ep = _gpu(p, 1, S, pr, periodic=periodic, cg_rtol=rtol, stream=stream)
         its = ep.stats()["cg_iters"]
         assert ep.solver_report()["passes"] == 1
         tau, nu = (t.cpu().numpy().astype(np.float64) for t in ep.sites())

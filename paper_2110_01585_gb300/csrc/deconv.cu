@@ -36,6 +36,7 @@
 #include <mutex>
 #include <new>
 #include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "internal.cuh"
@@ -1640,7 +1641,7 @@ __global__ void commit_kernel(double* X, const float* Ec, const int* act0, long 
 
 
 // ---------------------------------------------------------------------------
-// Circulant preconditioner on a power-of-two torus HP x WP that holds the image:
+// Circulant preconditioner on a torus HP x WP that holds the image (see torus()):
 //   M = H^T H / xi + dbar I,  dbar = mean(d),  M^{-1} r = F^{-1}[F r / (|h_f|^2 / xi + dbar)].
 // H^T H is circulant, so for an image of that size M differs from Q only by d - dbar on
 // the diagonal; CG on M^{-1} Q needs a few tens of iterations where Jacobi needs hundreds.
@@ -1664,7 +1665,7 @@ __global__ void commit_kernel(double* X, const float* Ec, const int* act0, long 
 // row or column), other sizes run Stockham passes in shared memory.
 struct FftDesc {
   int H, W;          // image
-  int HP, WP;        // power-of-two transform sizes, HP >= H, WP >= W
+  int HP, WP;        // transform sizes, HP >= H, WP >= W
   int R, pairs;
   int cw;            // columns per block in the column pass
   int rpb;           // rows per block in the row passes
@@ -2105,9 +2106,25 @@ __global__ void window_kernel(float* w, int n, int P) {
 // neighbouring entries; with w512^m at m the first step's reads met up to four to a bank):
 //   kTw512: w512^(t k1) at 64 k1 + t (t < 64, k1 < 8), then w64^(u k3) at 512 + 8 k3 + u
 //   w1024^m, m < 512
-//   256, 128 and 64 points: w_n^(t k1) at k1 T + t, T = n / 16
+//   the other warp transforms (kLens), one after another: w_n^(t k1) at k1 T + t, and for
+//   those of 12 T points w_T^(u k3) at n + 4 k3 + u
 constexpr int kTw512 = kF + 64;
-constexpr int kTwCount = kTw512 + kF + 256 + 128 + 64;
+constexpr int kLens[] = {64, 96, 128, 192, 256, 384};
+// elements per lane, lanes and twiddles of an n-point warp transform
+constexpr int warp_elems(int n) { return n % 3 == 0 ? 12 : 16; }
+constexpr int warp_lanes(int n) { return n / warp_elems(n); }
+constexpr int warp_tw(int n) { return n == kF ? kTw512 : warp_elems(n) == 16 ? n : n + warp_lanes(n); }
+// Where the table of the n-point warp transform lies in the twiddle buffer (n = 0: its end).
+constexpr int warp_twiddles(int n) {
+  if (n == kF) return 0;
+  int o = kTw512 + kF;
+  for (int len : kLens) {
+    if (len == n) break;
+    o += warp_tw(len);
+  }
+  return o;
+}
+constexpr int kTwCount = warp_twiddles(0);
 __global__ void twiddle_kernel(float2* tw) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
   if (m >= kTwCount) return;
@@ -2122,10 +2139,20 @@ __global__ void twiddle_kernel(float2* tw) {
     n = 2 * kF;
     e = m - kTw512;
   } else {
-    const int q = m - kTw512 - kF;
-    n = q < 256 ? 256 : q < 384 ? 128 : 64;
-    const int k = q < 256 ? q : q < 384 ? q - 256 : q - 384, T = n / 16;
-    e = (k % T) * (k / T);
+    int q = m - kTw512 - kF;
+    n = 0;
+    for (int len : {64, 96, 128, 192, 256, 384}) {
+      n = len;
+      if (q < warp_tw(len)) break;
+      q -= warp_tw(len);
+    }
+    const int T = warp_lanes(n);
+    if (q < n) {
+      e = (q % T) * (q / T);
+    } else {
+      e = ((q - n) & 3) * ((q - n) >> 2);
+      n = T;
+    }
   }
   float sn, cs;
   sincospif(-2.0f * (float)(e % n) / (float)n, &sn, &cs);
@@ -2171,10 +2198,17 @@ __device__ __forceinline__ void st_hint(float2* a, float2 v, uint64_t pol) {
                : "memory");
 }
 
-// Which passes take the warp transforms of 64 to 512 points (the others take the Stockham
-// ones): a block of the column pass holds 4096 / HP columns.
-inline bool warp_rows(const FftDesc& f) { return f.WP >= 64 && f.WP <= kF; }
-inline bool warp_cols(const FftDesc& f) { return f.HP >= 64 && f.HP <= kF && f.WP >= 4096 / f.HP; }
+// Which passes take the warp transforms (the others take the Stockham ones): a block of
+// the column pass holds 256 / T columns, and whole blocks make up WP.
+inline bool warp_len(int n) {
+  for (int len : kLens)
+    if (n == len) return true;
+  return n == kF;
+}
+inline bool warp_rows(const FftDesc& f) { return warp_len(f.WP); }
+inline bool warp_cols(const FftDesc& f) {
+  return warp_len(f.HP) && f.WP % (32 * kF512Warps / warp_lanes(f.HP)) == 0;
+}
 // and the 1024-point ones (below)
 inline bool fft1024_rows(const FftDesc& f) { return f.WP == 2 * kF; }
 inline bool fft1024_cols(const FftDesc& f) { return f.HP == 2 * kF && f.WP >= kF512Warps; }
@@ -2225,33 +2259,40 @@ __device__ __forceinline__ void fft512_warp(float2 (&v)[16], float2* xs, const f
   __syncwarp();  // the scratch is free again
 }
 
-// ---- register-resident transforms of 64, 128 and 256 points
+// ---- register-resident transforms of 64, 128 and 256, and of 96, 192 and 384 points
 //
-// T = n / 16 lanes hold one transform, 16 elements each (lane t keeps x[T m + t]), so a
-// warp runs 32 / T of them side by side with the registers of the 512-point one:
+// n = E T points: T lanes hold one transform, E elements each (lane t keeps x[T m + t]), so
+// that a warp runs 32 / T of them side by side.  E = 16 for the powers of two, with the
+// registers of the 512-point one:
 //   B_t[k1]      = w_n^(t k1) sum_m x[T m + t] w16^(m k1)      (in a lane)
 //   X[k1 + 16 k2] = sum_t B_t[k1] w_T^(t k2)
 // with one regrouping through the warp's scratch, after which lane t takes k1 = t + T j,
-// j < 16 / T: X[T (16 / T k2 + j) + t], the layout of the input.  For 17 pairs of a 256^2
-// image the preconditioner took 59 us in Stockham kernels (passes through shared memory
-// behind block barriers); its column and inverse row passes take 26 us here, and the
-// forward one is fused with the CG update.
+// j < 16 / T: X[T (16 / T k2 + j) + t], the layout of the input.  E = 12 for the others, where
+// the T points take two steps, M = T / 4 and 4, so that the last one's outputs lie 3 T apart,
+// a multiple of T, and fall in the input's layout again (t = 4 s + u):
+//   C_u[k1, k3]               = w_T^(u k3) sum_s B_(4 s + u)[k1] w_M^(s k3)
+//   X[k1 + 12 k3 + 12 M k4]    = sum_u C_u[k1, k3] w4^(u k4)
+// For 17 pairs of a 256^2 image the preconditioner took 59 us in Stockham kernels (passes
+// through shared memory behind block barriers); its column and inverse row passes take
+// 26 us here, and the forward one is fused with the CG update.
 //
 // Sizes per warp, in float2: kRow, from one transform's regrouping area to the next (entry
 // (k1, t) at k1 (T + 1) + t); kCol, from one staged column to the next in the column pass;
 // kScratch, from one warp's area to the next.  Their residues mod 16 keep the accesses of a
 // half-warp in distinct banks.
-template <int T>
+template <int kLen>
 struct Warp {
-  static constexpr int kN = 16 * T, kPer = 32 / T;
-  static constexpr int kTw = T == 32 ? kTw512 : kN;  // entries of the twiddle table
-  static constexpr int kRow = T == 32 ? 0 : T == 16 ? 272 : T == 8 ? 152 : 84;
-  static constexpr int kCol = T == 32 ? 0 : kN + 1;
-  static constexpr int kScratch = T == 32 ? kXs : T == 16 ? 546 : T == 8 ? 612 : 680;
+  static constexpr int kN = kLen, kE = warp_elems(kLen), kT = warp_lanes(kLen), kPer = 32 / kT;
+  static constexpr int kTw = warp_tw(kLen);  // entries of the twiddle table
+  static constexpr int kRow = kE == 12 ? (kT == 32 ? 432 : kT == 16 ? 240 : 120)
+                              : kT == 32 ? 0 : kT == 16 ? 272 : kT == 8 ? 152 : 84;
+  static constexpr int kCol = kLen == kF ? 0 : kN + 1;
+  static constexpr int kScratch = kE == 12 ? (kT == 32 ? 434 : kT == 16 ? 482 : 484)
+                                  : kT == 32 ? kXs : kT == 16 ? 546 : kT == 8 ? 612 : 680;
   static constexpr int kCols = kF512Warps * kPer;  // columns per block of the column pass
-  // rows per block of the row passes: four rounds of the block's warps for 512 points (one
-  // and two rounds were within 3% on 512^2 and 300 x 420), one for the others
-  static constexpr int kRows = T == 32 ? 4 * kF512Warps : kF512Warps * kPer;
+  // rows per block of the row passes: four rounds of the block's warps for a transform per
+  // warp (one to three rounds were within 3% on 512^2 and 300 x 420), one for the others
+  static constexpr int kRows = (kT == 32 ? 4 : 1) * kF512Warps * kPer;
   static_assert(kPer * kRow <= kScratch && kPer * kCol <= kScratch, "scratch");
 };
 
@@ -2285,14 +2326,43 @@ template <> __device__ __forceinline__ void dft_reg<16>(float2* v) {
   }
 }
 
+template <> __device__ __forceinline__ void dft_reg<3>(float2* v) {
+  const float s3 = 0.86602540378443864676f;
+  const float2 t1 = cadd(v[1], v[2]), d = csub(v[1], v[2]);
+  const float2 t2 = __ffma2_rn(t1, make_float2(-0.5f, -0.5f), v[0]);
+  v[0] = cadd(v[0], t1);
+  v[1] = make_float2(fmaf(s3, d.y, t2.x), fmaf(-s3, d.x, t2.y));
+  v[2] = make_float2(fmaf(-s3, d.y, t2.x), fmaf(s3, d.x, t2.y));
+}
+template <> __device__ __forceinline__ void dft_reg<12>(float2* v) {
+  // without twiddles (Good 1958): w12^(m k) = w4^(b k) w3^(a k) for m = 4 a + 3 b mod 12,
+  // and k is given by its residues mod 4 and 3
+  float2 c[4][3];
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) c[b][a] = v[(4 * a + 3 * b) % 12];
+    dft_reg<3>(c[b]);
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    float2 u[4] = {c[0][q], c[1][q], c[2][q], c[3][q]};
+    dft_reg<4>(u);
+#pragma unroll
+    for (int k = q; k < 12; k += 3) v[k] = u[k & 3];
+  }
+}
+
 // The warp's forward transforms in place; xs: the warp's scratch; tw: its kTw twiddles.
-template <int T>
-__device__ __forceinline__ void fft_warp(float2 (&v)[16], float2* xs, const float2* tw) {
-  if constexpr (T == 32) {
+template <int kLen>
+__device__ __forceinline__ void fft_warp(float2 (&v)[Warp<kLen>::kE], float2* xs, const float2* tw) {
+  using Wp = Warp<kLen>;
+  constexpr int T = Wp::kT, E = Wp::kE;
+  if constexpr (kLen == kF) {
     fft512_warp(v, xs, tw);
-  } else {
+  } else if constexpr (E == 16) {
     const int l = threadIdx.x & 31, t = l % T;
-    float2* x = xs + (l / T) * Warp<T>::kRow;
+    float2* x = xs + (l / T) * Wp::kRow;
     dft_reg<16>(v);
     x[t] = v[0];
 #pragma unroll
@@ -2310,25 +2380,67 @@ __device__ __forceinline__ void fft_warp(float2 (&v)[16], float2* xs, const floa
 #pragma unroll
       for (int k2 = 0; k2 < T; ++k2) v[16 / T * k2 + j] = b[j][k2];
     }
+  } else {
+    // M = T / 4; sub-transform (k1, u) by item q = k1 + E u of the transform's lanes
+    constexpr int M = T / 4, kItems = 4 * E, kRounds = (kItems + T - 1) / T;
+    constexpr int kPb = E + 1, kPc = E * M + (T == 8 ? 4 : 12);
+    static_assert(T * kPb <= Wp::kRow && 4 * kPc <= Wp::kRow, "scratch");
+    const int l = threadIdx.x & 31, t = l % T;
+    float2* x = xs + (l / T) * Wp::kRow;
+    dft_reg<E>(v);
+    x[t * kPb] = v[0];
+#pragma unroll
+    for (int k1 = 1; k1 < E; ++k1) x[t * kPb + k1] = cmul(v[k1], tw[k1 * T + t]);
+    __syncwarp();
+    float2 b[kRounds][M];
+#pragma unroll
+    for (int g = 0; g < kRounds; ++g) {
+      const int q = t + T * g, k1 = q % E, u = q / E;
+#pragma unroll
+      for (int s = 0; s < M; ++s)
+        b[g][s] = kItems % T == 0 || q < kItems ? x[(4 * s + u) * kPb + k1] : make_float2(0.f, 0.f);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int g = 0; g < kRounds; ++g) {
+      const int q = t + T * g, k1 = q % E, u = q / E;
+      dft_reg<M>(b[g]);
+      if (kItems % T == 0 || q < kItems) {
+        x[u * kPc + k1] = b[g][0];
+#pragma unroll
+        for (int k3 = 1; k3 < M; ++k3) x[u * kPc + k1 + E * k3] = cmul(b[g][k3], tw[kLen + 4 * k3 + u]);
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < E / 4; ++h) {
+      float2 c[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) c[u] = x[u * kPc + t + T * h];
+      dft_reg<4>(c);
+#pragma unroll
+      for (int k4 = 0; k4 < 4; ++k4) v[h + E / 4 * k4] = c[k4];
+    }
+    __syncwarp();  // the scratch is free again
   }
 }
 
-// The extension E along a row held by T lanes (W image columns in place): the copies past
+// The extension along a row held by T lanes (W image columns in place): the copies past
 // column W through the scratch, and the window wc.
-template <int T>
-__device__ __forceinline__ void extend_row(float2 (&v)[16], float2* xs, const float* wc, int W) {
-  constexpr int P = 16 * T;
+template <int kLen>
+__device__ __forceinline__ void extend_row(float2 (&v)[Warp<kLen>::kE], float2* xs, const float* wc, int W) {
+  constexpr int P = kLen, T = Warp<kLen>::kT, E = Warp<kLen>::kE;
   const int l = threadIdx.x & 31, t = l % T, ext = P - W, L = ext >> 1;
-  float2* x = xs + (l / T) * Warp<T>::kRow;
+  float2* x = xs + (l / T) * Warp<kLen>::kRow;
 #pragma unroll
-  for (int m = 0; m < 16; ++m) {
+  for (int m = 0; m < E; ++m) {
     const int c = T * m + t;
     if (c < L) x[c] = v[m];
     else if (c < W && c >= W - L) x[c - W + ext] = v[m];
   }
   __syncwarp();
 #pragma unroll
-  for (int m = 0; m < 16; ++m) {
+  for (int m = 0; m < E; ++m) {
     const int c = T * m + t;
     if (c >= W) v[m] = margin(c, W, P) >= 0 ? x[c - W] : make_float2(0.f, 0.f);
     v[m] = cscale(v[m], wc[c]);
@@ -2337,20 +2449,20 @@ __device__ __forceinline__ void extend_row(float2 (&v)[16], float2* xs, const fl
 }
 
 // E^T along a row: the windowed copies added to the image columns they copy.
-template <int T>
-__device__ __forceinline__ void fold_row(float2 (&v)[16], float2* xs, const float* wc, int W) {
-  constexpr int P = 16 * T;
+template <int kLen>
+__device__ __forceinline__ void fold_row(float2 (&v)[Warp<kLen>::kE], float2* xs, const float* wc, int W) {
+  constexpr int P = kLen, T = Warp<kLen>::kT, E = Warp<kLen>::kE;
   const int l = threadIdx.x & 31, t = l % T, ext = P - W, L = ext >> 1;
-  float2* x = xs + (l / T) * Warp<T>::kRow;
+  float2* x = xs + (l / T) * Warp<kLen>::kRow;
 #pragma unroll
-  for (int m = 0; m < 16; ++m) {
+  for (int m = 0; m < E; ++m) {
     const int c = T * m + t;
     v[m] = cscale(v[m], wc[c]);
     if (c >= W) x[c - W] = v[m];
   }
   __syncwarp();
 #pragma unroll
-  for (int m = 0; m < 16; ++m) {
+  for (int m = 0; m < E; ++m) {
     const int c = T * m + t;
     if (c < L) v[m] = cadd(v[m], x[c]);
     else if (c < W && c >= W - L) v[m] = cadd(v[m], x[c - W + ext]);
@@ -2358,10 +2470,11 @@ __device__ __forceinline__ void fold_row(float2 (&v)[16], float2* xs, const floa
   __syncwarp();
 }
 
-// fft_rows_fwd_kernel for WP = 16 T: rows [blockIdx.x kRows, + kRows), 32 / T per warp.
-template <int T>
+// fft_rows_fwd_kernel for the warp transforms: rows [blockIdx.x kRows, + kRows), 32 / T per warp.
+template <int kLen>
 __global__ void __launch_bounds__(32 * kF512Warps) warp_rows_fwd_kernel(FftDesc f, const float* __restrict__ Rr) {
-  using Wp = Warp<T>;
+  using Wp = Warp<kLen>;
+  constexpr int T = Wp::kT, E = Wp::kE;
   if (pair_idle(f, blockIdx.y)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0 && f.counters)
     atomicAdd(&f.counters[DC_CG_PRE_UNITS], 2 * blockIdx.y + 1 < f.R ? 2ull : 1ull);
@@ -2383,18 +2496,18 @@ __global__ void __launch_bounds__(32 * kF512Warps) warp_rows_fwd_kernel(FftDesc 
     const int row = base + l / T;
     const bool ok = row < rend;
     const long long p0 = (long long)row * f.W;
-    float2 v[16];
+    float2 v[E];
 #pragma unroll
-    for (int m = 0; m < 16; ++m) {
+    for (int m = 0; m < E; ++m) {
       const int c = T * m + t;
       v[m] = make_float2(0.f, 0.f);
       if (ok && c < f.W) v[m] = make_float2(ld_hint(r0p + p0 + c, keep), two ? ld_hint(r1p + p0 + c, keep) : 0.f);
     }
-    if (f.W < Wp::kN) extend_row<T>(v, scratch[w], f.wc, f.W);
-    fft_warp<T>(v, scratch[w], tw);
+    if (f.W < Wp::kN) extend_row<kLen>(v, scratch[w], f.wc, f.W);
+    fft_warp<kLen>(v, scratch[w], tw);
     if (ok) {
 #pragma unroll
-      for (int m = 0; m < 16; ++m) st_hint(out + (long long)row * Wp::kN + T * m + t, v[m], keep);
+      for (int m = 0; m < E; ++m) st_hint(out + (long long)row * Wp::kN + T * m + t, v[m], keep);
     }
   }
 }
@@ -2405,7 +2518,7 @@ __device__ __forceinline__ float still_active(const CgArgs& a, int j, double r2)
   return (r2 <= a.thr[j] || r2 > 16.0 * a.rr0[j]) ? 0.f : 1.f;
 }
 
-// The CG update fused with the forward row pass (rows of 64 to 512 points): for each system
+// The CG update fused with the forward row pass (warp transforms): for each system
 // of the pair that is active when the iteration starts, alpha = r.z / p.q from the
 // direction kernel's partials, e += alpha p and r -= alpha q, exactly as update_kernel
 // forms them; the new residual rows of the pair then go through the forward row
@@ -2418,9 +2531,10 @@ __device__ __forceinline__ float still_active(const CgArgs& a, int j, double r2)
 // done by the next direction kernel over its tile, where p is the direction it reads
 // anyway, or by the commit after a system's last iteration; the same operation on the
 // same values, so the results do not change.
-template <int T>
+template <int kLen>
 __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_update_rows_fwd_kernel(FftDesc f, CgArgs a, int it_arg) {
-  using Wp = Warp<T>;
+  using Wp = Warp<kLen>;
+  constexpr int T = Wp::kT, E = Wp::kE;
   const int pair = blockIdx.y;
   const int j0 = 2 * pair, j1 = 2 * pair + 1;
   const bool two = j1 < f.R;
@@ -2452,7 +2566,7 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_update_rows_fwd_kerne
     const int row = base + l / T;
     const int cols = row < rend ? f.W : 0;  // columns of this lane's row that exist
     const long long p0 = (long long)row * f.W;
-    float2 v[16];
+    float2 v[E];
     if (a.defer_e) {
       // r only, both systems' loads in flight together: e += alpha p is left to the
       // next direction kernel or the commit
@@ -2460,9 +2574,9 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_update_rows_fwd_kerne
       const float* Q1 = a.Qp + (long long)j1 * N + p0;
       float* R0 = a.Rr + (long long)j0 * N + p0;
       float* R1 = a.Rr + (long long)j1 * N + p0;
-      float qa[16], ra[16], qb[16], rb[16];
+      float qa[E], ra[E], qb[E], rb[E];
 #pragma unroll
-      for (int m = 0; m < 16; ++m) {
+      for (int m = 0; m < E; ++m) {
         const int c = T * m + t;
         qa[m] = ra[m] = qb[m] = rb[m] = 0.f;
         if (c < cols) {
@@ -2478,7 +2592,7 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_update_rows_fwd_kerne
       }
       const float al0 = alpha_s[0], al1 = alpha_s[1];
 #pragma unroll
-      for (int m = 0; m < 16; ++m) {
+      for (int m = 0; m < E; ++m) {
         const int c = T * m + t;
         v[m] = make_float2(0.f, 0.f);
         if (c < cols) {
@@ -2499,7 +2613,7 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_update_rows_fwd_kerne
       for (int u = 0; u < 2; ++u) {
         if (!(u ? act1 : act0)) {
 #pragma unroll
-          for (int m = 0; m < 16; ++m) (u ? v[m].y : v[m].x) = 0.f;
+          for (int m = 0; m < E; ++m) (u ? v[m].y : v[m].x) = 0.f;
           continue;
         }
         const long long o = (long long)(j0 + u) * N + p0;
@@ -2508,9 +2622,9 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_update_rows_fwd_kerne
         float* Ec = a.Ec + o;
         float* Rr = a.Rr + o;
         const float alpha = alpha_s[u];
-        float pv[16], qv[16], rv[16], ev[16];
+        float pv[E], qv[E], rv[E], ev[E];
 #pragma unroll
-        for (int m = 0; m < 16; ++m) {
+        for (int m = 0; m < E; ++m) {
           const int c = T * m + t;
           pv[m] = qv[m] = rv[m] = ev[m] = 0.f;
           if (c < cols) {
@@ -2521,7 +2635,7 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_update_rows_fwd_kerne
           }
         }
 #pragma unroll
-        for (int m = 0; m < 16; ++m) {
+        for (int m = 0; m < E; ++m) {
           const int c = T * m + t;
           float r = 0.f;
           if (c < cols) {
@@ -2534,11 +2648,11 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_update_rows_fwd_kerne
         }
       }
     }
-    if (f.W < Wp::kN) extend_row<T>(v, scratch[w], f.wc, f.W);
-    fft_warp<T>(v, scratch[w], tw);
+    if (f.W < Wp::kN) extend_row<kLen>(v, scratch[w], f.wc, f.W);
+    fft_warp<kLen>(v, scratch[w], tw);
     if (row < rend) {
 #pragma unroll
-      for (int m = 0; m < 16; ++m) st_hint(out + (long long)row * Wp::kN + T * m + t, v[m], keep);
+      for (int m = 0; m < E; ++m) st_hint(out + (long long)row * Wp::kN + T * m + t, v[m], keep);
     }
   }
   block_sumf<2>(rr0, rr1, 0.f, act0 ? a.part_rr + (long long)j0 * a.nb + blockIdx.x : nullptr,
@@ -2556,15 +2670,16 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_update_rows_fwd_kerne
   }
 }
 
-// fft_cols_filter_kernel for HP = 16 T: the block takes columns [blockIdx.x kCols, + kCols) of
+// fft_cols_filter_kernel for the warp transforms: the block takes columns [blockIdx.x kCols, + kCols) of
 // a pair, stages the tile in shared memory (row segments of 64 bytes and more from global
 // memory, extended to HP rows), and each group of T lanes transforms one column in
 // registers, filters it with filtT (the filter stored column-major, [c][i]), transforms
 // again and leaves it in its slot for the block's store of the fold to H rows.
-template <int T>
+template <int kLen>
 __global__ void __launch_bounds__(32 * kF512Warps, 3) warp_cols_filter_kernel(FftDesc f,
                                                                           const float* __restrict__ filtT) {
-  using Wp = Warp<T>;
+  using Wp = Warp<kLen>;
+  constexpr int T = Wp::kT, E = Wp::kE;
   loop_step(f);
   if (pair_idle(f, blockIdx.y)) return;
   __shared__ float2 tw[Wp::kTw];
@@ -2579,47 +2694,47 @@ __global__ void __launch_bounds__(32 * kF512Warps, 3) warp_cols_filter_kernel(Ff
   const uint64_t keep = l2_policy_keep();
   float2* const col = tp + c0 + cc;
   {
-    float2 x[16];  // all of the thread's tile loads in flight at once
+    float2 x[E];  // all of the thread's tile loads in flight at once
     if (f.H == Wp::kN) {
 #pragma unroll
-      for (int u = 0; u < 16; ++u) x[u] = ld_hint(col + (long long)(kStep * u + ro) * f.WP, keep);
+      for (int u = 0; u < E; ++u) x[u] = ld_hint(col + (long long)(kStep * u + ro) * f.WP, keep);
     } else {
 #pragma unroll
-      for (int u = 0; u < 16; ++u) {
+      for (int u = 0; u < E; ++u) {
         const int src = margin(kStep * u + ro, f.H, Wp::kN);
         x[u] = src >= 0 ? ld_hint(col + (long long)src * f.WP, keep) : make_float2(0.f, 0.f);
       }
 #pragma unroll
-      for (int u = 0; u < 16; ++u) x[u] = cscale(x[u], f.wr[kStep * u + ro]);
+      for (int u = 0; u < E; ++u) x[u] = cscale(x[u], f.wr[kStep * u + ro]);
     }
 #pragma unroll
-    for (int u = 0; u < 16; ++u) slot[kStep * u + ro] = x[u];
+    for (int u = 0; u < E; ++u) slot[kStep * u + ro] = x[u];
   }
   __syncthreads();
   float2* xs = cols + w * Wp::kScratch;
   float2* const mine = xs + (l / T) * Wp::kCol;
   const float* g = filtT + (long long)(c0 + w * Wp::kPer + l / T) * Wp::kN;
-  float gv[16];  // the filter column, loaded before the transform
+  float gv[E];  // the filter column, loaded before the transform
 #pragma unroll
-  for (int m = 0; m < 16; ++m) gv[m] = g[T * m + t];
-  float2 v[16];
+  for (int m = 0; m < E; ++m) gv[m] = g[T * m + t];
+  float2 v[E];
 #pragma unroll
-  for (int m = 0; m < 16; ++m) v[m] = mine[T * m + t];
+  for (int m = 0; m < E; ++m) v[m] = mine[T * m + t];
   __syncwarp();
-  fft_warp<T>(v, xs, tw);
+  fft_warp<kLen>(v, xs, tw);
   // filter, then the inverse transform as conj(F(conj(.)))
 #pragma unroll
-  for (int m = 0; m < 16; ++m) v[m] = make_float2(v[m].x * gv[m], -v[m].y * gv[m]);
-  fft_warp<T>(v, xs, tw);
+  for (int m = 0; m < E; ++m) v[m] = make_float2(v[m].x * gv[m], -v[m].y * gv[m]);
+  fft_warp<kLen>(v, xs, tw);
 #pragma unroll
-  for (int m = 0; m < 16; ++m) mine[T * m + t] = cconj(v[m]);
+  for (int m = 0; m < E; ++m) mine[T * m + t] = cconj(v[m]);
   __syncthreads();
   if (f.H == Wp::kN) {
 #pragma unroll
-    for (int u = 0; u < 16; ++u) st_hint(col + (long long)(kStep * u + ro) * f.WP, slot[kStep * u + ro], keep);
+    for (int u = 0; u < E; ++u) st_hint(col + (long long)(kStep * u + ro) * f.WP, slot[kStep * u + ro], keep);
   } else {
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
+    for (int u = 0; u < E; ++u) {
       const int i = kStep * u + ro;
       if (i < f.H)
         st_hint(col + (long long)i * f.WP, fold(i, f.H, Wp::kN, [&](int k) { return cscale(slot[k], f.wr[k]); }), keep);
@@ -2641,9 +2756,10 @@ __global__ void __launch_bounds__(32 * kF512Warps, 3) warp_cols_filter_kernel(Ff
 // Bound by its nine planes (36 bytes per pixel and system, and d): at 512^2 with 33 systems
 // 61 us, 5.7 TB/s.  Three kernels per iteration, 60 bytes in all, against four with the
 // stencil kernel and the same bytes (direction 53 us and update 28 us there).
-template <int T>
+template <int kLen>
 __global__ void __launch_bounds__(32 * kF512Warps, 2) pw_update_rows_fwd_kernel(FftDesc f, CgArgs a, int it_arg) {
-  using Wp = Warp<T>;
+  using Wp = Warp<kLen>;
+  constexpr int T = Wp::kT, E = Wp::kE;
   const int pair = blockIdx.y;
   const int j0 = 2 * pair, j1 = 2 * pair + 1;
   const bool two = j1 < f.R;
@@ -2669,18 +2785,18 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) pw_update_rows_fwd_kernel(
     const int row = base + l / T;
     const bool ok = row < rend;
     const long long p0 = (long long)row * Wp::kN + t;
-    float2 v[16];
+    float2 v[E];
 #pragma unroll
-    for (int m = 0; m < 16; ++m) v[m] = make_float2(0.f, 0.f);
+    for (int m = 0; m < E; ++m) v[m] = make_float2(0.f, 0.f);
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       if (!ok || !(u ? act1 : act0)) continue;
       const int j = j0 + u;
       const float beta = a.scal[4 * j + 1], alpha = a.scal[4 * j + 2];
       const long long o = (long long)j * N + p0;
-      constexpr int kB = 8;  // elements per lane whose loads are in flight together
+      constexpr int kB = E / 2;  // elements per lane whose loads are in flight together
 #pragma unroll
-      for (int b = 0; b < 16; b += kB) {
+      for (int b = 0; b < E; b += kB) {
         float zv[kB], rv[kB], sv[kB], pv[kB], ev[kB], dv[kB];
 #pragma unroll
         for (int k = 0; k < kB; ++k) {
@@ -2710,10 +2826,10 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) pw_update_rows_fwd_kernel(
         }
       }
     }
-    fft_warp<T>(v, scratch[w], tw);
+    fft_warp<kLen>(v, scratch[w], tw);
     if (ok) {
 #pragma unroll
-      for (int m = 0; m < 16; ++m) st_hint(out + p0 + T * m, v[m], keep);
+      for (int m = 0; m < E; ++m) st_hint(out + p0 + T * m, v[m], keep);
     }
   }
   block_sumf<2>(rr[0], rr[1], 0.f, act0 ? a.part_rr + (long long)j0 * a.nb + blockIdx.x : nullptr,
@@ -2724,12 +2840,13 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) pw_update_rows_fwd_kernel(
   }
 }
 
-// fft_rows_inv_kernel for WP = 16 T: rows [blockIdx.x rows_per, + rows_per), rows_per =
+// fft_rows_inv_kernel for the warp transforms: rows [blockIdx.x rows_per, + rows_per), rows_per =
 // ceil(H / nbz).  kPw: the image fills the torus, and the pass also sums (d - dbar) z^2.
-template <int T, bool kPw>
+template <int kLen, bool kPw>
 __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_rows_inv_kernel(FftDesc f, const float* __restrict__ Rr,
                                                                        float* Z, double* part_rz) {
-  using Wp = Warp<T>;
+  using Wp = Warp<kLen>;
+  constexpr int T = Wp::kT, E = Wp::kE;
   if (pair_idle(f, blockIdx.y)) return;
   __shared__ float2 tw[Wp::kTw];
   __shared__ float2 scratch[kF512Warps][Wp::kScratch];
@@ -2753,10 +2870,10 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_rows_inv_kernel(FftDe
     const int cols = ok ? f.W : 0;
     const long long p0 = (long long)row * f.W;
     // the row's transform input and both residuals, all loads in flight together
-    float2 v[16], rr[16];
-    float dv[kPw ? 16 : 1];
+    float2 v[E], rr[E];
+    float dv[kPw ? E : 1];
 #pragma unroll
-    for (int m = 0; m < 16; ++m) {
+    for (int m = 0; m < E; ++m) {
       const int c = T * m + t;
       v[m] = rr[m] = make_float2(0.f, 0.f);
       if (kPw) dv[m] = ok ? f.D[p0 + c] : 0.f;
@@ -2766,11 +2883,11 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_rows_inv_kernel(FftDe
         if (two) rr[m].y = ld_hint(Rr + (long long)j1 * N + p0 + c, release);
       }
     }
-    fft_warp<T>(v, scratch[w], tw);
-    if (!kPw && f.W < Wp::kN) fold_row<T>(v, scratch[w], f.wc, f.W);
+    fft_warp<kLen>(v, scratch[w], tw);
+    if (!kPw && f.W < Wp::kN) fold_row<kLen>(v, scratch[w], f.wc, f.W);
     float rz0 = 0.f, rz1 = 0.f, dz0 = 0.f, dz1 = 0.f;
 #pragma unroll
-    for (int m = 0; m < 16; ++m) {
+    for (int m = 0; m < E; ++m) {
       const int c = T * m + t;
       if (c < cols) {
         const long long p = p0 + c;
@@ -2806,7 +2923,7 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_rows_inv_kernel(FftDe
 
 // ---- one refinement pass of a square image that fills the torus, in one kernel
 //
-// H = W = 16 T (64 to 256) with pointwise products: one cluster of kSolveCtas CTAs runs all CG
+// H = W = 64, 128 or 256 with pointwise products: one cluster of kSolveCtas CTAs runs all CG
 // iterations of a pass for one pair of systems, from the first z = M^{-1} r to the commit
 // x += e.  CTA c owns an eighth of the rows, which stay its own from iteration to
 // iteration, and an eighth of the columns of the transform plane, which passes through L2.
@@ -2821,8 +2938,10 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_rows_inv_kernel(FftDe
 constexpr int kSolveCtas = 8;
 // Warps per CTA.  Two such CTAs fit an SM, so that the 17 pairs of the default 33 systems
 // are resident at once; with 16 warps a 256^2 pass was 10% slower.
-template <int T>
+template <int kLen>
 constexpr int solve_warps() { return 8; }
+// The sides that take this kernel.
+constexpr bool solve_len(int n) { return n == 64 || n == 128 || n == 256; }
 
 // Sums NV values per thread over the CTA and writes the sums to slot[rank] of every CTA of the
 // cluster; they are there after the next cluster barrier.
@@ -2854,17 +2973,18 @@ __device__ __forceinline__ void cluster_sum(cooperative_groups::cluster_group& c
   }
 }
 
-template <int T>
+template <int kLen>
 constexpr size_t solve_smem() {
-  return sizeof(float2) * (size_t)solve_warps<T>() * Warp<T>::kScratch;
+  return sizeof(float2) * (size_t)solve_warps<kLen>() * Warp<kLen>::kScratch;
 }
 
-template <int T>
-__global__ void __cluster_dims__(kSolveCtas, 1, 1) __launch_bounds__(32 * solve_warps<T>(), 16 / solve_warps<T>())
+template <int kLen>
+__global__ void __cluster_dims__(kSolveCtas, 1, 1) __launch_bounds__(32 * solve_warps<kLen>(), 16 / solve_warps<kLen>())
     pw_solve_kernel(FftDesc f, CgArgs a, const float* filtT, const LoopState* ls, int budget, int* pass_its) {
   namespace cg = cooperative_groups;
-  using Wp = Warp<T>;
-  constexpr int kN = Wp::kN, kPer = Wp::kPer, kSolveWarps = solve_warps<T>();
+  using Wp = Warp<kLen>;
+  constexpr int T = Wp::kT, E = Wp::kE;
+  constexpr int kN = Wp::kN, kPer = Wp::kPer, kSolveWarps = solve_warps<kLen>();
   constexpr int kOwn = kN / kSolveCtas;  // rows, and columns, of one CTA
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank();
@@ -2912,19 +3032,19 @@ __global__ void __cluster_dims__(kSolveCtas, 1, 1) __launch_bounds__(32 * solve_
       if (w * kPer < kTileC) {
         float2* const mine = xs + (l / T) * Wp::kCol;
         const float* g = filtT + (long long)(c0 + w * kPer + l / T) * kN;
-        float gv[16];
+        float gv[E];
 #pragma unroll
-        for (int m = 0; m < 16; ++m) gv[m] = g[T * m + t];
-        float2 v[16];
+        for (int m = 0; m < E; ++m) gv[m] = g[T * m + t];
+        float2 v[E];
 #pragma unroll
-        for (int m = 0; m < 16; ++m) v[m] = mine[T * m + t];
+        for (int m = 0; m < E; ++m) v[m] = mine[T * m + t];
         __syncwarp();
-        fft_warp<T>(v, xs, twr);
+        fft_warp<kLen>(v, xs, twr);
 #pragma unroll
-        for (int m = 0; m < 16; ++m) v[m] = make_float2(v[m].x * gv[m], -v[m].y * gv[m]);
-        fft_warp<T>(v, xs, twr);
+        for (int m = 0; m < E; ++m) v[m] = make_float2(v[m].x * gv[m], -v[m].y * gv[m]);
+        fft_warp<kLen>(v, xs, twr);
 #pragma unroll
-        for (int m = 0; m < 16; ++m) mine[T * m + t] = cconj(v[m]);
+        for (int m = 0; m < E; ++m) mine[T * m + t] = cconj(v[m]);
       }
       __syncthreads();
 #pragma unroll
@@ -2938,19 +3058,19 @@ __global__ void __cluster_dims__(kSolveCtas, 1, 1) __launch_bounds__(32 * solve_
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     for (int row = row0; row < row_end; row += kRowStep) {
       const long long p0 = (long long)row * kN + t;
-      float2 v[16];
-      float ra[16], rb[16], dv[16];
+      float2 v[E];
+      float ra[E], rb[E], dv[E];
 #pragma unroll
-      for (int m = 0; m < 16; ++m) {
+      for (int m = 0; m < E; ++m) {
         v[m] = cconj(__ldcg(tmp + p0 + T * m));
         ra[m] = a.Rr[j0 * N + p0 + T * m];
         rb[m] = two ? a.Rr[j1 * N + p0 + T * m] : 0.f;
         dv[m] = a.D[p0 + T * m];
       }
-      fft_warp<T>(v, xs, twr);
+      fft_warp<kLen>(v, xs, twr);
       float s0 = 0.f, s1 = 0.f, q0 = 0.f, q1 = 0.f;
 #pragma unroll
-      for (int m = 0; m < 16; ++m) {
+      for (int m = 0; m < E; ++m) {
         const float z0 = v[m].x * scale, z1 = -v[m].y * scale;
         a.Z[j0 * N + p0 + T * m] = z0;
         s0 = fmaf(ra[m], z0, s0);
@@ -3000,13 +3120,13 @@ __global__ void __cluster_dims__(kSolveCtas, 1, 1) __launch_bounds__(32 * solve_
   // the first z: forward rows of the true residual
   for (int row = row0; row < row_end; row += kRowStep) {
     const long long p0 = (long long)row * kN + t;
-    float2 v[16];
+    float2 v[E];
 #pragma unroll
-    for (int m = 0; m < 16; ++m)
+    for (int m = 0; m < E; ++m)
       v[m] = make_float2(a.Rr[j0 * N + p0 + T * m], two ? a.Rr[j1 * N + p0 + T * m] : 0.f);
-    fft_warp<T>(v, xs, twr);
+    fft_warp<kLen>(v, xs, twr);
 #pragma unroll
-    for (int m = 0; m < 16; ++m) tmp[p0 + T * m] = v[m];
+    for (int m = 0; m < E; ++m) tmp[p0 + T * m] = v[m];
   }
   cl.sync();
   columns();
@@ -3022,17 +3142,17 @@ __global__ void __cluster_dims__(kSolveCtas, 1, 1) __launch_bounds__(32 * solve_
     float rr[2] = {0.f, 0.f};
     for (int row = row0; row < row_end; row += kRowStep) {
       const long long p0 = (long long)row * kN + t;
-      float2 v[16];
+      float2 v[E];
 #pragma unroll
-      for (int m = 0; m < 16; ++m) v[m] = make_float2(0.f, 0.f);
+      for (int m = 0; m < E; ++m) v[m] = make_float2(0.f, 0.f);
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         if (!(u ? act1 : act0)) continue;
         const float beta = coef[u][0], alpha = coef[u][1];
         const long long o = (long long)(j0 + u) * N + p0;
-        constexpr int kB = 8;  // elements per lane whose loads are in flight together
+        constexpr int kB = E / 2;  // elements per lane whose loads are in flight together
 #pragma unroll
-        for (int b = 0; b < 16; b += kB) {
+        for (int b = 0; b < E; b += kB) {
           float zv[kB], rv[kB], sv[kB], pv[kB], ev[kB], dv[kB];
 #pragma unroll
           for (int k = 0; k < kB; ++k) {
@@ -3062,9 +3182,9 @@ __global__ void __cluster_dims__(kSolveCtas, 1, 1) __launch_bounds__(32 * solve_
           }
         }
       }
-      fft_warp<T>(v, xs, twr);
+      fft_warp<kLen>(v, xs, twr);
 #pragma unroll
-      for (int m = 0; m < 16; ++m) tmp[p0 + T * m] = v[m];
+      for (int m = 0; m < E; ++m) tmp[p0 + T * m] = v[m];
     }
     units += (unsigned long long)(act0 + act1);
     ++it;
@@ -3100,24 +3220,23 @@ __global__ void __cluster_dims__(kSolveCtas, 1, 1) __launch_bounds__(32 * solve_
   }
 }
 
-// Runs fn<T>() for the transform length n = 16 T.
+// Runs fn<n>() for a warp transform of n points.
 template <typename Fn>
 inline void with_warp(int n, Fn&& fn) {
   switch (n) {
-    case 64: fn(std::integral_constant<int, 4>()); return;
-    case 128: fn(std::integral_constant<int, 8>()); return;
-    case 256: fn(std::integral_constant<int, 16>()); return;
-    default: fn(std::integral_constant<int, 32>()); return;
+    case 64: fn(std::integral_constant<int, 64>()); return;
+    case 96: fn(std::integral_constant<int, 96>()); return;
+    case 128: fn(std::integral_constant<int, 128>()); return;
+    case 192: fn(std::integral_constant<int, 192>()); return;
+    case 256: fn(std::integral_constant<int, 256>()); return;
+    case 384: fn(std::integral_constant<int, 384>()); return;
+    default: fn(std::integral_constant<int, kF>()); return;
   }
 }
 inline int warp_rows_per_block(int n) {
   int r = 0;
   with_warp(n, [&](auto t) { r = Warp<decltype(t)::value>::kRows; });
   return r;
-}
-// Where the table of the n-point transform lies in the twiddle buffer (twiddle_kernel).
-inline int warp_twiddles(int n) {
-  return n == 512 ? 0 : kTw512 + kF + (n == 256 ? 0 : n == 128 ? 256 : 384);
 }
 
 // ---- register-resident 1024-point transforms
@@ -3780,7 +3899,7 @@ struct LikelihoodState {
   float* Qp = nullptr;
   double* part = nullptr;   // pq, rz[2], rr[2], bb
   int nbz = 0, nbmax = 0;
-  // circulant FFT preconditioner (power-of-two sizes)
+  // circulant FFT preconditioner
   bool fft = false;
   bool pw = false;          // pointwise products: the image fills the torus (pw_update_rows_fwd_kernel)
   bool solve = false;       // and is square: a pass is one kernel (pw_solve_kernel)
@@ -3905,14 +4024,14 @@ void precond_apply(LikelihoodState* L, double* rz_buf, bool cg, int first,
   if (stages & 1) {
     if (warp_rows(f)) {
       with_warp(f.WP, [&](auto t) {
-        constexpr int T = decltype(t)::value;
-        const dim3 grid((f.H + Warp<T>::kRows - 1) / Warp<T>::kRows, f.pairs);
+        constexpr int n = decltype(t)::value;
+        const dim3 grid((f.H + Warp<n>::kRows - 1) / Warp<n>::kRows, f.pairs);
         if (upd && L->pw)
-          pw_update_rows_fwd_kernel<T><<<grid, kWt, 0, s>>>(f, *upd, it);
+          pw_update_rows_fwd_kernel<n><<<grid, kWt, 0, s>>>(f, *upd, it);
         else if (upd)
-          warp_update_rows_fwd_kernel<T><<<grid, kWt, 0, s>>>(f, *upd, it);
+          warp_update_rows_fwd_kernel<n><<<grid, kWt, 0, s>>>(f, *upd, it);
         else
-          warp_rows_fwd_kernel<T><<<grid, kWt, 0, s>>>(f, L->Rr);
+          warp_rows_fwd_kernel<n><<<grid, kWt, 0, s>>>(f, L->Rr);
       });
     } else if (fft1024_rows(f)) {
       const dim3 grid((f.H + kRows1024 - 1) / kRows1024, f.pairs);
@@ -3928,8 +4047,8 @@ void precond_apply(LikelihoodState* L, double* rz_buf, bool cg, int first,
   if (!(stages & 2)) return;
   if (warp_cols(f))
     with_warp(f.HP, [&](auto t) {
-      constexpr int T = decltype(t)::value;
-      warp_cols_filter_kernel<T><<<dim3(f.WP / Warp<T>::kCols, f.pairs), kWt, 0, s>>>(f, f.filt);
+      constexpr int n = decltype(t)::value;
+      warp_cols_filter_kernel<n><<<dim3(f.WP / Warp<n>::kCols, f.pairs), kWt, 0, s>>>(f, f.filt);
     });
   else if (fft1024_cols(f))
     fft1024_cols_filter_kernel<<<dim3(f.WP / kF512Warps, f.pairs), kWt, sizeof(float2) * kF512Warps * kXs2, s>>>(
@@ -3938,11 +4057,11 @@ void precond_apply(LikelihoodState* L, double* rz_buf, bool cg, int first,
     fft_cols_filter_kernel<<<dim3(f.WP / f.cw, f.pairs), kFftThreads, L->smem_cols, s>>>(f);
   if (warp_rows(f))
     with_warp(f.WP, [&](auto t) {
-      constexpr int T = decltype(t)::value;
+      constexpr int n = decltype(t)::value;
       if (L->pw && cg)
-        warp_rows_inv_kernel<T, true><<<dim3(f.nbz, f.pairs), kWt, 0, s>>>(f, L->Rr, L->Z, rz_buf);
+        warp_rows_inv_kernel<n, true><<<dim3(f.nbz, f.pairs), kWt, 0, s>>>(f, L->Rr, L->Z, rz_buf);
       else
-        warp_rows_inv_kernel<T, false><<<dim3(f.nbz, f.pairs), kWt, 0, s>>>(f, L->Rr, L->Z, rz_buf);
+        warp_rows_inv_kernel<n, false><<<dim3(f.nbz, f.pairs), kWt, 0, s>>>(f, L->Rr, L->Z, rz_buf);
     });
   else if (fft1024_rows(f))
     fft1024_rows_inv_kernel<<<dim3(f.nbz, f.pairs), kWt, 0, s>>>(f, L->Rr, L->Z, rz_buf);
@@ -3965,9 +4084,10 @@ void launch_solve(LikelihoodState* L, const CgArgs& a, const LoopState* ls, int 
   f.max_iter = L->max_iter;
   f.counters = counters;
   with_warp(f.WP, [&](auto t) {
-    constexpr int T = decltype(t)::value;
-    pw_solve_kernel<T><<<f.pairs * kSolveCtas, 32 * solve_warps<T>(), solve_smem<T>(), s>>>(f, a, f.filt, ls, budget,
-                                                                                     &L->d_loop->pass_its);
+    constexpr int n = decltype(t)::value;
+    if constexpr (solve_len(n))
+      pw_solve_kernel<n><<<f.pairs * kSolveCtas, 32 * solve_warps<n>(), solve_smem<n>(), s>>>(
+          f, a, f.filt, ls, budget, &L->d_loop->pass_its);
   });
 }
 
@@ -4153,8 +4273,8 @@ bool raise_smem_limits() {
                        (const void*)residual_pair_kernel<15>,
                        (const void*)fft_rows_fwd_kernel, (const void*)fft_rows_inv_kernel,
                        (const void*)fft_cols_filter_kernel, (const void*)fft1024_cols_filter_kernel,
-                       (const void*)pw_solve_kernel<4>, (const void*)pw_solve_kernel<8>,
-                       (const void*)pw_solve_kernel<16>, (const void*)pw_solve_kernel<32>};
+                       (const void*)pw_solve_kernel<64>, (const void*)pw_solve_kernel<128>,
+                       (const void*)pw_solve_kernel<256>};
   for (const void* f : fns) {
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, f) != cudaSuccess) return false;
@@ -4164,6 +4284,59 @@ bool raise_smem_limits() {
   }
   done[dev] = true;
   return true;
+}
+
+}  // namespace
+
+namespace {
+
+// The preconditioner's torus, HP x WP, for a kh x kw blur of an H x W image: along each axis
+// the image's own length if a transform has it (the exact circulant), else a power of two
+// or 3 2^k whose margin and area cost least.  Measured per update of 33 systems:
+//   - iterations grow as the margin P - n falls below three blur widths, the more the less
+//     noise (9 x 9 blur at 30 dB and at sigma 0.1: margin 6 on 250^2 283 and 58 iterations
+//     against 129 and 49, margin 8 on 376^2 229 and 59 against 130 and 50, margin 12 on
+//     180^2 175 and 51 against 144 and 49), and at 40 dB up to six (188 x 166: 26 columns
+//     21 against 14): modelled as 1 + 0.2 (3 - x) + 0.05 (6 - x), x = margin / width;
+//   - an iteration is bound by latency and its other planes more than by the area (300^2:
+//     88 us on 384^2, 103 on 512^2; 250^2: 59 on 256^2, 76 on 384^2): 1 + area ratio / 3.
+// 250^2 with that blur: 27.7 and 5.9 ms for two sweeps on 256^2, 16.0 and 6.0 on 384^2, which
+// the rule takes; 376^2: 36.5 and 9.7 on 384^2, 24.7 and 9.8 on 512^2; 300^2: 21.5 and 8.7 on
+// 512^2, 18.3 and 7.5 on 384^2.  (Transforms of 160 and 320 points, 20 elements per lane,
+// were no faster than those of 192 and 384.)
+std::pair<int, int> torus(int H, int W, int kh, int kw) {
+  auto pow2 = [](int n) {
+    int p2 = 2;
+    while (p2 < n) p2 <<= 1;
+    return p2;
+  };
+  auto lengths = [&](int n) {
+    std::vector<int> out{pow2(n)};
+    for (int len : {64, 96, 128, 192, 256, 384, 512})
+      if (n > 32 && len >= n && len <= 2 * n && len != out[0]) out.push_back(len);
+    return out;
+  };
+  auto iterations = [](int P, int n, int k) {
+    const double x = (double)(P - n) / std::max(k - 1, 1);
+    return P == n ? 1.0 : 1.0 + 0.2 * std::max(0.0, 3.0 - x) + 0.05 * std::max(0.0, 6.0 - x);
+  };
+  std::pair<int, int> best{pow2(H), pow2(W)};
+  double best_cost = INFINITY;
+  for (int P : lengths(H))
+    for (int Q : lengths(W)) {
+      FftDesc f{};
+      f.HP = P;
+      f.WP = Q;
+      // the other column passes are for powers of two, and slower where this one could do
+      if ((P % 3 == 0 || (Q % 3 == 0 && warp_len(P))) && !warp_cols(f)) continue;
+      const double cost =
+          iterations(P, H, kh) * iterations(Q, W, kw) * (1.0 + (double)P * Q / (3.0 * H * W));
+      if (cost < best_cost) {
+        best_cost = cost;
+        best = {P, Q};
+      }
+    }
+  return best;
 }
 
 }  // namespace
@@ -4256,14 +4429,7 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
   c.tiles_x = (c.W + kTile - 1) / kTile;
   c.tiles_y = (c.H + kTile - 1) / kTile;
   L->nb = c.tiles_x * c.tiles_y;
-  // circulant preconditioner on the smallest power-of-two torus that holds the image
-  // (padding keeps it symmetric positive definite: crop * C^-1 * pad)
-  auto next_pow2 = [](int v) {
-    int p2 = 2;
-    while (p2 < v) p2 <<= 1;
-    return p2;
-  };
-  const int HP = next_pow2(c.H), WP = next_pow2(c.W);
+  const auto [HP, WP] = torus(c.H, c.W, kh, kw);
   L->fft = HP <= 8192 && WP <= 8192;
   // Sides that are not powers of two: a quarter of both targets.  How far a solution is from
   // the exact one at a given residual depends on the preconditioner: CG under the padded
@@ -4300,7 +4466,7 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
     L->pw = c.H == HP && c.W == WP && warp_rows(f);
     // 512^2: three kernels per iteration with 16 to 24 warps per SM are faster there (124
     // against 173 us) than one cluster of eight 8-warp CTAs per pair
-    L->solve = L->pw && HP == WP && HP <= 256;
+    L->solve = L->pw && HP == WP && solve_len(HP);
     L->smem_rows = sizeof(float2) * ((size_t)WP + (size_t)f.rpb * WP);
     L->smem_cols = sizeof(float2) * ((size_t)HP + (size_t)HP * f.cw);
   }

@@ -252,11 +252,12 @@ def test_deconv_mog2_prior_parity_and_no_em():
 
 
 @pytest.mark.parametrize("h,w,periodic", [(60, 60, 1), (64, 128, 1), (33, 67, 0), (100, 250, 1), (131, 256, 0),
-                                          (256, 40, 1), (300, 130, 1), (30, 511, 0), (520, 66, 1), (62, 1000, 1)])
+                                          (256, 40, 1), (300, 130, 1), (30, 511, 0), (520, 66, 1), (62, 1000, 1),
+                                          (96, 96, 1), (192, 98, 1), (97, 191, 0), (384, 70, 1), (78, 350, 1)])
 def test_deconv_parity_transform_sizes(h, w, periodic):
-    """Every length of the preconditioner's warp transforms (64 to 512 points) along rows
-    and columns, with 1024 and the shared-memory ones, with margins from none to
-    nearly half the transform, even and odd; the oracle solves by FP64 CG."""
+    """Every length of the preconditioner's warp transforms (64 to 512 points, powers of two
+    and 3 2^k) along rows and columns, with 1024 and the shared-memory ones, with margins
+    from none to nearly half the transform, even and odd; the oracle solves by FP64 CG."""
     p = syn.deconv_problem(h, w, kernel=syn.uniform_kernel(5), bsnr_db=30.0, beta0=2.0, seed=h + w,
                            grf_length=8.0)
     S = 3
@@ -269,19 +270,16 @@ def test_deconv_parity_transform_sizes(h, w, periodic):
     ep.close()
 
 
-def _emulated_iterations(p, pr, d, ncav, rtol, eta=3.2e-5):
+def _emulated_iterations(p, pr, d, ncav, rtol, torus, eta=3.2e-5):
     """Iterations of the first likelihood update (zero start): refinement passes of FP32 CG
-    preconditioned by the windowed periodic extension into the power-of-two torus, all
+    preconditioned by the windowed periodic extension into the torus, all
     systems in step, each pass down to max(eta |r|, rtol |b| / 2).  In FP32 as on the GPU:
     on these systems (flat regions have d near 1e-7) rounding costs CG iterations."""
     import scipy.fft as sf
     f4 = np.float32
     h, w = p.y.shape
 
-    def axis(n):
-        P = 2
-        while P < n:
-            P *= 2
+    def axis(n, P):
         L = (P - n) // 2
         i = np.arange(P)
         src = np.where(i < n, i, np.where(i < n + L, i - n, np.where(i >= P - L, i - P + n, -1)))
@@ -295,7 +293,7 @@ def _emulated_iterations(p, pr, d, ncav, rtol, eta=3.2e-5):
         assert np.allclose(E.T @ E, np.eye(n))
         return E
 
-    Er, Ec = axis(h), axis(w)
+    Er, Ec = axis(h, torus[0]), axis(w, torus[1])
     Er4, Ec4 = Er.astype(f4), Ec.astype(f4)
     k = p.kernel
     pad = np.zeros((Er.shape[0], Ec.shape[0]))
@@ -337,8 +335,10 @@ def _emulated_iterations(p, pr, d, ncav, rtol, eta=3.2e-5):
     return total
 
 
-@pytest.mark.parametrize("h,w,periodic", [(76, 108, 1), (45, 99, 0), (40, 140, 1), (128, 64, 1), (24, 600, 1)])
-def test_preconditioner_iterations_are_those_of_the_windowed_extension(h, w, periodic):
+@pytest.mark.parametrize("h,w,periodic,torus", [
+    (76, 108, 1, (96, 128)), (45, 99, 0, (64, 128)), (40, 140, 1, (64, 192)), (128, 64, 1, (128, 64)),
+    (24, 600, 1, (32, 1024)), (300, 90, 1, (384, 128)), (62, 62, 1, (96, 96))])
+def test_preconditioner_iterations_are_those_of_the_windowed_extension(h, w, periodic, torus):
     """The preconditioner shows in the iteration count alone: the count of the first
     likelihood update is that of the emulation.  The target, 1e-4, is one that a single
     refinement pass meets (at 1e-9 the FP32 floor decides how many passes follow); FP32
@@ -359,5 +359,5 @@ def test_preconditioner_iterations_are_those_of_the_windowed_extension(h, w, per
         assert ep.solver_report()["passes"] == 1
         tau, nu = (t.cpu().numpy().astype(np.float64) for t in ep.sites())
         ep.close()
-    ref = _emulated_iterations(p, pr, tau[1:].sum(axis=0), nu[1:].sum(axis=0), rtol=1e-4)
+    ref = _emulated_iterations(p, pr, tau[1:].sum(axis=0), nu[1:].sum(axis=0), 1e-4, torus)
     assert abs(its - ref) <= 3 + 0.1 * ref, (its, ref)

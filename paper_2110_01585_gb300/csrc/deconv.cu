@@ -1272,18 +1272,28 @@ __global__ void __launch_bounds__(kThreads, 5) direction_kernel(CgArgs a, int it
 // preconditioner, separable H^T H with equal half-widths HR).  The region holds
 // (system 0, system 1) float2 pairs, so that each tap of both stencil passes is one
 // packed FP32 FMA for the two systems, and the index arithmetic, the shared-memory
-// addressing and the loads of d serve both.  Row pass: two adjacent outputs per thread
-// from one window read as float4; column pass: four consecutive rows of one column per
-// thread, whose outputs stay in registers for the epilogue.  Per system and output
-// the taps are summed in the order of hth_tile_sep.  A system that has stopped is
-// neither read nor written.
+// addressing and the loads of d serve both.  Row pass: eight adjacent outputs per thread
+// from a window in registers, read as float4, a warp down 32 rows; two outputs per thread
+// took twice the shared-memory wavefronts, which bounded the 15 x 15 blur.  Column pass:
+// four consecutive rows of one column per thread, whose outputs stay in registers for the
+// epilogue.  Per system and output the taps are summed in the order of hth_tile_sep.  A
+// system that has stopped is neither read nor written.
+// Bound by the planes (z, p, e read, p, q, e written, 24 bytes per pixel and system, the
+// first two with the halo) and by the shared memory: 488^2 with 33 systems, 15 x 15 blur, 116 ->
+// 91 us (tiles of 64 rows, with half the halo per output, were no faster); rows that are no
+// multiple of four floats long staged two floats at a time, instead of one, and their e
+// updated along the rows, instead of four floats per lane: 458^2, 9 x 9, 99 -> 57 us.
+// Pitch of its region: a multiple of two that puts eight rows in distinct banks of 16 bytes.
+template <int HR>
+constexpr int kPairPitch = kTile + 2 * HR + 2;
 template <int HR>
 __global__ void __launch_bounds__(kThreads, HR >= 14 ? 3 : 5) direction_pair_kernel(CgArgs a, int it_arg) {
   constexpr int RH = kTile + 2 * HR, RW = kTile + 2 * HR, NT = 2 * HR + 1;
+  constexpr int RP = kPairPitch<HR>, TP = kTile + 2;  // pitches of the two buffers
   extern __shared__ float4 smem4[];
   float2* reg = reinterpret_cast<float2*>(smem4);  // RH x RW region pairs
-  float2* tmp = reg + RH * RW;                     // RH x kTile, after the row pass
-  __shared__ float2 taps2[2 * NT];                 // (g, g): row taps, then column taps
+  float2* tmp = reg + RH * RP;                     // RH x kTile, after the row pass
+  __shared__ __align__(16) float2 tapr[NT + 1], tapc[NT + 1];  // (g, g) of the row and column taps
   __shared__ int ctab[RW];
   const ConvDesc& c = a.c;
   const int j0 = 2 * blockIdx.z, j1 = j0 + 1;
@@ -1296,9 +1306,10 @@ __global__ void __launch_bounds__(kThreads, HR >= 14 ? 3 : 5) direction_pair_ker
   const int r0 = blockIdx.y * kTile, c0 = blockIdx.x * kTile;
   for (int i = threadIdx.x; i < 2 * NT; i += kThreads) {
     const float g = i < NT ? c.gr[i] : c.gc[i - NT];
-    taps2[i] = make_float2(g, g);
+    (i < NT ? tapr[i] : tapc[i - NT]) = make_float2(g, g);
   }
   column_table(ctab, c0 - HR, RW, c.W);
+  const int rows = min(kTile, c.H - r0) + 2 * HR;  // of the region
   const long long N = c.N;
   const long long o0 = (long long)j0 * N, o1 = (long long)j1 * N;
   const float* Pold = (it & 1) ? a.P : a.P2;
@@ -1314,7 +1325,8 @@ __global__ void __launch_bounds__(kThreads, HR >= 14 ? 3 : 5) direction_pair_ker
   if ((c.W & 3) == 0 && (HR & 3) == 0 && c0 >= HR && c0 + kTile + HR <= c.W) {
     // no column wraps: float4 quads of each plane
     // in rounds of KQ quads per thread, all loads of a round in flight together
-    constexpr int Q4 = RW / 4, NQ = RH * Q4, KQ = 2;
+    constexpr int Q4 = RW / 4, KQ = 2;
+    const int NQ = rows * Q4;
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int i0 = threadIdx.x; i0 < NQ; i0 += KQ * kThreads) {
     float4 zv0[KQ], zv1[KQ], pv0[KQ], pv1[KQ];
@@ -1351,14 +1363,54 @@ __global__ void __launch_bounds__(kThreads, HR >= 14 ? 3 : 5) direction_pair_ker
           v1.z = fmaf(beta1, pv1[k].z, v1.z);
           v1.w = fmaf(beta1, pv1[k].w, v1.w);
         }
-        float4* dst = reinterpret_cast<float4*>(reg + rr * RW + 4 * q);
+        float4* dst = reinterpret_cast<float4*>(reg + rr * RP + 4 * q);
         dst[0] = make_float4(v0.x, v1.x, v0.y, v1.y);
         dst[1] = make_float4(v0.z, v1.z, v0.w, v1.w);
       }
     }
     }
+  } else if ((c.W & 1) == 0) {
+    // even rows and an even first column: two neighbours stay neighbours across the wrap
+    constexpr int kBatch = 4, Q2 = RW / 2;
+    const int NQ = rows * Q2;
+    const float2 zero2 = make_float2(0.f, 0.f);
+    for (int i0 = threadIdx.x; i0 < NQ; i0 += kBatch * kThreads) {
+      float2 zs0[kBatch], zs1[kBatch], ps0[kBatch], ps1[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const int i = i0 + u * kThreads;
+        zs0[u] = zs1[u] = ps0[u] = ps1[u] = zero2;
+        if (i < NQ) {
+          const int rr = i / Q2, q = i - rr * Q2;
+          const long long p = (long long)wrapi(r0 - HR + rr, c.H) * c.W + ctab[2 * q];
+          if (act0) {
+            zs0[u] = *reinterpret_cast<const float2*>(a.Z + o0 + p);
+            if (it > 0) ps0[u] = *reinterpret_cast<const float2*>(Pold + o0 + p);
+          }
+          if (act1) {
+            zs1[u] = *reinterpret_cast<const float2*>(a.Z + o1 + p);
+            if (it > 0) ps1[u] = *reinterpret_cast<const float2*>(Pold + o1 + p);
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const int i = i0 + u * kThreads;
+        if (i < NQ) {
+          float2 v0 = zs0[u], v1 = zs1[u];
+          if (it > 0) {
+            v0.x = fmaf(beta0, ps0[u].x, v0.x);
+            v0.y = fmaf(beta0, ps0[u].y, v0.y);
+            v1.x = fmaf(beta1, ps1[u].x, v1.x);
+            v1.y = fmaf(beta1, ps1[u].y, v1.y);
+          }
+          *reinterpret_cast<float4*>(reg + i / Q2 * RP + 2 * (i % Q2)) = make_float4(v0.x, v1.x, v0.y, v1.y);
+        }
+      }
+    }
   } else {
-    constexpr int kBatch = 4, NE = RH * RW;
+    constexpr int kBatch = 4;
+    const int NE = rows * RW;
     for (int i0 = threadIdx.x; i0 < NE; i0 += kBatch * kThreads) {
       float zs0[kBatch], zs1[kBatch], ps0[kBatch], ps1[kBatch];
 #pragma unroll
@@ -1382,34 +1434,44 @@ __global__ void __launch_bounds__(kThreads, HR >= 14 ? 3 : 5) direction_pair_ker
       for (int u = 0; u < kBatch; ++u) {
         const int i = i0 + u * kThreads;
         if (i < NE)
-          reg[i] = it > 0 ? make_float2(fmaf(beta0, ps0[u], zs0[u]), fmaf(beta1, ps1[u], zs1[u]))
+          reg[i / RW * RP + i % RW] = it > 0 ? make_float2(fmaf(beta0, ps0[u], zs0[u]), fmaf(beta1, ps1[u], zs1[u]))
                           : make_float2(zs0[u], zs1[u]);
       }
     }
   }
   __syncthreads();
-  // row pass (column taps along the rows)
+  // row pass (column taps along the rows): eight adjacent outputs per thread from one
+  // window, a warp down the rows
   {
-    const int cp = threadIdx.x & 15;  // column pair 2 cp, 2 cp + 1 of the tile
-    for (int rr = threadIdx.x >> 4; rr < RH; rr += kThreads / 16) {
-      const float4* row4 = reinterpret_cast<const float4*>(reg + rr * RW + 2 * cp);
-      // window columns 2 q, 2 q + 1 arrive as one float4; tap b meets columns b, b + 1
-      float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
-      float4 t = row4[0];
+    const int rr = threadIdx.x & 63, cg = threadIdx.x >> 6;  // row, columns 8 cg .. 8 cg + 7
+    static_assert(RH <= 64 && kThreads == 256 && kTile == 32, "one round");
+    if (rr < rows) {
+      const float4* x4 = reinterpret_cast<const float4*>(reg + rr * RP + 8 * cg);
+      // input i of the window at win[i % 10]; tap t meets inputs t .. t + 7
+      float2 win[10], acc[8];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float4 x = x4[u];
+        win[2 * u] = make_float2(x.x, x.y);
+        win[2 * u + 1] = make_float2(x.z, x.w);
+        acc[2 * u] = acc[2 * u + 1] = make_float2(0.f, 0.f);
+      }
 #pragma unroll
       for (int q = 0; q < HR; ++q) {
-        const float4 u = row4[q + 1];
-        const float2 w0 = taps2[NT + 2 * q], w1 = taps2[NT + 2 * q + 1];
-        a0 = __ffma2_rn(w0, make_float2(t.x, t.y), a0);
-        a1 = __ffma2_rn(w0, make_float2(t.z, t.w), a1);
-        a0 = __ffma2_rn(w1, make_float2(t.z, t.w), a0);
-        a1 = __ffma2_rn(w1, make_float2(u.x, u.y), a1);
-        t = u;
+        const float4 x = x4[q + 4], g = *reinterpret_cast<const float4*>(tapc + 2 * q);
+        win[(2 * q + 8) % 10] = make_float2(x.x, x.y);
+        win[(2 * q + 9) % 10] = make_float2(x.z, x.w);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc[u] = __ffma2_rn(make_float2(g.x, g.y), win[(2 * q + u) % 10], acc[u]);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc[u] = __ffma2_rn(make_float2(g.z, g.w), win[(2 * q + 1 + u) % 10], acc[u]);
       }
-      const float2 wl = taps2[NT + 2 * HR];
-      a0 = __ffma2_rn(wl, make_float2(t.x, t.y), a0);
-      a1 = __ffma2_rn(wl, make_float2(t.z, t.w), a1);
-      *reinterpret_cast<float4*>(tmp + rr * kTile + 2 * cp) = make_float4(a0.x, a0.y, a1.x, a1.y);
+      const float2 g = tapc[2 * HR];
+      float4* out = reinterpret_cast<float4*>(tmp + rr * TP + 8 * cg);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) acc[u] = __ffma2_rn(g, win[(2 * HR + u) % 10], acc[u]);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) out[u] = make_float4(acc[2 * u].x, acc[2 * u].y, acc[2 * u + 1].x, acc[2 * u + 1].y);
     }
   }
   __syncthreads();
@@ -1418,14 +1480,14 @@ __global__ void __launch_bounds__(kThreads, HR >= 14 ? 3 : 5) direction_pair_ker
   float2 acc[4];
   {
     // a sliding window of four inputs: tap t meets rows tr0 + t .. tr0 + t + 3
-    float2 in0 = tmp[tr0 * kTile + tx], in1 = tmp[(tr0 + 1) * kTile + tx],
-           in2 = tmp[(tr0 + 2) * kTile + tx];
+    float2 in0 = tmp[tr0 * TP + tx], in1 = tmp[(tr0 + 1) * TP + tx],
+           in2 = tmp[(tr0 + 2) * TP + tx];
 #pragma unroll
     for (int o = 0; o < 4; ++o) acc[o] = make_float2(0.f, 0.f);
 #pragma unroll
     for (int t = 0; t < NT; ++t) {
-      const float2 in3 = tmp[(tr0 + t + 3) * kTile + tx];
-      const float2 wr = taps2[t];
+      const float2 in3 = tmp[(tr0 + t + 3) * TP + tx];
+      const float2 wr = tapr[t];
       acc[0] = __ffma2_rn(wr, in0, acc[0]);
       acc[1] = __ffma2_rn(wr, in1, acc[1]);
       acc[2] = __ffma2_rn(wr, in2, acc[2]);
@@ -1442,7 +1504,7 @@ __global__ void __launch_bounds__(kThreads, HR >= 14 ? 3 : 5) direction_pair_ker
     const int tr = tr0 + o, gr = r0 + tr, gcol = c0 + tx;
     if (gr >= c.H || gcol >= c.W) continue;
     const long long p = (long long)gr * c.W + gcol;
-    const float2 pv = reg[(tr + HR) * RW + tx + HR];
+    const float2 pv = reg[(tr + HR) * RP + tx + HR];
     const float d = a.D[p];
     if (act0) {
       const float q = acc[o].x * c.inv_xi + d * pv.x;
@@ -1466,10 +1528,10 @@ __global__ void __launch_bounds__(kThreads, HR >= 14 ? 3 : 5) direction_pair_ker
     // was active then)
     const float al0 = a.scal[4 * j0 + 2], al1 = act1 ? a.scal[4 * j1 + 2] : 0.f;
     const bool e_zero = it == 1;  // the correction starts at zero: not read
-    const int gr = r0 + (threadIdx.x >> 3), gc0 = c0 + (threadIdx.x & 7) * 4;
-    if (gr < c.H) {
-      const long long p = (long long)gr * c.W + gc0;
-      if ((c.W & 3) == 0 && gc0 + 4 <= c.W) {
+    if ((c.W & 3) == 0) {
+      const int gr = r0 + (threadIdx.x >> 3), gc0 = c0 + (threadIdx.x & 7) * 4;
+      if (gr < c.H && gc0 < c.W) {
+        const long long p = (long long)gr * c.W + gc0;
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           if (!(u ? act1 : act0)) continue;
@@ -1484,11 +1546,30 @@ __global__ void __launch_bounds__(kThreads, HR >= 14 ? 3 : 5) direction_pair_ker
           ev.w = fmaf(al, pv.w, ev.w);
           *reinterpret_cast<float4*>(a.Ec + q) = ev;
         }
-      } else {
-        for (int t = 0; t < 4 && gc0 + t < c.W; ++t) {
-          if (act0) a.Ec[o0 + p + t] = fmaf(al0, Pold[o0 + p + t], e_zero ? 0.f : a.Ec[o0 + p + t]);
-          if (act1) a.Ec[o1 + p + t] = fmaf(al1, Pold[o1 + p + t], e_zero ? 0.f : a.Ec[o1 + p + t]);
+      }
+    } else if (c0 + tx < c.W) {
+      // a row of the tile per warp and round, all loads in flight together
+      float pv[2][4], ev[2][4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int gr = r0 + (threadIdx.x >> 5) + 8 * k;
+        const long long p = (long long)gr * c.W + c0 + tx;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          pv[u][k] = ev[u][k] = 0.f;
+          if (gr < c.H && (u ? act1 : act0)) {
+            pv[u][k] = Pold[(u ? o1 : o0) + p];
+            if (!e_zero) ev[u][k] = a.Ec[(u ? o1 : o0) + p];
+          }
         }
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int gr = r0 + (threadIdx.x >> 5) + 8 * k;
+        const long long p = (long long)gr * c.W + c0 + tx;
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+          if (gr < c.H && (u ? act1 : act0)) a.Ec[(u ? o1 : o0) + p] = fmaf(u ? al1 : al0, pv[u][k], ev[u][k]);
       }
     }
   }
@@ -4128,8 +4209,8 @@ void launch_direction(const LikelihoodState* L, const CgArgs& a, int it, cudaStr
   const ConvDesc& c = L->c;
   if (pair_direction(L)) {
     const dim3 g(c.tiles_x, c.tiles_y, (L->R + 1) / 2);
-    // region (RH x RW) and row-pass output (RH x kTile) pairs
-    const size_t sm = sizeof(float2) * (size_t)(kTile + 2 * c.hr) * (2 * kTile + 2 * c.hr);
+    // the region and the row pass's output
+    const size_t sm = sizeof(float2) * (size_t)(kTile + 2 * c.hr) * ((kTile + 2 * c.hr + 2) + (kTile + 2));
     switch (c.hr) {
       case 2: direction_pair_kernel<2><<<g, kThreads, sm, s>>>(a, it); return;
       case 4: direction_pair_kernel<4><<<g, kThreads, sm, s>>>(a, it); return;

@@ -270,6 +270,23 @@ def test_deconv_parity_transform_sizes(h, w, periodic):
     ep.close()
 
 
+@pytest.mark.parametrize("h,w,kernel,periodic", [(70, 66, 15, 1), (40, 100, 15, 1), (45, 67, 15, 0), (68, 70, 9, 1),
+                                                 (72, 41, 9, 0), (66, 92, 5, 1), (34, 62, 3, 1)])
+def test_deconv_parity_stencil_forms(h, w, kernel, periodic):
+    """The paired stencil product for every halo, with rows of 4 k, even and odd lengths
+    (float4, float2 and scalar staging) and tiles cut by the image's edges."""
+    p = syn.deconv_problem(h, w, kernel=syn.uniform_kernel(kernel), bsnr_db=30.0, beta0=2.0, seed=h + w,
+                           grf_length=8.0)
+    S = 3
+    pr = probes(p, S, 54)
+    mu, var, ep = _gpu(p, 2, S, pr, periodic=periodic)
+    o = EPOracle("deconv", y32(p), p.xi, p.beta, h, w, kernel=p.kernel, site0="rbmc_cg", probes=pr,
+                 periodic=bool(periodic))
+    o.run(2)
+    assert_parity(mu, var, *o.posterior(), p.y)
+    ep.close()
+
+
 def _emulated_iterations(p, pr, d, ncav, rtol, torus, eta=3.2e-5):
     """Iterations of the first likelihood update (zero start): refinement passes of FP32 CG
     preconditioned by the windowed periodic extension into the torus, all

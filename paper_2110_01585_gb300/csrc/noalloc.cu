@@ -27,7 +27,7 @@ namespace {
 
 // Large images are cut into units of 16 row pairs of a 60-column strip, so 65536 units
 // hold images of up to about 65536 * 32 * 60 = 126 M pixels.  Shorter units are taken
-// only by images of fewer than 7296 of those, which have fewer than 2 * 7296 units.
+// only where an image has at most 18 * 1824 of them (unit_shift in prior_sweep.cu).
 constexpr int kNoAllocMaxBlocks = 65536;
 constexpr int kNoAllocDoubles = kNoAllocMaxBlocks + 8;
 constexpr int kMaxDevices = 64;

@@ -48,7 +48,7 @@ namespace {
 
 constexpr int kStripCols = 60;     // owned columns per warp (lanes 1..30, two each)
 constexpr int kMaxUnitShift = 4;   // at most 16 row-pair steps per work unit
-constexpr long long kWantUnits = 4 * 1824;  // units a whole image is cut into, if it has them
+constexpr int kSweepWarps = 152 * 12;  // warps the GPU holds, see unit_shift()
 constexpr int kWarpsPerBlock = 4;
 constexpr int kThreads = 32 * kWarpsPerBlock;
 constexpr int kMinBlocks = 3;      // blocks per SM the register budget is sized for
@@ -1045,19 +1045,29 @@ double prior_sweep_bytes_per_pixel(bool site0_from_y) {
   return site0_from_y ? (9 + 8) * 4.0 : (10 + 8) * 4.0;
 }
 
-// Row-pair steps per work unit, as a power of two: the longest unit (16 steps at most)
-// that still cuts the image into kWantUnits units, four per warp the GPU holds
-// (152 SMs x 12 warps), so that the warps' ranges differ by a quarter at most; small
-// images come down to units of one step.  A warp runs its steps one after another
-// (about 2.4 us each while few warps are resident, 3.7 us with twelve per SM), and a range
-// of any length starts with one warm-up step.  By size only, so that an image's E|u|
-// sums do not depend on the device or on the batch it is in.  With units of 16 steps
-// always, a 64^2 to 1024^2 sweep took 41-42 us, one warp's 17 steps; now 8.3 us at 64^2
-// and 15 us at 512^2.  Eight units per warp made 4096^2 1.3% slower (units of 8 steps,
-// whose FP64 sums cost more than the finer ranges gave).
+// Row-pair steps per work unit, as a power of two: the one whose longest range takes the
+// least time.  The GPU holds kSweepWarps warps; a warp runs its range of units step after
+// step (about 2.4 us each while few warps are resident, 3.7 us with twelve per SM), after
+// one warm-up step, and a unit's FP64 sums cost another 0.05 to 0.2 of a step.  Small
+// images come down to units of one step; the largest keep 16.  By size only, so that an
+// image's E|u| sums do not depend on the device or on the batch it is in.  With units of 16
+// steps always, a 64^2 to 1024^2 sweep took 41-42 us, one warp's 17 steps; now 8.3 us at
+// 64^2 and 12.4 us at 512^2.  Four units per warp, whatever ranges they gave, took 13.0 us
+// at 512^2, 76.5 against 75.1 at 2014 x 1513 and 92.3 against 87.1 at 2500 x 1800.
 static int unit_shift(int height, int width) {
-  int shift = kMaxUnitShift;
-  while (shift > 0 && (long long)strips_of(width) * units_per_strip(height, shift) < kWantUnits) --shift;
+  int shift = 0;
+  double least = 0.0;
+  for (int s = kMaxUnitShift; s >= 0; --s) {
+    const long long units = (long long)strips_of(width) * units_per_strip(height, s);
+    // 18 units per warp leave nothing to balance; and the scratch of the sweep that
+    // allocates nothing holds 65536
+    if (s < kMaxUnitShift && units > 18 * kSweepWarps) break;
+    const double steps = (double)((units + kSweepWarps - 1) / kSweepWarps) * ((1 << s) + 0.15) + 1.0;
+    if (s == kMaxUnitShift || steps < least) {
+      least = steps;
+      shift = s;
+    }
+  }
   return shift;
 }
 

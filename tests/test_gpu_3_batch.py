@@ -77,7 +77,7 @@ def test_batch_denoise_matches_oracle():
 
 @pytest.mark.parametrize("h,w", [(2, 2), (3, 61), (66, 120), (30000, 62)])
 def test_unit_lengths_batch_and_statistic(h, w):
-    """Work units of one row-pair step (the small sizes) and of four (30000 x 62): an
+    """Work units of one row-pair step (the small sizes) and of two (30000 x 62): an
     image swept in a batch with one of another unit length gives the bits of the image
     alone, and a_u, whose partial sums are one per unit, is the oracle's (FP32 terms of
     relative error below 1e-6 summed in FP32 per lane and unit, then in FP64)."""

@@ -116,8 +116,9 @@ typedef struct {
   int32_t cg_max_iter;   /* CONV_PERIODIC: cap on the conjugate-gradient iterations of one
                             likelihood-site update (all refinement passes together) */
   double cg_rtol;        /* CONV_PERIODIC: target of the true relative residual ||b - Q x|| /
-                            ||b|| of the mean solve (probe solves: max(cg_rtol, 1e-6)).  The
-                            residual is recomputed in float-float arithmetic between FP32
+                            ||b|| of the mean solve (probe solves: max(cg_rtol, 1e-6)); a
+                            quarter of both for images whose sides are not powers of two.
+                            The residual is recomputed in float-float arithmetic between FP32
                             CG passes; a solve also stops when a pass no longer halves a
                             residual already below 1e-6 (the evaluation floor).  Default 1e-9. */
   int32_t precision;     /* 0: FP32 with FP64 for edges whose tilted moments lose
@@ -282,18 +283,22 @@ ep_tv_status ep_tv_solve_host(const ep_tv_operator* op, const float* y_host,
 /* Kernel classes reported by the tracer. */
 typedef enum {
   EP_TV_K_PRIOR_SWEEP = 0,   /* fused V_1..V_4 prior-site pass, unit = pixel */
-  EP_TV_K_CG_DIRECTION = 1,  /* CG direction + H^T H stencil (with 512-point FFT rows and a
-                                separable blur also the previous iteration's correction
-                                update), unit = pixel of one active system */
-  EP_TV_K_CG_UPDATE = 2,     /* CG correction / residual update (with 512-point FFT rows: the
-                                residual update fused with the preconditioner's forward row
-                                pass), unit = pixel of one active system */
+  EP_TV_K_CG_DIRECTION = 1,  /* CG direction + H^T H stencil (with FFT rows of 64 to 1024 points
+                                and a separable blur also the previous iteration's correction
+                                update), unit = pixel of one active system; none for images
+                                that fill the preconditioner's torus */
+  EP_TV_K_CG_UPDATE = 2,     /* CG correction / residual update (with those FFT rows fused with
+                                the preconditioner's forward row pass; for images that fill the
+                                torus also the direction and its product; for 64^2, 128^2 and
+                                256^2 all iterations of a refinement pass in one launch),
+                                unit = pixel of one active system and iteration */
   EP_TV_K_CG_RESIDUAL = 3,   /* true CG residual of a refinement pass, unit = pixel of one
                                 system */
   EP_TV_K_SITE0 = 4,         /* likelihood-site update, unit = pixel */
   EP_TV_K_CG_PRECOND = 5,    /* FFT circulant preconditioner (3 kernels; 2 in CG iterations whose
-                                forward row pass runs with the update), unit = pixel of one
-                                transformed system (pairs of stopped systems are skipped) */
+                                forward row pass runs with the update; none where a pass is one
+                                launch), unit = pixel of one transformed system (pairs of
+                                stopped systems are skipped) */
   EP_TV_K_CS = 6,            /* compressive-sensing likelihood site (Woodbury, FP64-accurate)
                                 except its tensor-core products, unit = pixel; its per-unit
                                 figure is FP64 CUDA-core flops, not bytes */
@@ -408,7 +413,7 @@ size_t ep_tv_conv3x3_backward_work(int32_t n, int32_t cin, int32_t cout, int32_t
    Overwrites dweight (cout x cin x 3 x 3), dbias (cout) and, unless it is NULL,
    dx (n x cin x h x w; needs cin <= 32).  work: DEVICE scratch of at least
    ep_tv_conv3x3_backward_work bytes, owned by the caller.  The weight gradient
-   is summed per 16 x 16 tile and then over tiles in a fixed order
+   is summed per tile and then over tiles, by compensated sums in a fixed order
    (deterministic). */
 ep_tv_status ep_tv_conv3x3_backward(int32_t n, int32_t cin, int32_t cout, int32_t height,
                                     int32_t width, const float* x, const float* weight,

@@ -1742,8 +1742,8 @@ __global__ void commit_kernel(double* X, const float* Ec, const int* act0, long 
 // Two real systems share one complex transform (z = r_a + i r_b): the filter is
 // real and even in frequency, so the real and imaginary parts of the result are
 // M^{-1} r_a and M^{-1} r_b.  Rows, then columns (forward, filter, inverse in one
-// pass), then rows again; 512-point transforms are register-resident (one warp per
-// row or column), other sizes run Stockham passes in shared memory.
+// pass), then rows again; transforms of 64 to 1024 points are register-resident (a warp
+// per row or column, or for several), other sizes run Stockham passes in shared memory.
 struct FftDesc {
   int H, W;          // image
   int HP, WP;        // transform sizes, HP >= H, WP >= W
@@ -2162,7 +2162,7 @@ __global__ void __launch_bounds__(kFftThreads, 4) fft_rows_inv_kernel(FftDesc f,
 // transform, a pointwise filter and another transform chain in registers.
 constexpr int kF = 512;
 constexpr int kXs = 578;        // scratch / staged-column pitch in float2
-constexpr int kF512Warps = 8;   // warps per block of the 512-point kernels
+constexpr int kF512Warps = 8;   // warps per block of the kernels with warp transforms
 // The row passes take a warp's rows one after another, each row's loads all issued before
 // its transform starts (prefetching the next row during the transform measured slower:
 // it raises register pressure at the 128-register limit).
@@ -2358,7 +2358,7 @@ __device__ __forceinline__ void fft512_warp(float2 (&v)[16], float2* xs, const f
 // 26 us here, and the forward one is fused with the CG update.
 //
 // Sizes per warp, in float2: kRow, from one transform's regrouping area to the next (entry
-// (k1, t) at k1 (T + 1) + t); kCol, from one staged column to the next in the column pass;
+// (k1, t) at k1 (T + 1) + t, for E = 12 at 13 t + k1, then (u, j) at kPc u + j); kCol, from one staged column to the next in the column pass;
 // kScratch, from one warp's area to the next.  Their residues mod 16 keep the accesses of a
 // half-warp in distinct banks.
 template <int kLen>
@@ -4079,8 +4079,8 @@ int ilog2(int v) {
 // pass sets beta and r.z of the active systems (first: the first application of a
 // refinement pass, beta = 0); without it every system is transformed and the CG
 // scalars are left alone (launch-shape tuning).
-// stages: 1 = the forward row pass (fused with the CG update when upd is given:
-// 512-point rows only, see fused_update), 2 = the column and inverse row passes.
+// stages: 1 = the forward row pass (fused with the CG update when upd is given, see
+// fused_update), 2 = the column and inverse row passes.
 // step: graph replays, whose column pass then advances the inner loop and its
 // condition h_step (loop_step).
 void precond_apply(LikelihoodState* L, double* rz_buf, bool cg, int first,

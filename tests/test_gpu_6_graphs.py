@@ -99,6 +99,7 @@ def test_deconv_update_graph_equals_host_driven_loop(h, w, kernel, em):
 @pytest.mark.parametrize("h,w,S,max_iter", [
     (64, 64, 1, 0), (64, 64, 4, 0), (128, 128, 5, 0), (256, 256, 2, 0),  # a pass as one kernel
     (64, 128, 3, 0), (192, 96, 2, 0), (512, 64, 4, 0), (128, 384, 2, 0),  # three kernels per iteration
+    (32, 64, 2, 0), (32, 96, 3, 0), (1024, 64, 1, 0),                    # with the other column passes
     (64, 64, 2, 7), (128, 128, 1, 1), (128, 64, 2, 7), (38, 68, 2, 6)])  # the iteration budget runs out
 def test_deconv_pass_forms_graph_equals_host_driven_loop(h, w, S, max_iter):
     """Images that fill the preconditioner's torus (products formed pointwise, a pass

@@ -411,8 +411,9 @@ size_t ep_tv_conv3x3_backward_work(int32_t n, int32_t cin, int32_t cout, int32_t
 /* Gradients through one ep_tv_conv3x3_forward call given dy = dL/dy.  y is that
    call's output when it applied the ReLU (dy is masked by y > 0), else NULL.
    Overwrites dweight (cout x cin x 3 x 3), dbias (cout) and, unless it is NULL,
-   dx (n x cin x h x w; needs cin <= 32).  work: DEVICE scratch of at least
-   ep_tv_conv3x3_backward_work bytes, owned by the caller.  The weight gradient
+   dx (n x cin x h x w; needs cin <= 32).  dx may lie on any of the inputs (dx = dy is
+   the gradient in place), dweight and dbias on x, y or dy.  work: DEVICE scratch of at
+   least ep_tv_conv3x3_backward_work bytes, owned by the caller.  The weight gradient
    is summed per tile and then over tiles, by compensated sums in a fixed order
    (deterministic). */
 ep_tv_status ep_tv_conv3x3_backward(int32_t n, int32_t cin, int32_t cout, int32_t height,

@@ -471,6 +471,12 @@ bool dw_smem_ok() {
   return done[dev];
 }
 
+// Whether the ranges a .. a + na - 1 and b .. b + nb - 1 share memory.
+bool overlap(const float* a, long long na, const float* b, long long nb) {
+  const uintptr_t a0 = (uintptr_t)a, b0 = (uintptr_t)b;
+  return a0 < b0 + sizeof(float) * (size_t)nb && b0 < a0 + sizeof(float) * (size_t)na;
+}
+
 // Output groups and tile shape by the number of output channels: 8 or 16 outputs per thread
 // with tiles of 16 rows, or two groups of 16 with tiles of 8 (the same 128 threads).
 template <bool kGrad>
@@ -523,13 +529,28 @@ ep_tv_status ep_tv_conv3x3_backward(int32_t n, int32_t cin, int32_t cout, int32_
   const long long n_tiles = tiles(height, width) * n;
   const int nblk = dw_blocks(n_tiles);
   const long long stride = (long long)cout * cin * 9 + cout;
-  float* g = dx && y ? (float*)(part + nblk * stride) : nullptr;  // the masked gradient, for dx
+  // dx is formed last, after dweight and dbias are written and while other blocks write dx:
+  // from a copy of the (masked) gradient, unless it is dy itself and no output lies on it,
+  // and from a copy of the weights where dx lies on them
+  const long long n_dy = (long long)n * cout * height * width, n_dx = (long long)n * cin * height * width;
+  const long long n_w = (long long)cout * cin * 9;
+  const bool copy_g =
+      dx && (y || overlap(dx, n_dx, dy, n_dy) || overlap(dweight, n_w, dy, n_dy) || overlap(dbias, cout, dy, n_dy));
+  float* g = copy_g ? (float*)(part + nblk * stride) : nullptr;
   if (!dw_smem_ok()) return EP_TV_ERR_CUDA;
   conv3x3_dw_kernel<<<dim3(nblk, (cin + 31) / 32), kDwThreads, kDwSmem, s>>>(
       cin, cout, height, width, (width + kT - 1) / kT, n_tiles, x, dy, y, g, part);
   reduce_parts_kernel<<<(unsigned)((stride + 31) / 32), 256, 0, s>>>(part, stride, nblk, dweight, dbias,
                                                                      (long long)cout * cin * 9);
-  if (dx) launch_conv<true>(n, cout, cin, height, width, g ? g : dy, weight, nullptr, 0, dx, s);
+  if (!dx) return launch_status();
+  const float* w = weight;
+  if (overlap(dx, n_dx, weight, n_w)) {
+    // the partial gradients have been added up: their place holds the weights
+    if (cudaMemcpyAsync(part, weight, sizeof(float) * n_w, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+      return EP_TV_ERR_CUDA;
+    w = (const float*)part;
+  }
+  launch_conv<true>(n, cout, cin, height, width, g ? g : dy, w, nullptr, 0, dx, s);
   return launch_status();
 }
 

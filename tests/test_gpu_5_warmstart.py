@@ -216,3 +216,52 @@ def test_conv_tile_edges(n, cin, cout, h, w, relu):
     _close(db.cpu().numpy(), dbr)
     if dx is not None:
         _close(dx.cpu().numpy(), dxr)
+
+
+@pytest.mark.parametrize("relu", [0, 1])
+@pytest.mark.parametrize("h,w", [(40, 64), (17, 33)])
+@pytest.mark.parametrize("lies_on", ["dy", "dy_shifted", "x", "weight", "dw_on_dy", "db_on_dy"])
+def test_conv_backward_outputs_on_inputs(lies_on, h, w, relu):
+    """dx on dy (the gradient in place, whole and shifted by part of a plane), on x and on the
+    weights, and dweight or dbias on dy: the bits of the same call with separate buffers.
+    Several tiles of each image border on one another, with and without whole float4 rows."""
+    torch = cuda()
+    from paper_2110_01585_gb300 import _lib
+    lib = _lib.load()
+    n, c = 3, 8
+    rng = np.random.default_rng(h + relu)
+    x, dy = (_t(torch, rng.standard_normal((n, c, h, w))) for _ in range(2))
+    wt = _t(torch, rng.standard_normal((c, c, 3, 3)))
+    y = _t(torch, rng.standard_normal((n, c, h, w))) if relu else None
+    work = torch.empty(lib.ep_tv_conv3x3_backward_work(n, c, c, h, w), dtype=torch.uint8, device="cuda")
+    s = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    P = lambda t: ctypes.c_void_p(t.data_ptr()) if t is not None else ctypes.c_void_p()
+
+    def run(x, wt, dy, dx, dw, db):
+        assert lib.ep_tv_conv3x3_backward(n, c, c, h, w, P(x), P(wt), P(y), P(dy), P(dx), P(dw), P(db), P(work),
+                                          ctypes.c_size_t(work.numel()), s) == 0
+        return [t.clone() for t in (dx, dw, db)]
+
+    new = lambda: (torch.empty_like(x), torch.empty_like(wt), torch.empty(c, device="cuda"))
+    ref = run(x, wt, dy, *new())
+    dx, dw, db = new()
+    buf = torch.zeros(x.numel() + h * w, device="cuda")
+    head = buf[:x.numel()].view_as(x)
+    if lies_on == "dy":
+        dx = dy = dy.clone()
+    elif lies_on == "dy_shifted":
+        dy, dx = head.copy_(dy), buf[h * w:].view_as(x)
+    elif lies_on == "x":
+        dx = x = x.clone()
+    elif lies_on == "weight":
+        dx = head
+        wt = buf[5 * h * w:5 * h * w + wt.numel()].view_as(wt).copy_(wt)
+    elif lies_on == "dw_on_dy":
+        dy = dy.clone()
+        dw = dy.view(-1)[h * w:h * w + wt.numel()].view_as(wt)
+    else:
+        dy = dy.clone()
+        db = dy.view(-1)[:c]
+    got = run(x, wt, dy, dx, dw, db)
+    for a, b in zip(got, ref):
+        assert torch.equal(a, b)

@@ -1777,6 +1777,13 @@ struct FftDesc {
   int max_iter;
 };
 
+// The iteration that just ended was the pass's last (graph replays; loop_step has decided):
+// system j stops, also where only the budget is spent.  By the last block of its pair in
+// the inverse row pass, when every other block of the pair has read the flag.
+__device__ __forceinline__ void stop_when_spent(const FftDesc& f, int j) {
+  if (f.loop && !f.loop->live) f.scal_w[4 * j] = 0.f;
+}
+
 // The last block of a pair's inverse row pass sums the r.z partials of its two
 // systems and sets, for each system still active, beta = r.z(new) / r.z(old)
 // (0 in the first application of a refinement pass) and r.z = r.z(new).
@@ -1789,6 +1796,7 @@ __device__ __forceinline__ void rz_tail(const FftDesc& f, int pair, const double
   if ((threadIdx.x & 31) == 0 && f.act[4 * j] != 0.f) {
     f.scal_w[4 * j + 1] = f.first ? 0.f : (float)(rz / f.rzs[j]);
     f.rzs[j] = rz;
+    stop_when_spent(f, j);
   }
 }
 
@@ -1824,6 +1832,7 @@ __device__ __forceinline__ void pw_tail(const FftDesc& f, int pair, const double
   f.scal_w[4 * j + 2] = (float)alpha;
   f.alphas[j] = alpha;
   f.rzs[j] = rz;
+  stop_when_spent(f, j);
 }
 
 // Both systems of a pair have stopped in this CG iteration: their z is not used.
@@ -1837,21 +1846,18 @@ __device__ __forceinline__ bool pair_idle(const FftDesc& f, int pair) {
 // which every iteration launches): count the iteration, and go on while a system is
 // still active and the iteration budget lasts, as iter_kernel does.  A body of the loop
 // holds kUnroll iterations; those launched after the last one find every system stopped
-// (with the budget spent, by the flags cleared here) and are not counted.
+// and are not counted.  With the budget spent, the flags are cleared by the inverse row
+// pass (stop_when_spent): the column pass's other blocks are reading them here.
 __device__ __forceinline__ void loop_step(const FftDesc& f) {
   if (!f.loop || blockIdx.x != 0 || blockIdx.y != 0 || threadIdx.x >= 32 || !f.loop->live) return;
   int cnt = 0;
   for (int j = threadIdx.x; j < f.R; j += 32) cnt += f.act[4 * j] != 0.f;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, off);
-  const bool spent = f.loop->total + 1 >= f.max_iter;
-  __syncwarp();
-  if (spent)
-    for (int j = threadIdx.x; j < f.R; j += 32) f.scal_w[4 * j] = 0.f;
   if (threadIdx.x == 0) {
     f.loop->it += 1;
     f.loop->total += 1;
-    const int go = cnt > 0 && !spent;
+    const int go = cnt > 0 && f.loop->total < f.max_iter;
     f.loop->live = go;
     cudaGraphSetConditional(f.h_inner, go);
   }

@@ -128,3 +128,33 @@ def test_deconv_pass_forms_graph_equals_host_driven_loop(h, w, S, max_iter):
             assert g.stats()["cg_iters"] == max_iter and host.stats()["cg_iters"] == max_iter
         else:
             assert rep["relres_mean"] <= 1e-9 and rep["relres_probe_max"] <= 1e-6
+
+
+@pytest.mark.parametrize("h,w,kernel,S", [(64, 128, 5, 4),   # three kernels per iteration
+                                          (38, 68, 9, 5),    # stencil, warp transforms
+                                          (24, 520, 5, 2),   # 1024-point rows, columns in shared memory
+                                          (20, 24, 5, 3),    # shared-memory transforms, separate update
+                                          (64, 64, 5, 3)])   # a pass as one kernel
+@pytest.mark.parametrize("budget", [1, 2, 3, 4, 5, 9])
+def test_spent_iteration_budget_graph_equals_host_driven_loop(h, w, kernel, S, budget):
+    """The iteration budget runs out at every place of the loop body's four iterations, with
+    several pairs of systems: every iteration up to the last is whole in the graph, and those
+    launched after it change nothing.  Later sweeps start from what it left."""
+    from paper_2110_01585_gb300 import OP_CONV_PERIODIC
+    torch = cuda()
+    stream = torch.cuda.Stream()
+    p = syn.deconv_problem(h, w, kernel=syn.uniform_kernel(kernel), bsnr_db=30.0, beta0=2.0, seed=h + w,
+                           grf_length=8.0)
+    y = torch.as_tensor(p.y.astype(np.float32), device="cuda")
+    kw = dict(op=OP_CONV_PERIODIC, kernel=p.kernel, rbmc_samples=S, stream=stream, cg_max_iter=budget)
+    with EPTV(y, p.xi, p.beta, **kw) as g, EPTV(y, p.xi, p.beta, **kw) as host:
+        host.trace(True)
+        for _ in range(2):
+            g.sweep(1)
+            host.sweep(1)
+            got = [[t.view(torch.int32) for t in ep.sites() + ep.posterior()] for ep in (g, host)]
+            torch.cuda.synchronize()
+            assert all(torch.equal(a, b) for a, b in zip(*got))
+            assert g.stats()["cg_iters"] == host.stats()["cg_iters"] == budget
+        assert g.status() == host.status() != 0
+        assert g.graph_sweeps() == 2 and host.graph_sweeps() == 0

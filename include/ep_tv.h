@@ -414,7 +414,7 @@ size_t ep_tv_conv3x3_backward_work(int32_t n, int32_t cin, int32_t cout, int32_t
    dx (n x cin x h x w; needs cin <= 32).  dx may lie on any of the inputs (dx = dy is
    the gradient in place), dweight and dbias on x, y or dy.  work: DEVICE scratch of at
    least ep_tv_conv3x3_backward_work bytes, owned by the caller.  The weight gradient
-   is summed per tile and then over tiles, by compensated sums in a fixed order
+   is summed per tile in FP32 and then over tiles in FP64, in a fixed order
    (deterministic). */
 ep_tv_status ep_tv_conv3x3_backward(int32_t n, int32_t cin, int32_t cout, int32_t height,
                                     int32_t width, const float* x, const float* weight,

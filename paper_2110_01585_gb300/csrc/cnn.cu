@@ -207,10 +207,11 @@ __global__ void __launch_bounds__(128, 4) conv3x3_kernel(int cin, int cout, int 
 // pixels of a tile's row at a time share the inputs of their taps, so they cost seven loads
 // and 36 packed FMAs.  The next tile's x, dy and y arrive by asynchronous copies
 // meanwhile; dy and y are turned into the masked gradient, pixel-major, between tiles.
-// A tile's sums are FP32, as is their compensated sum over the block's tiles (Knuth's
-// TwoSum: hi + lo), which is stored in FP64.
+// A tile's sums are FP32; their sum over the block's tiles is FP64, as is the reduction over
+// blocks (a pair of FP32 sums with TwoSum holds fewer bits and makes NaN of an infinite
+// tile sum; it took 10 us less, the FP64 additions being two per clock and SM).
 // Measured at 32 -> 32 channels, 8 images of 128^2: 145 us with one output and channel per
-// thread and a pass for the mask (23 us) before, 84 here; the reduction 78 -> 6.5 us.
+// thread and a pass for the mask (23 us) before, 94 here; the reduction 78 -> 6.5 us.
 constexpr int kT = 16;        // tile side (pixels)
 constexpr int kDwThreads = 512;
 constexpr int kDwPitch = kT + 8;  // columns x0 - 4 .. x0 + 19
@@ -277,14 +278,9 @@ __global__ void __launch_bounds__(kDwThreads) conv3x3_dw_kernel(int cin, int cou
     }
     cp_commit();
   };
-  float2 hi[9], lo[9], bhi = make_float2(0.f, 0.f), blo = make_float2(0.f, 0.f);
+  double2 sum[9], bsum = make_double2(0.0, 0.0);
 #pragma unroll
-  for (int k = 0; k < 9; ++k) hi[k] = lo[k] = make_float2(0.f, 0.f);
-  auto two_sum = [](float& s, float& e, float v) {
-    const float t = __fadd_rn(s, v), bb = __fsub_rn(t, s);
-    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(v, bb)));
-    s = t;
-  };
+  for (int k = 0; k < 9; ++k) sum[k] = make_double2(0.0, 0.0);
   int buf = 0;
   if (blockIdx.x < n_tiles) stage(blockIdx.x, 0);
   for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, buf ^= 1) {
@@ -346,13 +342,21 @@ __global__ void __launch_bounds__(kDwThreads) conv3x3_dw_kernel(int cin, int cou
         }
       }
     }
+    if (tile == blockIdx.x) {
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      two_sum(hi[k].x, lo[k].x, acc[k].x);
-      two_sum(hi[k].y, lo[k].y, acc[k].y);
+      for (int k = 0; k < 9; ++k) sum[k] = make_double2((double)acc[k].x, (double)acc[k].y);
+      bsum = make_double2((double)bacc.x, (double)bacc.y);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 9; ++k) {
+        sum[k].x += (double)acc[k].x;
+        sum[k].y += (double)acc[k].y;
+      }
+      if (c == 0) {
+        bsum.x += (double)bacc.x;
+        bsum.y += (double)bacc.y;
+      }
     }
-    two_sum(bhi.x, blo.x, bacc.x);
-    two_sum(bhi.y, blo.y, bacc.y);
   }
   const long long stride = (long long)cout * cin * 9 + cout;
   double* out = part + blockIdx.x * stride;
@@ -362,12 +366,9 @@ __global__ void __launch_bounds__(kDwThreads) conv3x3_dw_kernel(int cin, int cou
     if (o >= cout) break;
     if (c < cc) {
 #pragma unroll
-      for (int k = 0; k < 9; ++k)
-        out[((long long)o * cin + c0 + c) * 9 + k] =
-            e ? (double)hi[k].y + (double)lo[k].y : (double)hi[k].x + (double)lo[k].x;
+      for (int k = 0; k < 9; ++k) out[((long long)o * cin + c0 + c) * 9 + k] = e ? sum[k].y : sum[k].x;
     }
-    if (c == 0 && c0 == 0)
-      out[(long long)cout * cin * 9 + o] = e ? (double)bhi.y + (double)blo.y : (double)bhi.x + (double)blo.x;
+    if (c == 0 && c0 == 0) out[(long long)cout * cin * 9 + o] = e ? bsum.y : bsum.x;
   }
 }
 

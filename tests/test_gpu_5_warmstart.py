@@ -265,3 +265,57 @@ def test_conv_backward_outputs_on_inputs(lies_on, h, w, relu):
     got = run(x, wt, dy, dx, dw, db)
     for a, b in zip(got, ref):
         assert torch.equal(a, b)
+
+
+def _weight_gradient(torch, x, dy):
+    from paper_2110_01585_gb300 import _lib
+    lib = _lib.load()
+    (n, cin, h, w), cout = x.shape, dy.shape[1]
+    xd, dyd = _t(torch, x), _t(torch, dy)
+    dw, db = torch.empty((cout, cin, 3, 3), device="cuda"), torch.empty(cout, device="cuda")
+    work = torch.empty(lib.ep_tv_conv3x3_backward_work(n, cin, cout, h, w), dtype=torch.uint8, device="cuda")
+    P = lambda t: ctypes.c_void_p(t.data_ptr() if t is not None else None)
+    assert lib.ep_tv_conv3x3_backward(n, cin, cout, h, w, P(xd), P(dw), P(None), P(dyd), P(None), P(dw), P(db), P(work),
+                                      ctypes.c_size_t(work.numel()),
+                                      ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+    return dw.cpu().numpy(), db.cpu().numpy()
+
+
+def test_weight_gradient_sums_tiles_in_fp64():
+    """One 16 x 16 tile per image; a value in every 152nd image, so that however the tiles are
+    spread over 152 blocks or fewer, the sum over tiles meets 2^50, 2^24, 1, -2^50, -2^24: 1 in FP64 in
+    any order, 0 in FP32 or in a pair of FP32 numbers that drops what neither holds."""
+    torch = cuda()
+    n = 4 * 152 + 1
+    x, dy = np.zeros((n, 2, 16, 16), np.float32), np.zeros((n, 2, 16, 16), np.float32)
+    vals = [2.0 ** 50, 2.0 ** 24, 1.0, -2.0 ** 50, -2.0 ** 24]
+    for i, v in enumerate(vals):
+        x[152 * i, 1, 7, 7], dy[152 * i, 0, 7, 7] = 1.0, v
+    dw, db = _weight_gradient(torch, x, dy)
+    ref = np.zeros((2, 2, 3, 3))
+    ref[0, 1, 1, 1] = 1.0
+    np.testing.assert_array_equal(dw, ref)
+    np.testing.assert_array_equal(db, [1.0, 0.0])
+
+
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_weight_gradient_keeps_infinities(sign):
+    """A product past FP32's range (or an infinite input) makes the sums it enters +-Inf, not
+    NaN, over several tiles of a block; Inf and -Inf, and zero times Inf, are NaN: as FP32
+    sums over each tile (one per image here) and FP64 sums over tiles give it."""
+    torch = cuda()
+    x, dy = np.zeros((4 * 152, 3, 16, 16), np.float32), np.zeros((4 * 152, 2, 16, 16), np.float32)
+    dy[:, :, 8, 8] = 2.0
+    x[0, 0, 8, 8] = sign * 3e38
+    x[152, 1, 8, 8] = sign * np.inf
+    x[0, 2, 8, 8], x[152, 2, 8, 8] = np.inf, -np.inf
+    dy[152, 1, 8, 8] = sign * np.inf
+    ref = np.zeros((2, 3, 3, 3), np.float32)
+    with np.errstate(over="ignore", invalid="ignore"):
+        for o, c, a, e in np.ndindex(*ref.shape):
+            shifted = np.roll(x[:, c], (1 - a, 1 - e), axis=(1, 2))
+            ref[o, c, a, e] = (dy[:, o] * shifted).sum(axis=(1, 2)).astype(np.float64).sum()
+    assert np.isinf(ref[:, :, 1, 1]).sum() >= 3 and np.isnan(ref[0, 2, 1, 1])
+    dw, db = _weight_gradient(torch, x, dy)
+    np.testing.assert_array_equal(dw, ref)
+    np.testing.assert_array_equal(db, [2.0 * 4 * 152, sign * np.inf])

@@ -396,8 +396,8 @@ __global__ void aty_kernel(const float* A, const float* y, int M, int N, float* 
 //   - the owned rows of the trailing update; the next diagonal block's written to every CTA;
 //   - at the end the owned columns of Z by block forward substitution.
 // Measured for 64 rows: 287 us as a one-block Cholesky with square root and division
-// per pivot and a one-thread-per-column inverse, 54 us in this form; 128 rows take 139 us,
-// against 98 for two halves and about 140 for the four products between them.
+// per pivot and a one-thread-per-column inverse, 59 us in this form; 128 rows take 147 us,
+// against 119 for two halves and about 140 for the four products between them.
 constexpr int kBlk = 128;
 constexpr int kBlkCtas = 8;
 constexpr int kBlkThreads = 256;
@@ -445,7 +445,7 @@ __global__ void __cluster_dims__(kBlkCtas, 1, 1) __launch_bounds__(kBlkThreads)
         if (i == j) piv = d;
         if ((tid >> 5) * 2 + 1 > j) {  // warps whose rows are all done have nothing to update
           const double t = cij * row[k];
-          const double r = recip_f64(d);
+          const double r = 1.0 / d;
           if (i > j) a = k == j ? -cij * r : fma(-t, r, a);
         }
       }

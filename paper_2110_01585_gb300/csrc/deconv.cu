@@ -2641,7 +2641,7 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_update_rows_fwd_kerne
   if (w < 2 && (w == 0 ? act0 : act1)) {
     const int j = j0 + w;
     const double pqs = group_sum(a.part_pq + (long long)j * a.nb, a.nb);
-    if (l == 0) alpha_s[w] = (float)(a.rzs[j] * recip_f64(pqs));
+    if (l == 0) alpha_s[w] = (float)(a.rzs[j] / pqs);
   }
   __syncthreads();
   const long long N = (long long)f.H * f.W;
@@ -3187,7 +3187,7 @@ __global__ void __cluster_dims__(kSolveCtas, 1, 1) __launch_bounds__(32 * solve_
       const double delta = gamma + __shfl_sync(0xffffffffu, x, 2 * (l & 1) + 1);
       double beta = 0.0, den = delta;
       if (!first) {
-        beta = gamma * recip_f64(gamma_old);
+        beta = gamma / gamma_old;
         den = delta - beta * beta * den_old;  // beta gamma / alpha(old), alpha(old) = gamma(old) / den(old)
         if (!(den > 0.0)) {
           beta = 0.0;
@@ -3196,7 +3196,7 @@ __global__ void __cluster_dims__(kSolveCtas, 1, 1) __launch_bounds__(32 * solve_
       }
       if (l < 2) {
         coef[l][0] = (float)beta;
-        coef[l][1] = (float)(gamma * recip_f64(den));
+        coef[l][1] = (float)(gamma / den);
       }
       gamma_old = gamma;
       den_old = den;
@@ -3421,7 +3421,7 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_update_rows_fwd_ke
   if (w < 2 && (w == 0 ? act0 : act1)) {
     const int j = j0 + w;
     const double pqs = group_sum(a.part_pq + (long long)j * a.nb, a.nb);
-    if (l == 0) alpha_s[w] = (float)(a.rzs[j] * recip_f64(pqs));
+    if (l == 0) alpha_s[w] = (float)(a.rzs[j] / pqs);
   }
   __syncthreads();
   const long long N = (long long)f.H * f.W;

@@ -171,14 +171,4 @@ void launch_site0_noise(float* tau0, float* nu0, const float* y, const float* xi
 void launch_posterior(const float* tau0, const float* nu0, const float* tp, const float* np,
                       long long n, float* mean, float* var, cudaStream_t s);
 
-// 1 / d to FP64 rounding from the hardware's approximation, by one third-order
-// (Householder) step: with e = 1 - d r0, 1 / d = r0 (1 + e + e^2 + O(e^3)), and e is below
-// 2^-19.  Three dependent FP64 operations.
-__device__ __forceinline__ double recip_f64(double d) {
-  double r0;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(d));
-  const double e = fma(-d, r0, 1.0);
-  return fma(r0, fma(e, e, e), r0);
-}
-
 }  // namespace eptv

@@ -52,7 +52,8 @@ typedef enum {
   EP_TV_ERR_NOMEM = 2,        /* device allocation failed */
   EP_TV_ERR_CUDA = 3,         /* a CUDA runtime call failed */
   EP_TV_ERR_NONFINITE = 4,    /* a site value became NaN or infinite */
-  EP_TV_ERR_CG_NOCONV = 5,    /* the likelihood-site solver hit its iteration cap */
+  EP_TV_ERR_CG_NOCONV = 5,    /* the likelihood-site solver hit its iteration cap before
+                                 the targets of cg_rtol */
   EP_TV_ERR_TIMEOUT = 6,      /* a bounded device-side wait gave up */
   EP_TV_ERR_STATE = 7,        /* context unusable after a latched device error */
   EP_TV_ERR_UNSUPPORTED = 8   /* valid request this build does not implement */
@@ -116,8 +117,9 @@ typedef struct {
   int32_t cg_max_iter;   /* CONV_PERIODIC: cap on the conjugate-gradient iterations of one
                             likelihood-site update (all refinement passes together) */
   double cg_rtol;        /* CONV_PERIODIC: target of the true relative residual ||b - Q x|| /
-                            ||b|| of the mean solve (probe solves: max(cg_rtol, 1e-6)); a
-                            quarter of both for images whose sides are not powers of two.
+                            ||b|| of the mean solve (probe solves: max(cg_rtol, 1e-6)).
+                            Images whose sides are not powers of two are solved to a
+                            quarter of both, as far as the cap on the iterations lets it.
                             The residual is recomputed in float-float arithmetic between FP32
                             CG passes; a solve also stops when a pass no longer halves a
                             residual already below 1e-6 (the evaluation floor).  Default 1e-9. */

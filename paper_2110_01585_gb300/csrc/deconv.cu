@@ -1091,8 +1091,10 @@ struct PassArgs {
 };
 
 // After a true residual and its thresholds: start another pass, or stop (converged, or
-// out of passes or iterations), as the host loop does.
-__device__ __forceinline__ void start_pass(const PassArgs& p, int active) {
+// out of passes or iterations), as the host loop does.  missed: systems beyond the
+// caller's target, which may be four times the one aimed at; with none of them a solve
+// that runs out has converged too.
+__device__ __forceinline__ void start_pass(const PassArgs& p, int active, int missed) {
   LoopState* ls = p.ls;
   ls->total += ls->pass_its;
   ls->pass_its = 0;
@@ -1103,25 +1105,28 @@ __device__ __forceinline__ void start_pass(const PassArgs& p, int active) {
     go = 1;
     ls->it = 0;
     ls->outer += 1;
+  } else {
+    ls->converged = missed == 0;
   }
   ls->live = (int)go;
   cudaGraphSetConditional(p.h_outer, go);
   if (p.inner) cudaGraphSetConditional(p.h_inner, go);
 }
 
-// Per system after a true residual: done if r.r <= rtol^2 b.b (threshold +inf),
+// Per system after a true residual: done if r.r <= rtol^2 b.b (threshold +inf; missed, the
+// count behind *active, if r.r is beyond slack^2 times that, the caller's target),
 // otherwise the inner loop runs until r.r <= max(eta^2 r.r, (rtol/2)^2 b.b).
 // Also starts the pass's CG scalars: active flag (and act0) = not done, beta = 0,
 // and for Jacobi r.z from the residual kernel's r.Minv.r partials.
 __global__ void thresholds_kernel(const double* part_rr, const double* part_bb,
                                   const double* part_rz, int fft, int R, int nb,
-                                  double rtol2_mean, double rtol2_probe, double eta2, double* thr,
+                                  double rtol2_mean, double rtol2_probe, double slack2, double eta2, double* thr,
                                   double* relres, double* prev_rr, double* rr0, int first_arg,
                                   int* active, float* scal, int* act0, double* rzs, PassArgs pass) {
   // the first true residual of this update (graph replays: passes started = 0)
   const int first = pass.ls ? (pass.ls->outer == 0) : first_arg;
-  __shared__ int cnt;
-  if (threadIdx.x == 0) cnt = 0;
+  __shared__ int cnt, missed;
+  if (threadIdx.x == 0) cnt = missed = 0;
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int j = warp; j < R; j += blockDim.x / 32) {
@@ -1155,6 +1160,7 @@ __global__ void thresholds_kernel(const double* part_rr, const double* part_bb,
       scal[4 * j + 3] = -1.f;  // its iteration (none yet)
       act0[j] = done ? 0 : 1;
       if (!done) atomicAdd(&cnt, 1);
+      if (!done && !(rr <= slack2 * rtol2 * bb)) atomicAdd(&missed, 1);
     }
     if (!fft) {
       double rz = 0;
@@ -1166,8 +1172,9 @@ __global__ void thresholds_kernel(const double* part_rr, const double* part_bb,
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    *active = cnt;
-    if (pass.ls) start_pass(pass, cnt);
+    active[0] = cnt;
+    active[1] = missed;
+    if (pass.ls) start_pass(pass, cnt, missed);
   }
 }
 
@@ -3979,6 +3986,7 @@ struct LikelihoodState {
   float* d_hf = nullptr;    // forward-blur taps FP32
   double rtol2_true = 0.0;  // target of the true relative residual of the mean solve, squared
   double rtol2_probe = 0.0; // the same for the probe solves
+  double slack2 = 1.0;      // the caller's targets over these, squared
   int max_outer = 24;
   float* Rr = nullptr;
   float* P = nullptr;
@@ -4000,7 +4008,7 @@ struct LikelihoodState {
   double* dbar = nullptr;
   int prep_blocks = 0;
   size_t smem_rows = 0, smem_cols = 0;
-  int* d_active = nullptr;
+  int* d_active = nullptr;  // systems still active, and those beyond the caller's target
   int* h_active = nullptr;  // pinned, 2 slots
   cudaEvent_t ev[2] = {nullptr, nullptr};
   int nb = 0;
@@ -4527,6 +4535,7 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
   if (L->fft && ((c.H & (c.H - 1)) || (c.W & (c.W - 1)))) {
     L->rtol2_true *= 0.0625;
     L->rtol2_probe *= 0.0625;
+    L->slack2 = 16.0;
   }
   L->nbz = L->nb;
   if (L->fft) {
@@ -4599,7 +4608,7 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
               cudaMalloc(&L->hth, 2 * sizeof(float) * L->fd.HP * L->fd.WP) == cudaSuccess &&
               cudaMalloc(&L->tw512, sizeof(float2) * kTwCount) == cudaSuccess &&
               cudaMalloc(&L->window, sizeof(float) * (L->fd.HP + L->fd.WP)) == cudaSuccess)) &&
-            cudaMalloc(&L->d_active, sizeof(int)) == cudaSuccess &&
+            cudaMalloc(&L->d_active, 2 * sizeof(int)) == cudaSuccess &&
             cudaMalloc(&L->d_relres, sizeof(double) * L->R) == cudaSuccess &&
             cudaMalloc(&L->d_prev_rr, sizeof(double) * L->R) == cudaSuccess &&
             cudaMalloc(&L->d_rr0, sizeof(double) * L->R) == cudaSuccess &&
@@ -4849,7 +4858,7 @@ bool build_update_graph(LikelihoodState* L, float* tau, float* nu, const float* 
     launch_residual(L, a, all, s);
     const PassArgs pass{L->d_loop, L->max_outer, L->max_iter, L->solve ? 0 : 1, h_outer, h_inner};
     thresholds_kernel<<<1, 1024, 0, s>>>(a.part_rr, a.part_bb, a.part_rz, a.fft, L->R, L->nb,
-                                         L->rtol2_true, L->rtol2_probe, kEta2, L->thr, L->d_relres,
+                                         L->rtol2_true, L->rtol2_probe, L->slack2, kEta2, L->thr, L->d_relres,
                                          L->d_prev_rr, L->d_rr0, 0, L->d_active, L->d_scal, L->d_act0,
                                          L->d_rzs, pass);
   };
@@ -4956,10 +4965,10 @@ ep_tv_status likelihood_update(LikelihoodState* L, float* tau, float* nu, const 
     launch_residual(L, a, outer == 0, s);
     tr->end(s, (double)(outer == 0 ? L->R : prev_active) * N);
     thresholds_kernel<<<1, 1024, 0, s>>>(a.part_rr, a.part_bb, a.part_rz, a.fft, L->R, L->nb,
-                                         L->rtol2_true, L->rtol2_probe, eta2, L->thr, L->d_relres,
+                                         L->rtol2_true, L->rtol2_probe, L->slack2, eta2, L->thr, L->d_relres,
                                          L->d_prev_rr, L->d_rr0, outer == 0, L->d_active, L->d_scal,
                                          L->d_act0, L->d_rzs, PassArgs{});
-    if (cudaMemcpyAsync(L->h_active, L->d_active, sizeof(int), cudaMemcpyDeviceToHost, s) !=
+    if (cudaMemcpyAsync(L->h_active, L->d_active, 2 * sizeof(int), cudaMemcpyDeviceToHost, s) !=
             cudaSuccess ||
         cudaMemcpyAsync(L->h_relres, L->d_relres, sizeof(double) * L->R, cudaMemcpyDeviceToHost,
                         s) != cudaSuccess ||
@@ -4979,7 +4988,10 @@ ep_tv_status likelihood_update(LikelihoodState* L, float* tau, float* nu, const 
       converged = true;
       break;
     }
-    if (outer >= L->max_outer || total >= L->max_iter) break;
+    if (outer >= L->max_outer || total >= L->max_iter) {
+      converged = L->h_active[1] == 0;
+      break;
+    }
     const int started = L->h_active[0];  // systems that iterate in this pass
     prev_active = started;
     if (L->solve) {

@@ -378,3 +378,27 @@ def test_preconditioner_iterations_are_those_of_the_windowed_extension(h, w, per
         ep.close()
     ref = _emulated_iterations(p, pr, tau[1:].sum(axis=0), nu[1:].sum(axis=0), 1e-4, torus)
     assert abs(its - ref) <= 3 + 0.1 * ref, (its, ref)
+
+
+@pytest.mark.parametrize("h,w", [(38, 68), (96, 96), (62, 62)])  # stencil, pointwise, paired stencil
+@pytest.mark.parametrize("traced", [False, True])                # the graph, and the host-driven loop
+def test_status_is_that_of_the_callers_target(h, w, traced):
+    """Sides that are not powers of two aim at a quarter of cg_rtol; an iteration cap that ends
+    a solve between the two raises no error, one that ends it before cg_rtol does."""
+    torch = cuda()
+    p = syn.deconv_problem(h, w, kernel=syn.uniform_kernel(5), bsnr_db=30.0, beta0=2.0, seed=h + w,
+                           grf_length=8.0)
+    y = torch.as_tensor(p.y.astype(np.float32), device="cuda")
+    rtol, seen = 1e-3, set()
+    for cap in range(1, 200):
+        with EPTV(y, p.xi, p.beta, op=OP_CONV_PERIODIC, kernel=p.kernel, rbmc_samples=2, cg_rtol=rtol,
+                  cg_max_iter=cap, stream=torch.cuda.Stream()) as ep:
+            ep.trace(traced)
+            ep.sweep(1)
+            st, rep = ep.status(), ep.solver_report()
+        worst = max(rep["relres_mean"], rep["relres_probe_max"])
+        assert st == (5 if worst > rtol else 0), (cap, worst, st)
+        seen.add("beyond" if worst > rtol else "between" if worst > 0.25 * rtol else "met")
+        if worst <= 0.25 * rtol:
+            break
+    assert seen == {"beyond", "between", "met"}

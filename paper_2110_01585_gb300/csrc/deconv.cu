@@ -2053,13 +2053,15 @@ __global__ void __launch_bounds__(kFftThreads, 4) fft_rows_fwd_kernel(FftDesc f,
   const float* r0p = Rr + (long long)j0 * N;
   const float* r1p = Rr + (long long)j1 * N;
   const bool two = j1 < f.R;
+  const bool fills = f.W == f.WP;  // neither copies nor a window
   stage_loads(s, f.rpb * f.WP, [&](int idx) {
     const int rr = idx / f.WP, cc = idx - rr * f.WP;
-    const int row = row0 + rr, src = margin(cc, f.W, f.WP);
+    const int row = row0 + rr, src = fills ? cc : margin(cc, f.W, f.WP);
     float2 v = make_float2(0.f, 0.f);
     if (row < f.H && src >= 0) {
       const long long p = (long long)row * f.W + src;
-      v = cscale(make_float2(r0p[p], two ? r1p[p] : 0.f), f.wc[cc]);
+      v = make_float2(r0p[p], two ? r1p[p] : 0.f);
+      if (!fills) v = cscale(v, f.wc[cc]);
     }
     return v;
   });
@@ -2086,8 +2088,10 @@ __global__ void __launch_bounds__(kFftThreads, 4) fft_cols_filter_kernel(FftDesc
   const int c0 = blockIdx.x * f.cw;
   float2* t = f.tmp + (long long)pair * f.H * f.WP;
   make_table(tw, f.HP);
+  const bool fills = f.H == f.HP;
   stage_loads(s, f.HP * f.cw, [&](int idx) {
     const int i = idx / f.cw, c = idx - i * f.cw;
+    if (fills) return t[(long long)i * f.WP + c0 + c];
     const int src = margin(i, f.H, f.HP);
     return src >= 0 ? cscale(t[(long long)src * f.WP + c0 + c], f.wr[i]) : make_float2(0.f, 0.f);
   });
@@ -2104,7 +2108,7 @@ __global__ void __launch_bounds__(kFftThreads, 4) fft_cols_filter_kernel(FftDesc
   for (int idx = threadIdx.x; idx < f.H * f.cw; idx += blockDim.x) {
     const int i = idx / f.cw, c = idx - i * f.cw;
     t[(long long)i * f.WP + c0 + c] =
-        cconj(fold(i, f.H, f.HP, [&](int k) { return cscale(s[k * f.cw + c], f.wr[k]); }));
+        cconj(fills ? s[idx] : fold(i, f.H, f.HP, [&](int k) { return cscale(s[k * f.cw + c], f.wr[k]); }));
   }
 }
 
@@ -2123,6 +2127,7 @@ __global__ void __launch_bounds__(kFftThreads, 4) fft_rows_inv_kernel(FftDesc f,
   const int rows_per = (f.H + f.nbz - 1) / f.nbz;
   const int rbeg = blockIdx.x * rows_per, rend = min(f.H, rbeg + rows_per);
   make_table(tw, f.WP);
+  const bool fills = f.W == f.WP;
   double acc0 = 0.0, acc1 = 0.0;
   const float2* tin = f.tmp + (long long)pair * f.H * f.WP;
   for (int r0 = rbeg; r0 < rend; r0 += f.rpb) {
@@ -2139,7 +2144,9 @@ __global__ void __launch_bounds__(kFftThreads, 4) fft_rows_inv_kernel(FftDesc f,
       const int row = r0 + rr;
       if (row >= rend) break;
       for (int cc = threadIdx.x; cc < f.W; cc += blockDim.x) {
-        const float2 v = cconj(fold(cc, f.W, f.WP, [&](int k) { return cscale(s[rr * f.WP + k], f.wc[k]); }));
+        const float2 v = cconj(fills ? s[rr * f.WP + cc] : fold(cc, f.W, f.WP, [&](int k) {
+          return cscale(s[rr * f.WP + k], f.wc[k]);
+        }));
         const long long p = (long long)row * f.W + cc;
         const float z0 = v.x * scale;
         Z[(long long)j0 * N + p] = z0;
@@ -3384,14 +3391,24 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_rows_fwd_kernel(Ff
   for (int row = blockIdx.x * rpb + w; row < rend; row += kF512Warps) {
     const long long p0 = (long long)row * f.W;
     float2 lo[16], hi[16];
+    if (f.W == 2 * kF) {
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const int c = 32 * q + l, c2 = c + kF;  // W > 512: c is an image column
-      lo[q] = cscale(make_float2(ld_hint(r0p + p0 + c, keep), two ? ld_hint(r1p + p0 + c, keep) : 0.f), f.wc[c]);
-      const int src = margin(c2, f.W, 2 * kF);
-      hi[q] = make_float2(0.f, 0.f);
-      if (src >= 0)
-        hi[q] = cscale(make_float2(ld_hint(r0p + p0 + src, keep), two ? ld_hint(r1p + p0 + src, keep) : 0.f), f.wc[c2]);
+      for (int q = 0; q < 16; ++q) {
+        const float* a = r0p + p0 + 32 * q + l;
+        const float* b = r1p + p0 + 32 * q + l;
+        lo[q] = make_float2(ld_hint(a, keep), two ? ld_hint(b, keep) : 0.f);
+        hi[q] = make_float2(ld_hint(a + kF, keep), two ? ld_hint(b + kF, keep) : 0.f);
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        const int c = 32 * q + l, c2 = c + kF;  // W > 512: c is an image column
+        lo[q] = cscale(make_float2(ld_hint(r0p + p0 + c, keep), two ? ld_hint(r1p + p0 + c, keep) : 0.f), f.wc[c]);
+        const int src = margin(c2, f.W, 2 * kF);
+        hi[q] = make_float2(0.f, 0.f);
+        if (src >= 0)
+          hi[q] = cscale(make_float2(ld_hint(r0p + p0 + src, keep), two ? ld_hint(r1p + p0 + src, keep) : 0.f), f.wc[c2]);
+      }
     }
     fft1024_warp(lo, hi, scratch[w], tw, tw2);
 #pragma unroll
@@ -3549,21 +3566,25 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_cols_filter_kernel
   const int c0 = blockIdx.x * kF512Warps;
   float2* t = f.tmp + (long long)blockIdx.y * f.H * f.WP;
   const int cc = threadIdx.x & 7, ro = threadIdx.x >> 3;  // 32 rows x 8 columns per block step
+  const bool fills = f.H == 2 * kF;  // neither copies nor a window
   const uint64_t keep = l2_policy_keep();
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     float2 x[16];  // half of the thread's tile loads in flight at once
+    if (fills) {
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int i = 32 * (16 * h + u) + ro;
-      const int src = margin(i, f.H, 2 * kF);
-      x[u] = src >= 0 ? ld_hint(t + (long long)src * f.WP + c0 + cc, keep) : make_float2(0.f, 0.f);
+      for (int u = 0; u < 16; ++u) x[u] = ld_hint(t + (long long)(32 * (16 * h + u) + ro) * f.WP + c0 + cc, keep);
+    } else {
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        const int src = margin(32 * (16 * h + u) + ro, f.H, 2 * kF);
+        x[u] = src >= 0 ? ld_hint(t + (long long)src * f.WP + c0 + cc, keep) : make_float2(0.f, 0.f);
+      }
+#pragma unroll
+      for (int u = 0; u < 16; ++u) x[u] = cscale(x[u], f.wr[32 * (16 * h + u) + ro]);
     }
 #pragma unroll
-    for (int u = 0; u < 16; ++u) {
-      const int i = 32 * (16 * h + u) + ro;
-      cols[cc * kXs2 + i] = cscale(x[u], f.wr[i]);
-    }
+    for (int u = 0; u < 16; ++u) cols[cc * kXs2 + 32 * (16 * h + u) + ro] = x[u];
   }
   __syncthreads();
   float2* xs = cols + w * kXs2;
@@ -3601,6 +3622,12 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) fft1024_cols_filter_kernel
     *reinterpret_cast<float4*>(xs + 64 * m + 2 * l) = make_float4(a.x, a.y, b.x, b.y);
   }
   __syncthreads();
+  if (fills) {
+#pragma unroll
+    for (int u = 0; u < 32; ++u)
+      st_hint(t + (long long)(32 * u + ro) * f.WP + c0 + cc, cols[cc * kXs2 + 32 * u + ro], keep);
+    return;
+  }
 #pragma unroll
   for (int u = 0; u < 32; ++u) {
     const int i = 32 * u + ro;

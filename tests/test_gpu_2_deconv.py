@@ -402,3 +402,18 @@ def test_status_is_that_of_the_callers_target(h, w, traced):
         if worst <= 0.25 * rtol:
             break
     assert seen == {"beyond", "between", "met"}
+
+
+@pytest.mark.parametrize("h,w", [(24, 1024), (1024, 24), (24, 2048), (2048, 24), (1300, 20), (20, 1300)])
+def test_deconv_parity_long_transforms(h, w):
+    """1024 points and the shared-memory transforms above, along rows and columns, with the
+    axis filled (no copies, no window) and with a margin; the oracle solves by FP64 CG."""
+    p = syn.deconv_problem(h, w, kernel=syn.uniform_kernel(5), bsnr_db=30.0, beta0=2.0, seed=h + w,
+                           grf_length=8.0)
+    S = 3
+    pr = probes(p, S, 56)
+    mu, var, ep = _gpu(p, 2, S, pr)
+    o = EPOracle("deconv", y32(p), p.xi, p.beta, h, w, kernel=p.kernel, site0="rbmc_cg", probes=pr)
+    o.run(2)
+    assert_parity(mu, var, *o.posterior(), p.y)
+    ep.close()

@@ -119,7 +119,8 @@ typedef struct {
   double cg_rtol;        /* CONV_PERIODIC: target of the true relative residual ||b - Q x|| /
                             ||b|| of the mean solve (probe solves: max(cg_rtol, 1e-6)).
                             Images whose sides are not powers of two are solved to a
-                            quarter of both, as far as the cap on the iterations lets it.
+                            quarter of the former and an eighth of the latter, as far as
+                            the cap on the iterations lets it.
                             The residual is recomputed in float-float arithmetic between FP32
                             CG passes; a solve also stops when a pass no longer halves a
                             residual already below 1e-6 (the evaluation floor).  Default 1e-9. */

@@ -1092,7 +1092,7 @@ struct PassArgs {
 
 // After a true residual and its thresholds: start another pass, or stop (converged, or
 // out of passes or iterations), as the host loop does.  missed: systems beyond the
-// caller's target, which may be four times the one aimed at; with none of them a solve
+// caller's target, which may be several times the one aimed at; with none of them a solve
 // that runs out has converged too.
 __device__ __forceinline__ void start_pass(const PassArgs& p, int active, int missed) {
   LoopState* ls = p.ls;
@@ -1113,14 +1113,17 @@ __device__ __forceinline__ void start_pass(const PassArgs& p, int active, int mi
   if (p.inner) cudaGraphSetConditional(p.h_inner, go);
 }
 
-// Per system after a true residual: done if r.r <= rtol^2 b.b (threshold +inf; missed, the
-// count behind *active, if r.r is beyond slack^2 times that, the caller's target),
+// Target of a probe's relative residual, squared, from the mean's (max(cg_rtol, 1e-6)).
+__host__ __device__ __forceinline__ double probe_target2(double rtol2) { return rtol2 < 1e-12 ? 1e-12 : rtol2; }
+
+// Per system after a true residual: done if r.r <= rtol^2 b.b (threshold +inf),
 // otherwise the inner loop runs until r.r <= max(eta^2 r.r, (rtol/2)^2 b.b).
 // Also starts the pass's CG scalars: active flag (and act0) = not done, beta = 0,
-// and for Jacobi r.z from the residual kernel's r.Minv.r partials.
+// and for Jacobi r.z from the residual kernel's r.Minv.r partials.  active[1]: how many
+// systems are beyond the caller's own targets (asked2 = cg_rtol^2, see likelihood_create).
 __global__ void thresholds_kernel(const double* part_rr, const double* part_bb,
                                   const double* part_rz, int fft, int R, int nb,
-                                  double rtol2_mean, double rtol2_probe, double slack2, double eta2, double* thr,
+                                  double rtol2_mean, double rtol2_probe, double asked2, double eta2, double* thr,
                                   double* relres, double* prev_rr, double* rr0, int first_arg,
                                   int* active, float* scal, int* act0, double* rzs, PassArgs pass) {
   // the first true residual of this update (graph replays: passes started = 0)
@@ -1160,7 +1163,7 @@ __global__ void thresholds_kernel(const double* part_rr, const double* part_bb,
       scal[4 * j + 3] = -1.f;  // its iteration (none yet)
       act0[j] = done ? 0 : 1;
       if (!done) atomicAdd(&cnt, 1);
-      if (!done && !(rr <= slack2 * rtol2 * bb)) atomicAdd(&missed, 1);
+      if (!done && !(rr <= (j == 0 ? asked2 : probe_target2(asked2)) * bb)) atomicAdd(&missed, 1);
     }
     if (!fft) {
       double rz = 0;
@@ -3993,7 +3996,7 @@ struct LikelihoodState {
   ConvDesc c;
   int S = 0, R = 0;
   float inv_xi = 0.f;
-  double rtol2 = 0.0;
+  double rtol2 = 0.0;       // the caller's cg_rtol, squared
   int max_iter = 0;
   unsigned long long seed = 0;
   float damping = 0.5f, min_tau = 1e-8f;
@@ -4013,7 +4016,6 @@ struct LikelihoodState {
   float* d_hf = nullptr;    // forward-blur taps FP32
   double rtol2_true = 0.0;  // target of the true relative residual of the mean solve, squared
   double rtol2_probe = 0.0; // the same for the probe solves
-  double slack2 = 1.0;      // the caller's targets over these, squared
   int max_outer = 24;
   float* Rr = nullptr;
   float* P = nullptr;
@@ -4527,7 +4529,7 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
   // H^T (y' - H z) / xi + (n' - d z) cancels between two terms several times
   // larger, which puts their FP32 floor near 1e-7.  A relative residual of 1e-6
   // moves an RB variance term by about Q_ii / d * 1e-6 relative, below 1e-4.
-  L->rtol2_probe = std::max(L->rtol2, 1e-12);
+  L->rtol2_probe = probe_target2(L->rtol2);
   L->max_iter = cfg.p->cg_max_iter;
   {
     const char* dbg = getenv("EPTV_DEBUG");
@@ -4553,16 +4555,18 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
   L->nb = c.tiles_x * c.tiles_y;
   const auto [HP, WP] = torus(c.H, c.W, kh, kw);
   L->fft = HP <= 8192 && WP <= 8192;
-  // Sides that are not powers of two: a quarter of both targets.  How far a solution is from
-  // the exact one at a given residual depends on the preconditioner: CG under the padded
-  // circulant without the window, which took two to seven times the iterations, ended closer.
-  // Over 17 warm-started restorations (15 x 15 Gaussian blur, sides 64 to 512) the posterior
-  // variances at the targets themselves were 1.4 to 5.6 times as far from an FP64 solution
-  // as under it, at 0.3 of them 0.6 to 1.2 times; a factor of 0.3 costs 10 to 15% time.
+  // Sides that are not powers of two: a quarter of the mean's target and an eighth of the
+  // probes'.  How far a solution is from the exact one at a given residual depends on how CG
+  // got there, and the circulant padded with zeros to a power of two, which these sizes took
+  // before the lengths 3 2^k and the window, needed two to seven times the iterations and ended
+  // closer.  Over 73 restorations (warm-started 15 x 15 blur; 9 x 9 and 5 x 3 blurs at 30 and
+  // 40 dB; sides 56 to 512, half of them filling their torus) the posterior variances were at
+  // most 1.41 times as far from an FP64 solution as then at a quarter of both targets, and
+  // 1.01 times here (0.57 in geometric mean), for 3.6% more time.  Sizes that fill their torus
+  // need it as much: at the targets themselves, 10 to 15% faster, up to 3.3 times (1.65).
   if (L->fft && ((c.H & (c.H - 1)) || (c.W & (c.W - 1)))) {
-    L->rtol2_true *= 0.0625;
-    L->rtol2_probe *= 0.0625;
-    L->slack2 = 16.0;
+    L->rtol2_true *= 1.0 / 16.0;
+    L->rtol2_probe *= 1.0 / 64.0;
   }
   L->nbz = L->nb;
   if (L->fft) {
@@ -4885,7 +4889,7 @@ bool build_update_graph(LikelihoodState* L, float* tau, float* nu, const float* 
     launch_residual(L, a, all, s);
     const PassArgs pass{L->d_loop, L->max_outer, L->max_iter, L->solve ? 0 : 1, h_outer, h_inner};
     thresholds_kernel<<<1, 1024, 0, s>>>(a.part_rr, a.part_bb, a.part_rz, a.fft, L->R, L->nb,
-                                         L->rtol2_true, L->rtol2_probe, L->slack2, kEta2, L->thr, L->d_relres,
+                                         L->rtol2_true, L->rtol2_probe, L->rtol2, kEta2, L->thr, L->d_relres,
                                          L->d_prev_rr, L->d_rr0, 0, L->d_active, L->d_scal, L->d_act0,
                                          L->d_rzs, pass);
   };
@@ -4992,7 +4996,7 @@ ep_tv_status likelihood_update(LikelihoodState* L, float* tau, float* nu, const 
     launch_residual(L, a, outer == 0, s);
     tr->end(s, (double)(outer == 0 ? L->R : prev_active) * N);
     thresholds_kernel<<<1, 1024, 0, s>>>(a.part_rr, a.part_bb, a.part_rz, a.fft, L->R, L->nb,
-                                         L->rtol2_true, L->rtol2_probe, L->slack2, eta2, L->thr, L->d_relres,
+                                         L->rtol2_true, L->rtol2_probe, L->rtol2, eta2, L->thr, L->d_relres,
                                          L->d_prev_rr, L->d_rr0, outer == 0, L->d_active, L->d_scal,
                                          L->d_act0, L->d_rzs, PassArgs{});
     if (cudaMemcpyAsync(L->h_active, L->d_active, 2 * sizeof(int), cudaMemcpyDeviceToHost, s) !=

@@ -435,3 +435,45 @@ def test_probes_of_ragged_sizes_are_solved_to_an_eighth(h, w):
         rep = ep.solver_report()
         assert ep.status() == 0
     assert rep["relres_probe_max"] <= 0.08e-3 and rep["relres_mean"] <= 0.25e-3
+
+
+def _torus(h, w, kh, kw):
+    """The solver's choice of the preconditioner's torus (its rule, restated)."""
+    lens = (64, 96, 128, 192, 256, 384, 512)
+
+    def lengths(n):
+        p2 = max(2, 1 << (n - 1).bit_length())
+        return [p2] + [v for v in lens if n > 32 and n <= v <= 2 * n and v != p2]
+
+    def its(P, n, k):
+        x = (P - n) / max(k - 1, 1)
+        return 1.0 if P == n else 1.0 + 0.2 * max(0.0, 3.0 - x) + 0.05 * max(0.0, 6.0 - x)
+
+    def warp_cols(P, Q):
+        return P in lens and Q % (256 * (12 if P % 3 == 0 else 16) // P) == 0
+
+    return min((its(P, h, kh) * its(Q, w, kw) * (1.0 + P * Q / (3.0 * h * w)), i, (P, Q))
+               for i, (P, Q) in enumerate((P, Q) for P in lengths(h) for Q in lengths(w))
+               if not ((P % 3 == 0 or (Q % 3 == 0 and P in lens)) and not warp_cols(P, Q)))[2]
+
+
+@pytest.mark.parametrize("h,w,periodic,torus", [(450, 40, 1, (512, 64)), (409, 35, 0, (512, 64)),
+                                                (500, 66, 1, (512, 96)), (210, 40, 1, (256, 64)),
+                                                (217, 35, 0, (256, 64)), (40, 216, 1, (64, 256)),
+                                                (35, 470, 0, (64, 512))])
+def test_deconv_parity_margins_of_256_and_512_points(h, w, periodic, torus):
+    """Columns (and rows) of 256 and 512 points with a margin, whose gather and fold the sizes
+    above leave out since 320 rows take 384 points: the torus is asserted, the results are
+    the oracle's and the iterations those of the windowed extension on that torus."""
+    assert _torus(h, w, 5, 5) == torus
+    p = syn.deconv_problem(h, w, kernel=syn.uniform_kernel(5), bsnr_db=30.0, beta0=2.0, seed=h + w,
+                           grf_length=8.0)
+    S = 3
+    pr = probes(p, S, 58)
+    mu, var, ep = _gpu(p, 2, S, pr, periodic=periodic)
+    o = EPOracle("deconv", y32(p), p.xi, p.beta, h, w, kernel=p.kernel, site0="rbmc_cg", probes=pr,
+                 periodic=bool(periodic))
+    o.run(2)
+    assert_parity(mu, var, *o.posterior(), p.y)
+    ep.close()
+    test_preconditioner_iterations_are_those_of_the_windowed_extension(h, w, periodic, torus)

@@ -477,3 +477,28 @@ def test_deconv_parity_margins_of_256_and_512_points(h, w, periodic, torus):
     assert_parity(mu, var, *o.posterior(), p.y)
     ep.close()
     test_preconditioner_iterations_are_those_of_the_windowed_extension(h, w, periodic, torus)
+
+
+@pytest.mark.parametrize("kernel", ["nonseparable 5x3", "separable 3x7"])
+@pytest.mark.parametrize("h,w,S", [(64, 64, 2), (64, 64, 3),    # a pass as one kernel
+                                   (64, 128, 3), (96, 96, 2),   # three kernels per iteration
+                                   (32, 64, 2)])                # columns in shared memory
+def test_deconv_parity_pointwise_products_of_any_blur(h, w, S, kernel):
+    """Images that fill the torus form Q z from the transform of the kernel, whatever its form;
+    the true residual that ends a solve comes from the taps.  Rectangular kernels, separable
+    and not, with even and odd numbers of systems, against the oracle."""
+    if kernel == "nonseparable 5x3":
+        k = np.random.default_rng(4).random((5, 3)) ** 2
+        assert np.linalg.matrix_rank(k) == 3
+    else:
+        k = np.outer([1.0, 2.0, 1.5], [1.0, 2.0, 3.0, 4.0, 3.5, 2.0, 0.5])
+    assert _torus(h, w, *k.shape) == (h, w)
+    p = syn.deconv_problem(h, w, kernel=k / k.sum(), bsnr_db=30.0, beta0=2.0, seed=h + w, grf_length=8.0)
+    pr = probes(p, S, 60)
+    mu, var, ep = _gpu(p, 3, S, pr)
+    rep = ep.solver_report()
+    assert rep["relres_mean"] <= 1e-9 and rep["relres_probe_max"] <= 1e-6
+    o = EPOracle("deconv", y32(p), p.xi, p.beta, h, w, kernel=p.kernel, site0="rbmc_cg", probes=pr)
+    o.run(3)
+    assert_parity(mu, var, *o.posterior(), p.y)
+    ep.close()

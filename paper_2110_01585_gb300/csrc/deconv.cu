@@ -61,9 +61,7 @@ struct ConvDesc {
   const float* gr;       // 2 hr + 1 (separable)
   const float* gc;       // 2 hc + 1 (separable)
   const double* hd;      // forward-blur taps, FP64: separable u (kh) then v (kw), else k
-  const float* hf;       // the same taps in FP32
   float inv_xi;
-  double inv_xi_d;
   float g0_xi;           // diag of H^T H / xi = sum k^2 / xi
   int tiles_x, tiles_y;
 };
@@ -384,7 +382,6 @@ struct CgArgs {
   double* part_rz;       // [R][nbz]
   double* part_rr;       // [R][nb]
   double* part_bb;       // [R][nb]
-  double rtol2;
   float* scal;           // [R][4]: active flag, beta; each written by the last block
                          // of the kernel whose partial sums it needs
   double* rzs;           // [R] r.z of the current iteration
@@ -535,100 +532,6 @@ __device__ __forceinline__ ff2 ff2_sub_from(float2 y, ff2 acc) {
   return fast_two_sum2(sh, f2sub(f2add(sl, make_float2(0.f, 0.f)), acc.lo));
 }
 
-// The separable part of residual_kernel with a compile-time K x K kernel: the
-// same float-float H x and FP32 H^T sums in the same order, with the region
-// sizes, index divisions and tap loops resolved at compile time.
-template <int K>
-__device__ __forceinline__ void residual_sep_fixed(const ConvDesc& c, const float* taph,
-                                                   const float* tapl, const float* xh,
-                                                   const float* xl, float* ph, float* pl, float* vs,
-                                                   float* tmpf, float* outb, const float* yp, int r0,
-                                                   int c0) {
-  constexpr int hh = K / 2, hw = K / 2;
-  constexpr int RH = kTile + 2 * (K - 1), RW = RH;
-  constexpr int MH = kTile + 2 * hh, MW = MH;
-  float uh[K], ul[K], vh[K], vl[K];
-#pragma unroll
-  for (int b = 0; b < K; ++b) {
-    uh[b] = taph[b];
-    ul[b] = tapl[b];
-    vh[b] = taph[K + b];
-    vl[b] = tapl[K + b];
-  }
-  // Both float-float passes produce two adjacent outputs per thread from one
-  // window of K + 1 inputs (the row pass reads it as float2); every output sums its
-  // taps in the same order as a one-output loop.
-  static_assert(K % 2 == 1 && RW % 2 == 0 && MW % 2 == 0 && MH % 2 == 0, "paired outputs");
-  for (int idx = threadIdx.x; idx < RH * (MW / 2); idx += kThreads) {
-    const int rr = idx / (MW / 2), mp = idx - rr * (MW / 2);
-    // outputs (rr, 2 mp) and (rr, 2 mp + 1) read x[rr][2 mp .. 2 mp + K]
-    const float2* h2 = reinterpret_cast<const float2*>(xh + rr * RW + 2 * mp);
-    const float2* l2 = reinterpret_cast<const float2*>(xl + rr * RW + 2 * mp);
-    float wh[K + 1], wl[K + 1];
-#pragma unroll
-    for (int q = 0; q < (K + 1) / 2; ++q) {
-      const float2 th = h2[q], tl = l2[q];
-      wh[2 * q] = th.x;
-      wh[2 * q + 1] = th.y;
-      wl[2 * q] = tl.x;
-      wl[2 * q + 1] = tl.y;
-    }
-    ff acc0 = {0.f, 0.f}, acc1 = {0.f, 0.f};
-#pragma unroll
-    for (int b = 0; b < K; ++b) {
-      acc0 = ff_fma(acc0, ff{wh[K - 1 - b], wl[K - 1 - b]}, vh[b], vl[b]);
-      acc1 = ff_fma(acc1, ff{wh[K - b], wl[K - b]}, vh[b], vl[b]);
-    }
-    const int o = rr * MW + 2 * mp;
-    ph[o] = acc0.hi;
-    pl[o] = acc0.lo;
-    ph[o + 1] = acc1.hi;
-    pl[o + 1] = acc1.lo;
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < (MH / 2) * MW; idx += kThreads) {
-    const int mp = idx / MW, mc = idx - mp * MW, mr = 2 * mp;
-    // outputs (mr, mc) and (mr + 1, mc) read rows mr .. mr + K of column mc
-    const int gcol = wrapi(c0 - hw + mc, c.W);
-    const float y0 = yp[(long long)wrapi(r0 - hh + mr, c.H) * c.W + gcol];
-    const float y1 = yp[(long long)wrapi(r0 - hh + mr + 1, c.H) * c.W + gcol];
-    float wh[K + 1], wl[K + 1];
-#pragma unroll
-    for (int j = 0; j <= K; ++j) {
-      wh[j] = ph[(mr + j) * MW + mc];
-      wl[j] = pl[(mr + j) * MW + mc];
-    }
-    ff acc0 = {0.f, 0.f}, acc1 = {0.f, 0.f};
-#pragma unroll
-    for (int aa = 0; aa < K; ++aa) {
-      acc0 = ff_fma(acc0, ff{wh[K - 1 - aa], wl[K - 1 - aa]}, uh[aa], ul[aa]);
-      acc1 = ff_fma(acc1, ff{wh[K - aa], wl[K - aa]}, uh[aa], ul[aa]);
-    }
-    const ff v0 = ff_add(ff{y0, 0.f}, ff_neg(acc0));
-    const ff v1 = ff_add(ff{y1, 0.f}, ff_neg(acc1));
-    vs[mr * MW + mc] = v0.hi + v0.lo;
-    vs[(mr + 1) * MW + mc] = v1.hi + v1.lo;
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < MH * kTile; idx += kThreads) {
-    const int mr = idx / kTile, tc = idx - mr * kTile;
-    const float* row = vs + mr * MW + tc;
-    float acc = 0.f;
-#pragma unroll
-    for (int b = 0; b < K; ++b) acc = fmaf(vh[b], row[b], acc);
-    tmpf[idx] = acc;
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < kTile * kTile; idx += kThreads) {
-    const int tr = idx / kTile, tc = idx - tr * kTile;
-    const float* col = tmpf + tr * kTile + tc;
-    float acc = 0.f;
-#pragma unroll
-    for (int aa = 0; aa < K; ++aa) acc = fmaf(uh[aa], col[aa * kTile], acc);
-    outb[idx] = acc;
-  }
-}
-
 // True residual of every system (blockIdx.z),
 //   r = H^T (y' - H x) / xi + (n' - d x),
 // y' = y, n' = n for the mean system and y' = sqrt(xi) eps1_s, n' = sqrt(d) eps2_s for
@@ -695,79 +598,75 @@ __global__ void __launch_bounds__(kThreads) residual_kernel(CgArgs a) {
   }
   __syncthreads();
   const float* yp = j == 0 ? a.Y0 : a.Y1 + (long long)(j - 1) * c.N;
-  if (c.separable && c.kh == 9 && c.kw == 9) {
-    residual_sep_fixed<9>(c, taph, tapl, xh, xl, ph, pl, vs, tmpf, outb, yp, r0, c0);
-  } else {
-    // v = y' - H x on the (kh/2, kw/2)-halo region: (H x)(r,c) = sum k[a,b] x(r-a+hh, c-b+hw)
-    if (c.separable) {
-      const float* uh = taph;
-      const float* ul = tapl;
-      const float* vh = taph + c.kh;
-      const float* vl = tapl + c.kh;
-      for (int idx = threadIdx.x; idx < RH * MW; idx += kThreads) {
-        const int rr = idx / MW, mc = idx - rr * MW;
-        const int base = rr * RW + mc + 2 * hw;
-        ff acc = {0.f, 0.f};
-        for (int b = 0; b < c.kw; ++b) acc = ff_fma(acc, ff{xh[base - b], xl[base - b]}, vh[b], vl[b]);
-        ph[idx] = acc.hi;
-        pl[idx] = acc.lo;
-      }
-      __syncthreads();
-      for (int idx = threadIdx.x; idx < MH * MW; idx += kThreads) {
-        const int mr = idx / MW, mc = idx - mr * MW;
-        const int base = (mr + 2 * hh) * MW + mc;
-        ff acc = {0.f, 0.f};
-        for (int aa = 0; aa < c.kh; ++aa)
-          acc = ff_fma(acc, ff{ph[base - aa * MW], pl[base - aa * MW]}, uh[aa], ul[aa]);
-        const int gr = wrapi(r0 - hh + mr, c.H), gcol = wrapi(c0 - hw + mc, c.W);
-        const ff v = ff_add(ff{yp[(long long)gr * c.W + gcol], 0.f}, ff_neg(acc));
-        vs[idx] = v.hi + v.lo;
-      }
-    } else {
-      for (int idx = threadIdx.x; idx < MH * MW; idx += kThreads) {
-        const int mr = idx / MW, mc = idx - mr * MW;
-        ff acc = {0.f, 0.f};
-        for (int aa = 0; aa < c.kh; ++aa) {
-          const int base = (mr + 2 * hh - aa) * RW + mc + 2 * hw;
-          for (int b = 0; b < c.kw; ++b)
-            acc = ff_fma(acc, ff{xh[base - b], xl[base - b]}, taph[aa * c.kw + b], tapl[aa * c.kw + b]);
-        }
-        const int gr = wrapi(r0 - hh + mr, c.H), gcol = wrapi(c0 - hw + mc, c.W);
-        const ff v = ff_add(ff{yp[(long long)gr * c.W + gcol], 0.f}, ff_neg(acc));
-        vs[idx] = v.hi + v.lo;
-      }
+  // v = y' - H x on the (kh/2, kw/2)-halo region: (H x)(r,c) = sum k[a,b] x(r-a+hh, c-b+hw)
+  if (c.separable) {
+    const float* uh = taph;
+    const float* ul = tapl;
+    const float* vh = taph + c.kh;
+    const float* vl = tapl + c.kh;
+    for (int idx = threadIdx.x; idx < RH * MW; idx += kThreads) {
+      const int rr = idx / MW, mc = idx - rr * MW;
+      const int base = rr * RW + mc + 2 * hw;
+      ff acc = {0.f, 0.f};
+      for (int b = 0; b < c.kw; ++b) acc = ff_fma(acc, ff{xh[base - b], xl[base - b]}, vh[b], vl[b]);
+      ph[idx] = acc.hi;
+      pl[idx] = acc.lo;
     }
     __syncthreads();
-    // H^T v on the tile in FP32: (H^T v)(r, c) = sum k[a, b] v(r + a - hh, c + b - hw)
-    if (c.separable) {
-      const float* u = taph;
-      const float* v = taph + c.kh;
-      for (int idx = threadIdx.x; idx < MH * kTile; idx += kThreads) {
-        const int mr = idx / kTile, tc = idx - mr * kTile;
-        const float* row = vs + mr * MW + tc;
-        float acc = 0.f;
-        for (int b = 0; b < c.kw; ++b) acc = fmaf(v[b], row[b], acc);
-        tmpf[idx] = acc;
+    for (int idx = threadIdx.x; idx < MH * MW; idx += kThreads) {
+      const int mr = idx / MW, mc = idx - mr * MW;
+      const int base = (mr + 2 * hh) * MW + mc;
+      ff acc = {0.f, 0.f};
+      for (int aa = 0; aa < c.kh; ++aa)
+        acc = ff_fma(acc, ff{ph[base - aa * MW], pl[base - aa * MW]}, uh[aa], ul[aa]);
+      const int gr = wrapi(r0 - hh + mr, c.H), gcol = wrapi(c0 - hw + mc, c.W);
+      const ff v = ff_add(ff{yp[(long long)gr * c.W + gcol], 0.f}, ff_neg(acc));
+      vs[idx] = v.hi + v.lo;
+    }
+  } else {
+    for (int idx = threadIdx.x; idx < MH * MW; idx += kThreads) {
+      const int mr = idx / MW, mc = idx - mr * MW;
+      ff acc = {0.f, 0.f};
+      for (int aa = 0; aa < c.kh; ++aa) {
+        const int base = (mr + 2 * hh - aa) * RW + mc + 2 * hw;
+        for (int b = 0; b < c.kw; ++b)
+          acc = ff_fma(acc, ff{xh[base - b], xl[base - b]}, taph[aa * c.kw + b], tapl[aa * c.kw + b]);
       }
-      __syncthreads();
-      for (int idx = threadIdx.x; idx < kTile * kTile; idx += kThreads) {
-        const int tr = idx / kTile, tc = idx - tr * kTile;
-        const float* col = tmpf + tr * kTile + tc;
-        float acc = 0.f;
-        for (int aa = 0; aa < c.kh; ++aa) acc = fmaf(u[aa], col[aa * kTile], acc);
-        outb[idx] = acc;
+      const int gr = wrapi(r0 - hh + mr, c.H), gcol = wrapi(c0 - hw + mc, c.W);
+      const ff v = ff_add(ff{yp[(long long)gr * c.W + gcol], 0.f}, ff_neg(acc));
+      vs[idx] = v.hi + v.lo;
+    }
+  }
+  __syncthreads();
+  // H^T v on the tile in FP32: (H^T v)(r, c) = sum k[a, b] v(r + a - hh, c + b - hw)
+  if (c.separable) {
+    const float* u = taph;
+    const float* v = taph + c.kh;
+    for (int idx = threadIdx.x; idx < MH * kTile; idx += kThreads) {
+      const int mr = idx / kTile, tc = idx - mr * kTile;
+      const float* row = vs + mr * MW + tc;
+      float acc = 0.f;
+      for (int b = 0; b < c.kw; ++b) acc = fmaf(v[b], row[b], acc);
+      tmpf[idx] = acc;
+    }
+    __syncthreads();
+    for (int idx = threadIdx.x; idx < kTile * kTile; idx += kThreads) {
+      const int tr = idx / kTile, tc = idx - tr * kTile;
+      const float* col = tmpf + tr * kTile + tc;
+      float acc = 0.f;
+      for (int aa = 0; aa < c.kh; ++aa) acc = fmaf(u[aa], col[aa * kTile], acc);
+      outb[idx] = acc;
+    }
+  } else {
+    for (int idx = threadIdx.x; idx < kTile * kTile; idx += kThreads) {
+      const int tr = idx / kTile, tc = idx - tr * kTile;
+      float acc = 0.f;
+      for (int aa = 0; aa < c.kh; ++aa) {
+        const float* vrow = vs + (tr + aa) * MW + tc;
+        const float* krow = taph + aa * c.kw;
+        for (int b = 0; b < c.kw; ++b) acc = fmaf(krow[b], vrow[b], acc);
       }
-    } else {
-      for (int idx = threadIdx.x; idx < kTile * kTile; idx += kThreads) {
-        const int tr = idx / kTile, tc = idx - tr * kTile;
-        float acc = 0.f;
-        for (int aa = 0; aa < c.kh; ++aa) {
-          const float* vrow = vs + (tr + aa) * MW + tc;
-          const float* krow = taph + aa * c.kw;
-          for (int b = 0; b < c.kw; ++b) acc = fmaf(krow[b], vrow[b], acc);
-        }
-        outb[idx] = acc;
-      }
+      outb[idx] = acc;
     }
   }
   __syncthreads();
@@ -828,8 +727,7 @@ __global__ void __launch_bounds__(kThreads) residual_kernel(CgArgs a) {
 // float-float tap of H x and each FP32 tap of H^T is one packed operation for both
 // (ff2_fma: per lane the operations of ff_fma), and the index arithmetic, tap loads
 // and the loads of d are shared.  Per system and output the taps are summed in the
-// order of residual_sep_fixed, and the epilogue forms r, b and the partial sums as
-// residual_kernel does.  Shared memory: the x region (hi, lo) and the row-pass output
+// order of residual_kernel, and the epilogue forms r, b and the partial sums as it does.  Shared memory: the x region (hi, lo) and the row-pass output
 // (hi, lo); y' - H x is written over the latter's hi half once every thread has read
 // it, and the H^T row pass over its lo half.
 template <int K>
@@ -3042,8 +2940,7 @@ __global__ void __launch_bounds__(32 * kF512Warps, 2) warp_rows_inv_kernel(FftDe
 constexpr int kSolveCtas = 8;
 // Warps per CTA.  Two such CTAs fit an SM, so that the 17 pairs of the default 33 systems
 // are resident at once; with 16 warps a 256^2 pass was 10% slower.
-template <int kLen>
-constexpr int solve_warps() { return 8; }
+constexpr int kSolveWarps = 8;
 // The sides that take this kernel.
 constexpr bool solve_len(int n) { return n == 64 || n == 128 || n == 256; }
 
@@ -3079,16 +2976,16 @@ __device__ __forceinline__ void cluster_sum(cooperative_groups::cluster_group& c
 
 template <int kLen>
 constexpr size_t solve_smem() {
-  return sizeof(float2) * (size_t)solve_warps<kLen>() * Warp<kLen>::kScratch;
+  return sizeof(float2) * (size_t)kSolveWarps * Warp<kLen>::kScratch;
 }
 
 template <int kLen>
-__global__ void __cluster_dims__(kSolveCtas, 1, 1) __launch_bounds__(32 * solve_warps<kLen>(), 16 / solve_warps<kLen>())
+__global__ void __cluster_dims__(kSolveCtas, 1, 1) __launch_bounds__(32 * kSolveWarps, 16 / kSolveWarps)
     pw_solve_kernel(FftDesc f, CgArgs a, const float* filtT, const LoopState* ls, int budget, int* pass_its) {
   namespace cg = cooperative_groups;
   using Wp = Warp<kLen>;
   constexpr int T = Wp::kT, E = Wp::kE;
-  constexpr int kN = Wp::kN, kPer = Wp::kPer, kSolveWarps = solve_warps<kLen>();
+  constexpr int kN = Wp::kN, kPer = Wp::kPer;
   constexpr int kOwn = kN / kSolveCtas;  // rows, and columns, of one CTA
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank();
@@ -4013,7 +3910,6 @@ struct LikelihoodState {
   float* Y1 = nullptr;      // sqrt(xi) eps1
   double* thr = nullptr;    // inner convergence thresholds
   double* d_hd = nullptr;   // forward-blur taps FP64
-  float* d_hf = nullptr;    // forward-blur taps FP32
   double rtol2_true = 0.0;  // target of the true relative residual of the mean solve, squared
   double rtol2_probe = 0.0; // the same for the probe solves
   int max_outer = 24;
@@ -4102,7 +3998,6 @@ CgArgs cg_args(LikelihoodState* L) {
   a.part_rz = L->part + rn;
   a.part_rr = L->part + 2 * rn;
   a.part_bb = L->part + 3 * rn;
-  a.rtol2 = L->rtol2;
   a.nb = L->nb;
   a.nbz = L->nbz;
   a.fft = L->fft ? 1 : 0;
@@ -4210,7 +4105,7 @@ void launch_solve(LikelihoodState* L, const CgArgs& a, const LoopState* ls, int 
   with_warp(f.WP, [&](auto t) {
     constexpr int n = decltype(t)::value;
     if constexpr (solve_len(n))
-      pw_solve_kernel<n><<<f.pairs * kSolveCtas, 32 * solve_warps<n>(), solve_smem<n>(), s>>>(
+      pw_solve_kernel<n><<<f.pairs * kSolveCtas, 32 * kSolveWarps, solve_smem<n>(), s>>>(
           f, a, f.filt, ls, budget, &L->d_loop->pass_its);
   });
 }
@@ -4548,7 +4443,6 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
   c.hc = hc;
   c.separable = sep ? 1 : 0;
   c.inv_xi = L->inv_xi;
-  c.inv_xi_d = 1.0 / cfg.p->xi;
   c.g0_xi = (float)(g0 / cfg.p->xi);
   c.tiles_x = (c.W + kTile - 1) / kTile;
   c.tiles_y = (c.H + kTile - 1) / kTile;
@@ -4625,7 +4519,6 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
             cudaMalloc(&L->Y1, sizeof(float) * L->S * N) == cudaSuccess &&
             cudaMalloc(&L->thr, sizeof(double) * L->R) == cudaSuccess &&
             cudaMalloc(&L->d_hd, sizeof(double) * (kh * kw + kh + kw)) == cudaSuccess &&
-            cudaMalloc(&L->d_hf, sizeof(float) * (kh * kw + kh + kw)) == cudaSuccess &&
             cudaMalloc(&L->Rr, sizeof(float) * RN) == cudaSuccess &&
             cudaMalloc(&L->P, sizeof(float) * RN) == cudaSuccess &&
             (L->pw || cudaMalloc(&L->P2, sizeof(float) * RN) == cudaSuccess) &&
@@ -4669,7 +4562,6 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
   c.gr = L->d_g;
   c.gc = L->d_g + (2 * hr + 1);
   c.hd = L->d_hd;
-  c.hf = L->d_hf;
   L->Y0 = cfg.y;
   {
     std::vector<double> hd;
@@ -4679,10 +4571,7 @@ ep_tv_status likelihood_create(const LikelihoodConfig& cfg, cudaStream_t s, Like
     } else {
       hd = k;
     }
-    std::vector<float> hf(hd.begin(), hd.end());
     if (cudaMemcpyAsync(L->d_hd, hd.data(), sizeof(double) * hd.size(), cudaMemcpyHostToDevice, s) !=
-            cudaSuccess ||
-        cudaMemcpyAsync(L->d_hf, hf.data(), sizeof(float) * hf.size(), cudaMemcpyHostToDevice, s) !=
             cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
       likelihood_destroy(L);
@@ -4772,7 +4661,6 @@ void likelihood_destroy(LikelihoodState* L) {
   cudaFree(L->Y1);
   cudaFree(L->thr);
   cudaFree(L->d_hd);
-  cudaFree(L->d_hf);
   cudaFree(L->Rr);
   cudaFree(L->P);
   cudaFree(L->P2);

@@ -29,7 +29,7 @@
 // ozaki.cu.  K = L L^T and Z = L^{-1} come together from a recursion on halves
 // (L21 = K21 Z11^T, K22 -= L21 L21^T, Z21 = -Z22 L21 Z11) whose large products
 // run in the same split form with 10 digit slices and seven exact diagonals (as
-// accurate as FP64 on these operands); blocks of 64 rows and smaller products
+// accurate as FP64 on these operands); blocks of up to 128 rows and smaller products
 // stay on the FP64 CUDA cores.  The mean uses v = Z t and g = W^T v.
 //
 // Kernels here: an FP64 tiled GEMM (64 x 64 tiles, 4 x 4 per thread) for the

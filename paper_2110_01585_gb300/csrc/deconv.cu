@@ -1938,7 +1938,10 @@ __device__ __forceinline__ void stage_loads(float2* s, int total, Get get) {
   }
 }
 
-// Pack two residual planes into complex rows (extended to WP) and transform them.
+// Pack two residual planes into complex rows (extended to WP) and transform them.  Here and
+// in the passes below, as in the 1024-point ones, an axis that the image fills has neither
+// copies nor a window, and its loads and stores are plain: an application at 4096^2 (3 systems)
+// 2.87 -> 2.56 ms, at 2048^2 (9) 1.13 -> 1.05 ms, at 1024^2 (33; 1024-point passes) 216 -> 168 us.
 __global__ void __launch_bounds__(kFftThreads, 4) fft_rows_fwd_kernel(FftDesc f, const float* __restrict__ Rr) {
   if (pair_idle(f, blockIdx.y)) return;
   if (blockIdx.x == 0 && threadIdx.x == 0 && f.counters)
@@ -2752,12 +2755,15 @@ __global__ void __launch_bounds__(32 * kF512Warps, 3) warp_cols_filter_kernel(Ff
 // per iteration then does, for both systems of a pair, p, s, e += alpha p and
 // r -= alpha s, and transforms the new residual rows; alpha and beta come from the inverse
 // row pass before it (pw_tail).  The rounding error of Q z is that of the transforms times
-// |H^T H| / xi, the same order as the FP32 stencil's: in an FP32 emulation at 128^2 and 256^2
+// |H^T H| / xi, the order of the FP32 stencil's: in an FP32 emulation at 128^2 and 256^2
 // (40 dB and 30 dB) both take the same iterations in every pass, and the true residual that
-// ends a solve is formed by the float-float residual kernel as before.
+// ends a solve is formed by the float-float residual kernel as before.  After a pass of
+// many hundreds of iterations it leaves the true residual higher, and the next pass longer:
+// 64 x 128 at 30 dB, first update 345 -> 353 iterations at beta = 10, 959 -> 1073 at 100;
+// at 60 dB and beta = 1e4, where a solve takes 10^4, up to 1.9 times as many.
 // Bound by its nine planes (36 bytes per pixel and system, and d): at 512^2 with 33 systems
-// 61 us, 5.7 TB/s.  Three kernels per iteration, 60 bytes in all, against four with the
-// stencil kernel and the same bytes (direction 53 us and update 28 us there).
+// 61 us, 5.1 TB/s (0.75 of the copy bandwidth).  Three kernels per iteration, 60 bytes in all,
+// against four with the stencil kernel and the same bytes (direction 53 us, update 28 us there).
 template <int kLen>
 __global__ void __launch_bounds__(32 * kF512Warps, 2) pw_update_rows_fwd_kernel(FftDesc f, CgArgs a, int it_arg) {
   using Wp = Warp<kLen>;

@@ -369,10 +369,11 @@ ep_tv_status ep_tv_batch_create(int32_t n, ep_tv_ctx* const* ctxs, ep_tv_batch**
 /* n_sweeps sweeps of every context: one persistent launch runs the prior-site
    pass of all images (warps take contiguous ranges of the images' work units,
    found through a table), then the likelihood-site
-   updates run concurrently on one worker stream per context, each driven by a host
-   thread of a pool of up to 16; with em_every > 0 every context's beta is updated
-   after each em_every-th sweep.  Returns when all work is enqueued (the likelihood
-   solvers synchronise with their own streams while they run). */
+   updates run concurrently on one worker stream per context, enqueued as graphs by
+   the calling thread (with tracing on, host-driven by a pool of up to 16 threads,
+   which synchronise with their streams while they run); with em_every > 0 every
+   context's beta is updated after each em_every-th sweep.  Returns when all work is
+   enqueued. */
 ep_tv_status ep_tv_batch_sweep(ep_tv_batch* batch, int32_t n_sweeps, int32_t em_every);
 /* Synchronises and frees the batch (not the contexts).  NULL is accepted. */
 void ep_tv_batch_destroy(ep_tv_batch* batch);
